@@ -22,10 +22,9 @@
 //                           running counts).
 //   k_permute               particles in tree order (sources, permutation,
 //                           grid coordinates).
-//   k_expand_count / k_expand_write  one level of cells from the previous one:
-//                           a cell with more than leaf_size particles (above
-//                           the last grid level) splits into the runs of its
-//                           particles' next key digit, found by binary search.
+//   k_levels / k_cells / k_links  every cell of every level at once, from the
+//                           number of key digits that neighbouring particles
+//                           share.
 //   k_moments               leaves sum their particles (all leaves in one
 //                           launch), then parents combine their children, one
 //                           level per launch, deepest first.
@@ -310,108 +309,223 @@ struct Cells {
     int32_t* nchild;
 };
 
-// The levels' first cells live on the device (lev[L] = first cell of level
-// L, lev[L + 1] = one past its last), so that a level is expanded without the
-// host reading its size: each kernel reads the bounds and runs a grid-stride
-// loop over 8 threads per cell (whole blocks per round, so that the
-// 8-lane shuffles and the ballots see every lane).  stop != 0 (the cell
-// capacity ran out) makes the rest of the expansion return at once.
+// All cells at once from the sorted keys, with no loop over levels.  With
+// cd(i, j) the number of leading key digits (levels) that particles i and j
+// share, the cell at level L that holds particle b has more than leaf_size
+// particles exactly when some window of leaf_size + 1 consecutive particles
+// that contains b shares L digits.  So the deepest cell that holds b, its
+// leaf, is at level
+//   D(b) = min(21, 1 + max over i in [b - leaf_size, b] of cd(i, i + leaf_size))
+// (0 when there is no such window), and the cells whose first particle is b
+// are those of levels cd(b - 1, b) + 1 .. D(b) (from level 0 for b = 0).
+// Cells are numbered by (level, first particle), which keeps a cell's
+// children consecutive: a cell's index is the start of its level plus the
+// number of cells of that level that start before it.
+//
+//   k_levels   both levels of every particle and, per tile, how many cells of
+//              each level start in it
+//   (scan)     counts in (level, tile) order: where each tile's cells of each
+//              level go; the last sum is the number of cells
+//   k_cells    the cells of a tile, ranked per level by warp ballots
+//   k_links    children and end of every cell
+//
+// Four to six launches, bound by their latency at small N and by the keys and
+// cell arrays they read and write at large N; expanding one level after
+// another took five launches per level for 22 possible levels, most of them
+// over few cells.  Device time of the two forms (Plummer, Hernquist at 2^23;
+// sums of launches under ncu): N = 4096 0.031 against 0.372 ms, 2^20 0.049
+// against 0.501 ms, 2^23 0.19 against 0.73 ms.
 
-// Thread (c, d): the start of the run of next-level digit >= d inside cell
-// c = lo + t / 8 (a split cell's keys are sorted and share the cell's prefix,
-// so its next digit does not decrease along the cell).  cnt[c - lo] = number
-// of non-empty runs (children); starts go to dig[(c - lo) * 8 + d].
-__global__ void k_expand_count(const int32_t* __restrict__ lev, int L, int leaf_size,
-                               const uint64_t* __restrict__ keys, Cells c, int32_t* __restrict__ dig,
-                               int32_t* __restrict__ cnt, const uint32_t* __restrict__ stop)
+constexpr int kLvTile = kRsTile;      // particles per block, in contiguous runs per warp
+constexpr int kLvRounds = kLvTile / kRsThreads;
+constexpr int kLvLeaf = 64;           // leaf sizes up to this take the window maximum in shared memory
+constexpr int kLv = kLevels + 1;      // levels 0 .. 21
+
+// Leading digits two keys share (21 for equal keys; bit 63 of a key is 0).
+__device__ __forceinline__ int common_digits(uint64_t a, uint64_t b)
 {
-    if (*stop) return;
-    const int32_t lo = lev[L], hi = lev[L + 1];
-    const int64_t nt = 8 * (int64_t)(hi - lo);
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nt; base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = base + threadIdx.x;
-        const int32_t cell = lo + (int32_t)(t >> 3);
-        const int d = (int)(t & 7);
-        const bool in = t < nt;
-        int32_t b = 0, e = 0;
-        bool split = false;
-        if (in) {
-            b = c.begin[cell];
-            e = c.end[cell];
-            split = e - b > leaf_size && L < kLevels;
+    const uint64_t x = a ^ b;
+    return x ? (__clzll((long long)x) - 1) / 3 : kLevels;
+}
+
+// Windows for leaf sizes above kLvLeaf, in global memory, padded in front by
+// leaf_size zeros: win[j] = 1 + cd(i, i + leaf) for i = j - leaf in [0, n -
+// leaf), else 0; then maxima over runs of 2, 4, ... windows by doubling.
+__global__ void k_win_init(const uint64_t* __restrict__ keys, int64_t n, int64_t leaf, uint8_t* __restrict__ win)
+{
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n + leaf) return;
+    const int64_t i = j - leaf;
+    win[j] = i >= 0 && i + leaf < n ? (uint8_t)(1 + common_digits(keys[i], keys[i + leaf])) : (uint8_t)0;
+}
+
+__global__ void k_win_double(const uint8_t* __restrict__ in, int64_t len, int64_t step, uint8_t* __restrict__ out)
+{
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= len) return;
+    const uint8_t a = in[j], b = j + step < len ? in[j + step] : (uint8_t)0;
+    out[j] = a > b ? a : b;
+}
+
+// lv[b] = lo | D << 8, lo the level of the first cell that starts at b (above
+// D when none does); hist[L * gridDim.x + blk]: cells of level L that start in
+// the tile.  win: NULL for leaf <= kLvLeaf, else the maxima over runs of span
+// windows (span the largest power of two <= leaf + 1).
+__global__ void __launch_bounds__(kRsThreads) k_levels(const uint64_t* __restrict__ keys, int64_t n, int64_t leaf,
+                                                        const uint8_t* __restrict__ win, int64_t span,
+                                                        uint16_t* __restrict__ lv, int32_t* __restrict__ hist)
+{
+    __shared__ uint64_t sk[kLvTile + 2 * kLvLeaf];
+    __shared__ uint8_t sw[kLvTile + kLvLeaf];
+    __shared__ int32_t wcnt[kRsWarps][kLv];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t t0 = (int64_t)blockIdx.x * kLvTile;
+    const int halo = win ? 1 : (int)leaf;  // keys staged before and after the tile
+    for (int j = threadIdx.x; j < kLvTile + 2 * halo; j += kRsThreads) {
+        const int64_t i = t0 - halo + j;
+        sk[j] = i >= 0 && i < n ? keys[i] : 0;
+    }
+    __syncthreads();
+    if (!win) {
+        for (int j = threadIdx.x; j < kLvTile + halo; j += kRsThreads) {
+            const int64_t i = t0 - halo + j;  // window [i, i + leaf]
+            sw[j] = i >= 0 && i + halo < n ? (uint8_t)(1 + common_digits(sk[j], sk[j + halo])) : (uint8_t)0;
         }
-        int32_t start = e;
-        if (split) {
-            const int shift = 3 * (kLevels - 1 - L);
-            int32_t l = b, r = e;  // first index in [b, e) with digit >= d
-            while (l < r) {
-                const int32_t m = l + ((r - l) >> 1);
-                if ((int)((keys[m] >> shift) & 7u) < d)
-                    l = m + 1;
-                else
-                    r = m;
+        __syncthreads();
+    }
+    int32_t mine = 0;  // lane L: cells of level L that start in the warp's run
+    for (int r = 0; r < kLvRounds; ++r) {
+        const int q = w * 32 * kLvRounds + r * 32 + lane;
+        const int64_t b = t0 + q;
+        int lo = kLv, dp = 0;
+        if (b < n) {
+            lo = b == 0 ? 0 : common_digits(sk[q + halo - 1], sk[q + halo]) + 1;
+            int m = 0;
+            if (win) {
+                const int m0 = win[b], m1 = win[b + leaf + 1 - span];
+                m = m0 > m1 ? m0 : m1;
+            } else {
+                for (int k = 0; k <= halo; ++k) m = sw[q + k] > m ? sw[q + k] : m;
             }
-            start = l;
+            dp = m < kLevels ? m : kLevels;
+            lv[b] = (uint16_t)(lo | (dp << 8));
         }
-        // run d is [start_d, start_{d+1}), start_8 = e
-        const int32_t next = __shfl_down_sync(kFull, start, 1, 8);
-        const int32_t nxt = d == 7 ? e : next;
-        const bool nonempty = split && start < nxt;
-        const unsigned m = __ballot_sync(kFull, nonempty);
-        if (in) {
-            dig[(int64_t)(cell - lo) * 8 + d] = start;
-            if (d == 0) cnt[cell - lo] = __popc((m >> (threadIdx.x & 24)) & 0xffu);
+        const bool any = lo <= dp && b < n;
+        const int l0 = __reduce_min_sync(kFull, any ? lo : kLv), l1 = __reduce_max_sync(kFull, any ? dp : -1);
+        for (int L = l0; L <= l1; ++L) {
+            const int c = __popc(__ballot_sync(kFull, any && lo <= L && L <= dp));
+            if (lane == L) mine += c;
+        }
+    }
+    if (lane < kLv) wcnt[w][lane] = mine;
+    __syncthreads();
+    if (threadIdx.x < kLv) {
+        int32_t c = 0;
+        for (int k = 0; k < kRsWarps; ++k) c += wcnt[k][threadIdx.x];
+        hist[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = c;
+    }
+}
+
+// Writes the cells that start in the tile.  offs: the exclusive scan of
+// k_levels' counts, *total their sum; block 0 writes the levels' first cells
+// lev[0 .. 22].  More than cap cells: nothing is written and stop is set.
+__global__ void __launch_bounds__(kRsThreads) k_cells(int64_t n, const uint16_t* __restrict__ lv,
+                                                       const int32_t* __restrict__ offs,
+                                                       const int64_t* __restrict__ total, int64_t cap, Cells c,
+                                                       int32_t* __restrict__ lev, uint32_t* __restrict__ stop)
+{
+    __shared__ int32_t wcnt[kRsWarps][kLv];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    if (*total > cap) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) *stop = 1u;
+        return;
+    }
+    if (blockIdx.x == 0 && threadIdx.x <= kLv)
+        lev[threadIdx.x] = threadIdx.x < kLv ? offs[(int64_t)threadIdx.x * gridDim.x] : (int32_t)*total;
+    const int64_t t0 = (int64_t)blockIdx.x * kLvTile + (int64_t)w * 32 * kLvRounds;
+    uint16_t v[kLvRounds];
+    int32_t mine = 0;
+#pragma unroll
+    for (int r = 0; r < kLvRounds; ++r) {
+        const int64_t b = t0 + r * 32 + lane;
+        v[r] = b < n ? lv[b] : (uint16_t)kLv;
+        const int lo = v[r] & 255, dp = v[r] >> 8;
+        const bool any = lo <= dp;
+        const int l0 = __reduce_min_sync(kFull, any ? lo : kLv), l1 = __reduce_max_sync(kFull, any ? dp : -1);
+        for (int L = l0; L <= l1; ++L) {
+            const int k = __popc(__ballot_sync(kFull, any && lo <= L && L <= dp));
+            if (lane == L) mine += k;
+        }
+    }
+    if (lane < kLv) wcnt[w][lane] = mine;
+    __syncthreads();
+    // lane L: index of the next cell of level L
+    int32_t next = 0;
+    if (lane < kLv) {
+        next = offs[(int64_t)lane * gridDim.x + blockIdx.x];
+        for (int k = 0; k < w; ++k) next += wcnt[k][lane];
+    }
+#pragma unroll
+    for (int r = 0; r < kLvRounds; ++r) {
+        const int64_t b = t0 + r * 32 + lane;
+        const int lo = v[r] & 255, dp = v[r] >> 8;
+        const bool any = lo <= dp;
+        const int l0 = __reduce_min_sync(kFull, any ? lo : kLv), l1 = __reduce_max_sync(kFull, any ? dp : -1);
+        int32_t up = 0;    // the last cell of level L - 1 that starts at or before b
+        int32_t mine_up = -1;  // the cell of level L - 1 that starts at b
+        for (int L = l0 > 0 ? l0 - 1 : 0; L <= l1; ++L) {
+            const bool on = any && lo <= L && L <= dp;
+            const unsigned m = __ballot_sync(kFull, on);
+            const int32_t base = __shfl_sync(kFull, next, L);
+            const int32_t id = base + __popc(m & lt);
+            if (on) {
+                c.begin[id] = (int32_t)b;
+                c.level[id] = L;
+                c.parent[id] = L == 0 ? -1 : up;
+                if (L == dp) c.child0[id] = 0;
+                if (mine_up >= 0) c.child0[mine_up] = id;
+                mine_up = id;
+            }
+            up = base + __popc(m & lt) - (on ? 0 : 1);
+            if (lane == L) next += __popc(m);
         }
     }
 }
 
-// Writes level L + 1: the children of level L's cells at lev[L + 1] +
-// coff[c - lo] (coff: the exclusive scan of cnt, *total its sum), and
-// lev[L + 2].  Children past cap are not written and set stop.
-__global__ void k_expand_write(int32_t* __restrict__ lev, int L, Cells c, const int32_t* __restrict__ dig,
-                               const int32_t* __restrict__ coff, const int64_t* __restrict__ total, int64_t cap,
-                               uint32_t* __restrict__ stop)
+// Of every cell: its children, the consecutive cells from child0 on that name
+// it as their parent, and its end, the first particle past it (a galloping
+// search over the keys' leading digits; a cell that splits holds at least
+// leaf_size + 1 particles).  One thread per cell, so that the searches'
+// dependent loads overlap: inside k_cells, one round of a warp after another,
+// they made it 40 us at N = 4096 (10 and 9.5 us apart) and 250 us at 2^23 (69
+// and 43).
+__global__ void k_links(int32_t n_cell, const uint64_t* __restrict__ keys, int64_t n, int64_t leaf_size, Cells c)
 {
-    if (*stop) return;
-    const int32_t lo = lev[L], hi = lev[L + 1];
-    const int32_t next_base = hi;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const int64_t end = (int64_t)hi + *total;
-        lev[L + 2] = (int32_t)(end < cap ? end : cap);
-        if (end > cap) *stop = 1u;
+    const int32_t cell = blockIdx.x * blockDim.x + threadIdx.x;
+    if (cell >= n_cell) return;
+    int32_t k = 0;
+    const int32_t c0 = c.child0[cell];
+    if (c0 > 0)
+        while (k < 8 && c0 + k < n_cell && c.parent[c0 + k] == cell) ++k;
+    c.nchild[cell] = k;
+    const int64_t b = c.begin[cell];
+    const int sh = 3 * (kLevels - c.level[cell]);
+    const uint64_t pre = keys[b] >> sh;
+    int64_t l = k > 0 ? b + leaf_size : b, hi, step = 1;
+    for (hi = l + step; hi < n && (keys[hi] >> sh) == pre; hi = l + step) {
+        l = hi;
+        step *= 2;
     }
-    const int64_t nt = 8 * (int64_t)(hi - lo);
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nt; base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = base + threadIdx.x;
-        const int32_t cell = lo + (int32_t)(t >> 3);
-        const int d = (int)(t & 7);
-        const bool in = t < nt;
-        int32_t start = 0, e = 0;
-        if (in) {
-            start = dig[(int64_t)(cell - lo) * 8 + d];
-            e = c.end[cell];
-        }
-        const int32_t next = __shfl_down_sync(kFull, start, 1, 8);
-        const int32_t nxt = d == 7 ? e : next;
-        const bool nonempty = in && start < nxt;  // a cell that does not split has start = end for every digit
-        const unsigned m = __ballot_sync(kFull, nonempty);
-        const unsigned mine = (m >> (threadIdx.x & 24)) & 0xffu;
-        if (!in) continue;
-        const int32_t first = next_base + coff[cell - lo];
-        if (d == 0) {
-            c.child0[cell] = mine ? first : 0;
-            c.nchild[cell] = __popc(mine);
-        }
-        if (nonempty) {
-            const int64_t k = (int64_t)first + __popc(mine & ((1u << d) - 1u));
-            if (k < cap) {
-                c.begin[k] = start;
-                c.end[k] = nxt;
-                c.level[k] = L + 1;
-                c.parent[k] = cell;
-            }
-        }
+    if (hi > n) hi = n;
+    while (hi - l > 1) {
+        const int64_t mid = l + ((hi - l) >> 1);
+        if ((keys[mid] >> sh) == pre)
+            l = mid;
+        else
+            hi = mid;
     }
+    c.end[cell] = (int32_t)hi;
 }
 
 // ---- moments ------------------------------------------------------------------------
@@ -797,60 +911,43 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(int32_t* __restrict
         if (e_ != cudaSuccess) return set_error(OTOO_ECUDA, "%s: %s", #expr, cudaGetErrorString(e_));  \
     } while (0)
 
-// exclusive scan of a[0, n) in place; the total to *total (device)
-// The same three scans over a[0, n) with n = lev[L + 1] - lev[L] read on the
-// device: grid-stride over blocks of kScanThreads (whole blocks per round).
-__global__ void __launch_bounds__(kScanThreads) k_scan_sums_lev(const int32_t* __restrict__ a,
-                                                                 const int32_t* __restrict__ lev, int L,
-                                                                 int64_t* __restrict__ bsum)
+// One block: an exclusive scan of a[0, n) in place, four elements per thread
+// and round, the total to *total.  For arrays of up to 16 * kScanThreads
+// elements, where the three launches below (2.8 us each at least) cost more
+// than the serial rounds (3.4 us at n = 512, 7.8 us at 11264).
+__global__ void __launch_bounds__(kScanThreads) k_scan_one(int32_t* __restrict__ a, int64_t n,
+                                                            int64_t* __restrict__ total)
 {
-    __shared__ int64_t ws[33];
-    const int64_t n = lev[L + 1] - lev[L];
-    for (int64_t blk = blockIdx.x; blk * kScanThreads < n; blk += gridDim.x) {
-        const int64_t i = blk * kScanThreads + threadIdx.x;
-        int64_t tot;
-        block_excl_scan64(i < n ? a[i] : 0, ws, &tot);
-        if (threadIdx.x == 0) bsum[blk] = tot;
-    }
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_top_lev(int64_t* __restrict__ bsum,
-                                                                const int32_t* __restrict__ lev, int L,
-                                                                int64_t* __restrict__ total)
-{
-    const int64_t n = lev[L + 1] - lev[L];
-    const int64_t nblk = (n + kScanThreads - 1) / kScanThreads;
     __shared__ int64_t ws[33];
     int64_t carry = 0;
-    for (int64_t b0 = 0; b0 < nblk; b0 += kScanThreads) {
-        const int64_t i = b0 + threadIdx.x;
+    for (int64_t b0 = 0; b0 < n; b0 += 4 * kScanThreads) {
+        const int64_t i = b0 + 4 * (int64_t)threadIdx.x;
+        int32_t v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = i + k < n ? a[i + k] : 0;
         int64_t tot;
-        const int64_t e = block_excl_scan64(i < nblk ? bsum[i] : 0, ws, &tot);
-        if (i < nblk) bsum[i] = carry + e;
+        int64_t e = carry + block_excl_scan64((int64_t)v[0] + v[1] + v[2] + v[3], ws, &tot);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i + k < n) a[i + k] = (int32_t)e;
+            e += v[k];
+        }
         carry += tot;
     }
     if (threadIdx.x == 0) *total = carry;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply_lev(int32_t* __restrict__ a,
-                                                                  const int32_t* __restrict__ lev, int L,
-                                                                  const int64_t* __restrict__ bsum)
-{
-    __shared__ int64_t ws[33];
-    const int64_t n = lev[L + 1] - lev[L];
-    for (int64_t blk = blockIdx.x; blk * kScanThreads < n; blk += gridDim.x) {
-        const int64_t i = blk * kScanThreads + threadIdx.x;
-        int64_t tot;
-        const int64_t e = block_excl_scan64(i < n ? a[i] : 0, ws, &tot) + bsum[blk];
-        if (i < n) a[i] = (int32_t)e;
-    }
-}
-
+// exclusive scan of a[0, n) in place; the total to *total (device)
 int scan32(int32_t* a, int64_t n, int64_t* bsum, int64_t* total, cudaStream_t s)
 {
     const int64_t nblk = (n + kScanThreads - 1) / kScanThreads;
     if (nblk == 0) {
         CUDA_TRY(cudaMemsetAsync(total, 0, sizeof(int64_t), s));
+        return OTOO_OK;
+    }
+    if (n <= 16 * kScanThreads) {
+        k_scan_one<<<1, kScanThreads, 0, s>>>(a, n, total);
+        CUDA_TRY(cudaGetLastError());
         return OTOO_OK;
     }
     k_scan_sums<<<(unsigned)nblk, kScanThreads, 0, s>>>(a, n, bsum);
@@ -994,34 +1091,32 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     if (st & kTreeBadSort) return set_error(OTOO_EDEVICE, "otoo_devtree_build: sort produced an invalid order");
     const uint64_t* skeys = keys[cur];
 
-    // cells, level by level, the levels' bounds on the device (one read at
-    // the end instead of one per level)
-    const int32_t root[6] = {0, (int32_t)n, 0, -1, 0, 0};
-    for (int k = 0; k < 6; ++k) {
-        int32_t* arr = k == 0 ? c.begin : k == 1 ? c.end : k == 2 ? c.level : k == 3 ? c.parent : k == 4 ? c.child0 : c.nchild;
-        CUDA_TRY(cudaMemcpyAsync(arr, &root[k], sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    }
+    // cells; the unsorted copy of the keys is dead, its memory holds the
+    // particles' levels (2 n bytes) and the windows of large leaf sizes
+    // (2 (n + leaf_size) bytes, leaf_size < n)
     int32_t* lev = reinterpret_cast<int32_t*>(base + ly.lev);
     uint32_t* stop = reinterpret_cast<uint32_t*>(lev + kLevels + 4);
+    CUDA_TRY(cudaMemsetAsync(lev, 0, 4 * (kLevels + 4) + 4, s));
+    uint16_t* lv = reinterpret_cast<uint16_t*>(keys[cur ^ 1]);
+    const uint8_t* win = nullptr;
+    int64_t span = 1;
+    const int64_t leaf = std::min<int64_t>(t->leaf_size, n);
+    if (leaf > kLvLeaf) {
+        const int64_t len = n + leaf;
+        uint8_t* wb[2] = {reinterpret_cast<uint8_t*>(lv + n), reinterpret_cast<uint8_t*>(lv + n) + len};
+        const unsigned g = (unsigned)((len + 255) / 256);
+        k_win_init<<<g, 256, 0, s>>>(skeys, n, leaf, wb[0]);
+        int k = 0;
+        for (; 2 * span <= leaf + 1; span *= 2, k ^= 1) k_win_double<<<g, 256, 0, s>>>(wb[k], len, span, wb[k ^ 1]);
+        win = wb[k];
+    }
+    k_levels<<<nblk, kRsThreads, 0, s>>>(skeys, n, leaf, win, span, lv, hist);
+    CUDA_TRY(cudaGetLastError());
     {
-        static const int32_t lev01[2] = {0, 1};
-        CUDA_TRY(cudaMemsetAsync(lev, 0, 4 * (kLevels + 4) + 4, s));
-        CUDA_TRY(cudaMemcpyAsync(lev, lev01, sizeof(lev01), cudaMemcpyHostToDevice, s));
+        const int r = scan32(hist, (int64_t)kLv * nblk, bsum, tot, s);
+        if (r) return r;
     }
-    int dev = 0, sms = 0;
-    CUDA_TRY(cudaGetDevice(&dev));
-    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // grid-stride rounds: enough blocks to fill the GPU, no more than the
-    // widest level could use (8 threads per cell, at most cap cells)
-    const unsigned eg = (unsigned)std::min<int64_t>((int64_t)sms * 8, (8 * cap + 255) / 256);
-    const unsigned sg = (unsigned)std::min<int64_t>((int64_t)sms * 2, (cap + kScanThreads - 1) / kScanThreads);
-    for (int L = 0; L <= kLevels; ++L) {
-        k_expand_count<<<eg, 256, 0, s>>>(lev, L, t->leaf_size, skeys, c, dig, cnt, stop);
-        k_scan_sums_lev<<<sg, kScanThreads, 0, s>>>(cnt, lev, L, bsum);
-        k_scan_top_lev<<<1, kScanThreads, 0, s>>>(bsum, lev, L, tot);
-        k_scan_apply_lev<<<sg, kScanThreads, 0, s>>>(cnt, lev, L, bsum);
-        k_expand_write<<<eg, 256, 0, s>>>(lev, L, c, dig, cnt, tot, cap, stop);
-    }
+    k_cells<<<nblk, kRsThreads, 0, s>>>(n, lv, hist, tot, cap, c, lev, stop);
     CUDA_TRY(cudaGetLastError());
     int32_t hlev[kLevels + 4];
     uint32_t hstop = 0;
@@ -1040,6 +1135,7 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     lev_lo.resize(depth + 2);
     const int32_t n_cell = lev_lo.back();
 
+    k_links<<<(unsigned)((n_cell + 127) / 128), 128, 0, s>>>(n_cell, skeys, n, leaf, c);
     // moments: every leaf in one launch, then the parents level by level,
     // deepest first
     k_moments<<<(unsigned)((n_cell + 127) / 128), 128, 0, s>>>(0, n_cell, t->src, c, mo, 1);

@@ -1,0 +1,32 @@
+"""The device tree at the edges of its kernels' tiles and leaf-size paths,
+against the host build (needs a GPU): bit-exact order, cells and groups,
+moments to rounding (check_tree of test_gpu_tree.py)."""
+import numpy as np
+import pytest
+
+from paper_1206_1199_gb300 import _lib as L
+from paper_1206_1199_gb300 import ic
+from test_gpu_tree import check_tree
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    return L.load()
+
+
+@pytest.mark.parametrize("n", [2, 31, 33, 2047, 2048, 2049, 4097])
+@pytest.mark.parametrize("leaf", [1, 8, 64, 65, 127, 300, 5000])
+def test_cells_at_tile_and_leaf_edges(n, leaf):
+    pos, mass = ic.hernquist(n, 61)
+    check_tree(pos, mass, leaf, 16 if leaf < 16 else 64)
+
+
+@pytest.mark.parametrize("leaf", [1, 8, 64, 100])
+def test_cells_of_coincident_and_lattice_particles(leaf):
+    # runs of equal keys longer than a tile, next to a lattice whose cell
+    # faces coincide with particle positions
+    g = np.stack(np.meshgrid(*[np.arange(8) / 8.0] * 3, indexing="ij"), -1).reshape(-1, 3)
+    pos = np.concatenate([g, np.full((2500, 3), 0.1), np.full((70, 3), 0.7)])
+    check_tree(pos, np.full(len(pos), 1.0 / len(pos), np.float32), leaf, 32)
