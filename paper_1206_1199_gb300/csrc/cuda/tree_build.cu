@@ -22,12 +22,12 @@
 //                           running counts).
 //   k_permute               particles in tree order (sources, permutation,
 //                           grid coordinates).
-//   k_levels / k_cells / k_links  every cell of every level at once, from the
+//   k_levels / k_cells      every cell of every level at once, from the
 //                           number of key digits that neighbouring particles
 //                           share.
-//   k_moments               leaves sum their particles (all leaves in one
-//                           launch), then parents combine their children, one
-//                           level per launch, deepest first.
+//   k_leaves / k_parents    the cells' links and the leaves' moments, then the
+//                           parents combine their children, deepest level
+//                           first, in one cooperative launch.
 //   k_bmax                  largest distance of a cell's particles from its
 //                           centre of mass (FP64, on the particles an FP32
 //                           bound leaves), or the SPH radius bound (FP32);
@@ -39,7 +39,6 @@
 
 #include <algorithm>
 #include <cstdint>
-#include <vector>
 
 #include "../common.h"
 #include "../treegeom.h"
@@ -58,6 +57,7 @@ constexpr int kBmaxChunk = 2048;                // particles per b_max work item
 // status bits
 constexpr uint32_t kTreeBadInput = 1u;   // a non-finite position or a mass <= 0
 constexpr uint32_t kTreeBadSort = 2u;    // the sorted order indexed outside the particles
+constexpr uint32_t kTreeStuck = 4u;      // a wait between blocks ran into its limit
 
 struct Geom {
     double lo[3], S, h, scale;
@@ -327,7 +327,7 @@ struct Cells {
 //   (scan)     counts in (level, tile) order: where each tile's cells of each
 //              level go; the last sum is the number of cells
 //   k_cells    the cells of a tile, ranked per level by warp ballots
-//   k_links    children and end of every cell
+//   k_leaves   children and end of every cell (and the leaves' moments)
 //
 // Four to six launches, bound by their latency at small N and by the keys and
 // cell arrays they read and write at large N; expanding one level after
@@ -493,41 +493,6 @@ __global__ void __launch_bounds__(kRsThreads) k_cells(int64_t n, const uint16_t*
     }
 }
 
-// Of every cell: its children, the consecutive cells from child0 on that name
-// it as their parent, and its end, the first particle past it (a galloping
-// search over the keys' leading digits; a cell that splits holds at least
-// leaf_size + 1 particles).  One thread per cell, so that the searches'
-// dependent loads overlap: inside k_cells, one round of a warp after another,
-// they made it 40 us at N = 4096 (10 and 9.5 us apart) and 250 us at 2^23 (69
-// and 43).
-__global__ void k_links(int32_t n_cell, const uint64_t* __restrict__ keys, int64_t n, int64_t leaf_size, Cells c)
-{
-    const int32_t cell = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= n_cell) return;
-    int32_t k = 0;
-    const int32_t c0 = c.child0[cell];
-    if (c0 > 0)
-        while (k < 8 && c0 + k < n_cell && c.parent[c0 + k] == cell) ++k;
-    c.nchild[cell] = k;
-    const int64_t b = c.begin[cell];
-    const int sh = 3 * (kLevels - c.level[cell]);
-    const uint64_t pre = keys[b] >> sh;
-    int64_t l = k > 0 ? b + leaf_size : b, hi, step = 1;
-    for (hi = l + step; hi < n && (keys[hi] >> sh) == pre; hi = l + step) {
-        l = hi;
-        step *= 2;
-    }
-    if (hi > n) hi = n;
-    while (hi - l > 1) {
-        const int64_t mid = l + ((hi - l) >> 1);
-        if ((keys[mid] >> sh) == pre)
-            l = mid;
-        else
-            hi = mid;
-    }
-    c.end[cell] = (int32_t)hi;
-}
-
 // ---- moments ------------------------------------------------------------------------
 
 struct Moments {
@@ -539,76 +504,290 @@ struct Moments {
                                 //   the SPH radius (FP32, zero-extended)
 };
 
-// Cells [lo, hi), one thread each, in one pass over the cell's members
-// (its particles for a leaf, its children for a parent): with x0 a member's
-// position (a leaf's first particle, a parent's heaviest child's centre of
-// mass) and d = x - x0, M = sum m, S1 = sum m d, S2 = sum m d d^T (+ the
-// child's own central second moment C_c), then com = x0 + S1 / M and the
-// central second moment C = S2 - S1 S1^T / M (the parallel-axis shift to the
-// centre of mass).  S1 S1^T / M = M g g^T with g = com - x0, while C holds
-// at least m_0 M / (M - m_0) g g^T (the reference member, mass m_0, against
-// the rest), so the subtraction loses about log2((M - m_0) / m_0) bits: under
-// 3 for a parent (the heaviest of up to 8 children), about log2 of the leaf
-// size for equal masses in a leaf.  Stored: m, com, C (Cxx Cyy Czz Cxy Cxz
-// Cyz) and B_2 = tr C; the records take the quadrupole Q = 3 C - tr(C) I.
-// mode 1: leaves only; 2: parents only (their children done); else all.
-__global__ void k_moments(int32_t lo, int32_t hi, const otoo_src* __restrict__ src, Cells c, Moments mo, int mode)
+// A positive float widened to double by integer operations on its bits (the
+// FP64 pipe, which the conversion instruction would occupy, is what bounds
+// these kernels); subnormal, infinite and NaN values take the conversion.
+__device__ __forceinline__ double widen(float f)
 {
-    const int32_t cell = lo + (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (cell >= hi) return;
-    const int32_t nch = c.nchild[cell];
-    if ((mode == 1 && nch != 0) || (mode == 2 && nch == 0)) return;
-    double m = 0, s1[3] = {0, 0, 0}, s2[6] = {0, 0, 0, 0, 0, 0}, x0[3];
-    if (nch == 0) {
-        const int32_t b = c.begin[cell], e = c.end[cell];
-        {
-            const otoo_src p = src[b];
-            x0[0] = p.x, x0[1] = p.y, x0[2] = p.z;
+    const uint32_t u = __float_as_uint(f);
+    if (u - 0x00800000u < 0x7f000000u) return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
+    return (double)f;
+}
+
+// Moments of every cell, in one pass over its members (its particles for a
+// leaf, its children for a parent): with x0 a member's position (a leaf's
+// first particle, a parent's heaviest child's centre of mass) and d = x - x0,
+// M = sum m, S1 = sum m d, S2 = sum m d d^T (+ the child's own central second
+// moment C_c), then com = x0 + S1 / M and the central second moment C = S2 -
+// S1 S1^T / M (the parallel-axis shift to the centre of mass).  S1 S1^T / M =
+// M g g^T with g = com - x0, while C holds at least m_0 M / (M - m_0) g g^T
+// (the reference member, mass m_0, against the rest), so the subtraction
+// loses about log2((M - m_0) / m_0) bits: under 3 for a parent (the heaviest
+// of up to 8 children), about log2 of the leaf size for equal masses in a
+// leaf.  Stored: m, com, C (Cxx Cyy Czz Cxy Cxz Cyz) and B_2 = tr C; the
+// records take the quadrupole Q = 3 C - tr(C) I.  GB300's FP64 pipe (1/76 of
+// the FP32 rate) bounds both kernels at large N, latency at small N.
+
+// One thread per cell: the cell's links (children: the consecutive cells from
+// child0 on that name it as their parent; end: the first particle past it, by
+// a galloping search over the keys' leading digits; a cell that splits holds
+// at least leaf_size + 1 particles), and for a leaf its moments.  The
+// reference particle's own terms are zero and are left out (a leaf of leaf size
+// 8 holds 2.7 particles on average): 17 us at N = 4096, 93 us at 2^20, 0.57 ms
+// at 2^23 with leaves of 16, links included.
+__global__ void __launch_bounds__(128) k_leaves(const int32_t* __restrict__ lev, const uint64_t* __restrict__ keys,
+                                                int64_t n, int64_t leaf_size, const otoo_src* __restrict__ src,
+                                                Cells c, Moments mo, int32_t* __restrict__ plist,
+                                                int32_t* __restrict__ pcount)
+{
+    const int32_t n_cell = lev[kLv];
+    for (int32_t cell = blockIdx.x * blockDim.x + threadIdx.x; cell < n_cell; cell += gridDim.x * blockDim.x) {
+        int32_t k = 0;
+        const int32_t c0 = c.child0[cell];
+        if (c0 > 0)
+            while (k < 8 && c0 + k < n_cell && c.parent[c0 + k] == cell) ++k;
+        c.nchild[cell] = k;
+        const int32_t b = c.begin[cell];
+        const int lvl = c.level[cell];
+        if (k > 0) {
+            // one atomic per warp and level (the cells of a warp are nearly
+            // always of one level)
+            const unsigned peers = __match_any_sync(__activemask(), lvl);
+            const int lane = threadIdx.x & 31, lead = __ffs(peers) - 1;
+            int32_t at = 0;
+            if (lane == lead) at = atomicAdd(pcount + lvl, __popc(peers));
+            at = __shfl_sync(peers, at, lead);
+            plist[lev[lvl] + at + __popc(peers & ((1u << lane) - 1u))] = cell;
         }
+        const int sh = 3 * (kLevels - lvl);
+        const uint64_t pre = keys[b] >> sh;
+        int64_t l = k > 0 ? b + leaf_size : b, hi, step = 1;
+        for (hi = l + step; hi < n && (keys[hi] >> sh) == pre; hi = l + step) {
+            l = hi;
+            step *= 2;
+        }
+        if (hi > n) hi = n;
+        while (hi - l > 1) {
+            const int64_t mid = l + ((hi - l) >> 1);
+            if ((keys[mid] >> sh) == pre)
+                l = mid;
+            else
+                hi = mid;
+        }
+        const int32_t e = (int32_t)hi;
+        c.end[cell] = e;
+        mo.dmax2[cell] = 0ull;
+        if (k > 0) continue;
+        const otoo_src p0 = src[b];
+        double m = widen(p0.m);
+        double* q = mo.q + 6 * (int64_t)cell;
+        double* com = mo.com + 3 * (int64_t)cell;
+        if (e - b == 1) {
+            mo.m[cell] = m;
+            com[0] = p0.x, com[1] = p0.y, com[2] = p0.z;
+            q[0] = q[1] = q[2] = q[3] = q[4] = q[5] = 0.0;
+            mo.b2[cell] = 0.0;
+            continue;
+        }
+        double s1[3] = {0, 0, 0}, s2[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll 1
-        for (int32_t i = b; i < e; ++i) {
+        for (int32_t i = b + 1; i < e; ++i) {
             const otoo_src p = src[i];
-            const double mi = p.m;
-            const double dx = p.x - x0[0], dy = p.y - x0[1], dz = p.z - x0[2];
+            const double mi = widen(p.m);
+            const double dx = p.x - p0.x, dy = p.y - p0.y, dz = p.z - p0.z;
             const double mx = mi * dx, my = mi * dy, mz = mi * dz;
             m += mi;
             s1[0] += mx, s1[1] += my, s1[2] += mz;
             s2[0] = fma(mx, dx, s2[0]), s2[1] = fma(my, dy, s2[1]), s2[2] = fma(mz, dz, s2[2]);
             s2[3] = fma(mx, dy, s2[3]), s2[4] = fma(mx, dz, s2[4]), s2[5] = fma(my, dz, s2[5]);
         }
-    } else {
-        const int32_t c0 = c.child0[cell];
-        int32_t kh = c0;  // the heaviest child (positive doubles order like their bits)
-        unsigned long long mh = 0;
-        for (int32_t k = c0; k < c0 + nch; ++k) {
-            const unsigned long long mb = (unsigned long long)__double_as_longlong(mo.m[k]);
-            if (mb > mh) mh = mb, kh = k;
+        const double inv = 1.0 / m;
+        const double gx = s1[0] * inv, gy = s1[1] * inv, gz = s1[2] * inv;  // com - x0
+        mo.m[cell] = m;
+        com[0] = p0.x + gx;
+        com[1] = p0.y + gy;
+        com[2] = p0.z + gz;
+        const double cxx = fma(-s1[0], gx, s2[0]), cyy = fma(-s1[1], gy, s2[1]), czz = fma(-s1[2], gz, s2[2]);
+        q[0] = cxx, q[1] = cyy, q[2] = czz;
+        q[3] = fma(-s1[0], gy, s2[3]), q[4] = fma(-s1[0], gz, s2[4]), q[5] = fma(-s1[1], gz, s2[5]);
+        mo.b2[cell] = cxx + cyy + czz;
+    }
+}
+
+// A grid-wide barrier of a cooperative launch: bar counts arrivals (zero
+// before the launch).  The wait is bounded (about a second); a block that
+// gives up sets the status bit and the others see it, so that the kernel ends
+// in any case.  False: leave the kernel.
+__device__ __forceinline__ bool grid_wait(uint32_t* bar, uint32_t round, uint32_t* status)
+{
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        const uint32_t want = round * gridDim.x;
+        int good = 0;
+        for (int spin = 0; spin < (1 << 22); ++spin) {
+            if (*(volatile uint32_t*)bar >= want) {
+                good = 1;
+                break;
+            }
+            if (spin > 64) __nanosleep(100);
+            if ((spin & 1023) == 1023 && (*(volatile uint32_t*)status & kTreeStuck)) break;
         }
-        for (int a = 0; a < 3; ++a) x0[a] = mo.com[3 * kh + a];
-#pragma unroll 1
-        for (int32_t k = c0; k < c0 + nch; ++k) {
-            const double mk = mo.m[k];
-            const double dx = mo.com[3 * k] - x0[0], dy = mo.com[3 * k + 1] - x0[1], dz = mo.com[3 * k + 2] - x0[2];
-            const double mx = mk * dx, my = mk * dy, mz = mk * dz;
-            m += mk;
-            s1[0] += mx, s1[1] += my, s1[2] += mz;
-            s2[0] = fma(mx, dx, s2[0] + mo.q[6 * k]), s2[1] = fma(my, dy, s2[1] + mo.q[6 * k + 1]);
-            s2[2] = fma(mz, dz, s2[2] + mo.q[6 * k + 2]), s2[3] = fma(mx, dy, s2[3] + mo.q[6 * k + 3]);
-            s2[4] = fma(mx, dz, s2[4] + mo.q[6 * k + 4]), s2[5] = fma(my, dz, s2[5] + mo.q[6 * k + 5]);
+        if (!good) atomicOr(status, kTreeStuck);
+        __threadfence();
+        ok = good;
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
+// One parent per eight lanes (lane j of eight holds child j of ch0, ch0 + 1,
+// ...; nch = 0: none, the lanes only take part in the shuffles).
+__device__ __forceinline__ void combine_children(int32_t cell, int nch, int32_t ch0, int j, const Moments& mo)
+{
+    const bool on = j < nch;
+    const int64_t ch = on ? ch0 + j : 0;
+    double v[10], x[3] = {0, 0, 0};
+#pragma unroll
+    for (int q = 0; q < 10; ++q) v[q] = 0.0;
+    if (on) {
+        v[0] = __ldcg(mo.m + ch);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) x[q] = __ldcg(mo.com + 3 * (int64_t)ch + q);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) v[4 + q] = __ldcg(mo.q + 6 * (int64_t)ch + q);
+    }
+    // the heaviest child, the first of equals (positive doubles order
+    // like their bits)
+    unsigned long long mb = (unsigned long long)__double_as_longlong(v[0]);
+    int jh = j;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        const unsigned long long mo_ = __shfl_xor_sync(kFull, mb, o, 8);
+        const int jo = __shfl_xor_sync(kFull, jh, o, 8);
+        if (mo_ > mb || (mo_ == mb && jo < jh)) mb = mo_, jh = jo;
+    }
+    double x0[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) x0[q] = __shfl_sync(kFull, x[q], jh, 8);
+    if (on) {
+        const double dx = x[0] - x0[0], dy = x[1] - x0[1], dz = x[2] - x0[2];
+        v[1] = v[0] * dx, v[2] = v[0] * dy, v[3] = v[0] * dz;
+        v[4] = fma(v[1], dx, v[4]), v[5] = fma(v[2], dy, v[5]), v[6] = fma(v[3], dz, v[6]);
+        v[7] = fma(v[1], dy, v[7]), v[8] = fma(v[1], dz, v[8]), v[9] = fma(v[2], dz, v[9]);
+    }
+    // lanes with bit 2 clear keep sums 0..4, the others 5..9; then of
+    // those five the first three or the last two, then two or one
+    double a[5];
+    const bool b2 = j & 4, b1 = j & 2, b0 = j & 1;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        const double got = __shfl_xor_sync(kFull, b2 ? v[q] : v[5 + q], 4, 8);
+        a[q] = (b2 ? v[5 + q] : v[q]) + got;
+    }
+    double d[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const double hi3 = q < 2 ? a[3 + q] : 0.0;
+        const double got = __shfl_xor_sync(kFull, b1 ? a[q] : hi3, 2, 8);
+        d[q] = (b1 ? hi3 : a[q]) + got;
+    }
+    double s[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const double hi2 = q < 1 ? d[2] : 0.0;
+        const double got = __shfl_xor_sync(kFull, b0 ? d[q] : hi2, 1, 8);
+        s[q] = (b0 ? hi2 : d[q]) + got;
+    }
+    // sums now: lane 0: 0, 1; 1: 2; 2: 3, 4; 4: 5, 6; 5: 7; 6: 8, 9
+    const double M = __shfl_sync(kFull, s[0], 0, 8);
+    double s1[3], g[3], s2[6];
+    s1[0] = __shfl_sync(kFull, s[1], 0, 8);
+    s1[1] = __shfl_sync(kFull, s[0], 1, 8);
+    s1[2] = __shfl_sync(kFull, s[0], 2, 8);
+    s2[0] = __shfl_sync(kFull, s[1], 2, 8);
+    s2[1] = __shfl_sync(kFull, s[0], 4, 8);
+    s2[2] = __shfl_sync(kFull, s[1], 4, 8);
+    s2[3] = __shfl_sync(kFull, s[0], 5, 8);
+    s2[4] = __shfl_sync(kFull, s[0], 6, 8);
+    s2[5] = __shfl_sync(kFull, s[1], 6, 8);
+    const double inv = 1.0 / (nch > 0 ? M : 1.0);  // (a zero divisor takes the division's slow path)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) g[q] = s1[q] * inv;  // com - x0
+    // lane 0 .. 5: one entry of C = S2 - S1 g^T; lane 6: M; lanes 0 .. 2 also com
+    const double ca = j == 0 || j == 3 || j == 4 ? s1[0] : j == 1 || j == 5 ? s1[1] : s1[2];
+    const double cg = j == 0 ? g[0] : j == 1 || j == 3 ? g[1] : g[2];
+    double sv = s2[0];
+#pragma unroll
+    for (int q = 1; q < 6; ++q) sv = j == q ? s2[q] : sv;
+    const double cv = fma(-ca, cg, sv);
+    const double c1 = __shfl_sync(kFull, cv, 1, 8), c2 = __shfl_sync(kFull, cv, 2, 8);
+    if (nch == 0) return;
+    if (j < 6) mo.q[6 * (int64_t)cell + j] = cv;
+    if (j < 3) {
+        const double xr = j == 0 ? x0[0] : j == 1 ? x0[1] : x0[2], gr = j == 0 ? g[0] : j == 1 ? g[1] : g[2];
+        mo.com[3 * (int64_t)cell + j] = xr + gr;
+    }
+    if (j == 6) mo.m[cell] = M;
+    if (j == 0) mo.b2[cell] = cv + c1 + c2;
+}
+
+// Parents, deepest level first, eight lanes per parent (lane j holds child j):
+// the children's loads and products run side by side, then the ten sums are
+// halved over the lanes (a lane ends with one or two of them), so four parents
+// cost a warp about 40 FP64 instructions in a short chain; one thread per
+// parent is a chain of 8 dependent loads and 200 FP64 instructions.  One
+// cooperative launch walks the levels: a level of at most kSoloParents parents
+// is block 0's alone (block barriers), the others take a grid barrier before
+// and after, and each warp has its first parents' links in registers when the
+// barrier opens.  40 us at N = 4096, 97 us at 2^20, 0.20 ms at 2^23 (Plummer);
+// leaves and parents together 58, 190 and 770 us against 149, 382 and 1056 us
+// with one thread per cell and one launch per level, the links not counted
+// there.  The line at 64 parents: 16 warps of one SM take them in one round.
+// plist: k_leaves' parents of each level, pcount of them from
+// the level's first cell on.  mo's arrays are read past L1 (other blocks of
+// this launch write them).
+constexpr int kSoloParents = 64;
+
+__global__ void __launch_bounds__(512) k_parents(const int32_t* __restrict__ lev, Cells c, Moments mo,
+                                                  const int32_t* __restrict__ plist,
+                                                  const int32_t* __restrict__ pcount, uint32_t* __restrict__ bar,
+                                                  uint32_t* __restrict__ status)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    uint32_t round = 0;
+    bool wide_done = false;  // a level shared by all blocks has been summed since the last barrier
+    for (int L = kLevels - 1; L >= 0; --L) {
+        const int32_t np = pcount[L];
+        if (np == 0) continue;
+        const bool solo = np <= kSoloParents;
+        // neighbouring parents go to different SMs (each has one narrow FP64 pipe)
+        const int64_t nwarp = solo ? nw : (int64_t)gridDim.x * nw;
+        const int64_t warp = solo ? wid : (int64_t)wid * gridDim.x + blockIdx.x;
+        const int32_t* pl = plist + lev[L];
+        int64_t k = 4 * warp + (lane >> 3);
+        int32_t cell = 0, n = 0, c0 = 0;
+        auto links = [&]() {
+            cell = k < np ? pl[k] : 0;
+            n = k < np ? c.nchild[cell] : 0;
+            c0 = k < np ? c.child0[cell] : 0;
+        };
+        if (!solo || blockIdx.x == 0) links();
+        if (wide_done || !solo) {
+            if (!grid_wait(bar, ++round, status)) return;
+        } else {
+            __syncthreads();
+        }
+        wide_done = !solo;
+        if (solo && blockIdx.x != 0) continue;
+        for (int64_t w0 = 4 * warp; w0 < np; w0 += 4 * nwarp) {
+            combine_children(cell, n, c0, lane & 7, mo);
+            k += 4 * nwarp;
+            if (w0 + 4 * nwarp < np) links();
         }
     }
-    const double inv = 1.0 / m;
-    const double gx = s1[0] * inv, gy = s1[1] * inv, gz = s1[2] * inv;  // com - x0
-    mo.m[cell] = m;
-    mo.com[3 * cell] = x0[0] + gx;
-    mo.com[3 * cell + 1] = x0[1] + gy;
-    mo.com[3 * cell + 2] = x0[2] + gz;
-    const double cxx = fma(-s1[0], gx, s2[0]), cyy = fma(-s1[1], gy, s2[1]), czz = fma(-s1[2], gz, s2[2]);
-    double* q = mo.q + 6 * (int64_t)cell;
-    q[0] = cxx, q[1] = cyy, q[2] = czz;
-    q[3] = fma(-s1[0], gy, s2[3]), q[4] = fma(-s1[0], gz, s2[4]), q[5] = fma(-s1[1], gz, s2[5]);
-    mo.b2[cell] = cxx + cyy + czz;
-    mo.dmax2[cell] = 0ull;
 }
 
 // FP32 distance |c~ - x~_j| between a cell's rounded centre of mass c~ and a
@@ -995,7 +1174,8 @@ Layout layout(int64_t n, int64_t cap)
     l.cnt = take(4 * (big + 1));
     l.flag = take(4 * (n + 1));
     l.tot = take(64);
-    l.lev = take(4 * (kLevels + 4) + 4);  // level bounds, then the stop word
+    l.lev = take(4 * 64);  // level bounds, then the stop word; word 32: the grid barrier;
+                           // words 33..: parents per level
     l.total = o;
     return l;
 }
@@ -1096,7 +1276,7 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     // (2 (n + leaf_size) bytes, leaf_size < n)
     int32_t* lev = reinterpret_cast<int32_t*>(base + ly.lev);
     uint32_t* stop = reinterpret_cast<uint32_t*>(lev + kLevels + 4);
-    CUDA_TRY(cudaMemsetAsync(lev, 0, 4 * (kLevels + 4) + 4, s));
+    CUDA_TRY(cudaMemsetAsync(lev, 0, 4 * 64, s));
     uint16_t* lv = reinterpret_cast<uint16_t*>(keys[cur ^ 1]);
     const uint8_t* win = nullptr;
     int64_t span = 1;
@@ -1128,20 +1308,23 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
         return set_error(OTOO_ENOMEM, "otoo_devtree_build: more than cap_cell = %lld cells", (long long)cap);
     }
     // level L holds [hlev[L], hlev[L + 1]); the last non-empty level is the depth
-    std::vector<int32_t> lev_lo(hlev, hlev + kLevels + 3);
     int depth = 0;
-    for (int L = 0; L <= kLevels + 1; ++L)
+    for (int L = 0; L <= kLevels; ++L)
         if (hlev[L + 1] > hlev[L]) depth = L;
-    lev_lo.resize(depth + 2);
-    const int32_t n_cell = lev_lo.back();
+    const int32_t n_cell = hlev[kLv];
 
-    k_links<<<(unsigned)((n_cell + 127) / 128), 128, 0, s>>>(n_cell, skeys, n, leaf, c);
-    // moments: every leaf in one launch, then the parents level by level,
-    // deepest first
-    k_moments<<<(unsigned)((n_cell + 127) / 128), 128, 0, s>>>(0, n_cell, t->src, c, mo, 1);
-    for (int L = depth; L >= 0; --L) {
-        const int32_t lo = lev_lo[L], hi = lev_lo[L + 1];
-        if (hi > lo) k_moments<<<(unsigned)((hi - lo + 127) / 128), 128, 0, s>>>(lo, hi, t->src, c, mo, 2);
+    // links, leaves, then the parents level by level, deepest first
+    int dev = 0, sms = 0;
+    CUDA_TRY(cudaGetDevice(&dev));
+    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int32_t* pcount = lev + 33;  // one count per level
+    k_leaves<<<(unsigned)((n_cell + 127) / 128), 128, 0, s>>>(lev, skeys, n, leaf, t->src, c, mo, dig, pcount);
+    if (depth > 0) {
+        uint32_t* bar = reinterpret_cast<uint32_t*>(lev) + 32;
+        void* args[] = {&lev, &c, &mo, &dig, &pcount, &bar, &status};
+        // one block per SM at most, no more than the widest level could use
+        const unsigned pg = (unsigned)std::min<int64_t>(sms, (n_cell + 63) / 64);
+        CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_parents, dim3(pg), dim3(512), args, 0, s));
     }
     CUDA_TRY(cudaGetLastError());
     const bool sph = t->mac == OTOO_MAC_SPH;
@@ -1182,7 +1365,9 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     k_group_write<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, flag, cnt, t->group_first);
     int64_t G = 0;
     CUDA_TRY(cudaMemcpyAsync(&G, tot, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(cudaMemcpyAsync(&st, status, sizeof(st), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaStreamSynchronize(s));
+    if (st & kTreeStuck) return set_error(OTOO_EDEVICE, "otoo_devtree_build: a wait between blocks ran into its limit");
     k_group_count<<<(unsigned)((G + 255) / 256), 256, 0, s>>>(n, (int32_t)G, t->group_first, t->group_count);
     CUDA_TRY(cudaGetLastError());
     t->n_cell = n_cell;
