@@ -15,11 +15,10 @@
 //   k_bbox / k_bbox_final   min/max of the positions (order-preserving integer
 //                           keys: exact), then the root cube.
 //   k_keys                  grid coordinates and Hilbert key per particle.
-//   k_rs_hist / k_rs_scatter  stable LSD radix sort of (key, index), 8 bits
-//                           per pass: per-block digit counts, a scan of the
-//                           counts (digit-major), a scatter that ranks equal
-//                           digits in input order (warp match + per-warp
-//                           running counts).
+//   k_sort_pass / k_sort_tile  stable LSD radix sort of (key, index), 8 bits
+//                           per pass: one launch per pass with a decoupled
+//                           look-back between tiles, or all passes in one
+//                           block for at most one tile.
 //   k_permute               particles in tree order (sources, permutation,
 //                           grid coordinates).
 //   k_levels / k_cells      every cell of every level at once, from the
@@ -48,10 +47,10 @@ using namespace otoo;
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kRsThreads = 256;                 // radix sort: threads per block
-constexpr int kRsItems = 8;                     // keys per thread
-constexpr int kRsTile = kRsThreads * kRsItems;  // keys per block
-constexpr int kRsWarps = kRsThreads / 32;
+constexpr int kLvThreads = 256;  // cells: threads per block
+constexpr int kLvWarps = kLvThreads / 32;
+constexpr int kLvTile = 2048;    // particles per block, in contiguous runs per warp
+constexpr int kLv = kLevels + 1;  // levels 0 .. 21
 constexpr int kBmaxChunk = 2048;                // particles per b_max work item
 
 // status bits
@@ -151,124 +150,266 @@ __global__ void __launch_bounds__(256) k_bbox_final(const long long* __restrict_
 
 // ---- keys ---------------------------------------------------------------------
 
-__global__ void k_keys(const double* __restrict__ pos, int64_t n, const Geom* __restrict__ g,
-                       uint64_t* __restrict__ keys, uint32_t* __restrict__ vals)
+// One key per particle, and the counts of all eight digits of all keys
+// (ghist[pass][digit], zero before the launch) that the sort's passes start
+// from: shared-memory counts per block (increments of one address by a whole
+// warp count as one), one global atomic per block and digit present.
+__global__ void __launch_bounds__(256) k_keys(const double* __restrict__ pos, int64_t n, const Geom* __restrict__ g,
+                                              uint64_t* __restrict__ keys, int32_t* __restrict__ ghist)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t x = quantize(pos[3 * i], g->lo[0], g->scale);
-    const uint32_t y = quantize(pos[3 * i + 1], g->lo[1], g->scale);
-    const uint32_t z = quantize(pos[3 * i + 2], g->lo[2], g->scale);
-    keys[i] = hilbert_key(x, y, z);
-    vals[i] = (uint32_t)i;
+    __shared__ int32_t h[8 * 256];
+    for (int j = threadIdx.x; j < 8 * 256; j += 256) h[j] = 0;
+    __syncthreads();
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+        const uint32_t x = quantize(pos[3 * i], g->lo[0], g->scale);
+        const uint32_t y = quantize(pos[3 * i + 1], g->lo[1], g->scale);
+        const uint32_t z = quantize(pos[3 * i + 2], g->lo[2], g->scale);
+        const uint64_t k = hilbert_key(x, y, z);
+        keys[i] = k;
+#pragma unroll
+        for (int p = 0; p < 8; ++p) atomicAdd(&h[256 * p + (int)((k >> (8 * p)) & 255u)], 1);
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < 8 * 256; j += 256)
+        if (h[j]) atomicAdd(ghist + j, h[j]);
 }
 
 // ---- stable LSD radix sort ----------------------------------------------------
-// Block b counts the digits of its tile (hist, digit-major: hist[d * nblk +
-// b]); an exclusive scan of hist gives each (digit, block) its output start.
-// The scatter ranks each key after the keys of smaller digit in its tile and
-// after the keys of equal digit that precede it (earlier warps of the block,
-// earlier rounds and lower lanes of the warp), which keeps the sort stable;
-// it stages the tile in that order in shared memory and then writes each
-// digit's run of the tile to consecutive addresses from the run's global
-// start (coalesced stores instead of one scattered store per key).
+// Eight passes of eight bits over (key, index), one launch each (Adinets and
+// Merrill, "Onesweep", 2022, after Merrill and Garland's decoupled look-back,
+// 2016).  A tile of 4096 keys ranks its keys by digit in input order (warp
+// ballots of the digit's bits and per-warp running counts: stable), publishes its count of every
+// digit, and finds how many keys of each digit precede it by walking back over
+// the earlier tiles' published words (an aggregate, or a whole prefix that
+// ends the walk), one digit per thread.  Tiles take their number from a
+// ticket, so a tile only waits for tiles that already run.  The tile is staged
+// in digit order in shared memory and each digit's run goes to consecutive
+// addresses.  A pass reads and writes every pair once (24 bytes per key) and
+// is bound by its barriers and ranking at large n (2.6 TB/s; the warp match
+// instruction in place of the ballots made it a third slower), by latency at small n.
+// Sums of launches under ncu, against the form before (counts, a scan and a
+// scatter per pass over tiles of 2048 keys, 40 launches): N = 4096 33 against
+// 150 us (one tile, one launch), 100003 83 against 212, 2^20 138 against 293,
+// 2^23 0.63 against 1.23 ms.
+// Every wait is bounded; a tile that gives up sets the status bit (the others
+// then stop waiting too) and its writes stay inside the arrays.
 
-__global__ void __launch_bounds__(kRsThreads) k_rs_hist(const uint64_t* __restrict__ keys, int64_t n, int shift,
-                                                         int32_t* __restrict__ hist, int nblk)
+constexpr int kSortThreads = 512;
+constexpr int kSortItems = 8;
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kSortTile = kSortThreads * kSortItems;
+constexpr uint32_t kSortAgg = 1u << 30, kSortPre = 2u << 30, kSortVal = kSortAgg - 1u;  // counts below 2^30
+
+struct SortShared {
+    uint64_t key[kSortTile];
+    uint32_t val[kSortTile];
+    int32_t wcount[kSortWarps][256];
+    int32_t dstart[256], gstart[256];
+    int32_t wsum[2][8];
+    int32_t tile;
+};
+
+// Ranks the tile's keys (warp w owns a contiguous run) and fills dstart; each
+// thread gets the tile position of its keys and thread d < 256 the tile's
+// count of digit d.
+__device__ __forceinline__ int32_t sort_rank(SortShared& sh, const uint64_t key[kSortItems], int64_t left, int shift,
+                                             int32_t lp[kSortItems])
 {
-    __shared__ int32_t h[256];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRsTile;
-    for (int k = 0; k < kRsItems; ++k) {
-        const int64_t i = base + (int64_t)k * kRsThreads + threadIdx.x;
-        if (i < n) atomicAdd(&h[(int)((keys[i] >> shift) & 255u)], 1);
-    }
-    __syncthreads();
-    hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = h[threadIdx.x];
-}
-
-static_assert(kRsThreads == 256, "the scatter gives each of the 256 digits one thread");
-
-__global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const uint64_t* __restrict__ kin,
-                                                            const uint32_t* __restrict__ vin, int64_t n, int shift,
-                                                            const int32_t* __restrict__ offs, int nblk,
-                                                            uint64_t* __restrict__ kout, uint32_t* __restrict__ vout)
-{
-    __shared__ int32_t wcount[kRsWarps][256];
-    __shared__ int32_t dstart[256], gstart[256], wsum[kRsWarps];
-    __shared__ uint64_t skey[kRsTile];
-    __shared__ uint32_t sval[kRsTile];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    for (int d = lane; d < 256; d += 32) wcount[w][d] = 0;
+    for (int d = lane; d < 256; d += 32) sh.wcount[w][d] = 0;
     __syncwarp();
-    // warp w owns the contiguous run [base, base + 32 kRsItems) of the tile
-    const int64_t b0 = (int64_t)blockIdx.x * kRsTile;
-    const int64_t base = b0 + (int64_t)w * 32 * kRsItems;
-    uint64_t key[kRsItems];
-    uint32_t val[kRsItems];
-    int dig[kRsItems];
 #pragma unroll
-    for (int r = 0; r < kRsItems; ++r) {
-        const int64_t i = base + r * 32 + lane;
-        const bool ok = i < n;
-        key[r] = ok ? kin[i] : 0;
-        val[r] = ok ? vin[i] : 0;
-        dig[r] = ok ? (int)((key[r] >> shift) & 255u) : 256;
-        const unsigned peers = __match_any_sync(kFull, dig[r]);
-        if (ok && (peers & lt) == 0) wcount[w][dig[r]] += __popc(peers);
+    for (int r = 0; r < kSortItems; ++r) {
+        const bool ok = w * 32 * kSortItems + r * 32 + lane < left;
+        const int d = ok ? (int)((key[r] >> shift) & 255u) : 256;
+        unsigned peers = __ballot_sync(kFull, ok);
+        if (!ok) peers = ~peers;
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const bool one = (d >> b) & 1;
+            const unsigned m = __ballot_sync(kFull, one);
+            peers &= one ? m : ~m;
+        }
+        const int lead = __ffs(peers) - 1;
+        int32_t before = 0;
+        if (ok && lane == lead) {
+            before = sh.wcount[w][d];
+            sh.wcount[w][d] = before + __popc(peers);
+        }
         __syncwarp();
+        lp[r] = __shfl_sync(kFull, before, lead) + __popc(peers & lt);
     }
     __syncthreads();
-    // digit d = thread: exclusive prefix over the warps, the tile's count of
-    // d, and (a block-wide scan over digits) the start of d's run in the tile
-    {
-        const int d = threadIdx.x;
-        int32_t run = 0;
-        for (int k = 0; k < kRsWarps; ++k) {
-            const int32_t c = wcount[k][d];
-            wcount[k][d] = run;
-            run += c;
+    int32_t cnt = 0, incl = 0;
+    if (threadIdx.x < 256) {
+        for (int k = 0; k < kSortWarps; ++k) {
+            const int32_t c = sh.wcount[k][threadIdx.x];
+            sh.wcount[k][threadIdx.x] = cnt;
+            cnt += c;
         }
-        int32_t incl = run;
+        incl = cnt;
+#pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int32_t t = __shfl_up_sync(kFull, incl, o);
             if (lane >= o) incl += t;
         }
-        if (lane == 31) wsum[w] = incl;
-        __syncthreads();
-        int32_t excl = incl - run;
-        for (int k = 0; k < w; ++k) excl += wsum[k];
-        dstart[d] = excl;
-        gstart[d] = offs[(int64_t)d * nblk + blockIdx.x];
-        for (int k = 0; k < kRsWarps; ++k) wcount[k][d] += excl;
+        if (lane == 31) sh.wsum[0][w] = incl;
+    }
+    __syncthreads();
+    if (threadIdx.x < 256) {
+        int32_t e = incl - cnt;
+        for (int k = 0; k < w; ++k) e += sh.wsum[0][k];
+        sh.dstart[threadIdx.x] = e;
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kRsItems; ++r) {
-        const unsigned peers = __match_any_sync(kFull, dig[r]);
-        const bool ok = dig[r] < 256;
-        int32_t lp = 0;
-        if (ok) lp = wcount[w][dig[r]] + __popc(peers & lt);
-        __syncwarp();
-        if (ok && (peers & lt) == 0) wcount[w][dig[r]] += __popc(peers);
-        __syncwarp();
+    for (int r = 0; r < kSortItems; ++r) {
+        const bool ok = w * 32 * kSortItems + r * 32 + lane < left;
         if (ok) {
-            skey[lp] = key[r];
-            sval[lp] = val[r];
+            const int d = (int)((key[r] >> shift) & 255u);
+            lp[r] += sh.wcount[w][d] + sh.dstart[d];
         }
     }
+    return cnt;
+}
+
+// ghist: this pass's digit counts; ticket: this pass's tile counter (zero);
+// look: this pass's published words (zero), look_next: the next pass's, zeroed
+// here (the pass before this one is done with them).  vin NULL: the index
+// itself (first pass).
+__global__ void __launch_bounds__(kSortThreads, 3) k_sort_pass(const uint64_t* __restrict__ kin,
+                                                             const uint32_t* __restrict__ vin, int64_t n, int shift,
+                                                             const int32_t* __restrict__ ghist,
+                                                             uint32_t* __restrict__ ticket,
+                                                             uint32_t* __restrict__ look,
+                                                             uint32_t* __restrict__ look_next,
+                                                             uint64_t* __restrict__ kout,
+                                                             uint32_t* __restrict__ vout,
+                                                             uint32_t* __restrict__ status)
+{
+    extern __shared__ __align__(16) unsigned char sort_smem[];
+    SortShared& sh = *reinterpret_cast<SortShared*>(sort_smem);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0) sh.tile = (int32_t)atomicAdd(ticket, 1u);
     __syncthreads();
-    // the tile's valid keys fill [0, nvalid) of the staging in digit order
-    const int nvalid = (int)(n - b0 < kRsTile ? n - b0 : kRsTile);
-    for (int j = threadIdx.x; j < nvalid; j += kRsThreads) {
-        const uint64_t k = skey[j];
-        const int d = (int)((k >> shift) & 255u);
-        const int64_t gp = (int64_t)gstart[d] + (j - dstart[d]);
-        kout[gp] = k;
-        vout[gp] = sval[j];
+    const int32_t tile = sh.tile;
+    const int64_t b0 = (int64_t)tile * kSortTile;
+    const int64_t left = n - b0;
+    uint64_t key[kSortItems];
+    int32_t lp[kSortItems];
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r) {
+        const int q = w * 32 * kSortItems + r * 32 + lane;
+        key[r] = q < left ? kin[b0 + q] : 0;
     }
+    const int32_t cnt = sort_rank(sh, key, left, shift, lp);
+    const int d = threadIdx.x;
+    volatile uint32_t* my = look + (int64_t)tile * 256;
+    if (d < 256) {
+        my[d] = (tile == 0 ? kSortPre : kSortAgg) | (uint32_t)cnt;
+        look_next[(int64_t)tile * 256 + d] = 0u;
+    }
+    // the tile in digit order, while the look-back's words arrive
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r) {
+        const int q = w * 32 * kSortItems + r * 32 + lane;
+        if (q < left) {
+            sh.key[lp[r]] = key[r];
+            sh.val[lp[r]] = vin ? vin[b0 + q] : (uint32_t)(b0 + q);
+        }
+    }
+    if (d < 256) {
+        // keys of smaller digits, then keys of this digit in earlier tiles
+        const int32_t gh = ghist[d];
+        int32_t incl = gh;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t t = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) sh.wsum[1][w] = incl;
+        uint32_t before = 0;
+        bool done = tile == 0;
+        // eight earlier tiles' words at a time, so that the walk does not wait
+        // for one load after another
+        for (int32_t t = tile - 1; !done;) {
+            uint32_t v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                v[k] = t - k >= 0 ? *(const volatile uint32_t*)(look + (int64_t)(t - k) * 256 + d) : kSortPre;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (done) continue;
+                for (int spin = 0; v[k] < kSortAgg; ++spin) {
+                    if (spin >= (1 << 20) || ((spin & 255) == 255 && (*(volatile uint32_t*)status & kTreeStuck))) {
+                        atomicOr(status, kTreeStuck);
+                        v[k] = kSortPre;
+                        break;
+                    }
+                    v[k] = *(const volatile uint32_t*)(look + (int64_t)(t - k) * 256 + d);
+                }
+                before += v[k] & kSortVal;
+                done = v[k] >= kSortPre;
+            }
+            t -= 8;
+        }
+        if (tile > 0) my[d] = kSortPre | ((before + (uint32_t)cnt) & kSortVal);
+        sh.gstart[d] = incl - gh + (int32_t)before;
+    }
+    __syncthreads();
+    if (d < 256) {
+        int32_t e = 0;
+        for (int k = 0; k < w; ++k) e += sh.wsum[1][k];
+        sh.gstart[d] += e - sh.dstart[d];
+    }
+    __syncthreads();
+    const int nvalid = (int)(left < kSortTile ? left : kSortTile);
+    for (int j = threadIdx.x; j < nvalid; j += kSortThreads) {
+        const uint64_t k = sh.key[j];
+        const int64_t gp = (int64_t)sh.gstart[(int)((k >> shift) & 255u)] + j;
+        if (gp >= 0 && gp < n) {  // (always, unless a wait gave up)
+            kout[gp] = k;
+            vout[gp] = sh.val[j];
+        }
+    }
+}
+
+// The whole sort of at most one tile: all passes in one block.
+__global__ void __launch_bounds__(kSortThreads) k_sort_tile(const uint64_t* __restrict__ kin, int64_t n,
+                                                             uint64_t* __restrict__ kout, uint32_t* __restrict__ vout)
+{
+    extern __shared__ __align__(16) unsigned char sort_smem[];
+    SortShared& sh = *reinterpret_cast<SortShared*>(sort_smem);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint64_t key[kSortItems];
+    uint32_t val[kSortItems];
+    int32_t lp[kSortItems];
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r) {
+        const int q = w * 32 * kSortItems + r * 32 + lane;
+        key[r] = q < n ? kin[q] : 0;
+        val[r] = (uint32_t)q;
+    }
+    for (int shift = 0;; shift += 8) {
+        sort_rank(sh, key, n, shift, lp);
+        if (shift == 56) break;
+        // (every thread has read its digits' starts: dstart and wcount are
+        // rewritten only after the barriers below)
+#pragma unroll
+        for (int r = 0; r < kSortItems; ++r)
+            if (w * 32 * kSortItems + r * 32 + lane < n) sh.key[lp[r]] = key[r], sh.val[lp[r]] = val[r];
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kSortItems; ++r) {
+            const int q = w * 32 * kSortItems + r * 32 + lane;
+            if (q < n) key[r] = sh.key[q], val[r] = sh.val[q];
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r)
+        if (w * 32 * kSortItems + r * 32 + lane < n) kout[lp[r]] = key[r], vout[lp[r]] = val[r];
 }
 
 // ---- tree order ------------------------------------------------------------------
@@ -336,10 +477,8 @@ struct Cells {
 // sums of launches under ncu): N = 4096 0.031 against 0.372 ms, 2^20 0.049
 // against 0.501 ms, 2^23 0.19 against 0.73 ms.
 
-constexpr int kLvTile = kRsTile;      // particles per block, in contiguous runs per warp
-constexpr int kLvRounds = kLvTile / kRsThreads;
+constexpr int kLvRounds = kLvTile / kLvThreads;
 constexpr int kLvLeaf = 64;           // leaf sizes up to this take the window maximum in shared memory
-constexpr int kLv = kLevels + 1;      // levels 0 .. 21
 
 // Leading digits two keys share (21 for equal keys; bit 63 of a key is 0).
 __device__ __forceinline__ int common_digits(uint64_t a, uint64_t b)
@@ -371,23 +510,23 @@ __global__ void k_win_double(const uint8_t* __restrict__ in, int64_t len, int64_
 // D when none does); hist[L * gridDim.x + blk]: cells of level L that start in
 // the tile.  win: NULL for leaf <= kLvLeaf, else the maxima over runs of span
 // windows (span the largest power of two <= leaf + 1).
-__global__ void __launch_bounds__(kRsThreads) k_levels(const uint64_t* __restrict__ keys, int64_t n, int64_t leaf,
+__global__ void __launch_bounds__(kLvThreads) k_levels(const uint64_t* __restrict__ keys, int64_t n, int64_t leaf,
                                                         const uint8_t* __restrict__ win, int64_t span,
                                                         uint16_t* __restrict__ lv, int32_t* __restrict__ hist)
 {
     __shared__ uint64_t sk[kLvTile + 2 * kLvLeaf];
     __shared__ uint8_t sw[kLvTile + kLvLeaf];
-    __shared__ int32_t wcnt[kRsWarps][kLv];
+    __shared__ int32_t wcnt[kLvWarps][kLv];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t t0 = (int64_t)blockIdx.x * kLvTile;
     const int halo = win ? 1 : (int)leaf;  // keys staged before and after the tile
-    for (int j = threadIdx.x; j < kLvTile + 2 * halo; j += kRsThreads) {
+    for (int j = threadIdx.x; j < kLvTile + 2 * halo; j += kLvThreads) {
         const int64_t i = t0 - halo + j;
         sk[j] = i >= 0 && i < n ? keys[i] : 0;
     }
     __syncthreads();
     if (!win) {
-        for (int j = threadIdx.x; j < kLvTile + halo; j += kRsThreads) {
+        for (int j = threadIdx.x; j < kLvTile + halo; j += kLvThreads) {
             const int64_t i = t0 - halo + j;  // window [i, i + leaf]
             sw[j] = i >= 0 && i + halo < n ? (uint8_t)(1 + common_digits(sk[j], sk[j + halo])) : (uint8_t)0;
         }
@@ -421,7 +560,7 @@ __global__ void __launch_bounds__(kRsThreads) k_levels(const uint64_t* __restric
     __syncthreads();
     if (threadIdx.x < kLv) {
         int32_t c = 0;
-        for (int k = 0; k < kRsWarps; ++k) c += wcnt[k][threadIdx.x];
+        for (int k = 0; k < kLvWarps; ++k) c += wcnt[k][threadIdx.x];
         hist[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = c;
     }
 }
@@ -429,12 +568,12 @@ __global__ void __launch_bounds__(kRsThreads) k_levels(const uint64_t* __restric
 // Writes the cells that start in the tile.  offs: the exclusive scan of
 // k_levels' counts, *total their sum; block 0 writes the levels' first cells
 // lev[0 .. 22].  More than cap cells: nothing is written and stop is set.
-__global__ void __launch_bounds__(kRsThreads) k_cells(int64_t n, const uint16_t* __restrict__ lv,
+__global__ void __launch_bounds__(kLvThreads) k_cells(int64_t n, const uint16_t* __restrict__ lv,
                                                        const int32_t* __restrict__ offs,
                                                        const int64_t* __restrict__ total, int64_t cap, Cells c,
                                                        int32_t* __restrict__ lev, uint32_t* __restrict__ stop)
 {
-    __shared__ int32_t wcnt[kRsWarps][kLv];
+    __shared__ int32_t wcnt[kLvWarps][kLv];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     if (*total > cap) {
@@ -1153,13 +1292,16 @@ Layout layout(int64_t n, int64_t cap)
         o += up(bytes);
         return at;
     };
-    const int64_t nblk = (n + kRsTile - 1) / kRsTile;
+    const int64_t nblk = (n + kLvTile - 1) / kLvTile;
     const int64_t big = n > cap ? n : cap;
     l.keys0 = take(8 * n);
     l.keys1 = take(8 * n);
     l.vals0 = take(4 * n);
     l.vals1 = take(4 * n);
-    l.hist = take(4 * 256 * nblk);
+    // the sort's counts, tickets and two sets of published words; later the
+    // cells' counts (kLv per tile of kLvTile)
+    const int64_t ntile = (n + kSortTile - 1) / kSortTile;
+    l.hist = take(4 * std::max<int64_t>(256 * (9 + 2 * ntile), kLv * nblk));
     l.bsum = take(8 * ((256 * nblk + 8 * big) / kScanThreads + 8));
     l.part = take(8 * 6 * 1024);
     l.geom = take(sizeof(Geom));
@@ -1246,19 +1388,31 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     const int nbb = (int)std::min<int64_t>(1024, (n + 255) / 256);
     k_bbox<<<nbb, 256, 0, s>>>(pos, mass, n, part, status);
     k_bbox_final<<<1, 256, 0, s>>>(part, nbb, geom);
-    k_keys<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(pos, n, geom, keys[0], vals[0]);
+    int dev = 0, sms = 0;
+    CUDA_TRY(cudaGetDevice(&dev));
+    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int nblk = (int)((n + kLvTile - 1) / kLvTile);
+    const int ntile = (int)((n + kSortTile - 1) / kSortTile);
+    // digit counts and tickets of the eight passes, then the first pass's words
+    int32_t* ghist = reinterpret_cast<int32_t*>(base + ly.hist);
+    uint32_t* ticket = reinterpret_cast<uint32_t*>(ghist + 8 * 256);
+    uint32_t* look[2] = {ticket + 256, ticket + 256 + (size_t)256 * ntile};
+    CUDA_TRY(cudaMemsetAsync(ghist, 0, 4 * (8 * 256 + 256 + (size_t)256 * ntile), s));
+    k_keys<<<(unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)sms * 8), 256, 0, s>>>(pos, n, geom, keys[0], ghist);
     CUDA_TRY(cudaGetLastError());
-    const int nblk = (int)((n + kRsTile - 1) / kRsTile);
+    CUDA_TRY(cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortShared)));
+    CUDA_TRY(cudaFuncSetAttribute(k_sort_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortShared)));
     int cur = 0;
-    for (int shift = 0; shift < 64; shift += 8) {
-        k_rs_hist<<<nblk, kRsThreads, 0, s>>>(keys[cur], n, shift, hist, nblk);
-        const int r = scan32(hist, (int64_t)256 * nblk, bsum, tot, s);
-        if (r) return r;
-        k_rs_scatter<<<nblk, kRsThreads, 0, s>>>(keys[cur], vals[cur], n, shift, hist, nblk, keys[cur ^ 1],
-                                                 vals[cur ^ 1]);
-        CUDA_TRY(cudaGetLastError());
-        cur ^= 1;
+    if (ntile == 1) {
+        k_sort_tile<<<1, kSortThreads, sizeof(SortShared), s>>>(keys[0], n, keys[1], vals[1]);
+        cur = 1;
+    } else {
+        for (int p = 0; p < 8; ++p, cur ^= 1)
+            k_sort_pass<<<ntile, kSortThreads, sizeof(SortShared), s>>>(
+                keys[cur], p ? vals[cur] : nullptr, n, 8 * p, ghist + 256 * p, ticket + p, look[p & 1],
+                look[(p & 1) ^ 1], keys[cur ^ 1], vals[cur ^ 1], status);
     }
+    CUDA_TRY(cudaGetLastError());
     k_permute<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(pos, mass, vals[cur], n, geom, t->src, t->perm, gq,
                                                           status);
     CUDA_TRY(cudaGetLastError());
@@ -1268,6 +1422,7 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     CUDA_TRY(cudaMemcpyAsync(&hg, geom, sizeof(hg), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaStreamSynchronize(s));
     if (st & kTreeBadInput) return set_error(OTOO_EINVAL, "otoo_devtree_build: non-finite position or mass <= 0");
+    if (st & kTreeStuck) return set_error(OTOO_EDEVICE, "otoo_devtree_build: a wait between blocks ran into its limit");
     if (st & kTreeBadSort) return set_error(OTOO_EDEVICE, "otoo_devtree_build: sort produced an invalid order");
     const uint64_t* skeys = keys[cur];
 
@@ -1290,13 +1445,13 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
         for (; 2 * span <= leaf + 1; span *= 2, k ^= 1) k_win_double<<<g, 256, 0, s>>>(wb[k], len, span, wb[k ^ 1]);
         win = wb[k];
     }
-    k_levels<<<nblk, kRsThreads, 0, s>>>(skeys, n, leaf, win, span, lv, hist);
+    k_levels<<<nblk, kLvThreads, 0, s>>>(skeys, n, leaf, win, span, lv, hist);
     CUDA_TRY(cudaGetLastError());
     {
         const int r = scan32(hist, (int64_t)kLv * nblk, bsum, tot, s);
         if (r) return r;
     }
-    k_cells<<<nblk, kRsThreads, 0, s>>>(n, lv, hist, tot, cap, c, lev, stop);
+    k_cells<<<nblk, kLvThreads, 0, s>>>(n, lv, hist, tot, cap, c, lev, stop);
     CUDA_TRY(cudaGetLastError());
     int32_t hlev[kLevels + 4];
     uint32_t hstop = 0;
@@ -1314,9 +1469,6 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     const int32_t n_cell = hlev[kLv];
 
     // links, leaves, then the parents level by level, deepest first
-    int dev = 0, sms = 0;
-    CUDA_TRY(cudaGetDevice(&dev));
-    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     int32_t* pcount = lev + 33;  // one count per level
     k_leaves<<<(unsigned)((n_cell + 127) / 128), 128, 0, s>>>(lev, skeys, n, leaf, t->src, c, mo, dig, pcount);
     if (depth > 0) {

@@ -30,3 +30,17 @@ def test_cells_of_coincident_and_lattice_particles(leaf):
     g = np.stack(np.meshgrid(*[np.arange(8) / 8.0] * 3, indexing="ij"), -1).reshape(-1, 3)
     pos = np.concatenate([g, np.full((2500, 3), 0.1), np.full((70, 3), 0.7)])
     check_tree(pos, np.full(len(pos), 1.0 / len(pos), np.float32), leaf, 32)
+
+
+@pytest.mark.parametrize("n", [4095, 4096, 4097, 8192, 12289, 70001])
+@pytest.mark.parametrize("model", ["uniform", "hernquist", "pairs"])
+def test_order_across_sort_tiles(n, model):
+    # one tile and several, the last one full, nearly empty and ragged; in
+    # "pairs" every position occurs many times, so equal keys span the tiles
+    # and the order among them is the callers'
+    if model == "pairs":
+        p, _ = ic.plummer(37, 62)
+        pos = p[np.arange(n) % 37]
+    else:
+        pos, _ = ic.make(model, n, 62)
+    check_tree(pos, np.full(n, 1.0 / n, np.float32), 8, 64)
