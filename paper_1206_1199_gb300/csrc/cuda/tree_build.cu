@@ -12,8 +12,8 @@
 // host's direct sums to rounding.
 //
 // Kernels
-//   k_bbox / k_bbox_final   min/max of the positions (order-preserving integer
-//                           keys: exact), then the root cube.
+//   k_bbox                  min/max of the positions (order-preserving integer
+//                           keys: exact); its last block sets the root cube.
 //   k_keys                  grid coordinates and Hilbert key per particle.
 //   k_sort_pass / k_sort_tile  stable LSD radix sort of (key, index), 8 bits
 //                           per pass: one launch per pass with a decoupled
@@ -31,9 +31,10 @@
 //                           centre of mass (FP64, on the particles an FP32
 //                           bound leaves), or the SPH radius bound (FP32);
 //                           chunks of particles, atomic max.
-//   k_records               sources, quadrupoles and walk records of the cells.
-//   k_group_flags           first particle of every group (maximal cells with
+//   k_records               sources, quadrupoles and walk records of the cells,
+//                           first particle of every group (maximal cells with
 //                           at most n_crit particles; larger leaves in chunks).
+//   k_group_sums / k_group_write  the groups in tree order.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -62,6 +63,19 @@ struct Geom {
     double lo[3], S, h, scale;
 };
 
+// What one build keeps in one place on the device: zeroed before the first
+// kernel, copied to the host once after the last (kernels read the counts of
+// the cells and groups here, so that nothing waits for the host in between).
+struct Head {
+    Geom g;
+    int64_t cells, groups;        // totals (cells: also when they exceed the capacity)
+    int32_t lev[kLevels + 4];     // first cell of each level; lev[22]: the number of cells
+    int32_t pcount[kLevels + 1];  // parents per level
+    uint32_t status, stop;        // error bits; more cells than the capacity
+    uint32_t bar, done;           // arrivals: grid barrier of k_parents, blocks of k_bbox
+    uint32_t extra;               // k_bmax's work items of the larger cells
+};
+
 __device__ __forceinline__ long long dkey(double x)
 {
     const long long b = __double_as_longlong(x);
@@ -72,7 +86,7 @@ __device__ __forceinline__ double dval(long long k) { return __longlong_as_doubl
 // ---- bounding box ------------------------------------------------------------
 
 __global__ void __launch_bounds__(256) k_bbox(const double* __restrict__ pos, const float* __restrict__ mass, int64_t n,
-                                              long long* __restrict__ part, uint32_t* __restrict__ status)
+                                              long long* __restrict__ part, Head* __restrict__ head)
 {
     long long lo[3], hi[3];
     for (int a = 0; a < 3; ++a) lo[a] = 0x7fffffffffffffffLL, hi[a] = -lo[a] - 1;
@@ -88,8 +102,9 @@ __global__ void __launch_bounds__(256) k_bbox(const double* __restrict__ pos, co
         const float m = mass[i];
         bad |= !(m > 0.0f) || !isfinite(m);
     }
-    if (bad) atomicOr(status, kTreeBadInput);
+    if (bad) atomicOr(&head->status, kTreeBadInput);
     __shared__ long long s[6][8];
+    __shared__ bool last;
     for (int a = 0; a < 3; ++a) {
         for (int o = 16; o > 0; o >>= 1) {
             const long long t0 = __shfl_xor_sync(kFull, lo[a], o), t1 = __shfl_xor_sync(kFull, hi[a], o);
@@ -108,29 +123,27 @@ __global__ void __launch_bounds__(256) k_bbox(const double* __restrict__ pos, co
             v = threadIdx.x < 3 ? (t < v ? t : v) : (t > v ? t : v);
         }
         part[6 * blockIdx.x + threadIdx.x] = v;
+        __threadfence();
     }
-}
-
-// One block of 256 threads: each thread folds a stride of the block
-// partials, then the warps and the block reduce; thread 0 sets the cube.
-__global__ void __launch_bounds__(256) k_bbox_final(const long long* __restrict__ part, int nb, Geom* __restrict__ g)
-{
-    long long lo[3], hi[3];
+    __syncthreads();
+    // the block that finishes last folds the partials and sets the root cube
+    if (threadIdx.x == 0) last = atomicAdd(&head->done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
     for (int a = 0; a < 3; ++a) lo[a] = 0x7fffffffffffffffLL, hi[a] = -lo[a] - 1;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x)
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
         for (int a = 0; a < 3; ++a) {
-            const long long l = part[6 * b + a], h = part[6 * b + 3 + a];
+            const long long l = __ldcg(part + 6 * b + a), h = __ldcg(part + 6 * b + 3 + a);
             lo[a] = l < lo[a] ? l : lo[a];
             hi[a] = h > hi[a] ? h : hi[a];
         }
-    __shared__ long long s[6][8];
     for (int a = 0; a < 3; ++a)
         for (int o = 16; o > 0; o >>= 1) {
             const long long t0 = __shfl_xor_sync(kFull, lo[a], o), t1 = __shfl_xor_sync(kFull, hi[a], o);
             lo[a] = t0 < lo[a] ? t0 : lo[a];
             hi[a] = t1 > hi[a] ? t1 : hi[a];
         }
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 0)
         for (int a = 0; a < 3; ++a) s[a][w] = lo[a], s[3 + a][w] = hi[a];
     __syncthreads();
@@ -142,6 +155,7 @@ __global__ void __launch_bounds__(256) k_bbox_final(const long long* __restrict_
             hi[a] = s[3 + a][k] > hi[a] ? s[3 + a][k] : hi[a];
         }
     }
+    Geom* g = &head->g;
     double mn[3], mx[3];
     for (int a = 0; a < 3; ++a) mn[a] = dval(lo[a]), mx[a] = dval(hi[a]);
     root_cube(mn, mx, g->lo, &g->S, &g->h);
@@ -667,89 +681,102 @@ __device__ __forceinline__ double widen(float f)
 // records take the quadrupole Q = 3 C - tr(C) I.  GB300's FP64 pipe (1/76 of
 // the FP32 rate) bounds both kernels at large N, latency at small N.
 
+// The end of a cell and, for a leaf (nch = 0), its moments.
+__device__ __forceinline__ void close_cell(int32_t cell, int32_t b, int lvl, int32_t nch,
+                                           const uint64_t* __restrict__ keys, int64_t n, int64_t leaf_size,
+                                           const otoo_src* __restrict__ src, const Cells& c, const Moments& mo)
+{
+    const int sh = 3 * (kLevels - lvl);
+    const uint64_t pre = keys[b] >> sh;
+    int64_t l = nch > 0 ? b + leaf_size : b, hi, step = 1;
+    for (hi = l + step; hi < n && (keys[hi] >> sh) == pre; hi = l + step) {
+        l = hi;
+        step *= 2;
+    }
+    if (hi > n) hi = n;
+    while (hi - l > 1) {
+        const int64_t mid = l + ((hi - l) >> 1);
+        if ((keys[mid] >> sh) == pre)
+            l = mid;
+        else
+            hi = mid;
+    }
+    const int32_t e = (int32_t)hi;
+    c.end[cell] = e;
+    mo.dmax2[cell] = 0ull;
+    if (nch > 0) return;
+    const otoo_src p0 = src[b];
+    double m = widen(p0.m);
+    double* q = mo.q + 6 * (int64_t)cell;
+    double* com = mo.com + 3 * (int64_t)cell;
+    if (e - b == 1) {
+        mo.m[cell] = m;
+        com[0] = p0.x, com[1] = p0.y, com[2] = p0.z;
+        q[0] = q[1] = q[2] = q[3] = q[4] = q[5] = 0.0;
+        mo.b2[cell] = 0.0;
+        return;
+    }
+    double s1[3] = {0, 0, 0}, s2[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll 1
+    for (int32_t i = b + 1; i < e; ++i) {
+        const otoo_src p = src[i];
+        const double mi = widen(p.m);
+        const double dx = p.x - p0.x, dy = p.y - p0.y, dz = p.z - p0.z;
+        const double mx = mi * dx, my = mi * dy, mz = mi * dz;
+        m += mi;
+        s1[0] += mx, s1[1] += my, s1[2] += mz;
+        s2[0] = fma(mx, dx, s2[0]), s2[1] = fma(my, dy, s2[1]), s2[2] = fma(mz, dz, s2[2]);
+        s2[3] = fma(mx, dy, s2[3]), s2[4] = fma(mx, dz, s2[4]), s2[5] = fma(my, dz, s2[5]);
+    }
+    const double inv = 1.0 / m;
+    const double gx = s1[0] * inv, gy = s1[1] * inv, gz = s1[2] * inv;  // com - x0
+    mo.m[cell] = m;
+    com[0] = p0.x + gx;
+    com[1] = p0.y + gy;
+    com[2] = p0.z + gz;
+    const double cxx = fma(-s1[0], gx, s2[0]), cyy = fma(-s1[1], gy, s2[1]), czz = fma(-s1[2], gz, s2[2]);
+    q[0] = cxx, q[1] = cyy, q[2] = czz;
+    q[3] = fma(-s1[0], gy, s2[3]), q[4] = fma(-s1[0], gz, s2[4]), q[5] = fma(-s1[1], gz, s2[5]);
+    mo.b2[cell] = cxx + cyy + czz;
+}
+
 // One thread per cell: the cell's links (children: the consecutive cells from
 // child0 on that name it as their parent; end: the first particle past it, by
 // a galloping search over the keys' leading digits; a cell that splits holds
 // at least leaf_size + 1 particles), and for a leaf its moments.  The
 // reference particle's own terms are zero and are left out (a leaf of leaf size
-// 8 holds 2.7 particles on average): 17 us at N = 4096, 93 us at 2^20, 0.57 ms
-// at 2^23 with leaves of 16, links included.
+// 8 holds 2.7 particles on average): 17 us at N = 4096, 93-97 us at 2^20, 0.57
+// to 0.64 ms at 2^23 with leaves of 16, links included.
 __global__ void __launch_bounds__(128) k_leaves(const int32_t* __restrict__ lev, const uint64_t* __restrict__ keys,
                                                 int64_t n, int64_t leaf_size, const otoo_src* __restrict__ src,
                                                 Cells c, Moments mo, int32_t* __restrict__ plist,
                                                 int32_t* __restrict__ pcount)
 {
     const int32_t n_cell = lev[kLv];
-    for (int32_t cell = blockIdx.x * blockDim.x + threadIdx.x; cell < n_cell; cell += gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); w0 < n_cell;
+         w0 += (int64_t)gridDim.x * blockDim.x) {
+        const bool in = w0 + lane < n_cell;
+        const int32_t cell = (int32_t)(in ? w0 + lane : w0);
         int32_t k = 0;
-        const int32_t c0 = c.child0[cell];
+        const int32_t c0 = in ? c.child0[cell] : 0;
         if (c0 > 0)
             while (k < 8 && c0 + k < n_cell && c.parent[c0 + k] == cell) ++k;
-        c.nchild[cell] = k;
-        const int32_t b = c.begin[cell];
         const int lvl = c.level[cell];
-        if (k > 0) {
-            // one atomic per warp and level (the cells of a warp are nearly
-            // always of one level)
-            const unsigned peers = __match_any_sync(__activemask(), lvl);
-            const int lane = threadIdx.x & 31, lead = __ffs(peers) - 1;
-            int32_t at = 0;
-            if (lane == lead) at = atomicAdd(pcount + lvl, __popc(peers));
-            at = __shfl_sync(peers, at, lead);
-            plist[lev[lvl] + at + __popc(peers & ((1u << lane) - 1u))] = cell;
+        __syncwarp();
+        // parents into their level's list, one atomic per warp and level (a
+        // warp's cells are nearly always of one level)
+        const unsigned peers = __match_any_sync(kFull, k > 0 ? lvl : -1 - lane);
+        const int lead = __ffs(peers) - 1;
+        int32_t at = 0;
+        if (k > 0 && lane == lead) at = atomicAdd(pcount + lvl, __popc(peers));
+        at = __shfl_sync(kFull, at, lead);
+        if (k > 0) plist[lev[lvl] + at + __popc(peers & ((1u << lane) - 1u))] = cell;
+        if (in) {
+            c.nchild[cell] = k;
+            close_cell(cell, c.begin[cell], lvl, k, keys, n, leaf_size, src, c, mo);
         }
-        const int sh = 3 * (kLevels - lvl);
-        const uint64_t pre = keys[b] >> sh;
-        int64_t l = k > 0 ? b + leaf_size : b, hi, step = 1;
-        for (hi = l + step; hi < n && (keys[hi] >> sh) == pre; hi = l + step) {
-            l = hi;
-            step *= 2;
-        }
-        if (hi > n) hi = n;
-        while (hi - l > 1) {
-            const int64_t mid = l + ((hi - l) >> 1);
-            if ((keys[mid] >> sh) == pre)
-                l = mid;
-            else
-                hi = mid;
-        }
-        const int32_t e = (int32_t)hi;
-        c.end[cell] = e;
-        mo.dmax2[cell] = 0ull;
-        if (k > 0) continue;
-        const otoo_src p0 = src[b];
-        double m = widen(p0.m);
-        double* q = mo.q + 6 * (int64_t)cell;
-        double* com = mo.com + 3 * (int64_t)cell;
-        if (e - b == 1) {
-            mo.m[cell] = m;
-            com[0] = p0.x, com[1] = p0.y, com[2] = p0.z;
-            q[0] = q[1] = q[2] = q[3] = q[4] = q[5] = 0.0;
-            mo.b2[cell] = 0.0;
-            continue;
-        }
-        double s1[3] = {0, 0, 0}, s2[6] = {0, 0, 0, 0, 0, 0};
-#pragma unroll 1
-        for (int32_t i = b + 1; i < e; ++i) {
-            const otoo_src p = src[i];
-            const double mi = widen(p.m);
-            const double dx = p.x - p0.x, dy = p.y - p0.y, dz = p.z - p0.z;
-            const double mx = mi * dx, my = mi * dy, mz = mi * dz;
-            m += mi;
-            s1[0] += mx, s1[1] += my, s1[2] += mz;
-            s2[0] = fma(mx, dx, s2[0]), s2[1] = fma(my, dy, s2[1]), s2[2] = fma(mz, dz, s2[2]);
-            s2[3] = fma(mx, dy, s2[3]), s2[4] = fma(mx, dz, s2[4]), s2[5] = fma(my, dz, s2[5]);
-        }
-        const double inv = 1.0 / m;
-        const double gx = s1[0] * inv, gy = s1[1] * inv, gz = s1[2] * inv;  // com - x0
-        mo.m[cell] = m;
-        com[0] = p0.x + gx;
-        com[1] = p0.y + gy;
-        com[2] = p0.z + gz;
-        const double cxx = fma(-s1[0], gx, s2[0]), cyy = fma(-s1[1], gy, s2[1]), czz = fma(-s1[2], gz, s2[2]);
-        q[0] = cxx, q[1] = cyy, q[2] = czz;
-        q[3] = fma(-s1[0], gy, s2[3]), q[4] = fma(-s1[0], gz, s2[4]), q[5] = fma(-s1[1], gz, s2[5]);
-        mo.b2[cell] = cxx + cyy + czz;
+        __syncwarp();
     }
 }
 
@@ -939,13 +966,6 @@ __device__ __forceinline__ float bmax_dist(const float4 cc, const float4 p, floa
     return sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
 }
 
-// Work items, one warp each: warp w < n_cell takes the first kBmaxChunk
-// particles of cell w; warp n_cell + k takes extra chunk k of the cells that
-// hold more (extra_off: exclusive prefix over cells of their chunk counts
-// minus one, so only those few warps search it).  The chunk's largest value
-// goes to the cell by an atomic max on its bits (non-negative floating-point
-// values order like their bit patterns).
-//
 // pk[j] = (x_j, y_j, z_j rounded to FP32, h_j or 0) in tree order,
 // cf[cell] = (com rounded to FP32, e_c).  Rounding a value v to FP32 moves it
 // by at most 2^-24 |v| per coordinate, so |com - x_j| lies within
@@ -960,90 +980,131 @@ __device__ __forceinline__ float bmax_dist(const float4 cc, const float4 p, floa
 //
 // Absolute MAC: the largest squared distance in FP64, as the host computes
 // it; dmax2 holds double bits.  A first FP32 pass finds a lower bound L on
-// the chunk's largest distance; the FP64 distance is then taken only for the
-// particles whose FP32 upper bound reaches L.  That set holds every particle
-// whose FP64 value could be the largest (their exact distances lie within
-// 2^-40 or so of the largest, far inside the bounds' margin), so the result
-// is the same bits as the FP64 maximum over all particles.
-__global__ void k_bmax(int64_t n_items, int32_t n_cell, const int32_t* __restrict__ extra_off,
-                       const otoo_src* __restrict__ src, const float4* __restrict__ pk,
-                       const float4* __restrict__ cf, Cells c, Moments mo, int sph)
+// the largest distance of the lanes' particles; the FP64 distance is then
+// taken only for the particles whose FP32 upper bound reaches L.  That set
+// holds every particle whose FP64 value could be the largest (their exact
+// distances lie within 2^-40 or so of the largest, far inside the bounds'
+// margin), so the result is the same bits as the FP64 maximum over all
+// particles.
+//
+// kW lanes (8 or 32) share the particles [i0, i1) of one cell; the lanes of a
+// warp run the same number of rounds (trips, uniform).  Returns the bits of
+// the kW lanes' maximum in every lane.
+template <int kW>
+__device__ __forceinline__ unsigned long long bmax_of(int64_t i0, int64_t i1, int trips, int j, float4 cc,
+                                                      const double* __restrict__ com,
+                                                      const otoo_src* __restrict__ src,
+                                                      const float4* __restrict__ pk, int sph)
 {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (w >= n_items) return;
-    int32_t cell;
-    int64_t chunk;
-    if (w < n_cell) {
-        cell = (int32_t)w;
-        chunk = 0;
-    } else {
-        const int64_t k = w - n_cell;
-        int32_t l = 0, r = n_cell;  // last cell with extra_off <= k
-        while (r - l > 1) {
-            const int32_t m = l + ((r - l) >> 1);
-            if (extra_off[m] <= k)
-                l = m;
-            else
-                r = m;
-        }
-        cell = l;
-        chunk = 1 + k - extra_off[cell];
-    }
-    const int32_t b = c.begin[cell], e = c.end[cell];
-    const int64_t i0 = b + chunk * kBmaxChunk;
-    const int64_t i1 = i0 + kBmaxChunk < e ? i0 + kBmaxChunk : e;
-    const float4 cc = cf[cell];
-    if (sph) {
-        float vmax = 0.f;
-        for (int64_t i = i0 + lane; i < i1; i += 32) {
+    float lo = 0.f;
+    for (int t = 0; t < trips; ++t) {
+        const int64_t i = i0 + (int64_t)t * kW + j;
+        if (i < i1) {
             const float4 p = pk[i];
             float ej;
             const float d = bmax_dist(cc, p, ej);
-            vmax = fmaxf(vmax, d + (p.w + ej));
+            lo = fmaxf(lo, sph ? d + (p.w + ej) : d * (1.0f - 0x1p-20f) - 2.0f * (ej + cc.w));
         }
-        for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(kFull, vmax, o));
-        if (lane == 0)
-            atomicMax(mo.dmax2 + cell, (unsigned long long)__float_as_uint((vmax + cc.w) * (1.0f + 0x1p-20f)));
-        return;
     }
-    float lo = 0.f;
-    for (int64_t i = i0 + lane; i < i1; i += 32) {
-        float ej;
-        const float d = bmax_dist(cc, pk[i], ej);
-        lo = fmaxf(lo, d * (1.0f - 0x1p-20f) - 2.0f * (ej + cc.w));
-    }
-    for (int o = 16; o > 0; o >>= 1) lo = fmaxf(lo, __shfl_xor_sync(kFull, lo, o));
-    const double cx = mo.com[3 * cell], cy = mo.com[3 * cell + 1], cz = mo.com[3 * cell + 2];
+    __syncwarp();
+#pragma unroll
+    for (int o = kW / 2; o > 0; o >>= 1) lo = fmaxf(lo, __shfl_xor_sync(kFull, lo, o));
+    if (sph) return (unsigned long long)__float_as_uint((lo + cc.w) * (1.0f + 0x1p-20f));
+    const double cx = com[0], cy = com[1], cz = com[2];
     unsigned long long d2max = 0;
-    for (int64_t i = i0 + lane; i < i1; i += 32) {
-        float ej;
-        const float d = bmax_dist(cc, pk[i], ej);
-        if (!((d + 2.0f * (ej + cc.w)) * (1.0f + 0x1p-20f) < lo)) {  // NaN bounds count as candidates
+    for (int t = 0; t < trips; ++t) {
+        const int64_t i = i0 + (int64_t)t * kW + j;
+        bool near = false;
+        if (i < i1) {
+            float ej;
+            const float d = bmax_dist(cc, pk[i], ej);
+            near = !((d + 2.0f * (ej + cc.w)) * (1.0f + 0x1p-20f) < lo);  // NaN bounds count as candidates
+        }
+        if (near) {
             const otoo_src p = src[i];
             const double dx = cx - p.x, dy = cy - p.y, dz = cz - p.z;
             const unsigned long long v = (unsigned long long)__double_as_longlong(dx * dx + dy * dy + dz * dz);
             d2max = v > d2max ? v : d2max;
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
+    __syncwarp();
+#pragma unroll
+    for (int o = kW / 2; o > 0; o >>= 1) {
         const unsigned long long v = __shfl_xor_sync(kFull, d2max, o);
         d2max = v > d2max ? v : d2max;
     }
-    if (lane == 0) atomicMax(mo.dmax2 + cell, d2max);
+    return d2max;
 }
 
-// Chunks of kBmaxChunk particles beyond the first, per cell, and the cell's
-// FP32 centre of mass with its rounding bound e_c (k_bmax).
-__global__ void k_chunks(int32_t n_cell, Cells c, const double* __restrict__ com, int32_t* __restrict__ extra,
-                         float4* __restrict__ cf)
+// Cells of up to kBmaxSmall particles, four per warp (eight lanes each: an
+// FP64 instruction on the narrow pipe serves four cells, where one warp per
+// cell left most of its lanes idle); larger cells as the work items
+// items[0, head->extra) = (cell, chunk of kBmaxChunk particles), one warp each,
+// folded into the cell by an atomic max on the bits (non-negative
+// floating-point values order like their bit patterns).
+constexpr int kBmaxSmall = 64;
+
+__global__ void __launch_bounds__(256) k_bmax(const Head* __restrict__ head, const int2* __restrict__ items,
+                                              const otoo_src* __restrict__ src, const float4* __restrict__ pk,
+                                              const float4* __restrict__ cf, Cells c, Moments mo, int sph)
 {
-    const int32_t cell = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= n_cell) return;
-    const int32_t cnt = c.end[cell] - c.begin[cell];
-    extra[cell] = (cnt + kBmaxChunk - 1) / kBmaxChunk - 1;
-    const float x = (float)com[3 * cell], y = (float)com[3 * cell + 1], z = (float)com[3 * cell + 2];
-    cf[cell] = make_float4(x, y, z, 0x1p-23f * (fabsf(x) + fabsf(y) + fabsf(z)));
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int32_t n_cell = head->lev[kLv];
+    const int64_t nbig = head->extra, n_units = nbig + ((int64_t)n_cell + 3) / 4;
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < n_units; w += nwarp) {
+        if (w < nbig) {
+            const int2 it = items[w];
+            const int64_t i0 = c.begin[it.x] + (int64_t)it.y * kBmaxChunk, e = c.end[it.x];
+            const int64_t i1 = i0 + kBmaxChunk < e ? i0 + kBmaxChunk : e;
+            const unsigned long long v = bmax_of<32>(i0, i1, (int)((i1 - i0 + 31) / 32), lane, cf[it.x],
+                                                     mo.com + 3 * (int64_t)it.x, src, pk, sph);
+            if (lane == 0) atomicMax(mo.dmax2 + it.x, v);
+        } else {
+            const int64_t k = 4 * (w - nbig) + (lane >> 3);
+            const int32_t cell = (int32_t)(k < n_cell ? k : n_cell - 1);
+            const int32_t b = c.begin[cell], e = c.end[cell];
+            // a single particle is its own centre of mass: distance 0
+            const bool on = k < n_cell && e - b <= kBmaxSmall && (sph || e - b > 1);
+            const int trips = __reduce_max_sync(kFull, on ? (e - b + 7) / 8 : 0);
+            const unsigned long long v = bmax_of<8>(b, on ? e : b, trips, lane & 7, cf[cell],
+                                                    mo.com + 3 * (int64_t)cell, src, pk, sph);
+            if (on && (lane & 7) == 0) mo.dmax2[cell] = v;
+        }
+    }
+}
+
+// The work items of the cells of more than kBmaxSmall particles (any order;
+// one atomic per warp), and every cell's FP32 centre of mass with its rounding
+// bound e_c.
+__global__ void __launch_bounds__(128) k_chunks(Head* __restrict__ head, Cells c, const double* __restrict__ com,
+                                                int2* __restrict__ items, float4* __restrict__ cf)
+{
+    const int32_t n_cell = head->lev[kLv];
+    const int lane = threadIdx.x & 31;
+    for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); w0 < n_cell;
+         w0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t cell = w0 + lane;
+        const bool in = cell < n_cell;
+        const int32_t cnt = in ? c.end[cell] - c.begin[cell] : 0;
+        const int32_t more = cnt > kBmaxSmall ? (cnt + kBmaxChunk - 1) / kBmaxChunk : 0;
+        int32_t incl = more;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t t = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += t;
+        }
+        uint32_t at = 0;
+        const int32_t all = __shfl_sync(kFull, incl, 31);
+        if (lane == 0 && all > 0) at = atomicAdd(&head->extra, (uint32_t)all);
+        at = __shfl_sync(kFull, at, 0) + (uint32_t)(incl - more);
+        for (int32_t k = 0; k < more; ++k) items[at + k] = make_int2((int)cell, k);
+        if (in) {
+            const float x = (float)com[3 * cell], y = (float)com[3 * cell + 1], z = (float)com[3 * cell + 2];
+            cf[cell] = make_float4(x, y, z, 0x1p-23f * (fabsf(x) + fabsf(y) + fabsf(z)));
+        }
+        __syncwarp();
+    }
 }
 
 // Tree-order FP32 positions with each particle's SPH radius, or 0 without h
@@ -1061,18 +1122,28 @@ __global__ void k_bpack(int64_t n, const otoo_src* __restrict__ src, const float
 
 struct RecArgs {
     int64_t n_part;
-    int32_t n_cell, use_quad, mac, n_crit;
+    int32_t use_quad, mac, n_crit;
     double delta, m_limit;
 };
 
-__global__ void k_records(RecArgs ra, const Geom* __restrict__ g, Cells c, Moments mo, const int32_t* __restrict__ gq,
-                          otoo_src* __restrict__ src, otoo_quad* __restrict__ quad, otoo_wcell* __restrict__ wc,
-                          otoo_wcell64* __restrict__ wc64, int32_t* __restrict__ level_out)
+// The records of one cell, and the groups that start in it: a group starts at
+// the first particle of each maximal cell with at most n_crit particles, and
+// every n_crit particles inside a leaf that holds more (one bit per particle
+// in bits).
+__device__ __forceinline__ void cell_records(const RecArgs& ra, int32_t cell, const Geom* __restrict__ g,
+                                             const Cells& c, const Moments& mo, const int32_t* __restrict__ gq,
+                                             otoo_src* __restrict__ src, otoo_quad* __restrict__ quad,
+                                             otoo_wcell* __restrict__ wc, otoo_wcell64* __restrict__ wc64,
+                                             int32_t* __restrict__ level_out, uint32_t* __restrict__ bits)
 {
-    const int32_t cell = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= ra.n_cell) return;
     const int L = c.level[cell];
-    const int32_t b = c.begin[cell];
+    const int32_t b = c.begin[cell], e = c.end[cell], par = c.parent[cell];
+    if (par < 0 || c.end[par] - c.begin[par] > ra.n_crit) {
+        if (e - b <= ra.n_crit)
+            atomicOr(bits + (b >> 5), 1u << (b & 31));
+        else if (c.nchild[cell] == 0)
+            for (int64_t k = b; k < e; k += ra.n_crit) atomicOr(bits + (k >> 5), 1u << (k & 31));
+    }
     const int sh = kLevels - L;
     const double side = cube_side(g->h, L);
     double lo[3], gc[3], com[3];
@@ -1081,7 +1152,7 @@ __global__ void k_records(RecArgs ra, const Geom* __restrict__ g, Cells c, Momen
         const int64_t org = sh >= kLevels ? 0 : (gcoord >> sh) << sh;
         lo[a] = cube_lo(g->lo[a], org, g->h);
         gc[a] = cube_centre(lo[a], side);
-        com[a] = mo.com[3 * cell + a];
+        com[a] = mo.com[3 * (int64_t)cell + a];
     }
     const double m = mo.m[cell];
     otoo_src s;
@@ -1114,7 +1185,7 @@ __global__ void k_records(RecArgs ra, const Geom* __restrict__ g, Cells c, Momen
     w.nchild = c.nchild[cell];
     w.child0 = w.nchild > 0 ? c.child0[cell] : 0;
     w.begin = b;
-    w.end = c.end[cell];
+    w.end = e;
     w.rb = (float)rb;
     wc[cell] = w;
     otoo_wcell64 w64;
@@ -1126,35 +1197,89 @@ __global__ void k_records(RecArgs ra, const Geom* __restrict__ g, Cells c, Momen
     level_out[cell] = L;
 }
 
-// A group starts at the first particle of each maximal cell with at most
-// n_crit particles, and every n_crit particles inside a leaf that holds more.
-__global__ void k_group_flags(RecArgs ra, Cells c, int32_t* __restrict__ flag)
+__global__ void __launch_bounds__(128) k_records(RecArgs ra, const Head* __restrict__ head, Cells c, Moments mo,
+                                                 const int32_t* __restrict__ gq, otoo_src* __restrict__ src,
+                                                 otoo_quad* __restrict__ quad, otoo_wcell* __restrict__ wc,
+                                                 otoo_wcell64* __restrict__ wc64, int32_t* __restrict__ level_out,
+                                                 uint32_t* __restrict__ bits)
 {
-    const int32_t cell = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= ra.n_cell) return;
-    const int32_t b = c.begin[cell], e = c.end[cell], p = c.parent[cell];
-    const int32_t cnt = e - b;
-    const bool parent_big = p < 0 || c.end[p] - c.begin[p] > ra.n_crit;
-    if (!parent_big) return;
-    if (cnt <= ra.n_crit) {
-        flag[b] = 1;
-    } else if (c.nchild[cell] == 0) {
-        for (int32_t k = b; k < e; k += ra.n_crit) flag[k] = 1;
+    const int32_t n_cell = head->lev[kLv];
+    for (int32_t cell = blockIdx.x * blockDim.x + threadIdx.x; cell < n_cell; cell += gridDim.x * blockDim.x)
+        cell_records(ra, cell, &head->g, c, mo, gq, src, quad, wc, wc64, level_out, bits);
+}
+
+// Groups in tree order from their first particles' bits: words of 32 particles,
+// kGroupWords words per block.  k_group_sums counts a block's bits, k_group_write
+// adds up the blocks before its own and writes its groups; a group ends where
+// the next bit is set.  Two launches and n / 8 bytes, against a flag per
+// particle, a copy, a three-launch scan, a compaction and a pass for the counts
+// (seven launches).
+constexpr int kGroupWords = 1024;
+
+__global__ void __launch_bounds__(256) k_group_sums(const uint32_t* __restrict__ bits, int64_t nw,
+                                                     int32_t* __restrict__ bsum)
+{
+    __shared__ int32_t s[8];
+    int32_t v = 0;
+    for (int k = 0; k < kGroupWords / 256; ++k) {
+        const int64_t i = (int64_t)blockIdx.x * kGroupWords + k * 256 + threadIdx.x;
+        if (i < nw) v += __popc(bits[i]);
+    }
+    v = __reduce_add_sync(kFull, v);
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < 8; ++k) v += s[k];
+        bsum[blockIdx.x] = v;
     }
 }
 
-__global__ void k_group_write(int64_t n, const int32_t* __restrict__ flag, const int32_t* __restrict__ gidx,
-                              int32_t* __restrict__ first)
+__global__ void __launch_bounds__(256) k_group_write(const uint32_t* __restrict__ bits, int64_t nw, int64_t n,
+                                                      const int32_t* __restrict__ bsum, int32_t* __restrict__ first,
+                                                      int32_t* __restrict__ count, Head* __restrict__ head,
+                                                      uint32_t* __restrict__ status_out)
 {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n && flag[k]) first[gidx[k]] = (int32_t)k;
-}
-
-__global__ void k_group_count(int64_t n, int32_t G, const int32_t* __restrict__ first, int32_t* __restrict__ count)
-{
-    const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= G) return;
-    count[g] = (g + 1 < G ? first[g + 1] : (int32_t)n) - first[g];
+    __shared__ int32_t s[2][8];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    // groups of the blocks before this one
+    int32_t v = 0;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += 256) v += bsum[b];
+    v = __reduce_add_sync(kFull, v);
+    // this block's words, four consecutive ones per thread
+    const int64_t i0 = (int64_t)blockIdx.x * kGroupWords + 4 * threadIdx.x;
+    uint32_t m[4];
+    int32_t mine = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        m[k] = i0 + k < nw ? bits[i0 + k] : 0u;
+        mine += __popc(m[k]);
+    }
+    int32_t incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) s[0][w] = incl;
+    if (lane == 0) s[1][w] = v;
+    __syncthreads();
+    int32_t g = incl - mine;
+    for (int k = 0; k < 8; ++k) g += s[1][k] + (k < w ? s[0][k] : 0);
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 255) {
+        head->groups = g + mine;
+        status_out[0] = head->status;
+    }
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k)
+        for (uint32_t x = m[k]; x; x &= x - 1u, ++g) {
+            const int64_t p = 32 * (i0 + k) + (__ffs(x) - 1);
+            // the next bit: in this word, or in the first word after it that has one
+            uint32_t up = x & (x - 1u);
+            int64_t j = i0 + k;
+            while (!up && ++j < nw) up = bits[j];
+            first[g] = (int32_t)p;
+            count[g] = (int32_t)((up ? 32 * j + (__ffs(up) - 1) : n) - p);
+        }
 }
 
 // ---- scans (exclusive, in place, int32) --------------------------------------------
@@ -1277,8 +1402,8 @@ int scan32(int32_t* a, int64_t n, int64_t* bsum, int64_t* total, cudaStream_t s)
 
 // Scratch layout (byte offsets, each part 256-byte aligned).
 struct Layout {
-    size_t keys0, keys1, vals0, vals1, hist, bsum, part, geom, gq, cells[6], mom_m, mom_com, mom_q, mom_b2,
-        mom_dmax, dig, cnt, flag, tot, lev, total;
+    size_t keys0, keys1, vals0, vals1, head, bits, hist, bsum, part, gq, cells[6], mom_m, mom_com, mom_q, mom_b2,
+        mom_dmax, dig, total;
 };
 
 size_t up(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -1293,18 +1418,21 @@ Layout layout(int64_t n, int64_t cap)
         return at;
     };
     const int64_t nblk = (n + kLvTile - 1) / kLvTile;
-    const int64_t big = n > cap ? n : cap;
     l.keys0 = take(8 * n);
     l.keys1 = take(8 * n);
     l.vals0 = take(4 * n);
     l.vals1 = take(4 * n);
+    // zeroed together before the first kernel: the head, a bit per particle,
+    // the sort's counts and first words
+    l.head = take(sizeof(Head));
+    l.bits = take(4 * ((n + 31) / 32));
     // the sort's counts, tickets and two sets of published words; later the
     // cells' counts (kLv per tile of kLvTile)
     const int64_t ntile = (n + kSortTile - 1) / kSortTile;
     l.hist = take(4 * std::max<int64_t>(256 * (9 + 2 * ntile), kLv * nblk));
-    l.bsum = take(8 * ((256 * nblk + 8 * big) / kScanThreads + 8));
+    // block sums of the cells' scan, later the groups' per block
+    l.bsum = take(8 * ((256 * nblk + n) / kScanThreads + 8));
     l.part = take(8 * 6 * 1024);
-    l.geom = take(sizeof(Geom));
     l.gq = take(12 * n);
     for (int k = 0; k < 6; ++k) l.cells[k] = take(4 * cap);
     l.mom_m = take(8 * cap);
@@ -1313,11 +1441,6 @@ Layout layout(int64_t n, int64_t cap)
     l.mom_b2 = take(8 * cap);
     l.mom_dmax = take(8 * cap);
     l.dig = take(32 * cap);
-    l.cnt = take(4 * (big + 1));
-    l.flag = take(4 * (n + 1));
-    l.tot = take(64);
-    l.lev = take(4 * 64);  // level bounds, then the stop word; word 32: the grid barrier;
-                           // words 33..: parents per level
     l.total = o;
     return l;
 }
@@ -1362,7 +1485,10 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     int32_t* hist = reinterpret_cast<int32_t*>(base + ly.hist);
     int64_t* bsum = reinterpret_cast<int64_t*>(base + ly.bsum);
     long long* part = reinterpret_cast<long long*>(base + ly.part);
-    Geom* geom = reinterpret_cast<Geom*>(base + ly.geom);
+    Head* head = reinterpret_cast<Head*>(base + ly.head);
+    Geom* geom = &head->g;
+    uint32_t* bits = reinterpret_cast<uint32_t*>(base + ly.bits);
+    const int64_t nw = (n + 31) / 32;
     int32_t* gq = reinterpret_cast<int32_t*>(base + ly.gq);
     Cells c;
     c.begin = reinterpret_cast<int32_t*>(base + ly.cells[0]);
@@ -1378,26 +1504,21 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     mo.b2 = reinterpret_cast<double*>(base + ly.mom_b2);
     mo.dmax2 = reinterpret_cast<unsigned long long*>(base + ly.mom_dmax);
     int32_t* dig = reinterpret_cast<int32_t*>(base + ly.dig);
-    int32_t* cnt = reinterpret_cast<int32_t*>(base + ly.cnt);
-    int32_t* flag = reinterpret_cast<int32_t*>(base + ly.flag);
-    int64_t* tot = reinterpret_cast<int64_t*>(base + ly.tot);
-    uint32_t* status = t->status;
-
-    // root cube, keys, sort
-    CUDA_TRY(cudaMemsetAsync(status, 0, 2 * sizeof(uint32_t), s));
-    const int nbb = (int)std::min<int64_t>(1024, (n + 255) / 256);
-    k_bbox<<<nbb, 256, 0, s>>>(pos, mass, n, part, status);
-    k_bbox_final<<<1, 256, 0, s>>>(part, nbb, geom);
+    uint32_t* status = &head->status;
     int dev = 0, sms = 0;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+
+    // root cube, keys, sort
     const int nblk = (int)((n + kLvTile - 1) / kLvTile);
     const int ntile = (int)((n + kSortTile - 1) / kSortTile);
     // digit counts and tickets of the eight passes, then the first pass's words
-    int32_t* ghist = reinterpret_cast<int32_t*>(base + ly.hist);
+    int32_t* ghist = hist;
     uint32_t* ticket = reinterpret_cast<uint32_t*>(ghist + 8 * 256);
     uint32_t* look[2] = {ticket + 256, ticket + 256 + (size_t)256 * ntile};
-    CUDA_TRY(cudaMemsetAsync(ghist, 0, 4 * (8 * 256 + 256 + (size_t)256 * ntile), s));
+    CUDA_TRY(cudaMemsetAsync(head, 0, ly.hist - ly.head + 4 * (8 * 256 + 256 + (size_t)256 * ntile), s));
+    const int nbb = (int)std::min<int64_t>(1024, (n + 255) / 256);
+    k_bbox<<<nbb, 256, 0, s>>>(pos, mass, n, part, head);
     k_keys<<<(unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)sms * 8), 256, 0, s>>>(pos, n, geom, keys[0], ghist);
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortShared)));
@@ -1416,22 +1537,12 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     k_permute<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(pos, mass, vals[cur], n, geom, t->src, t->perm, gq,
                                                           status);
     CUDA_TRY(cudaGetLastError());
-    uint32_t st = 0;
-    CUDA_TRY(cudaMemcpyAsync(&st, status, sizeof(st), cudaMemcpyDeviceToHost, s));
-    Geom hg;
-    CUDA_TRY(cudaMemcpyAsync(&hg, geom, sizeof(hg), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    if (st & kTreeBadInput) return set_error(OTOO_EINVAL, "otoo_devtree_build: non-finite position or mass <= 0");
-    if (st & kTreeStuck) return set_error(OTOO_EDEVICE, "otoo_devtree_build: a wait between blocks ran into its limit");
-    if (st & kTreeBadSort) return set_error(OTOO_EDEVICE, "otoo_devtree_build: sort produced an invalid order");
     const uint64_t* skeys = keys[cur];
 
     // cells; the unsorted copy of the keys is dead, its memory holds the
     // particles' levels (2 n bytes) and the windows of large leaf sizes
     // (2 (n + leaf_size) bytes, leaf_size < n)
-    int32_t* lev = reinterpret_cast<int32_t*>(base + ly.lev);
-    uint32_t* stop = reinterpret_cast<uint32_t*>(lev + kLevels + 4);
-    CUDA_TRY(cudaMemsetAsync(lev, 0, 4 * 64, s));
+    int32_t* lev = head->lev;
     uint16_t* lv = reinterpret_cast<uint16_t*>(keys[cur ^ 1]);
     const uint8_t* win = nullptr;
     int64_t span = 1;
@@ -1448,80 +1559,72 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     k_levels<<<nblk, kLvThreads, 0, s>>>(skeys, n, leaf, win, span, lv, hist);
     CUDA_TRY(cudaGetLastError());
     {
-        const int r = scan32(hist, (int64_t)kLv * nblk, bsum, tot, s);
+        const int r = scan32(hist, (int64_t)kLv * nblk, bsum, &head->cells, s);
         if (r) return r;
     }
-    k_cells<<<nblk, kLvThreads, 0, s>>>(n, lv, hist, tot, cap, c, lev, stop);
+    k_cells<<<nblk, kLvThreads, 0, s>>>(n, lv, hist, &head->cells, cap, c, lev, &head->stop);
     CUDA_TRY(cudaGetLastError());
-    int32_t hlev[kLevels + 4];
-    uint32_t hstop = 0;
-    CUDA_TRY(cudaMemcpyAsync(hlev, lev, sizeof(hlev), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaMemcpyAsync(&hstop, stop, sizeof(hstop), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    if (hstop) {
-        t->n_cell = -1;
-        return set_error(OTOO_ENOMEM, "otoo_devtree_build: more than cap_cell = %lld cells", (long long)cap);
-    }
-    // level L holds [hlev[L], hlev[L + 1]); the last non-empty level is the depth
-    int depth = 0;
-    for (int L = 0; L <= kLevels; ++L)
-        if (hlev[L + 1] > hlev[L]) depth = L;
-    const int32_t n_cell = hlev[kLv];
 
-    // links, leaves, then the parents level by level, deepest first
-    int32_t* pcount = lev + 33;  // one count per level
-    k_leaves<<<(unsigned)((n_cell + 127) / 128), 128, 0, s>>>(lev, skeys, n, leaf, t->src, c, mo, dig, pcount);
-    if (depth > 0) {
-        uint32_t* bar = reinterpret_cast<uint32_t*>(lev) + 32;
+    // links, leaves, then the parents level by level (grid-stride over the
+    // cells: their number is on the device)
+    const unsigned cg = (unsigned)std::min<int64_t>((cap + 127) / 128, (int64_t)sms * 16);
+    int32_t* pcount = head->pcount;
+    k_leaves<<<cg, 128, 0, s>>>(lev, skeys, n, leaf, t->src, c, mo, dig, pcount);
+    if (n > leaf) {
+        uint32_t* bar = &head->bar;
         void* args[] = {&lev, &c, &mo, &dig, &pcount, &bar, &status};
-        // one block per SM at most, no more than the widest level could use
-        const unsigned pg = (unsigned)std::min<int64_t>(sms, (n_cell + 63) / 64);
+        const unsigned pg = (unsigned)std::min<int64_t>(sms, (cap + 63) / 64);  // at most one block per SM
         CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_parents, dim3(pg), dim3(512), args, 0, s));
     }
     CUDA_TRY(cudaGetLastError());
     const bool sph = t->mac == OTOO_MAC_SPH;
     if (t->mac == OTOO_MAC_SW || sph) {
-        // The sorted keys and the expansion digits are dead once the cells
-        // exist: keys0..keys1 (two adjacent 256-byte-aligned parts of 8 n
-        // bytes) hold the FP32 particles, dig (32 cap bytes) the FP32 centres.
+        // The sorted keys, the sort's values and the parents' lists are dead
+        // once the moments exist: keys0..keys1 (two adjacent 256-byte-aligned
+        // parts of 8 n bytes) hold the FP32 particles, vals0..vals1 the larger
+        // cells' work items (8 bytes each; a level has at most n / 64 cells of
+        // more than 64 particles and n / 2048 further chunks, 22 levels: below
+        // 3 n bytes of 8 n), dig (32 cap bytes) the FP32 centres.
         float4* pk = reinterpret_cast<float4*>(base + ly.keys0);
         float4* cf = reinterpret_cast<float4*>(dig);
-        k_chunks<<<(unsigned)((n_cell + 255) / 256), 256, 0, s>>>(n_cell, c, mo.com, cnt, cf);
+        int2* extra = reinterpret_cast<int2*>(base + ly.vals0);
+        k_chunks<<<cg, 128, 0, s>>>(head, c, mo.com, extra, cf);
         k_bpack<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, t->src, sph ? t->h_sph : nullptr, t->perm, pk);
-        const int r = scan32(cnt, n_cell, bsum, tot, s);
-        if (r) return r;
-        int64_t n_extra = 0;
-        CUDA_TRY(cudaMemcpyAsync(&n_extra, tot, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        CUDA_TRY(cudaStreamSynchronize(s));
-        const int64_t n_items = n_cell + n_extra;
-        k_bmax<<<(unsigned)((n_items * 32 + 255) / 256), 256, 0, s>>>(n_items, n_cell, cnt, t->src, pk, cf, c, mo,
-                                                                      sph ? 1 : 0);
+        k_bmax<<<(unsigned)std::min<int64_t>((cap + 31) / 32, (int64_t)sms * 8), 256, 0, s>>>(
+            head, extra, t->src, pk, cf, c, mo, sph ? 1 : 0);
         CUDA_TRY(cudaGetLastError());
     }
     RecArgs ra;
     ra.n_part = n;
-    ra.n_cell = n_cell;
     ra.use_quad = t->use_quad ? 1 : 0;
     ra.mac = t->mac;
     ra.n_crit = t->n_crit;
     ra.delta = t->delta;
     ra.m_limit = t->m_limit;
-    k_records<<<(unsigned)((n_cell + 127) / 128), 128, 0, s>>>(ra, geom, c, mo, gq, t->src, t->quad, t->cell,
-                                                               t->cell64, t->cell_level);
+    k_records<<<cg, 128, 0, s>>>(ra, head, c, mo, gq, t->src, t->quad, t->cell, t->cell64, t->cell_level, bits);
     // groups
-    CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(int32_t) * (size_t)n, s));
-    k_group_flags<<<(unsigned)((n_cell + 255) / 256), 256, 0, s>>>(ra, c, flag);
-    CUDA_TRY(cudaMemcpyAsync(cnt, flag, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s));
-    const int r = scan32(cnt, n, bsum, tot, s);
-    if (r) return r;
-    k_group_write<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, flag, cnt, t->group_first);
-    int64_t G = 0;
-    CUDA_TRY(cudaMemcpyAsync(&G, tot, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaMemcpyAsync(&st, status, sizeof(st), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
-    if (st & kTreeStuck) return set_error(OTOO_EDEVICE, "otoo_devtree_build: a wait between blocks ran into its limit");
-    k_group_count<<<(unsigned)((G + 255) / 256), 256, 0, s>>>(n, (int32_t)G, t->group_first, t->group_count);
+    int32_t* gsum = reinterpret_cast<int32_t*>(bsum);
+    const unsigned gg = (unsigned)((nw + kGroupWords - 1) / kGroupWords);
+    k_group_sums<<<gg, 256, 0, s>>>(bits, nw, gsum);
+    k_group_write<<<gg, 256, 0, s>>>(bits, nw, n, gsum, t->group_first, t->group_count, head, t->status);
     CUDA_TRY(cudaGetLastError());
+    Head h;
+    CUDA_TRY(cudaMemcpyAsync(&h, head, sizeof(h), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(cudaStreamSynchronize(s));
+    if (h.status & kTreeBadInput) return set_error(OTOO_EINVAL, "otoo_devtree_build: non-finite position or mass <= 0");
+    if (h.status & kTreeStuck) return set_error(OTOO_EDEVICE, "otoo_devtree_build: a wait between blocks ran into its limit");
+    if (h.status & kTreeBadSort) return set_error(OTOO_EDEVICE, "otoo_devtree_build: sort produced an invalid order");
+    if (h.stop) {
+        t->n_cell = -1;
+        return set_error(OTOO_ENOMEM, "otoo_devtree_build: more than cap_cell = %lld cells", (long long)cap);
+    }
+    // level L holds [lev[L], lev[L + 1]); the last non-empty level is the depth
+    int depth = 0;
+    for (int L = 0; L <= kLevels; ++L)
+        if (h.lev[L + 1] > h.lev[L]) depth = L;
+    const Geom& hg = h.g;
+    const int32_t n_cell = h.lev[kLv];
+    const int64_t G = h.groups;
     t->n_cell = n_cell;
     t->n_groups = G;
     t->depth = depth;

@@ -44,3 +44,22 @@ def test_order_across_sort_tiles(n, model):
     else:
         pos, _ = ic.make(model, n, 62)
     check_tree(pos, np.full(n, 1.0 / n, np.float32), 8, 64)
+
+
+@pytest.mark.parametrize("mac", ["sw", "sph"])
+def test_repeated_builds_are_bit_equal(mac):
+    # cells of 1, of a few, of more than 64 and of more than 2048 particles
+    # (the forms of the radius pass), built many times: the same records
+    import torch
+
+    from paper_1206_1199_gb300 import system as S
+    pos, mass = ic.hernquist(30000, 53)
+    p, m = torch.from_numpy(pos).cuda(), torch.from_numpy(mass).cuda()
+    h = torch.from_numpy(ic.sph_radii(pos, mass, 64, "hernquist")).cuda() if mac == "sph" else None
+    ref = None
+    for _ in range(200):
+        dt = S.DeviceTree.build(p, m, 8, 64, True, "cuda", mac, 1e-5 if mac == "sw" else 0.0, 0.0, h_sph=h)
+        got = [dt.bufs[k].clone() for k in ("cell", "cell64", "first", "count")]
+        if ref is None:
+            ref = got
+        assert all(torch.equal(a, b) for a, b in zip(ref, got))
