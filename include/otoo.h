@@ -385,7 +385,12 @@ int64_t otoo_force_static_capacity(void);
    errors:  for each target t, i = targets[t] (an index into src),
      accel[t] = sum_{j != i} m_j r / (r^2 + eps2)^(3/2),
      pot[t]   = -sum_{j != i} m_j / (r^2 + eps2)^(1/2),   r = x_j - x_i,
-   over the n_src sources src[0, n_src) (pass the particles only).
+   over the n_src sources src[0, n_src) (pass the particles only).  From 65536
+   sources on, pairs are evaluated in two-float arithmetic (relative error of a
+   pair about 2^-47, unbiased; sums in three floats and FP64), whose sums are
+   closer to the exact ones than FP64 pairs summed one after another; systems
+   whose softening is below 2^-30 of the largest coordinate, or whose scale
+   leaves the FP32 exponents, take FP64 pairs at every size.
    Device arrays: src [n_src], targets [n_tgt] int64, accel [n_tgt][3],
    pot [n_tgt], scratch >= 4 * otoo_direct_chunks(n_src, n_tgt) * n_tgt
    doubles, status one uint32 (bit 2 set when a target index is out of
