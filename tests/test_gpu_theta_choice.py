@@ -18,18 +18,16 @@ def every_angle(net, feats, count, grid, target, theta0, fallback):
     with np.errstate(all="ignore"):
         y = net.predict(rows).reshape(g, k)
     th, tg = net.learned_theta(feats, count, grid, target, theta0, fallback)
-    want = np.full(g, np.float32(grid[0]))
-    for i in range(g):
-        ok = [np.float32(grid[j]) for j in range(k) if y[i, j] <= tg[i]]
-        if ok:
-            want[i] = max(want[i], max(ok))
-        if np.isnan(tg[i]) or not np.isfinite(y[i]).all():
-            want[i] = fallback
+    gv = np.asarray(grid, np.float32)
+    with np.errstate(invalid="ignore"):
+        ok = y <= tg[:, None]
+    want = np.maximum(np.where(ok, gv[None], gv[0]).max(1), gv[0])
+    want[np.isnan(tg) | ~np.isfinite(y).all(1)] = fallback
     return th, want
 
 
 @pytest.mark.parametrize("grid", [(0.7,), (0.5, 0.9), tuple(0.3 + 0.1 * k for k in range(13)), (0.9, 0.4, 1.2, 0.4)])
-@pytest.mark.parametrize("n", [1, 63, 64, 65, 500])
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 500, 9501, 38001])
 @pytest.mark.parametrize("case", ["plain", "large_weight", "large_input", "nan_weight"])
 def test_choice_equals_the_evaluation_of_every_angle(grid, n, case):
     L.load()
