@@ -78,16 +78,18 @@ typedef struct otoo_params {
 
 typedef struct otoo_tune {
     int32_t block;                 /* threads per CTA: 64, 128 or 256 (the FP32 form runs
-                                      one independent work item per warp; block, iblock
-                                      and tile must name a compiled variant) */
+                                      one independent work item per warp, or, with few items,
+                                      one per CTA of 128 threads with the same results;
+                                      block, iblock and tile must name a compiled variant) */
     int32_t iblock;                /* target particles per thread: 1, 2 or 4; a work item
                                       holds at most 32 * iblock targets */
     int32_t tile;                  /* list entries per staged tile: 64, 128 or 256 (FP32
                                       form; the FP64 form stages 128 entries per tile) */
     int32_t split;                 /* max list entries per work item (>= 32) */
     int32_t ctas_per_sm;           /* resident CTAs per SM for the persistent grid (0 = auto) */
-    int32_t packed;                /* FP32 form: 1 = pairs of list entries evaluated with packed
-                                      two-wide FP32 instructions, 0 = one entry at a time */
+    int32_t packed;                /* FP32 form: selects the compiled variants (block, iblock,
+                                      tile) that a tuning may name; both 0 and 1 evaluate pairs
+                                      of list entries with packed two-wide FP32 instructions */
 } otoo_tune;
 
 /* ---- device-side layout (what the host library exports and the caller

@@ -13,8 +13,8 @@
 // Kernels of one step (recorded into a CUDA graph):
 //   k_split       FP32 form only: each source position as a float pair
 //                 (hi, lo), once per step -- the FP64 work of the step.
-//   k_force_warp  FP32 form: one work item per warp, no block-wide barrier;
-//                 FP32 pairs on group-centre-relative coordinates, plain FP32
+//   k_force_warp2 FP32 form: one work item per warp (small launches: per CTA);
+//                 packed two-wide FP32 pairs on group-centre-relative coordinates, plain FP32
 //                 sums between Kahan-compensated flushes, FP64 merge of the
 //                 lane-level j-split and FP64 outputs.
 //   k_force_f64   FP64 form (comparison form): one work item per CTA, every
@@ -96,6 +96,21 @@ __device__ __forceinline__ void write_target(const otoo_dev_system& sys, const o
     }
 }
 
+// The same for one component c of a target (0 .. 2 acceleration, 3 potential).
+__device__ __forceinline__ void write_component(const otoo_dev_system& sys, const otoo_group& grp,
+                                                const otoo_item& item, int i, int c, double a,
+                                                double* __restrict__ accel, double* __restrict__ pot)
+{
+    const int ig = item.i0 + i;
+    if (item.slot < 0) {
+        const int64_t t = (int64_t)grp.first + ig;
+        const int64_t o = sys.perm ? sys.perm[t] : t;
+        (c < 3 ? accel[3 * o + c] : pot[o]) = a;
+    } else {
+        sys.partial[((int64_t)item.slot * sys.n_crit_max + ig) * 4 + c] = a;
+    }
+}
+
 // Position split for the FP32 form, once per step: hi = x rounded to FP32,
 // lo = (x - hi) rounded to FP32.  A centre-relative coordinate is then
 // (hi - c) + lo in FP32 with c an FP32 value: hi - c is exact for every entry
@@ -128,7 +143,6 @@ __global__ void k_centre_relative(const float4* __restrict__ pairs, int64_t n, f
     out[3 * s + 2] = rel32(h.z, l.z, cz);
 }
 
-#include "force_warp.cuh"
 #include "force_warp2.cuh"
 
 // FP64 form: one work item per CTA of B threads, IB targets per thread,
@@ -310,22 +324,42 @@ __global__ void k_merge(const otoo_dev_system sys, double* __restrict__ accel, d
 
 using Kernel = void (*)(const otoo_dev_system, double*, double*);
 
-Kernel pick_f32(int B, int IB, int tile, int packed)
+// The compiled tunings: threads per CTA, targets per lane, entries per tile.
+// packed is part of the tuning's name only: one entry per instruction was slower
+// at every size measured (merger, N = 10^6, n_crit 64: 2.94 ms against 2.72 ms,
+// tiles of 128 entries), so both values run the packed arithmetic.
+struct ForceKernel {
+    Kernel one, team;  // a work item per warp; a work item per CTA of kTeamWarps warps
+    int team_smem;
+};
+constexpr int kTeamWarps = 4;
+// Items per SM up to which a CTA of four warps takes one item: below, the
+// longest items (64 targets against the whole list) set the launch's time;
+// above, the team's barriers cost more than its shorter tail gives.  One item
+// per warp / per CTA (128, 2, 128 tuning, theta 0.6, quadrupole cells): N = 4096
+// (307 items) 92 / 48 us, 30000 (2039) 265 / 115, 100003 (6615) 408 / 283,
+// 200000 (8759) 831 / 731, 400000 (18094) 1426 / 1523, 2^20 (46109) 3951 / 4303.
+constexpr int64_t kTeamItems = 80;
+
+template <int NW, int IB, int SPL>
+constexpr ForceKernel force_kernel()
 {
-    const int spl = tile / 32;
+    return {k_force_warp2<NW, IB, SPL>, k_force_warp2<kTeamWarps, IB, SPL, true>,
+            (int)sizeof(TeamPart<IB>) * kTeamWarps};
+}
+
+ForceKernel pick_f32(int B, int IB, int tile, int packed)
+{
 #define PICK(NW_, IB_, SPL_) \
-    if (B == NW_ * 32 && IB == IB_ && spl == SPL_) return k_force_warp<NW_, IB_, SPL_>;
-#define PICK2(NW_, IB_, SPL_) \
-    if (B == NW_ * 32 && IB == IB_ && spl == SPL_) return k_force_warp2<NW_, IB_, SPL_>;
+    if (B == NW_ * 32 && IB == IB_ && tile == SPL_ * 32) return force_kernel<NW_, IB_, SPL_>();
+    PICK(4, 1, 4) PICK(4, 2, 4) PICK(4, 2, 8) PICK(2, 2, 4)
     if (packed) {
-        PICK2(4, 1, 4) PICK2(4, 2, 4) PICK2(4, 2, 8) PICK2(2, 2, 4) PICK2(2, 1, 4) PICK2(4, 1, 8)
-        return nullptr;
+        PICK(2, 1, 4) PICK(4, 1, 8)
+    } else {
+        PICK(4, 2, 2) PICK(4, 4, 4) PICK(4, 4, 8) PICK(2, 4, 4) PICK(8, 2, 4) PICK(8, 1, 4)
     }
-    PICK(4, 1, 4) PICK(4, 2, 2) PICK(4, 2, 4) PICK(4, 2, 8) PICK(4, 4, 4) PICK(4, 4, 8)
-    PICK(2, 2, 4) PICK(2, 4, 4) PICK(8, 2, 4) PICK(8, 1, 4)
 #undef PICK
-#undef PICK2
-    return nullptr;
+    return {nullptr, nullptr, 0};
 }
 
 // FP64 form: B threads per CTA for a plan made with iblock targets per lane
@@ -340,7 +374,7 @@ Kernel pick_f64(int IB)
 int check_tune(const otoo_tune* t)
 {
     OTOO_REQUIRE(t, OTOO_EINVAL, "tune is NULL");
-    OTOO_REQUIRE(pick_f32(t->block, t->iblock, t->tile, t->packed) != nullptr, OTOO_EINVAL,
+    OTOO_REQUIRE(pick_f32(t->block, t->iblock, t->tile, t->packed).one != nullptr, OTOO_EINVAL,
                  "unsupported tune: block %d, iblock %d, tile %d", t->block, t->iblock, t->tile);
     OTOO_REQUIRE(t->split >= 32, OTOO_EINVAL, "split must be >= 32");
     OTOO_REQUIRE(t->ctas_per_sm >= 0 && t->ctas_per_sm <= 32, OTOO_EINVAL, "ctas_per_sm out of range");
@@ -384,15 +418,20 @@ int enqueue_force(const otoo_dev_system* sys, double* accel, double* pot, int pr
                   cudaStream_t s)
 {
     const bool fp64 = precision == OTOO_FP64;
-    Kernel fn = fp64 ? pick_f64(t->iblock) : pick_f32(t->block, t->iblock, t->tile, t->packed);
-    const int block = fp64 ? 128 : t->block;
+    const ForceKernel fk = fp64 ? ForceKernel{pick_f64(t->iblock), nullptr, 0}
+                                : pick_f32(t->block, t->iblock, t->tile, t->packed);
     int dev = 0, nsm = 0, occ = 0;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, 0));
+    const bool team = !fp64 && sys->n_items <= kTeamItems * nsm;
+    Kernel fn = team ? fk.team : fk.one;
+    const int block = fp64 ? 128 : team ? 32 * kTeamWarps : t->block;
+    const int smem = team ? fk.team_smem : 0;
+    if (team) CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, smem));
     if (occ < 1) return set_error(OTOO_EINVAL, "force kernel does not fit on an SM");
     const int per_sm = t->ctas_per_sm > 0 ? std::min(t->ctas_per_sm, occ) : occ;
-    const int64_t units = fp64 ? sys->n_items : ((int64_t)sys->n_items + block / 32 - 1) / (block / 32);
+    const int64_t units = fp64 || team ? sys->n_items : ((int64_t)sys->n_items + block / 32 - 1) / (block / 32);
     const int grid = (int)std::min<int64_t>(units, (int64_t)nsm * per_sm);
     CUDA_TRY(cudaMemsetAsync(sys->counter, 0, 2 * sizeof(uint32_t), s));
     if (!fp64) {
@@ -401,7 +440,7 @@ int enqueue_force(const otoo_dev_system* sys, double* accel, double* pot, int pr
         CUDA_TRY(cudaGetLastError());
     }
     if (grid > 0) {
-        fn<<<grid, block, 0, s>>>(*sys, accel, pot);
+        fn<<<grid, block, smem, s>>>(*sys, accel, pot);
         CUDA_TRY(cudaGetLastError());
     }
     if (sys->n_splits > 0) {

@@ -1,10 +1,22 @@
-// FP32 force kernel with packed two-wide FP32 arithmetic (included by
-// force.cu after force_warp.cuh).
+// FP32 force kernel with packed two-wide FP32 arithmetic, one work item per
+// warp (included by force.cu, inside its anonymous namespace, after the pair
+// laws and the item helpers).
 //
-// The same work decomposition as k_force_warp (one work item per warp, IB
-// targets per lane, lane subsets interleaved over the staged entries), but a
-// lane evaluates two consecutive list entries at once: the shared-memory tile
-// holds "pair records" whose fields are (entry 2m, entry 2m+1) float pairs,
+// Layout of one item on the warp: the item's ni targets sit in
+// P = ceil(ni / IB) lane slots (IB targets per lane, register-resident) and
+// the warp's nsub = 32 / P lane subsets take interleaved records of each
+// staged tile, so one shared-memory read of a record feeds 2 IB pairs.  A tile
+// holds up to 32 SPL list entries: every lane loads its entries (index, then
+// the source's per-step float pair from k_split and, for a cell, its
+// quadrupole), converts them to group-centre-relative FP32 and writes them to
+// the warp's shared-memory tile, padded with zero-mass records so that every
+// active lane runs the same trip count.  No block-wide barrier; a lane sums
+// pairs in plain FP32 over a tile and adds the tile sum to its
+// Kahan-compensated running sum, and the lane subsets are merged with a
+// compensated FP32 sum in a fixed pairwise order and converted to FP64 once.
+//
+// A lane evaluates two consecutive list entries at once: the shared-memory
+// tile holds "pair records" whose fields are (entry 2m, entry 2m+1) float pairs,
 // and every FP32 operation of the pair law is a packed fma/mul/add.f32x2
 // (PTX) acting on both entries.  A packed instruction issues once for two
 // FP32 operations, so the FP32 pipe rather than instruction issue bounds the
@@ -20,8 +32,8 @@
 // The packed arithmetic (f2 operations, pair_mono2, pair_quad2, the record
 // layout and the evaluation loops) is in pair.cuh.
 
-// Packed operands take register pairs: fewer resident warps than the scalar
-// kernel, each with twice the independent FP32 work per instruction.
+// Packed operands take register pairs: 16 resident warps per SM at IB = 2 (128
+// registers), each with twice the independent FP32 work per instruction.
 #ifndef OTOO_W2_WARPS
 #define OTOO_W2_WARPS 16  // resident warps per SM asked for at IB >= 2
 #endif
@@ -31,9 +43,20 @@
 #ifndef OTOO_W2_MUNROLL
 #define OTOO_W2_MUNROLL 3  // pair records per step of the particle loop (3: 45.1 ms, 2: 45.3, 4: 45.6)
 #endif
-constexpr int warp2_min_blocks(int nw, int ib) { return (ib == 1 ? 20 : OTOO_W2_WARPS) / nw; }
+constexpr int warp2_min_blocks(int nw, int ib) { return (ib == 1 ? 20 : ib == 2 ? OTOO_W2_WARPS : 12) / nw; }
 
-template <int NW, int IB, int SPL>
+// kTeam: a work item per CTA instead of one per warp.  The CTA's warps take the
+// item's tiles in turn and write each tile's lane sums to shared memory; warp w
+// mod 4 keeps the compensated running sums of component w of every target and
+// adds the tiles in list order, so the results are the one-warp form's bit for
+// bit.  For launches with few items per resident warp, where the longest items
+// set the time (kTeamItems).
+template <int IB>
+struct TeamPart {
+    float s[2][4 * IB][32];  // double-buffered: [component + 4 target][lane] of one warp's tile
+};
+
+template <int NW, int IB, int SPL, bool kTeam = false>
 __global__ void __launch_bounds__(NW * 32, warp2_min_blocks(NW, IB)) k_force_warp2(const otoo_dev_system sys,
                                                                                   double* __restrict__ accel,
                                                                                   double* __restrict__ pot)
@@ -42,6 +65,9 @@ __global__ void __launch_bounds__(NW * 32, warp2_min_blocks(NW, IB)) k_force_war
     constexpr int TP = T / 2;            // pair records per tile at most
     constexpr int PPL = (TP + 31) / 32;  // pair records staged per lane
     __shared__ float4 s_rec[NW][kCellRecF4 * TP];
+    extern __shared__ __align__(16) unsigned char team_smem[];  // kTeam: TeamPart per warp
+    TeamPart<IB>* team = reinterpret_cast<TeamPart<IB>*>(team_smem);
+    __shared__ int s_ticket;
 
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
@@ -53,8 +79,15 @@ __global__ void __launch_bounds__(NW * 32, warp2_min_blocks(NW, IB)) k_force_war
 
     for (;;) {
         int it = 0;
-        if (lane == 0) it = (int)atomicAdd(sys.counter, 1u);
-        it = __shfl_sync(kFull, it, 0);
+        if constexpr (kTeam) {
+            __syncthreads();  // (the sums and the ticket of the item before are done with)
+            if (threadIdx.x == 0) s_ticket = (int)atomicAdd(sys.counter, 1u);
+            __syncthreads();
+            it = s_ticket;
+        } else {
+            if (lane == 0) it = (int)atomicAdd(sys.counter, 1u);
+            it = __shfl_sync(kFull, it, 0);
+        }
         if (it >= sys.n_items) break;
 
         const otoo_item item = sys.items[it];
@@ -119,101 +152,155 @@ __global__ void __launch_bounds__(NW * 32, warp2_min_blocks(NW, IB)) k_force_war
                     nidx[pp][h] = k < cnt ? __ldg(lst + base + k) : 0;
                 }
         };
-        if (nt > 0) load_idx(0);
-
-        for (int t = 0; t < nt; ++t) {
-            const bool cell = t < ntc;
-            const bool cq = cell && has_quad;
-            const int base = cell ? c0 + t * TE : p0 + (t - ntc) * TE;
-            const int cnt = cell ? min(TE, c1 - base) : min(TE, p1 - base);
-            const int npair = (cnt + 1) / 2;
-            const int npair_pad = (npair + nsub - 1) / nsub * nsub;
-
-            // stage this lane's pair records: loads of both entries first
+        // kTeam: warp w takes tiles w, w + NW, ...; every warp runs the same rounds
+        const int step = kTeam ? NW : 1;
+        const int t_end = kTeam ? (nt + NW - 1) / NW * NW : nt;
+        const int t_first = kTeam ? wid : 0;
+        if (t_first < nt) load_idx(t_first);
+        int buf = 0;
+        float tS[IB], tC[IB];  // kTeam: running sums of component wid & 3
+        if constexpr (kTeam) {
 #pragma unroll
-            for (int pp = 0; pp < PPL; ++pp) {
-                const int m = lane + 32 * pp;
-                if (m >= npair_pad) continue;
-                float4 hh[2], ll[2], qa[2], qb[2];
-                bool real[2];
+            for (int k = 0; k < IB; ++k) tS[k] = tC[k] = 0.f;
+        }
+
+        for (int t = t_first; t < t_end; t += step) {
+            if (!kTeam || t < nt) {
+                const bool cell = t < ntc;
+                const bool cq = cell && has_quad;
+                const int base = cell ? c0 + t * TE : p0 + (t - ntc) * TE;
+                const int cnt = cell ? min(TE, c1 - base) : min(TE, p1 - base);
+                const int npair = (cnt + 1) / 2;
+                const int npair_pad = (npair + nsub - 1) / nsub * nsub;
+
+                // stage this lane's pair records: loads of both entries first
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int k = 2 * m + h;
-                    real[h] = k < cnt;
-                    hh[h] = ll[h] = qa[h] = qb[h] = zero4;
-                    if (real[h]) {
-                        const int idx = nidx[pp][h];
-                        const bool good =
-                            cell ? (idx >= sys.n_part && idx < sys.n_src) : (idx >= 0 && idx < sys.n_part);
-                        if (good) {
-                            // a source's float pair and a cell's quadrupole: one 32-byte load each
-                            ld256x2(ff + 2 * (int64_t)idx, hh[h], ll[h]);
-                            if (cq) ld256x2(reinterpret_cast<const float4*>(sys.quad + (idx - sys.n_part)), qa[h], qb[h]);
+                for (int pp = 0; pp < PPL; ++pp) {
+                    const int m = lane + 32 * pp;
+                    if (m >= npair_pad) continue;
+                    float4 hh[2], ll[2], qa[2], qb[2];
+                    bool real[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int k = 2 * m + h;
+                        real[h] = k < cnt;
+                        hh[h] = ll[h] = qa[h] = qb[h] = zero4;
+                        if (real[h]) {
+                            const int idx = nidx[pp][h];
+                            const bool good =
+                                cell ? (idx >= sys.n_part && idx < sys.n_src) : (idx >= 0 && idx < sys.n_part);
+                            if (good) {
+                                // a source's float pair and a cell's quadrupole: one 32-byte load each
+                                ld256x2(ff + 2 * (int64_t)idx, hh[h], ll[h]);
+                                if (cq) ld256x2(reinterpret_cast<const float4*>(sys.quad + (idx - sys.n_part)), qa[h], qb[h]);
+                            } else {
+                                atomicOr(status, kBadIndex);
+                                real[h] = false;
+                            }
+                        }
+                    }
+                    float x[2], y[2], z[2], w[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        // padding and rejected entries loaded as zeros: mass (and
+                        // quadrupole) 0, so they add exactly nothing
+                        x[h] = rel32(hh[h].x, ll[h].x, cx);
+                        y[h] = rel32(hh[h].y, ll[h].y, cy);
+                        z[h] = rel32(hh[h].z, ll[h].z, cz);
+                        w[h] = hh[h].w;
+                    }
+                    put_rec2(rec, m, cq, x, y, z, w, qa, qb, eps2);
+                }
+                if (t + step < nt) load_idx(t + step);
+                __syncwarp();
+
+                if (active) {
+                    Acc2 P2[IB];
+#pragma unroll
+                    for (int k = 0; k < IB; ++k) P2[k].v[0] = P2[k].v[1] = P2[k].v[2] = P2[k].v[3] = zero2;
+                    const int niter = npair_pad / nsub;
+                    if (cq)
+                        eval_cells2<IB, OTOO_W2_QUNROLL>(rec, js, nsub, niter, nx, ny, nz, e2, P2);
+                    else
+                        eval_parts2<IB, OTOO_W2_MUNROLL>(rec, js, nsub, niter, nx, ny, nz, e2, P2);
+#pragma unroll
+                    for (int k = 0; k < IB; ++k) {
+                        float s[4];
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            float lo, hi;
+                            f2unpack(P2[k].v[c], lo, hi);
+                            s[c] = lo + hi;
+                        }
+                        if constexpr (kTeam) {
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) team[wid].s[buf][4 * k + c][lane] = s[c];
                         } else {
-                            atomicOr(status, kBadIndex);
-                            real[h] = false;
+                            acc[k].add(s);
                         }
                     }
                 }
-                float x[2], y[2], z[2], w[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    // padding and rejected entries loaded as zeros: mass (and
-                    // quadrupole) 0, so they add exactly nothing
-                    x[h] = rel32(hh[h].x, ll[h].x, cx);
-                    y[h] = rel32(hh[h].y, ll[h].y, cy);
-                    z[h] = rel32(hh[h].z, ll[h].z, cz);
-                    w[h] = hh[h].w;
-                }
-                put_rec2(rec, m, cq, x, y, z, w, qa, qb, eps2);
+                __syncwarp();
             }
-            if (t + 1 < nt) load_idx(t + 1);
-            __syncwarp();
-
-            if (active) {
-                Acc2 P2[IB];
+            if constexpr (kTeam) {
+                __syncthreads();
+                // Acc::add of this round's tiles in list order
+                const int live = min(NW, nt - (t - wid));
+                if (wid < 4 && active) {
+                    for (int w = 0; w < live; ++w)
 #pragma unroll
-                for (int k = 0; k < IB; ++k) P2[k].v[0] = P2[k].v[1] = P2[k].v[2] = P2[k].v[3] = zero2;
-                const int niter = npair_pad / nsub;
-                if (cq)
-                    eval_cells2<IB, OTOO_W2_QUNROLL>(rec, js, nsub, niter, nx, ny, nz, e2, P2);
-                else
-                    eval_parts2<IB, OTOO_W2_MUNROLL>(rec, js, nsub, niter, nx, ny, nz, e2, P2);
+                        for (int k = 0; k < IB; ++k) {
+                            const float y = __fsub_rn(team[w].s[buf][4 * k + wid][lane], tC[k]);
+                            const float u = __fadd_rn(tS[k], y);
+                            tC[k] = __fsub_rn(__fsub_rn(u, tS[k]), y);
+                            tS[k] = u;
+                        }
+                }
+                buf ^= 1;
+            }
+        }
+        if constexpr (kTeam) {
+            if (wid < 4) {
 #pragma unroll
                 for (int k = 0; k < IB; ++k) {
-                    float s[4];
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        float lo, hi;
-                        f2unpack(P2[k].v[c], lo, hi);
-                        s[c] = lo + hi;
+                    float S = tS[k], C = tC[k];
+                    merge_subsets(S, C, js, nsub, P);
+                    double a = (double)S - (double)C;
+                    const int i = islot + k * P;
+                    if (js == 0 && i < ni) {
+                        if (wid == 3) {
+                            a = -a;
+                            if (item.j0 == 0) {
+                                const float4 h = __ldg(ff + 2 * ((int64_t)grp.first + item.i0 + i));
+                                a += (double)(h.w * rsqrt_r(eps2));
+                            }
+                        }
+                        write_component(sys, grp, item, i, wid, a, accel, pot);
                     }
-                    acc[k].add(s);
                 }
             }
-            __syncwarp();
-        }
-
-        // merge the lane subsets into the js == 0 lanes (pairwise, in a fixed
-        // order) with a compensated FP32 sum; one conversion to FP64 per output
+        } else {
+            // merge the lane subsets into the js == 0 lanes (pairwise, in a fixed
+            // order) with a compensated FP32 sum; one conversion to FP64 per output
 #pragma unroll
-        for (int k = 0; k < IB; ++k) {
-            double a[4];
+            for (int k = 0; k < IB; ++k) {
+                double a[4];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                float S = acc[k].s[c], C = acc[k].c[c];
-                merge_subsets(S, C, js, nsub, P);
-                a[c] = (double)S - (double)C;
-            }
-            a[3] = -a[3];
-            const int i = islot + k * P;
-            if (js == 0 && i < ni) {
-                if (item.j0 == 0) {
-                    // the self pair added exactly -m_i rsqrt(eps^2) in FP32: take the same value out
-                    const float4 h = __ldg(ff + 2 * ((int64_t)grp.first + item.i0 + i));
-                    a[3] += (double)(h.w * rsqrt_r(eps2));
+                for (int c = 0; c < 4; ++c) {
+                    float S = acc[k].s[c], C = acc[k].c[c];
+                    merge_subsets(S, C, js, nsub, P);
+                    a[c] = (double)S - (double)C;
                 }
-                write_target(sys, grp, item, i, a, accel, pot);
+                a[3] = -a[3];
+                const int i = islot + k * P;
+                if (js == 0 && i < ni) {
+                    if (item.j0 == 0) {
+                        // the self pair added exactly -m_i rsqrt(eps^2) in FP32: take the same value out
+                        const float4 h = __ldg(ff + 2 * ((int64_t)grp.first + item.i0 + i));
+                        a[3] += (double)(h.w * rsqrt_r(eps2));
+                    }
+                    write_target(sys, grp, item, i, a, accel, pot);
+                }
             }
         }
     }
