@@ -17,8 +17,9 @@
 //                   block-level scans with the block offsets.
 //   k_walk<true>    pass 2: the same walk, entries written at the offsets.
 //   k_plan_count    per group: particle and list chunks (the cost model of the
-//                   host plan), cost class histogram.
-//   k_plan_cursor   start of each cost class, most expensive class first.
+//                   host plan), cost class histogram, sums per block.
+//   k_plan_scan     prefixes of the block sums; start of each cost class, most
+//                   expensive class first.
 //   k_plan_fill     work items and split records.
 #include <cuda_runtime.h>
 
@@ -1338,15 +1339,6 @@ struct GroupOff {
     otoo_group* g;
     __device__ void operator()(int64_t i, int64_t v) const { g[i].list_off = v; }
 };
-struct I32In {
-    const int32_t* p;
-    __device__ int64_t operator()(int64_t i) const { return p[i]; }
-};
-struct I32Out {
-    int32_t* p;
-    __device__ void operator()(int64_t i, int64_t v) const { p[i] = (int32_t)v; }
-};
-
 __device__ int64_t block_excl_scan(int64_t v, int64_t* warp_s, int64_t* total)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1445,44 +1437,68 @@ int64_t scan_blocks(int64_t n) { return (n + kScanBlock - 1) / kScanBlock; }
 // ---- device plan ------------------------------------------------------------
 
 struct PlanScratch {
-    int64_t* bsum;    // scan block sums (2 scans, one after the other)
+    int64_t* slots;   // [blocks] partial slots of each block's groups, then their exclusive prefix
+    int64_t* splits;  // [blocks] split lists of each block's groups, then their exclusive prefix
     int32_t* hist;    // [kClasses] items per cost class
     int32_t* cursor;  // [kClasses] next free item position of each class
-    int32_t* nic;     // [G] particle chunks
-    int32_t* nch;     // [G] list chunks
-    int32_t* slot0;   // [G] slots (n_chunks when > 1), then their exclusive prefix
-    int32_t* sidx;    // [G] 1 when the list is split, then the split record index
-    int32_t* cls;     // [G] cost class
+    int32_t* split;   // the list chunk length the counts were made with
 };
-
-PlanScratch plan_layout(int32_t* base, int64_t G)
-{
-    PlanScratch p;
-    const int64_t nb = scan_blocks(G) + 1;
-    p.bsum = reinterpret_cast<int64_t*>(base);
-    int32_t* q = base + 2 * nb;
-    p.hist = q;
-    p.cursor = q + kClasses;
-    q += 2 * kClasses;
-    p.nic = q;
-    p.nch = q + G;
-    p.slot0 = q + 2 * G;
-    p.sidx = q + 3 * G;
-    p.cls = q + 4 * G;
-    return p;
-}
 
 // The plan kernels run 256 threads per block, one group each.  The chunk
 // table (a kernel parameter) is copied to shared memory first: threads index
 // it by their own group sizes, which the parameter bank would serialise.
-// Counts and totals are summed per block in shared memory, so each block
-// makes one global atomic per class and per total instead of one per group.
+// Counts and totals are summed per warp and block, so each block makes one
+// global atomic per class and per total.  Three launches: k_plan_count also
+// leaves each block's sums of slots and split lists, k_plan_scan turns them and
+// the class counts into prefixes, k_plan_fill adds the prefix inside the block.
+// With 64-bit shared-memory atomics per group, two three-launch scans over all
+// groups and a one-thread prefix of the classes, ten launches took 49 us for
+// 260 groups and 84 us for 221169; these take 16 and 40 us.
 constexpr int kPlanThreads = 256;
+constexpr int kPlanWarps = kPlanThreads / 32;
+
+PlanScratch plan_layout(int32_t* base, int64_t G)
+{
+    const int64_t nb = (G + kPlanThreads - 1) / kPlanThreads;
+    PlanScratch p;
+    p.slots = reinterpret_cast<int64_t*>(base);
+    p.splits = p.slots + nb;
+    p.hist = reinterpret_cast<int32_t*>(p.splits + nb);
+    p.cursor = p.hist + kClasses;
+    p.split = p.cursor + kClasses;
+    return p;
+}
 
 __device__ void plan_table_to_shared(const ChunkTable& tab, ChunkTable& st)
 {
     for (int k = threadIdx.x; k <= kMaxGroup; k += blockDim.x) st.last[k] = tab.last[k];
     if (threadIdx.x == 0) st.ib = tab.ib;
+}
+
+// A group's particle chunks (plan_chunks.h), list chunks and cost class, the
+// host plan's: class = quarter octaves of the largest item's ni * (j1 - j0).
+// nic = nch = 0 for an empty list or a group size out of range.
+__device__ __forceinline__ void plan_group(const otoo_group& gr, const ChunkTable& st, int32_t split, int32_t& nic,
+                                           int32_t& nch, int32_t& cls)
+{
+    nic = nch = cls = 0;
+    const int64_t len = (int64_t)gr.n_cell + gr.n_part;
+    if (len <= 0 || gr.count <= 0 || gr.count > kMaxGroup) return;
+    int32_t big = 0;
+    nic = chunk_count(st, gr.count, &big);
+    nch = (int32_t)((len + split - 1) / split);
+    const int64_t c0 = (int64_t)big * ((len + nch - 1) / nch);
+    const int msb = 63 - __clzll((long long)c0);
+    const int frac = msb >= 2 ? (int)((c0 >> (msb - 2)) & 3) : (int)((c0 << (2 - msb)) & 3);
+    cls = 4 * msb + frac;
+    if (cls >= kClasses) cls = kClasses - 1;
+}
+
+__device__ __forceinline__ int64_t warp_sum64(int64_t v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    return v;
 }
 
 __global__ void __launch_bounds__(kPlanThreads) k_plan_count(const otoo_group* __restrict__ groups, int32_t G,
@@ -1491,104 +1507,119 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_count(const otoo_group* _
 {
     __shared__ ChunkTable st;
     __shared__ int32_t shist[kClasses];
-    __shared__ unsigned long long s_items, s_split_groups, s_split_chunks, s_max;
+    __shared__ int64_t s_sum[3][kPlanWarps];  // items, split lists, slots
+    __shared__ int32_t s_max[kPlanWarps];
     plan_table_to_shared(tab, st);
     for (int c = threadIdx.x; c < kClasses; c += blockDim.x) shist[c] = 0;
-    if (threadIdx.x == 0) s_items = s_split_groups = s_split_chunks = s_max = 0;
     __syncthreads();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
+    int32_t nic = 0, nch = 0, cls = 0, cnt = 1;
     if (g < G) {
         const otoo_group gr = groups[g];
-        atomicMax(&s_max, (unsigned long long)(gr.count > 1 ? gr.count : 1));
-        const int64_t len = (int64_t)gr.n_cell + gr.n_part;
-        int32_t nic = 0, nch = 0, cls = 0;
-        if (len > 0 && gr.count > 0 && gr.count <= kMaxGroup) {
-            // the host plan's particle chunks (plan_chunks.h)
-            int32_t big = 0;
-            nic = chunk_count(st, gr.count, &big);
-            nch = (int32_t)((len + split - 1) / split);
-            // cost class: 4 * log2 of the largest item's ni * (j1 - j0), in quarter octaves
-            const int64_t c0 = (int64_t)big * ((len + nch - 1) / nch);
-            const int msb = 63 - __clzll((long long)c0);
-            const int frac = msb >= 2 ? (int)((c0 >> (msb - 2)) & 3) : (int)((c0 << (2 - msb)) & 3);
-            cls = 4 * msb + frac;
-            if (cls >= kClasses) cls = kClasses - 1;
-            atomicAdd(shist + cls, nic * nch);
-            atomicAdd(&s_items, (unsigned long long)(nic * nch));
-            if (nch > 1) {
-                atomicAdd(&s_split_groups, 1ull);
-                atomicAdd(&s_split_chunks, (unsigned long long)nch);
-            }
-        }
-        p.nic[g] = nic;
-        p.nch[g] = nch;
-        p.slot0[g] = nch > 1 ? nch : 0;
-        p.sidx[g] = nch > 1 ? 1 : 0;
-        p.cls[g] = cls;
+        cnt = gr.count > 1 ? gr.count : 1;
+        plan_group(gr, st, split, nic, nch, cls);
+        if (nic > 0) atomicAdd(shist + cls, nic * nch);
     }
+    __syncwarp();
+    const int64_t items = warp_sum64((int64_t)nic * nch), slots = warp_sum64(nch > 1 ? nch : 0);
+    const int32_t splits = __reduce_add_sync(kFull, nch > 1 ? 1 : 0), mx = __reduce_max_sync(kFull, cnt);
+    if (lane == 0) s_sum[0][w] = items, s_sum[1][w] = splits, s_sum[2][w] = slots, s_max[w] = mx;
     __syncthreads();
     for (int c = threadIdx.x; c < kClasses; c += blockDim.x)
         if (shist[c]) atomicAdd(p.hist + c, shist[c]);
     if (threadIdx.x == 0) {
-        unsigned long long* t = reinterpret_cast<unsigned long long*>(totals);
-        if (s_items) atomicAdd(t, s_items);
-        if (s_split_groups) {
-            atomicAdd(t + 1, s_split_groups);
-            atomicAdd(t + 2, s_split_chunks);
+        int64_t a[3] = {0, 0, 0};
+        int32_t m = 1;
+        for (int k = 0; k < kPlanWarps; ++k) {
+            for (int q = 0; q < 3; ++q) a[q] += s_sum[q][k];
+            m = s_max[k] > m ? s_max[k] : m;
         }
-        atomicMax(t + 3, s_max);
+        unsigned long long* t = reinterpret_cast<unsigned long long*>(totals);
+        if (a[0]) atomicAdd(t, (unsigned long long)a[0]);
+        if (a[1]) {
+            atomicAdd(t + 1, (unsigned long long)a[1]);
+            atomicAdd(t + 2, (unsigned long long)a[2]);
+        }
+        atomicMax(t + 3, (unsigned long long)m);
+        p.splits[blockIdx.x] = a[1];
+        p.slots[blockIdx.x] = a[2];
+        if (blockIdx.x == 0) *p.split = split;
     }
 }
 
-__global__ void k_plan_cursor(PlanScratch p)
+// One block: exclusive prefixes of the blocks' slots and split lists, and the
+// start of each cost class, most expensive class first.
+__global__ void __launch_bounds__(kScanThreads) k_plan_scan(PlanScratch p, int32_t nblk,
+                                                             const int64_t* __restrict__ totals)
 {
-    if (threadIdx.x != 0) return;
-    int32_t pos = 0;
-    for (int c = kClasses - 1; c >= 0; --c) {
-        p.cursor[c] = pos;
-        pos += p.hist[c];
+    __shared__ int64_t ws[33];
+    const int c = kClasses - 1 - (int)threadIdx.x;
+    int64_t tot;
+    const int64_t pos = block_excl_scan(c >= 0 ? p.hist[c] : 0, ws, &tot);
+    if (c >= 0) p.cursor[c] = (int32_t)pos;
+    if (totals[1] == 0) return;  // no list is split: no slots
+    for (int a = 0; a < 2; ++a) {
+        int64_t* v = a ? p.splits : p.slots;
+        int64_t carry = 0;
+        for (int32_t b0 = 0; b0 < nblk; b0 += kScanThreads) {
+            const int32_t i = b0 + threadIdx.x;
+            const int64_t e = block_excl_scan(i < nblk ? v[i] : 0, ws, &tot);
+            if (i < nblk) v[i] = carry + e;
+            carry += tot;
+        }
     }
 }
 
 __global__ void __launch_bounds__(kPlanThreads) k_plan_fill(const otoo_group* __restrict__ groups, int32_t G,
                                                             const ChunkTable tab, PlanScratch p,
+                                                            const int64_t* __restrict__ totals,
                                                             otoo_item* __restrict__ items, int64_t items_cap,
                                                             otoo_split* __restrict__ splits, int64_t splits_cap,
                                                             uint32_t* __restrict__ status)
 {
     __shared__ ChunkTable st;
     __shared__ int32_t scount[kClasses], sbase[kClasses];
+    __shared__ int64_t ws[33];
     plan_table_to_shared(tab, st);
     for (int c = threadIdx.x; c < kClasses; c += blockDim.x) scount[c] = 0;
     __syncthreads();
     // the block's items of each class take one run of that class's items
     const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-    const int32_t nic = g < G ? p.nic[g] : 0, nch = g < G ? p.nch[g] : 0;
+    otoo_group gr = {};
+    int32_t nic = 0, nch = 0, cls = 0;
+    if (g < G) {
+        gr = groups[g];
+        plan_group(gr, st, *p.split, nic, nch, cls);
+    }
     const bool on = nic > 0 && nch > 0;
-    const int32_t cls = on ? p.cls[g] : 0;
     const int32_t local = on ? atomicAdd(scount + cls, nic * nch) : 0;
+    // first slot and split record of the group, in group order
+    int64_t slot0 = 0, si = 0;
+    if (totals[1] != 0) {  // (uniform)
+        int64_t tot;
+        slot0 = p.slots[blockIdx.x] + block_excl_scan(nch > 1 ? nch : 0, ws, &tot);
+        si = p.splits[blockIdx.x] + block_excl_scan(nch > 1 ? 1 : 0, ws, &tot);
+    }
     __syncthreads();
     for (int c = threadIdx.x; c < kClasses; c += blockDim.x)
         if (scount[c]) sbase[c] = atomicAdd(p.cursor + c, scount[c]);
     __syncthreads();
     if (!on) return;
-    const otoo_group gr = groups[g];
     const int64_t len = (int64_t)gr.n_cell + gr.n_part;
-    const int32_t slot0 = p.slot0[g];
     const int32_t pos = sbase[cls] + local;
     if ((int64_t)pos + nic * nch > items_cap) {
         atomicOr(status, kWalkNoRoom);
         return;
     }
     if (nch > 1) {
-        const int32_t si = p.sidx[g];
         if (si >= splits_cap) {
             atomicOr(status, kWalkNoRoom);
             return;
         }
         otoo_split s;
         s.g = g;
-        s.slot0 = slot0;
+        s.slot0 = (int32_t)slot0;
         s.n_chunks = nch;
         s.pad = 0;
         splits[si] = s;
@@ -1603,7 +1634,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_fill(const otoo_group* __
             it.ni = ni;
             it.j0 = (int32_t)(len * q / nch);
             it.j1 = (int32_t)(len * (q + 1) / nch);
-            it.slot = nch > 1 ? slot0 + q : -1;
+            it.slot = nch > 1 ? (int32_t)slot0 + q : -1;
             it.pad0 = it.pad1 = 0;
             items[k++] = it;
         }
@@ -1826,7 +1857,7 @@ int otoo_walk_check_status(const otoo_dev_walk* w, void* stream)
 int64_t otoo_plan_scratch_ints(int64_t n_groups)
 {
     if (n_groups < 0) n_groups = 0;
-    return 2 * (scan_blocks(n_groups) + 1) + 2 * kClasses + 5 * n_groups;
+    return 4 * ((n_groups + kPlanThreads - 1) / kPlanThreads + 1) + 2 * kClasses + 2;
 }
 
 int otoo_plan_count(const otoo_group* groups, int32_t n_groups, const otoo_tune* tune, int32_t* plan_scratch,
@@ -1843,10 +1874,7 @@ int otoo_plan_count(const otoo_group* groups, int32_t n_groups, const otoo_tune*
     CUDA_TRY(cudaMemsetAsync(p.hist, 0, kClasses * sizeof(int32_t), s));
     k_plan_count<<<(n_groups + kPlanThreads - 1) / kPlanThreads, kPlanThreads, 0, s>>>(
         groups, n_groups, chunk_table(ib), tune->split, p, plan_totals);
-    CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(excl_scan(I32In{p.slot0}, I32Out{p.slot0}, n_groups, p.bsum, nullptr, s));
-    CUDA_TRY(excl_scan(I32In{p.sidx}, I32Out{p.sidx}, n_groups, p.bsum, nullptr, s));
-    k_plan_cursor<<<1, 32, 0, s>>>(p);
+    k_plan_scan<<<1, kScanThreads, 0, s>>>(p, (n_groups + kPlanThreads - 1) / kPlanThreads, plan_totals);
     CUDA_TRY(cudaGetLastError());
     return OTOO_OK;
 }
@@ -1865,7 +1893,8 @@ int otoo_plan_fill(const otoo_group* groups, int32_t n_groups, const otoo_tune* 
     const int32_t ib = tune->iblock > 1 ? tune->iblock : 1;
     PlanScratch p = plan_layout(plan_scratch, n_groups);
     k_plan_fill<<<(n_groups + kPlanThreads - 1) / kPlanThreads, kPlanThreads, 0, s>>>(
-        groups, n_groups, chunk_table(ib), p, items, items_capacity, splits, splits_capacity, counter + 1);
+        groups, n_groups, chunk_table(ib), p, plan_totals, items, items_capacity, splits, splits_capacity,
+        counter + 1);
     CUDA_TRY(cudaGetLastError());
     return OTOO_OK;
 }
