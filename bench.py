@@ -3,9 +3,9 @@ interaction list on one GB300 (interactions per second and ms per step).
 
 Default workload: Hernquist halo N = 2^23 (a = 1, truncated at 100 a), eps
 5e-4, theta 0.5, quadrupole cells, FP32 centre-relative pairs with Kahan
-sums (FP64 form timed beside it).  A step is one otoo_force call (CUDA graph:
-ticket reset, persistent force kernel, chunk merge) over device-resident
-groups and lists; the host tree and walk are built once before timing.
+sums (FP64 form timed beside it).  A step is one otoo_force call (float-pair
+split with the ticket reset, persistent force kernel, chunk merge) over
+device-resident groups and lists; the host tree and walk are built once before timing.
 
 Prints one JSON line (rank 0).  --impl reference times the FP64 CPU oracle
 (the only reference this method has) on a bounded sample of the same
@@ -787,7 +787,7 @@ def run_paper_workloads(args, dev_name, tune, stream):
 
 def run_batch(args, dev_name):
     """64 independent Plummer/King systems of uneven size packed into one
-    ragged buffer and evaluated by one graph-launched force step."""
+    ragged buffer and evaluated by one force step."""
     import torch
 
     from paper_1206_1199_gb300 import _lib as L

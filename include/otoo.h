@@ -304,8 +304,8 @@ int otoo_default_tune(int32_t n_crit, otoo_tune* tune);
    host link takes these writes during the kernel, which replaces the copy
    that would follow it).
    precision: OTOO_FP32K or OTOO_FP64.  tune: the tuning the plan was made with.
-   The step (ticket reset, persistent force kernel, chunk merge) is recorded
-   once per distinct argument set into a CUDA graph and replayed on stream.
+   The step's kernels (float-pair split with the ticket reset, persistent force
+   kernel, chunk merge) are launched on stream, which may be captured.
    Every work item, list index and split record is bounds-checked on the
    device before it is used (groups, list, sources, and the partial slots
    against sys->partial_doubles); a bad one is skipped, its targets are not

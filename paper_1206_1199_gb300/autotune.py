@@ -70,7 +70,7 @@ def _time_step(dev, lists, tune, reps=3, inner=3):
     n = lists.n_part
     acc = torch.empty((n, 3), dtype=torch.float64, device=dev.bufs["src"].device)
     pot = torch.empty(n, dtype=torch.float64, device=dev.bufs["src"].device)
-    S.force(dev, acc, pot, L.OTOO_FP32K, tune)  # also records the graph
+    S.force(dev, acc, pot, L.OTOO_FP32K, tune)
     best = float("inf")
     for _ in range(reps):
         torch.cuda.synchronize()

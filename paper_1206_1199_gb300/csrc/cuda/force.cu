@@ -5,14 +5,16 @@
 // cell acting as a virtual particle at its centre of mass), Section III-D
 // (the GPU evaluates the interactions of a group that shares one walk).  The
 // quadrupole cell term, the FP32 centre-relative arithmetic with per-thread
-// Kahan sums, the persistent load-balanced launch and the CUDA graph are this
-// library's design for sm_103a; the pair law with Plummer softening is a
+// Kahan sums and the persistent load-balanced launch are this library's design for sm_103a; the pair law with Plummer softening is a
 // reading (the paper keeps a softening length per particle but does not print
 // the law).
 //
-// Kernels of one step (recorded into a CUDA graph):
+// Kernels of one step (two or three launches; a recorded CUDA graph replayed
+// as fast for unchanged arguments, but a time loop's counts change from step to
+// step, and recording it anew took 50 us at N = 4096):
 //   k_split       FP32 form only: each source position as a float pair
-//                 (hi, lo), once per step -- the FP64 work of the step.
+//                 (hi, lo), once per step -- the FP64 work of the step; clears
+//                 the work ticket and the status word.
 //   k_force_warp2 FP32 form: one work item per warp (small launches: per CTA);
 //                 packed two-wide FP32 pairs on group-centre-relative coordinates, plain FP32
 //                 sums between Kahan-compensated flushes, FP64 merge of the
@@ -27,7 +29,6 @@
 #include <cstdint>
 #include <cstring>
 #include <mutex>
-#include <vector>
 
 #include "../common.h"
 
@@ -117,9 +118,13 @@ __device__ __forceinline__ void write_component(const otoo_dev_system& sys, cons
 // within a factor of two of c (Sterbenz), so near entries keep the accuracy of
 // an FP64 subtraction rounded once to FP32, and far entries stay within about
 // one FP32 ulp of it.
-__global__ void k_split(const otoo_src* __restrict__ src, float4* __restrict__ out, int64_t n)
+// counter (or NULL): the work ticket and status word of the force kernel that
+// follows, cleared here instead of by a launch of its own.
+__global__ void k_split(const otoo_src* __restrict__ src, float4* __restrict__ out, int64_t n,
+                        uint32_t* __restrict__ counter)
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s < 2 && counter) counter[s] = 0u;
     if (s >= n) return;
     double x, y, z;
     float m;
@@ -320,7 +325,7 @@ __global__ void k_merge(const otoo_dev_system sys, double* __restrict__ accel, d
 }
 
 // ---------------------------------------------------------------------------
-// host side: kernel choice, launch shape, CUDA graph cache
+// host side: kernel choice, launch shape
 
 using Kernel = void (*)(const otoo_dev_system, double*, double*);
 
@@ -400,14 +405,14 @@ int read_status(const uint32_t* counter, void* stream)
     return OTOO_OK;
 }
 
-// Records the launches of one force step on stream s.
 }  // namespace
 
 int otoo::enqueue_split(const otoo_src* src, float* out, int64_t n, void* stream)
 {
     if (n <= 0) return OTOO_OK;
     const int64_t nb = (n + 255) / 256;
-    k_split<<<(unsigned)nb, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(src, reinterpret_cast<float4*>(out), n);
+    k_split<<<(unsigned)nb, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(src, reinterpret_cast<float4*>(out), n,
+                                                                              nullptr);
     CUDA_TRY(cudaGetLastError());
     return OTOO_OK;
 }
@@ -433,10 +438,11 @@ int enqueue_force(const otoo_dev_system* sys, double* accel, double* pot, int pr
     const int per_sm = t->ctas_per_sm > 0 ? std::min(t->ctas_per_sm, occ) : occ;
     const int64_t units = fp64 || team ? sys->n_items : ((int64_t)sys->n_items + block / 32 - 1) / (block / 32);
     const int grid = (int)std::min<int64_t>(units, (int64_t)nsm * per_sm);
-    CUDA_TRY(cudaMemsetAsync(sys->counter, 0, 2 * sizeof(uint32_t), s));
-    if (!fp64) {
+    if (fp64) {
+        CUDA_TRY(cudaMemsetAsync(sys->counter, 0, 2 * sizeof(uint32_t), s));
+    } else {
         const int64_t nb = (sys->n_src + 255) / 256;
-        k_split<<<(unsigned)nb, 256, 0, s>>>(sys->src, reinterpret_cast<float4*>(sys->split), sys->n_src);
+        k_split<<<(unsigned)nb, 256, 0, s>>>(sys->src, reinterpret_cast<float4*>(sys->split), sys->n_src, sys->counter);
         CUDA_TRY(cudaGetLastError());
     }
     if (grid > 0) {
@@ -449,26 +455,6 @@ int enqueue_force(const otoo_dev_system* sys, double* accel, double* pot, int pr
     }
     return OTOO_OK;
 }
-
-struct GraphKey {
-    otoo_dev_system sys;
-    double* accel;
-    double* pot;
-    int precision, device;
-    otoo_tune tune;
-    bool operator==(const GraphKey& o) const { return std::memcmp(this, &o, sizeof(GraphKey)) == 0; }
-};
-
-struct GraphEntry {
-    GraphKey key;
-    cudaGraphExec_t exec;
-    uint64_t last_use;
-};
-
-std::mutex g_graph_mu;
-std::vector<GraphEntry> g_graphs;
-uint64_t g_graph_clock = 0;
-constexpr size_t kMaxGraphs = 16;
 
 int validate_sys(const otoo_dev_system* sys)
 {
@@ -505,54 +491,7 @@ int otoo_force(const otoo_dev_system* sys, double* accel, double* pot, int32_t p
     if (rc) return rc;
     OTOO_REQUIRE(precision == OTOO_FP64 || sys->split != nullptr, OTOO_EINVAL,
                  "OTOO_FP32K needs the split scratch (32 bytes per source)");
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    GraphKey key;
-    std::memset(&key, 0, sizeof(key));
-    key.sys = *sys;
-    key.accel = accel;
-    key.pot = pot;
-    key.precision = precision;
-    CUDA_TRY(cudaGetDevice(&key.device));
-    key.tune = *tune;
-    std::lock_guard<std::mutex> lock(g_graph_mu);
-    for (GraphEntry& e : g_graphs) {
-        if (e.key == key) {
-            e.last_use = ++g_graph_clock;
-            CUDA_TRY(cudaGraphLaunch(e.exec, s));
-            return OTOO_OK;
-        }
-    }
-    // record the step into a graph on a private stream
-    cudaStream_t cs;
-    CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-    cudaGraph_t graph = nullptr;
-    cudaError_t ce = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-    if (ce != cudaSuccess) {
-        cudaStreamDestroy(cs);
-        return set_error(OTOO_ECUDA, "cudaStreamBeginCapture: %s", cudaGetErrorString(ce));
-    }
-    rc = enqueue_force(sys, accel, pot, precision, tune, cs);
-    ce = cudaStreamEndCapture(cs, &graph);
-    cudaStreamDestroy(cs);
-    if (rc) {
-        if (graph) cudaGraphDestroy(graph);
-        return rc;
-    }
-    if (ce != cudaSuccess) return set_error(OTOO_ECUDA, "cudaStreamEndCapture: %s", cudaGetErrorString(ce));
-    cudaGraphExec_t exec;
-    ce = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (ce != cudaSuccess) return set_error(OTOO_ECUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(ce));
-    if (g_graphs.size() >= kMaxGraphs) {
-        size_t old = 0;
-        for (size_t k = 1; k < g_graphs.size(); ++k)
-            if (g_graphs[k].last_use < g_graphs[old].last_use) old = k;
-        cudaGraphExecDestroy(g_graphs[old].exec);
-        g_graphs.erase(g_graphs.begin() + old);
-    }
-    g_graphs.push_back(GraphEntry{key, exec, ++g_graph_clock});
-    CUDA_TRY(cudaGraphLaunch(exec, s));
-    return OTOO_OK;
+    return enqueue_force(sys, accel, pot, precision, tune, reinterpret_cast<cudaStream_t>(stream));
 }
 
 int otoo_check_status(const otoo_dev_system* sys, void* stream)
@@ -601,7 +540,7 @@ extern "C" int otoo_centre_relative(const otoo_src* src, int64_t n, const double
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     float4* pairs = static_cast<float4*>(scratch);
     const unsigned nb = (unsigned)((n + 255) / 256);
-    k_split<<<nb, 256, 0, s>>>(src, pairs, n);
+    k_split<<<nb, 256, 0, s>>>(src, pairs, n, nullptr);
     CUDA_TRY(cudaGetLastError());
     k_centre_relative<<<nb, 256, 0, s>>>(pairs, n, (float)c[0], (float)c[1], (float)c[2], out);
     CUDA_TRY(cudaGetLastError());

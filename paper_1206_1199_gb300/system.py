@@ -348,8 +348,7 @@ def _stream(stream, device):
 
 class BufferPool:
     """Device buffers kept between steps (grown when too small), so that a
-    loop of device walks and force steps reuses the same memory and the
-    force step's recorded graph."""
+    loop of device walks and force steps reuses the same memory."""
 
     def __init__(self, device):
         self.device = device
