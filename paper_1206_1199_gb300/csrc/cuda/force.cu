@@ -19,8 +19,8 @@
 //                 packed two-wide FP32 pairs on group-centre-relative coordinates, plain FP32
 //                 sums between Kahan-compensated flushes, FP64 merge of the
 //                 lane-level j-split and FP64 outputs.
-//   k_force_f64   FP64 form (comparison form): one work item per CTA, every
-//                 pair in FP64.
+//   k_force_f64   FP64 form (comparison form): one work item per CTA, FP64
+//                 pairs (the quadrupole part in two-float arithmetic).
 //   k_merge       FP64 sum of the chunk partials of split lists, in chunk
 //                 order (deterministic).
 #include <cuda_runtime.h>
@@ -41,6 +41,7 @@ constexpr uint32_t kBadItem = 1u;
 constexpr uint32_t kBadIndex = 2u;
 
 #include "pair.cuh"
+#include "twofloat.cuh"
 
 __device__ __forceinline__ void load_src(const otoo_src* src, int64_t idx, double& x, double& y, double& z, float& m)
 {
@@ -74,8 +75,9 @@ __device__ __forceinline__ bool item_ok(const otoo_dev_system& sys, const otoo_i
 }
 
 // Final write of one target: the output, or the FP64 partial of the item's
-// list chunk.  The kernels take the self pair (r = 0, which adds -m_i / eps
-// to phi_i) out of the item whose list chunk starts at entry 0.
+// list chunk.  The FP32 kernels take the self pair (r = 0, which adds -m_i / eps
+// to phi_i) out of the item whose list chunk starts at entry 0; the FP64 form
+// gives it no mass.
 __device__ __forceinline__ void write_target(const otoo_dev_system& sys, const otoo_group& grp, const otoo_item& item,
                                              int i, const double a[4], double* __restrict__ accel,
                                              double* __restrict__ pot)
@@ -151,14 +153,22 @@ __global__ void k_centre_relative(const float4* __restrict__ pairs, int64_t n, f
 #include "force_warp2.cuh"
 
 // FP64 form: one work item per CTA of B threads, IB targets per thread,
-// B entries staged per tile, every pair in FP64.
+// B entries staged per tile; particles and monopoles in FP64, of a quadrupole
+// cell the monopole part (pair_quad_mixed).  Bound by the FP64 pipe, 18
+// operations per pair.  N = 2^17 (4.7e8 pairs, 70% with cells): 17.1 ms against
+// 28.3 ms with the quadrupole part in FP64 too (38 operations); error against
+// extended precision on the same lists (2-norm, accelerations) 4.5e-16 both, the
+// potentials' 1.7e-16 and 1.6e-16; over four models, theta 0.5 to 0.9,
+// softenings 1e-4 to 0.3 and lengths of 1 and 1e12 accelerations 1.3e-16 to
+// 5.5e-16 (within 6% of each other), potentials 1.3e-16 to 1.8e-16 (0.92 to 1.07).
 template <int B, int IB>
 __global__ void __launch_bounds__(B) k_force_f64(const otoo_dev_system sys, double* __restrict__ accel,
                                                  double* __restrict__ pot)
 {
     __shared__ V4<double> s_src[B];
-    __shared__ V4<double> s_qa[B];
-    __shared__ V4<double> s_qb[B];
+    __shared__ float4 s_qa[B];
+    __shared__ float4 s_qb[B];
+    __shared__ int s_idx[B];  // particle entries: their source index
     __shared__ double s_red[B * IB * 4];
     __shared__ int s_ticket;
 
@@ -189,9 +199,13 @@ __global__ void __launch_bounds__(B) k_force_f64(const otoo_dev_system sys, doub
 
         double xi[IB], yi[IB], zi[IB];
         Acc<double> acc[IB];
+        QuadSum qsum[IB];
+        int self[IB];  // the target's own source index
 #pragma unroll
         for (int k = 0; k < IB; ++k) {
             const int i = islot + k * P;
+            qsum[k].zero();
+            self[k] = active && i < ni ? grp.first + item.i0 + i : -1;
             xi[k] = yi[k] = zi[k] = 0.0;
             if (active && i < ni) {
                 double x, y, z;
@@ -225,6 +239,7 @@ __global__ void __launch_bounds__(B) k_force_f64(const otoo_dev_system sys, doub
                         atomicOr(status, kBadIndex);
                     }
                     s_src[tid] = v;
+                    s_idx[tid] = good ? idx : -2;
                     if (quad) {
                         float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
                         if (good) {
@@ -232,9 +247,8 @@ __global__ void __launch_bounds__(B) k_force_f64(const otoo_dev_system sys, doub
                             a = __ldg(qp);
                             b = __ldg(qp + 1);
                         }
-                        s_qa[tid] = V4<double>{a.x, a.y, a.z, a.w};
-                        // (xz, yz, B_2 eps^2, -) for the softened quadrupole term
-                        s_qb[tid] = V4<double>{b.x, b.y, (double)b.z * eps2, 0.0};
+                        s_qa[tid] = a;
+                        s_qb[tid] = b;
                     }
                 }
                 __syncthreads();
@@ -245,16 +259,19 @@ __global__ void __launch_bounds__(B) k_force_f64(const otoo_dev_system sys, doub
                     if (quad) {
                         for (int j = js; j < cnt; j += nsplit) {
                             const V4<double> s = s_src[j];
-                            const V4<double> qa = s_qa[j];
-                            const V4<double> qb = s_qb[j];
+                            const float4 qa = s_qa[j], qb = s_qb[j];
 #pragma unroll
-                            for (int k = 0; k < IB; ++k) pair_quad(s, qa, qb, xi[k], yi[k], zi[k], eps2, p[k]);
+                            for (int k = 0; k < IB; ++k)
+                                pair_quad_mixed(s, qa, qb, xi[k], yi[k], zi[k], eps2, p[k], qsum[k]);
                         }
                     } else {
                         for (int j = js; j < cnt; j += nsplit) {
                             const V4<double> s = s_src[j];
+                            const int idx = s_idx[j];
 #pragma unroll
-                            for (int k = 0; k < IB; ++k) pair_mono(s, xi[k], yi[k], zi[k], eps2, p[k]);
+                            for (int k = 0; k < IB; ++k)
+                                pair_mono(V4<double>{s.x, s.y, s.z, idx == self[k] ? 0.0 : s.w}, xi[k], yi[k], zi[k],
+                                          eps2, p[k]);  // j != i
                         }
                     }
 #pragma unroll
@@ -265,6 +282,8 @@ __global__ void __launch_bounds__(B) k_force_f64(const otoo_dev_system sys, doub
         }
 
         if (active) {
+#pragma unroll
+            for (int k = 0; k < IB; ++k) qsum[k].fold(acc[k].s);
 #pragma unroll
             for (int k = 0; k < IB; ++k)
 #pragma unroll
@@ -277,13 +296,6 @@ __global__ void __launch_bounds__(B) k_force_f64(const otoo_dev_system sys, doub
             for (int j = 0; j < nsplit; ++j)
 #pragma unroll
                 for (int c = 0; c < 4; ++c) a[c] += s_red[((j * P + sl) * IB + k) * 4 + c];
-            if (item.j0 == 0) {
-                // the self pair added -m_i rsqrt(eps^2) in FP64: take it out
-                double x, y, z;
-                float m;
-                load_src(sys.src, (int64_t)grp.first + item.i0 + i, x, y, z, m);
-                a[3] += (double)m * rsqrt(eps2);
-            }
             write_target(sys, grp, item, i, a, accel, pot);
         }
         __syncthreads();

@@ -10,9 +10,6 @@
 template <typename R> struct V4;
 template <> struct __align__(16) V4<float> { float x, y, z, w; };
 template <> struct __align__(32) V4<double> { double x, y, z, w; };
-template <typename R> struct V2;
-template <> struct __align__(8) V2<float> { float x, y; };
-template <> struct __align__(16) V2<double> { double x, y; };
 
 // FP32 reciprocal square root: the hardware approximation (PTX
 // rsqrt.approx.ftz.f32, relative error about 2^-23); the argument r^2 + eps^2
@@ -81,35 +78,6 @@ __device__ __forceinline__ void pair_mono(const V4<R>& s, R xi, R yi, R zi, R ep
     p[2] = fma(mq3, rz, p[2]);
 }
 
-// Quadrupole cell: the second-order Taylor term of the softened pair law
-// about the cell's centre of mass.  With q = (r^2 + eps^2)^(-1/2), the
-// traceless Q and w = r.Q.r - B_2 eps^2 (B_2 = sum m |x - com|^2; the B_2
-// part vanishes without softening):
-//   phi -= m q + (1/2) w q^5,  a += (m q^3 + (5/2) w q^7) r - q^5 Q r.
-// qa = (Qxx, Qyy, Qzz, Qxy), qb = (Qxz, Qyz, B_2 eps^2, -).
-template <typename R>
-__device__ __forceinline__ void pair_quad(const V4<R>& s, const V4<R>& qa, const V4<R>& qb, R xi, R yi, R zi,
-                                          R eps2, R p[4])
-{
-    const R rx = s.x - xi, ry = s.y - yi, rz = s.z - zi;
-    const R r2 = fma(rx, rx, fma(ry, ry, fma(rz, rz, eps2)));
-    const R q = rsqrt_r(r2);
-    const R q2 = q * q;
-    const R mq = s.w * q;
-    const R qr0 = fma(qa.x, rx, fma(qa.w, ry, qb.x * rz));
-    const R qr1 = fma(qa.w, rx, fma(qa.y, ry, qb.y * rz));
-    const R qr2 = fma(qb.x, rx, fma(qb.y, ry, qa.z * rz));
-    const R w = fma(rx, qr0, fma(ry, qr1, fma(rz, qr2, -qb.z)));
-    const R q5 = q * (q2 * q2);
-    const R t = w * q5;
-    p[3] -= fma(R(0.5), t, mq);
-    // radial coefficient m q^3 + (5/2) w q^7 = q^2 (m q + (5/2) w q^5)
-    const R cr = q2 * fma(R(2.5), t, mq);
-    p[0] = fma(cr, rx, fma(-q5, qr0, p[0]));
-    p[1] = fma(cr, ry, fma(-q5, qr1, p[1]));
-    p[2] = fma(cr, rz, fma(-q5, qr2, p[2]));
-}
-
 typedef unsigned long long f2;
 
 __device__ __forceinline__ f2 f2pack(float lo, float hi)
@@ -174,8 +142,13 @@ __device__ __forceinline__ void pair_mono2(f2 sx, f2 sy, f2 sz, f2 m, f2 nx, f2 
     A.v[2] = f2fma(mq3, rz, A.v[2]);
 }
 
-// Two quadrupole cells against one target: the law of pair_quad with the
-// fields of -Q, n = -Q r and u = r.n + B_2 eps^2 = -w (te = B_2 eps^2):
+// Two quadrupole cells against one target.  A cell's term is the second-order
+// Taylor term of the softened pair law about its centre of mass: with q = (r^2 +
+// eps^2)^(-1/2), the traceless Q and w = r.Q.r - B_2 eps^2 (B_2 = sum
+// m |x - com|^2; the B_2 part vanishes without softening),
+//   phi -= m q + (1/2) w q^5,  a += (m q^3 + (5/2) w q^7) r - q^5 Q r.
+// Here with the fields of -Q, n = -Q r and u = r.n + B_2 eps^2 = -w (te =
+// B_2 eps^2):
 //   A[3] += m q - (1/2) u q^5,  A[0..2] += (m q^3 - (5/2) u q^7) r + q^5 n;
 // mhalf = (-1/2, -1/2), m5half = (-5/2, -5/2).
 __device__ __forceinline__ void pair_quad2(f2 sx, f2 sy, f2 sz, f2 m, f2 nqxx, f2 nqyy, f2 nqzz, f2 nqxy, f2 nqxz,
