@@ -489,7 +489,7 @@ typedef struct otoo_dev_walk {
     int32_t set;                   /* groups one warp walks together (consecutive in group
                                       order; each cell's record loaded once and tested per
                                       group): 1..8, or 0 = up to 8 while every resident warp
-                                      gets about three sets.  Same entries per group for
+                                      gets about one set.  Same entries per group for
                                       every value (their order within a group may differ).
                                       Other values: OTOO_EINVAL */
     double theta;                  /* opening angle when theta_per_group is NULL (>= 0) */

@@ -5,17 +5,18 @@
 // minimum distance, after Barnes 1990) and Section II-A (the traversal rules:
 // accept a cell, open a cell into its children, take a leaf's particles).
 // The paper walks with one work-item per group along next/more links; here
-// one warp walks one group over a shared-memory stack, 32 cells at a time,
-// and writes the group's list for the force kernels (the host walk's lists,
+// one warp walks a set of neighbouring groups over a shared-memory stack, 64
+// cells at a time, and writes each group's list for the force kernels (the host walk's lists,
 // entry for entry, as sets per group).
 //
 // Kernels
-//   k_walk<false>   pass 1: the group's box (warp min/max over its particles),
-//                   the walk, entry counts into the group record.
+//   k_walk_set<0>   pass 1: the groups' boxes (warp min/max over their particles),
+//                   the walk, entry counts into the group records.
 //   k_scan_*        exclusive prefix sums in group order (list offsets, plan
 //                   slots): block sums, one-CTA scan of the block sums,
 //                   block-level scans with the block offsets.
-//   k_walk<true>    pass 2: the same walk, entries written at the offsets.
+//   k_walk_set<1>   pass 2: the same walk, entries written at the offsets.
+//   k_walk_set<2>   both in one pass, entries written into fixed slots.
 //   k_plan_count    per group: particle and list chunks (the cost model of the
 //                   host plan), cost class histogram, sums per block.
 //   k_plan_scan     prefixes of the block sums; start of each cost class, most
@@ -51,6 +52,8 @@ constexpr int kTotals = 6;          // walk totals: entries, interactions, cell 
                                     // largest n_cell, largest n_part, groups beyond their slots
 
 #include "pair.cuh"
+
+constexpr double kCubeAngle = 0.57;  // below 1/sqrt(3) = 0.5774 the test needs no cube overlap part
 
 // status bits (counter[1])
 constexpr uint32_t kWalkBadRecord = 1u;   // a cell record failed its bounds check
@@ -214,70 +217,6 @@ __device__ __forceinline__ int mac_filter_sw(const otoo_wcell& w, const BoxF& g)
     return -1;
 }
 
-// mac_filter and mac_filter_sw with the parts that depend on the cell alone
-// computed once per cell by the caller (the set walk tests one cell against
-// several groups): acell = |com_hi[0]| + |com_hi[1]| + |com_hi[2]| and, for
-// the opening angle, thr = side / theta + s as mac_filter rounds it.  Only K
-// (the scale of the rounding bound) is summed in another order, which moves
-// it by a few FP32 roundings, far inside the margins.
-template <bool kOverlap>
-__device__ __forceinline__ int mac_filter_pc(const otoo_wcell& w, const BoxF& g, float acell, float thr)
-{
-    float u[3], au = 0.f;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        u[a] = __fadd_rn(__fsub_rn(w.com_hi[a], g.c32[a]), __fsub_rn(w.com_lo[a], g.cl32[a]));
-        au += fabsf(u[a]);
-    }
-    const float K = au + g.B + thr + w.side + (g.A + acell) * 0x1p-24f;
-    if (kOverlap) {
-        const float del = K * 0x1p-18f;
-        bool sep = false, ovl = true;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const float lo = __fsub_rn(u[a], w.e[a]);
-            const float hi = __fadd_rn(lo, w.side);
-            sep = sep || (lo > g.bh[a] + del) || (g.bl[a] > hi + del);
-            ovl = ovl && (lo < g.bh[a] - del) && (g.bl[a] < hi - del);
-        }
-        if (ovl) return 0;
-        if (!sep) return -1;
-    }
-    float d2 = 0.f;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const float d = fmaxf(0.f, fmaxf(g.bl[a] - u[a], u[a] - g.bh[a]));
-        d2 = fmaf(d, d, d2);
-    }
-    const float thr2 = thr * thr, m = K * K * 0x1p-16f;
-    if (d2 > thr2 + m) return 1;
-    if (d2 < thr2 - m) return 0;
-    return -1;
-}
-
-__device__ __forceinline__ int mac_filter_sw_pc(const otoo_wcell& w, const BoxF& g, float acell)
-{
-    const float rb = w.rb;
-    if (!(rb <= 3.0e38f)) return 0;
-    float u[3], au = 0.f;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        u[a] = __fadd_rn(__fsub_rn(w.com_hi[a], g.c32[a]), __fsub_rn(w.com_lo[a], g.cl32[a]));
-        au += fabsf(u[a]);
-    }
-    const float K = au + g.B + rb + (g.A + acell) * 0x1p-24f;
-    float d2 = 0.f;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const float d = fmaxf(0.f, fmaxf(g.bl[a] - u[a], u[a] - g.bh[a]));
-        d2 = fmaf(d, d, d2);
-    }
-    const float rb2 = rb * rb, m = K * K * 0x1p-16f;
-    if (d2 > rb2 + m) return 1;
-    if (d2 < rb2 - m) return 0;
-    return -1;
-}
-
 __device__ __forceinline__ otoo_wcell load_wcell(const otoo_wcell* __restrict__ cell, int k)
 {
     float v[16];
@@ -316,23 +255,19 @@ __device__ __forceinline__ long long dkey(double x)
 }
 __device__ __forceinline__ double dval(long long k) { return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL)); }
 
+// Of signed 64-bit keys: the high words, then the low words of the lanes that
+// hold that high word (two reductions instead of five rounds of shuffles).
 __device__ __forceinline__ long long warp_min(long long v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const long long t = __shfl_xor_sync(kFull, v, o);
-        v = t < v ? t : v;
-    }
-    return v;
+    const int h = (int)(v >> 32), m = __reduce_min_sync(kFull, h);
+    const unsigned l = __reduce_min_sync(kFull, h == m ? (unsigned)v : 0xffffffffu);
+    return ((long long)m << 32) | l;
 }
 __device__ __forceinline__ long long warp_max(long long v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const long long t = __shfl_xor_sync(kFull, v, o);
-        v = t > v ? t : v;
-    }
-    return v;
+    const int h = (int)(v >> 32), m = __reduce_max_sync(kFull, h);
+    const unsigned l = __reduce_max_sync(kFull, h == m ? (unsigned)v : 0u);
+    return ((long long)m << 32) | l;
 }
 
 // A stack entry is a run of consecutive cells (the children of one cell):
@@ -354,9 +289,9 @@ struct GroupWalk {
 };
 
 // The box of particles [first, first + count) (min/max on order-preserving
-// integer keys, exact), its FP32 form for the filter, and the group's rule.
-__device__ __forceinline__ void group_walk_setup(const WalkArgs& a, int g, int32_t first, int32_t count, int lane,
-                                                 GroupWalk& w)
+// integer keys, exact).
+__device__ __forceinline__ void group_box(const WalkArgs& a, int32_t first, int32_t count, int lane, double lo[3],
+                                          double hi[3])
 {
     long long klo[3], khi[3];
 #pragma unroll
@@ -369,12 +304,22 @@ __device__ __forceinline__ void group_walk_setup(const WalkArgs& a, int g, int32
         klo[1] = ky < klo[1] ? ky : klo[1], khi[1] = ky > khi[1] ? ky : khi[1];
         klo[2] = kz < klo[2] ? kz : klo[2], khi[2] = kz > khi[2] ? kz : khi[2];
     }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        lo[k] = dval(warp_min(klo[k]));
+        hi[k] = dval(warp_max(khi[k]));
+    }
+}
+
+// A group's box, its FP32 form for the filter, and the group's rule.
+__device__ __forceinline__ void group_walk_setup(const WalkArgs& a, int g, int32_t first, int32_t count, int lane,
+                                                 GroupWalk& w)
+{
+    group_box(a, first, count, lane, w.blo, w.bhi);
     w.bf.B = 0.f;
     w.bf.A = 0.f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        w.blo[k] = dval(warp_min(klo[k]));
-        w.bhi[k] = dval(warp_max(khi[k]));
         w.c[k] = __dmul_rn(__dadd_rn(w.blo[k], w.bhi[k]), 0.5);
         w.bf.c32[k] = __double2float_rn(w.c[k]);
         w.bf.cl32[k] = __double2float_rn(__dsub_rn(w.c[k], (double)w.bf.c32[k]));
@@ -391,7 +336,7 @@ __device__ __forceinline__ void group_walk_setup(const WalkArgs& a, int g, int32
     // the per-group choices as bits of an integer, taken through an opaque
     // move: the compiler must not re-derive them from theta inside the
     // walk loop, where FP64 compares would occupy GB300's narrow FP64 pipe
-    int fl = (!w.sw && !(w.theta > 0.0) ? 1 : 0) | (w.theta < 0.57 ? 2 : 0);  // 0.57 < 1/sqrt(3) = 0.5774
+    int fl = (!w.sw && !(w.theta > 0.0) ? 1 : 0) | (w.theta < kCubeAngle ? 2 : 0);
     asm volatile("mov.b32 %0, %0;" : "+r"(fl));
     w.open_all = (fl & 1) != 0;
     w.small_angle = (fl & 2) != 0;
@@ -509,153 +454,7 @@ __device__ __forceinline__ void walk_push(uint32_t* stk, int& sp, const StepCell
     __syncwarp();
 }
 
-// One warp per group (atomic ticket).  The stack holds runs of sibling
-// cells; each step takes up to kWide = 32 kWalkHalves cells from the top runs
-// (walk_take; lane j tests the cells at positions j, j + 32, ...), emits
-// accepted cells and rejected leaves' particles in position order and pushes
-// one run per rejected inner cell (its children, walk_push).  A kWide-cell
-// step adds at most kWide entries and runs only with kWide + 1 + kMaxLevels
-// entries free; otherwise the step takes one cell, which adds at most one
-// entry, and only when it descends a level (a tree has at most kMaxLevels
-// levels below any cell), so the stack never overflows.
-// kMode 0: count (group records, totals); 1: fill the list at the offsets
-// of pass 0; 2: single pass -- count as pass 0 and write each group's entries
-// into its fixed slot of list (capacity cells + pcap particles per slot):
-// cells backwards from slot position capacity - 1, particles forwards from
-// capacity, so that they end up contiguous, cells first, and the slots serve
-// as the list (list_off set here; groups that outgrow their slot get -1).
-template <int kMode>
-__global__ void __launch_bounds__(kWalkWarps * 32, OTOO_WALK_MIN_BLOCKS) k_walk(WalkArgs a, otoo_group* __restrict__ groups,
-                                                          int32_t* __restrict__ list, int64_t capacity, int64_t pcap)
-{
-    constexpr bool kFill = kMode == 1;
-    constexpr bool kCount = kMode != 1;
-    constexpr bool kWrite = kMode != 0;
-    __shared__ uint32_t stack_s[kWalkWarps][kStack];
-    const int lane = threadIdx.x & 31;
-    uint32_t* stk = stack_s[threadIdx.x >> 5];
-    const unsigned lt = (1u << lane) - 1u;
-    uint32_t* status = a.counter + 1;
-    if (kFill && a.totals[0] > capacity) {
-        if (threadIdx.x == 0) atomicOr(status, kWalkNoRoom);
-        return;
-    }
-    for (;;) {
-        int g = 0;
-        if (lane == 0) g = (int)atomicAdd(a.counter, 1u);
-        g = __shfl_sync(kFull, g, 0);
-        if (g >= a.n_groups) break;
-        const int32_t first = a.gfirst[g], count = a.gcount[g];
-        if (first < 0 || count < 1 || count > kMaxGroup || (int64_t)first + count > a.n_part) {
-            if (lane == 0) {
-                atomicOr(status, kWalkBadGroup);
-                if (kCount) {
-                    otoo_group z = {};
-                    z.first = first;
-                    z.eps2 = a.eps2;
-                    z.theta = -1.f;
-                    groups[g] = z;
-                }
-            }
-            continue;
-        }
-        GroupWalk w;
-        group_walk_setup(a, g, first, count, lane, w);
-        int64_t off_c = 0, off_p = 0;
-        int32_t want_c = 0, want_p = 0;
-        if (kMode == 2) {
-            // cell r at off_c - r, particle k at off_p + k
-            off_p = (int64_t)g * (capacity + pcap) + capacity;
-            off_c = off_p - 1;
-            want_c = (int32_t)capacity;
-            want_p = (int32_t)pcap;
-        }
-        if (kFill) {
-            const otoo_group gr = groups[g];
-            off_c = gr.list_off;
-            want_c = gr.n_cell;
-            want_p = gr.n_part;
-            off_p = off_c + want_c;
-            if (off_c < 0 || want_c < 0 || want_p < 0 || off_p + want_p > capacity) {
-                if (lane == 0) atomicOr(status, kWalkNoRoom);
-                continue;
-            }
-        }
-        int32_t ncell = 0, npart = 0;
-        int sp = 0;
-        if (w.theta >= 0.0) {
-            if (lane == 0) stk[0] = run(0, 1);
-            sp = 1;
-        }
-        __syncwarp();
-        int64_t budget = a.n_cell;  // a tree visits each cell at most once
-        bool failed = false;
-        while (sp > 0) {
-            StepCells sc;
-            if (!walk_take(a, w, stk, sp, budget, lane, sc, status)) {
-                failed = true;
-                break;
-            }
-            // accepted cells, in position order
-#pragma unroll
-            for (int h = 0; h < kWalkHalves; ++h) {
-                const unsigned am = __ballot_sync(kFull, sc.kind[h] == 1 && !w.drop);
-                if (kWrite && sc.kind[h] == 1 && !w.drop) {
-                    const int32_t r = ncell + __popc(am & lt);
-                    if (r < want_c) list[kMode == 2 ? off_c - r : off_c + r] = (int32_t)(a.n_part + sc.node[h]);
-                }
-                ncell += __popc(am);
-            }
-            // particles of rejected leaves, in position order
-#pragma unroll
-            for (int h = 0; h < kWalkHalves; ++h) {
-                if (!__any_sync(kFull, sc.kind[h] == 2)) continue;
-                const int np = sc.kind[h] == 2 ? sc.pe[h] - sc.pb[h] : 0;
-                const int pin = warp_incl_scan(np, lane);
-                if (kWrite && np > 0) {
-                    const int32_t base = npart + pin - np;
-                    for (int k = 0; k < np; ++k)
-                        if (base + k < want_p) list[off_p + base + k] = sc.pb[h] + k;
-                }
-                npart += __shfl_sync(kFull, pin, 31);
-            }
-            walk_push(stk, sp, sc, lt);
-        }
-        if (failed && lane == 0) atomicOr(status, kWalkOverflow);
-        if (kCount) {
-            if (lane == 0) {
-                otoo_group r;
-                r.first = first;
-                r.count = count;
-                r.n_cell = ncell;
-                r.n_part = npart;
-                // pass 0: the offsets come from the scan that follows
-                r.list_off = kMode == 2 ? (ncell <= want_c && npart <= want_p ? off_p - ncell : -1) : 0;
-                r.eps2 = a.eps2;
-                r.cx = w.c[0];
-                r.cy = w.c[1];
-                r.cz = w.c[2];
-                r.theta = (float)w.theta;
-                r.sys = 0;
-                groups[g] = r;
-                const int64_t len = (int64_t)ncell + npart;
-                atomicAdd(reinterpret_cast<unsigned long long*>(a.totals), (unsigned long long)len);
-                atomicAdd(reinterpret_cast<unsigned long long*>(a.totals + 1), (unsigned long long)(len * count));
-                atomicAdd(reinterpret_cast<unsigned long long*>(a.totals + 2),
-                          (unsigned long long)((int64_t)ncell * count));
-                atomicMax(reinterpret_cast<unsigned long long*>(a.totals + 3), (unsigned long long)ncell);
-                atomicMax(reinterpret_cast<unsigned long long*>(a.totals + 4), (unsigned long long)npart);
-                if (kMode == 2 && (ncell > want_c || npart > want_p))
-                    atomicAdd(reinterpret_cast<unsigned long long*>(a.totals + 5), 1ull);
-            }
-        } else if (lane == 0 && (ncell != want_c || npart != want_p)) {
-            atomicOr(status, kWalkMismatch);
-        }
-    }
-}
-
-
-// ---- the walk of a set of groups ----------------------------------------------
+// ---- the walk over lists -------------------------------------------------------
 //
 // Groups that are neighbours in tree order lie close together, and their walks
 // test mostly the same cells: for the sets of groups under one parent cell of
@@ -664,65 +463,110 @@ __global__ void __launch_bounds__(kWalkWarps * 32, OTOO_WALK_MIN_BLOCKS) k_walk(
 // cells.  k_walk_set walks up to kSet consecutive groups with one warp: every
 // stack run carries the mask of the set's groups for which the run's cells
 // are still open (all their ancestors rejected), a taken cell's record is
-// loaded once and tested against each group of its mask with that group's
-// own test (the FP32 filter and the FP64 fallback of k_walk), and each group
-// keeps its own counts and list slots.  A cell a group accepts is emitted
-// for that group, a rejected leaf's particles go to every group that rejected
-// it, and an inner cell rejected by any group is opened with the mask of the
-// groups that rejected it.  Restricted to one group, the walk visits exactly
-// the cells the group's own walk visits and takes the same decisions, so
-// each group's entries are those of k_walk (as sets; the order of a group's
-// entries is the union walk's).  The stack bound of k_walk holds unchanged
-// (one run per opened cell).
+// loaded once and tested against each group of its mask, and each group keeps
+// its own counts and list slots.  A cell a group accepts is emitted for that
+// group, a rejected leaf's particles go to every group that rejected it, and
+// an inner cell rejected by any group is opened with the mask of the groups
+// that rejected it.  Restricted to one group, the walk visits exactly the
+// cells the group's own walk visits and takes the same decisions (those of the
+// FP64 test), so each group's entries are the same set whatever the sets are;
+// their order is the union walk's.
+//
+// The stack holds runs of sibling cells; each step takes up to kWide = 32
+// kWalkHalves cells from the top runs (set_take; lane j tests the cells at
+// positions j, j + 32, ...) and pushes one run per rejected inner cell
+// (set_push).  A kWide-cell step adds at most kWide entries and runs only with
+// kWide + 1 + kMaxLevels entries free; otherwise the step takes one cell,
+// which adds at most one entry, and only when it descends a level (a tree has
+// at most kMaxLevels levels below any cell), so the stack never overflows.
+//
+// Bound by instruction issue.  Everything of the test that the cell alone
+// decides (its centre of mass relative to the set's common centre, the squared
+// distances beyond which it is accepted and below which it is rejected) is
+// computed once per cell, with the rounding margin of the set's largest
+// group, and the groups are taken in a loop that the whole warp runs in step:
+// a test is 12 operations and two comparisons, its accepted cells are written
+// in the same turn.  Before, every lane went through its own cell's groups with
+// their own margins (5.8 tests of 18 lanes a step where four of 27 do, N = 2^20
+// taken two groups at a time; 977 instructions a step in all) and a second
+// loop wrote the entries.  Plummer N = 2^20, n_crit 128: 1.24 -> 0.81 ms (980
+// -> 642 million instructions) in sets of two, 0.68 ms in the sets taken now;
+// Hernquist N = 2^23 6.37 -> 3.81 ms; absolute MAC, N = 2^23 1.90 -> 1.42 ms.
 
 constexpr int kSet = 8;  // groups per set at most (one bit each in a run's mask)
 
-// One group of a set: its rule and box (as GroupWalk) and where its entries go.
+// One group of a set: its box relative to the set's centre, its rule, and where
+// its entries go.
 struct SetGroup {
-    BoxF bf;
-    double blo[3], bhi[3], c[3];
-    double theta;
-    float invth;
+    float bl[3], bh[3];
+    float invth;           // 1 / theta rounded to FP32
     int32_t flags;         // 1: opening angle 0 (nothing accepted), 2: theta < 1/sqrt(3)
-    int32_t first, count;
+    double blo[3], bhi[3]; // the particles' box
+    double theta;          // opening angle (0 for the absolute MAC / SPH)
     int64_t off_c, off_p;  // where cell r and particle k go (cells backwards in the single pass)
     int32_t want_c, want_p;
 };
 
-// Cells of one set-walk step: lane j holds positions j + 32 h of the taken
-// runs; acc / rej: masks of the groups that accept / reject the cell.
-struct SetStep {
-    int node[kWalkHalves], c0[kWalkHalves], nch[kWalkHalves], pb[kWalkHalves], pe[kWalkHalves];
-    unsigned acc[kWalkHalves], rej[kWalkHalves];
+// What the set's groups have in common.
+struct SetRule {
+    float4 c;   // centre of the set rounded to FP32; 1 / theta (if it is one for all)
+    float4 cl;  // the centre's low words; sum over axes of |c| 2^-24 + the largest group's sum of max(|bl|, |bh|)
 };
 
-// The decision of group j of a set on cell nd (record c): 1 accept, 0 reject.
-// acell, thr_u: the cell's own parts of the filter (thr_u for the set's
-// common angle, used when uni).
-__device__ __forceinline__ int set_decide(const WalkArgs& a, const SetGroup& g, bool sw, const otoo_wcell& c, int nd,
-                                          float acell, float thr_u, bool uni)
+// One cell of a step in the filter: the centre of mass relative to the set's
+// centre, the distance test's two limits, and what the cube test needs.
+struct SetCell {
+    float u[3], tu, tl;
+    float e[3], side, s, K, del;
+};
+
+// The limits for threshold thr (a length): the squared distance decides when it
+// differs from thr^2 by more than 2^-16 K^2.  Every rounded quantity is within
+// 2^-20 K of its exact value (K: sum of the magnitudes the test combines, plus
+// 2^-24 of the absolute coordinates for the truncated low words), so what the
+// limits decide the exact arithmetic and the host's FP64 decide the same way.
+__device__ __forceinline__ void set_limits(SetCell& c, float thr)
 {
-    if (sw) {
-        int dec = a.exact ? -1 : mac_filter_sw_pc(c, g.bf, acell);
-        if (dec < 0) dec = sw_exact(a.cell64, nd, g.blo, g.bhi) ? 1 : 0;
-        return dec;
-    }
-    if (g.flags & 1) return 0;
-    const float thr = uni ? thr_u : __fadd_rn(__fmul_rn(c.side, g.invth), c.s);
-    int dec = a.exact ? -1 : (g.flags & 2) ? mac_filter_pc<false>(c, g.bf, acell, thr)
-                                           : mac_filter_pc<true>(c, g.bf, acell, thr);
-    if (dec < 0) dec = mac_exact(a.cell64, nd, g.blo, g.bhi, g.theta) ? 1 : 0;
-    return dec;
+    const float K = c.K + thr, thr2 = thr * thr, m = K * K * 0x1p-16f;
+    c.tu = thr2 + m;
+    c.tl = thr2 - m;
+    c.del = K * 0x1p-18f;
 }
 
-// walk_take for a set: takes up to kWide cells with their runs' masks and
-// tests each against the groups of its mask.
-__device__ __forceinline__ bool set_take(const WalkArgs& a, const SetGroup* sg, bool sw, float invth_u, bool uni,
-                                         uint32_t* stk, uint8_t* msk, int& sp, int64_t& budget, int lane, SetStep& st,
-                                         uint32_t* status)
+__device__ __forceinline__ SetCell set_cell(const otoo_wcell& w, const SetRule& r, bool sw, bool none, bool exact)
+{
+    SetCell c;
+    const float4 h = r.c, l = r.cl;
+    c.u[0] = __fadd_rn(__fsub_rn(w.com_hi[0], h.x), __fsub_rn(w.com_lo[0], l.x));
+    c.u[1] = __fadd_rn(__fsub_rn(w.com_hi[1], h.y), __fsub_rn(w.com_lo[1], l.y));
+    c.u[2] = __fadd_rn(__fsub_rn(w.com_hi[2], h.z), __fsub_rn(w.com_lo[2], l.z));
+    float au = 0.f, ac = 0.f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        au += fabsf(c.u[a]);
+        ac += fabsf(w.com_hi[a]);
+        c.e[a] = w.e[a];
+    }
+    c.side = w.side;
+    c.s = w.s;
+    c.K = au + l.w + ac * 0x1p-24f + (sw ? 0.f : w.side);
+    set_limits(c, sw ? w.rb : __fadd_rn(__fmul_rn(w.side, h.w), w.s));
+    if (exact) c.tu = __int_as_float(0x7f800000), c.tl = -c.tu;
+    // angle 0, or an infinite r_b (delta = 0): nothing is accepted
+    if (none || (sw && !(w.rb <= 3.0e38f))) c.tu = c.tl = __int_as_float(0x7f800000);
+    return c;
+}
+
+// Takes up to kWide cells from the top runs of the stack (the last run may be
+// split, its rest goes back): the cell at position lane + 32 h and the mask of
+// its groups (0: no cell there).  False when the stack or the cell budget ran
+// out (the walk stops).
+__device__ __forceinline__ bool set_take(uint32_t* stk, uint8_t* msk, int& sp, int& budget, int lane,
+                                         int node[kWalkHalves], unsigned cm[kWalkHalves])
 {
     if (sp + 2 > kStack) return false;
     const int wcap = sp + kWide + 1 + kMaxLevels <= kStack ? kWide : 1;
+    // the top runs: lane l reads the l-th entry from the top
     const int nr = sp < 32 ? sp : 32;
     uint32_t e = 0;
     unsigned em = 0;
@@ -734,18 +578,21 @@ __device__ __forceinline__ bool set_take(const WalkArgs& a, const SetGroup* sg, 
     }
     const int rinc = warp_incl_scan(rn, lane);
     const int rstart = rinc - rn;
+    // runs wholly taken, and a run cut at wcap
     const bool whole = lane < nr && rinc <= wcap;
     const bool cut = lane < nr && rstart < wcap && rinc > wcap;
     const int nwhole = __popc(__ballot_sync(kFull, whole));
     const unsigned cutm = __ballot_sync(kFull, cut);
     const int in_whole = __shfl_sync(kFull, rinc, nwhole > 0 ? nwhole - 1 : 0);
     const int W = cutm ? wcap : (nwhole > 0 ? in_whole : 0);
+    // start positions of the taken runs, 32 positions per mask word
     unsigned starts[kWalkHalves];
 #pragma unroll
     for (int h = 0; h < kWalkHalves; ++h)
         starts[h] = __reduce_or_sync(kFull, (whole || cut) && rstart >= 32 * h && rstart < 32 * h + 32
                                                 ? (1u << (rstart - 32 * h))
                                                 : 0u);
+    // the run that continues after the cut goes back on the stack first
     sp -= nwhole + (cutm ? 1 : 0);
     if (cut) {
         const int taken = wcap - rstart;
@@ -755,74 +602,78 @@ __device__ __forceinline__ bool set_take(const WalkArgs& a, const SetGroup* sg, 
     sp += cutm ? 1 : 0;
     budget -= W;
     if (budget < 0) return false;
-    unsigned cm[kWalkHalves];
+    // position q lies in the run whose start is the last one <= q
 #pragma unroll
     for (int h = 0; h < kWalkHalves; ++h) {
         int r = -1;
 #pragma unroll
         for (int k = 0; k <= h; ++k) r += __popc(starts[k] & (k < h ? 0xffffffffu : (2u << lane) - 1u));
-        const uint32_t er = __shfl_sync(kFull, e, r < 0 ? 0 : r);
-        const int sr = __shfl_sync(kFull, rstart, r < 0 ? 0 : r);
-        cm[h] = __shfl_sync(kFull, em, r < 0 ? 0 : r);
+        r = r < 0 ? 0 : r;
+        const uint32_t er = __shfl_sync(kFull, e, r);
+        const int sr = __shfl_sync(kFull, rstart, r);
+        const unsigned mr = __shfl_sync(kFull, em, r);
         const int q = lane + 32 * h;
-        st.node[h] = q < W ? (int)(er & kRunMask) + (q - sr) : -1;
-        st.acc[h] = st.rej[h] = 0u;
-        st.c0[h] = st.nch[h] = st.pb[h] = st.pe[h] = 0;
+        node[h] = (int)(er & kRunMask) + (q - sr);
+        cm[h] = q < W ? mr : 0u;
     }
     __syncwarp();
-#pragma unroll
-    for (int h = 0; h < kWalkHalves; ++h) {
-        if (lane + 32 * h >= W) continue;
-        const int nd = st.node[h];
-        bool ok = nd >= 0 && nd < a.n_cell;
-        if (ok) {
-            const otoo_wcell c = load_wcell(a.cell, nd);
-            st.nch[h] = c.nchild;
-            st.c0[h] = c.child0;
-            st.pb[h] = c.begin;
-            st.pe[h] = c.end;
-            ok = st.nch[h] >= 0 && st.nch[h] <= 8 &&
-                 (st.nch[h] == 0 || (st.c0[h] > nd && (int64_t)st.c0[h] + st.nch[h] <= a.n_cell)) &&
-                 st.pb[h] >= 0 && st.pb[h] <= st.pe[h] && (int64_t)st.pe[h] <= a.n_part;
-            if (ok) {
-                const float acell = fabsf(c.com_hi[0]) + fabsf(c.com_hi[1]) + fabsf(c.com_hi[2]);
-                const float thr_u = __fadd_rn(__fmul_rn(c.side, invth_u), c.s);
-                unsigned ac = 0u;
-                for (unsigned m = cm[h] & ((1u << kSet) - 1u); m; m &= m - 1u) {
-                    const int j = __ffs(m) - 1;
-                    if (set_decide(a, sg[j], sw, c, nd, acell, thr_u, uni)) ac |= 1u << j;
-                }
-                st.acc[h] = ac;
-                st.rej[h] = cm[h] & ((1u << kSet) - 1u) & ~ac;
-            }
-        }
-        if (!ok) atomicOr(status, kWalkBadRecord);
-    }
     return true;
 }
 
-// walk_push for a set: one run per inner cell some group rejected, with the
-// mask of the groups that rejected it; the lowest position's run on top.
-__device__ __forceinline__ void set_push(uint32_t* stk, uint8_t* msk, int& sp, const SetStep& st, unsigned lt)
+// Rejected leaves of a walk with the masks of the groups that rejected them, in
+// the order their particles are listed: a ring per warp.  A step finds one to
+// six of them among its 64 cells; their particles are counted, scanned and
+// written for 32 leaves at once (set_flush).  A step adds at most kWide with
+// fewer than 32 held, so the ring is never full.
+constexpr int kLeafRing = 128;
+static_assert(kLeafRing >= kWide + 32 && (kLeafRing & (kLeafRing - 1)) == 0, "leaf ring");
+struct LeafRing {
+    int2 range[kLeafRing];  // first particle, one past the last
+    uint8_t mask[kLeafRing];
+};
+
+// Lists the particles of the ring's n <= 32 oldest leaves for the groups that
+// rejected them (lane j holds group j's count).
+template <bool kWrite>
+__device__ __forceinline__ void set_flush(const LeafRing& q, int head, int n, int lane, const SetGroup* sg,
+                                          int32_t* __restrict__ list, int& my_np)
 {
-#pragma unroll
-    for (int h = kWalkHalves - 1; h >= 0; --h) {
-        const bool op = st.rej[h] != 0u && st.nch[h] > 0;
-        const unsigned om = __ballot_sync(kFull, op);
-        const int no = __popc(om);
-        if (op) {
-            const int at = sp + no - 1 - __popc(om & lt);
-            stk[at] = run(st.c0[h], st.nch[h]);
-            msk[at] = (uint8_t)st.rej[h];
-        }
-        sp += no;
-    }
     __syncwarp();
+    int2 r = make_int2(0, 0);
+    unsigned m = 0u;
+    if (lane < n) {
+        r = q.range[(head + lane) & (kLeafRing - 1)];
+        m = q.mask[(head + lane) & (kLeafRing - 1)];
+    }
+    // (not unrolled: the walk loop must stay small for the instruction cache)
+#pragma unroll 1
+    for (unsigned gm = __reduce_or_sync(kFull, m); gm; gm &= gm - 1u) {
+        const int j = __ffs(gm) - 1;
+        const int np = (m >> j) & 1u ? r.y - r.x : 0;
+        const int pin = warp_incl_scan(np, lane);
+        const int had = __shfl_sync(kFull, my_np, j);
+        if (kWrite) {
+            const int32_t base = had + pin - np;
+            const int c = min(np, sg[j].want_p - base);
+            int32_t* o = list + sg[j].off_p + base;
+            for (int k = 0; k < c; ++k) o[k] = r.x + k;
+        }
+        const int sum = __shfl_sync(kFull, pin, 31);
+        if (lane == j) my_np = had + sum;
+    }
 }
 
-// One warp per set of gs <= kSet consecutive groups (atomic ticket over
-// sets); kMode as k_walk's.
-template <int kMode>
+// One warp per set of gs <= kSet consecutive groups (atomic ticket over sets).
+// kMode 0: count (group records, totals); 1: fill the list at the offsets
+// of pass 0; 2: single pass -- count as pass 0 and write each group's entries
+// into its fixed slot of list (capacity cells + pcap particles per slot):
+// cells backwards from slot position capacity - 1, particles forwards from
+// capacity, so that they end up contiguous, cells first, and the slots serve
+// as the list (list_off set here; groups that outgrow their slot get -1).
+// kGen: opening angles per group, or 1/sqrt(3) and more (plain_rule says which
+// form a walk needs); without it the loop over the groups holds five values of
+// a cell instead of twelve.
+template <int kMode, bool kGen>
 __global__ void __launch_bounds__(kWalkWarps * 32, OTOO_WALK_MIN_BLOCKS)
     k_walk_set(WalkArgs a, int32_t n_sets, int32_t gs, otoo_group* __restrict__ groups, int32_t* __restrict__ list,
                int64_t capacity, int64_t pcap)
@@ -833,13 +684,17 @@ __global__ void __launch_bounds__(kWalkWarps * 32, OTOO_WALK_MIN_BLOCKS)
     __shared__ uint32_t stack_s[kWalkWarps][kStack];
     __shared__ uint8_t mask_s[kWalkWarps][kStack];
     __shared__ SetGroup sg_s[kWalkWarps][kSet];
+    __shared__ LeafRing ring_s[kWalkWarps];
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
     uint32_t* stk = stack_s[wid];
     uint8_t* msk = mask_s[wid];
     SetGroup* sg = sg_s[wid];
+    LeafRing& ring = ring_s[wid];
     const unsigned lt = (1u << lane) - 1u;
     uint32_t* status = a.counter + 1;
+    // the absolute MAC and the SPH radius share the test d_min > r_b; an
+    // SPH walk drops the cells that pass it (no neighbour inside)
     const bool sw = a.mac == OTOO_MAC_SW || a.mac == OTOO_MAC_SPH;
     const bool drop = a.mac == OTOO_MAC_SPH;
     if (kFill && a.totals[0] > capacity) {
@@ -853,7 +708,6 @@ __global__ void __launch_bounds__(kWalkWarps * 32, OTOO_WALK_MIN_BLOCKS)
         if (set >= n_sets) break;
         const int g0 = set * gs;
         const int ng = min(gs, a.n_groups - g0);
-        unsigned live = 0u;   // groups that walk
         unsigned valid = 0u;  // groups with a record to write (pass 0 / single pass) or check (pass 1)
         for (int j = 0; j < ng; ++j) {
             const int g = g0 + j;
@@ -871,54 +725,90 @@ __global__ void __launch_bounds__(kWalkWarps * 32, OTOO_WALK_MIN_BLOCKS)
                 }
                 continue;
             }
-            GroupWalk w;
-            group_walk_setup(a, g, first, count, lane, w);
+            double lo[3], hi[3];
+            group_box(a, first, count, lane, lo, hi);
+            if (lane == 0)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) sg[j].blo[k] = lo[k], sg[j].bhi[k] = hi[k];
+            valid |= 1u << j;
+        }
+        // lane j: group j's rule and offsets
+        bool mine = lane < ng && ((valid >> lane) & 1u);
+        bool walks = false;
+        float my_inv = 0.f;
+        int my_fl = 0;
+        if (mine) {
+            SetGroup& q = sg[lane];
+            const double theta = sw ? 0.0 : a.tpg ? (double)a.tpg[g0 + lane] : a.theta;
             int64_t off_c = 0, off_p = 0;
             int32_t want_c = 0, want_p = 0;
             if (kMode == 2) {
-                off_p = (int64_t)g * (capacity + pcap) + capacity;
+                // cell r at off_c - r, particle k at off_p + k
+                off_p = (int64_t)(g0 + lane) * (capacity + pcap) + capacity;
                 off_c = off_p - 1;
                 want_c = (int32_t)capacity;
                 want_p = (int32_t)pcap;
             }
             if (kFill) {
-                const otoo_group gr = groups[g];
+                const otoo_group gr = groups[g0 + lane];
                 off_c = gr.list_off;
                 want_c = gr.n_cell;
                 want_p = gr.n_part;
                 off_p = off_c + want_c;
                 if (off_c < 0 || want_c < 0 || want_p < 0 || off_p + want_p > capacity) {
-                    if (lane == 0) atomicOr(status, kWalkNoRoom);
-                    continue;
+                    atomicOr(status, kWalkNoRoom);
+                    mine = false;
                 }
             }
-            if (lane == 0) {
-                SetGroup& q = sg[j];
-                q.bf = w.bf;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) q.blo[k] = w.blo[k], q.bhi[k] = w.bhi[k], q.c[k] = w.c[k];
-                q.theta = w.theta;
-                q.invth = w.invth;
-                q.flags = (w.open_all ? 1 : 0) | (w.small_angle ? 2 : 0);
-                q.first = first;
-                q.count = count;
-                q.off_c = off_c;
-                q.off_p = off_p;
-                q.want_c = want_c;
-                q.want_p = want_p;
-            }
-            valid |= 1u << j;
-            if (w.theta >= 0.0) live |= 1u << j;
+            my_fl = (!sw && !(theta > 0.0) ? 1 : 0) | (theta < kCubeAngle ? 2 : 0);
+            // 1/theta within 2^-23 (the filter's margins allow 2^-21)
+            my_inv = sw || (my_fl & 1) ? 0.f : __frcp_rn(__double2float_rn(theta));
+            q.theta = theta;
+            q.invth = my_inv;
+            q.flags = my_fl;
+            q.off_c = off_c;
+            q.off_p = off_p;
+            q.want_c = want_c;
+            q.want_p = want_p;
+            walks = mine && theta >= 0.0;
         }
+        const unsigned live = __ballot_sync(kFull, walks);  // groups that walk
         __syncwarp();
-        // one opening angle for all walking groups: the threshold side /
-        // theta + s is computed once per cell
-        float invth_u = 0.f;
-        bool uni = false;
+        // the set's centre: that of the box of its walking groups
+        SetRule rule = {};
+        bool uni = true, none = false, overlap = false;  // one angle; nothing accepted; the test needs the cubes
         if (live) {
-            invth_u = sg[__ffs(live) - 1].invth;
-            uni = true;
-            for (unsigned m = live; m; m &= m - 1u) uni = uni && sg[__ffs(m) - 1].invth == invth_u;
+            double lo[3], hi[3];
+            const int j0 = __ffs(live) - 1;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                lo[k] = dval(warp_min(dkey(sg[walks ? lane : j0].blo[k])));
+                hi[k] = dval(warp_max(dkey(sg[walks ? lane : j0].bhi[k])));
+            }
+            float B = 0.f, A = 0.f, ch[3], cl[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const double c = __dmul_rn(__dadd_rn(lo[k], hi[k]), 0.5);
+                ch[k] = __double2float_rn(c);
+                cl[k] = __double2float_rn(__dsub_rn(c, (double)ch[k]));
+                A += fabsf(ch[k]);
+                if (walks) {
+                    SetGroup& q = sg[lane];
+                    q.bl[k] = __double2float_rn(__dsub_rn(q.blo[k], c));
+                    q.bh[k] = __double2float_rn(__dsub_rn(q.bhi[k], c));
+                    B += fmaxf(fabsf(q.bl[k]), fabsf(q.bh[k]));
+                }
+            }
+            // (B >= 0: its bits are ordered as the value)
+            B = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(B)));
+            const float inv0 = __shfl_sync(kFull, my_inv, j0);
+            const int fl0 = __shfl_sync(kFull, my_fl, j0);
+            uni = __all_sync(kFull, !walks || (my_inv == inv0 && my_fl == fl0));
+            none = (fl0 & 1) != 0;
+            overlap = !sw && __any_sync(kFull, walks && !(my_fl & 2));
+            rule.c = make_float4(ch[0], ch[1], ch[2], inv0);
+            rule.cl = make_float4(cl[0], cl[1], cl[2], B + A * 0x1p-24f);
+            __syncwarp();
         }
         int my_nc = 0, my_np = 0;  // lane j: counts of group j
         int sp = 0;
@@ -930,92 +820,170 @@ __global__ void __launch_bounds__(kWalkWarps * 32, OTOO_WALK_MIN_BLOCKS)
             sp = 1;
         }
         __syncwarp();
-        int64_t budget = a.n_cell;  // the union of the walks visits each cell at most once
+        int budget = (int)a.n_cell;  // the union of the walks visits each cell at most once
         bool failed = false;
+        int head = 0, held = 0;  // the ring's leaves
         while (sp > 0) {
-            SetStep st;
-            if (!set_take(a, sg, sw, invth_u, uni, stk, msk, sp, budget, lane, st, status)) {
+            // at, num: an inner cell's first child and -(number of children), a leaf's
+            // first particle and one past its last
+            int node[kWalkHalves], at[kWalkHalves], num[kWalkHalves];
+            unsigned cm[kWalkHalves], acc[kWalkHalves];
+            SetCell sc[kWalkHalves];
+            if (!set_take(stk, msk, sp, budget, lane, node, cm)) {
                 failed = true;
                 break;
             }
-            // accepted cells, per group, in position order
-            unsigned acc_any = 0u, leaf_any = 0u;
 #pragma unroll
             for (int h = 0; h < kWalkHalves; ++h) {
-                acc_any |= st.acc[h];
-                leaf_any |= st.nch[h] == 0 ? st.rej[h] : 0u;
+                const int nd = node[h];
+                otoo_wcell c = {};
+                bool ok = nd >= 0 && nd < a.n_cell;
+                if (cm[h] && ok) c = load_wcell(a.cell, nd);
+                ok = ok && c.nchild >= 0 && c.nchild <= 8 &&
+                     (c.nchild == 0 || (c.child0 > nd && (int64_t)c.child0 + c.nchild <= a.n_cell)) && c.begin >= 0 &&
+                     c.begin <= c.end && (int64_t)c.end <= a.n_part;
+                at[h] = c.nchild ? c.child0 : c.begin;
+                num[h] = c.nchild ? -c.nchild : c.end;
+                if (cm[h] && !ok) {
+                    atomicOr(status, kWalkBadRecord);
+                    cm[h] = 0u;
+                }
+                acc[h] = 0u;
+                sc[h] = set_cell(c, rule, sw, none, a.exact != 0);
             }
-            acc_any = drop ? 0u : __reduce_or_sync(kFull, acc_any);
-            leaf_any = __reduce_or_sync(kFull, leaf_any);
-            // (loops over the groups present, not unrolled: the walk loop must
-            // stay small for the instruction cache)
+            // group by group: the decisions, and its accepted cells in position order
+            // (not unrolled: the walk loop must stay small for the instruction cache)
+            unsigned any = 0u;
+#pragma unroll
+            for (int h = 0; h < kWalkHalves; ++h) any |= cm[h];
 #pragma unroll 1
-            for (unsigned gm = acc_any; gm; gm &= gm - 1u) {
+            for (unsigned gm = __reduce_or_sync(kFull, any); gm; gm &= gm - 1u) {
                 const int j = __ffs(gm) - 1;
-                const int64_t oc = sg[j].off_c;
-                const int32_t wc = sg[j].want_c;
-                int n = __shfl_sync(kFull, my_nc, j);
+                const SetGroup& q = sg[j];
+                float bl[3], bh[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) bl[k] = q.bl[k], bh[k] = q.bh[k];
+                if (kGen && !uni) {
+#pragma unroll
+                    for (int h = 0; h < kWalkHalves; ++h) {
+                        set_limits(sc[h], __fadd_rn(__fmul_rn(sc[h].side, q.invth), sc[h].s));
+                        if (a.exact) sc[h].tu = __int_as_float(0x7f800000), sc[h].tl = -sc[h].tu;
+                        if (q.flags & 1) sc[h].tu = sc[h].tl = __int_as_float(0x7f800000);
+                    }
+                }
+                bool in[kWalkHalves], tc[kWalkHalves];
 #pragma unroll
                 for (int h = 0; h < kWalkHalves; ++h) {
-                    const bool mine = (st.acc[h] >> j) & 1u;
-                    const unsigned am = __ballot_sync(kFull, mine);
-                    if (kWrite && mine) {
+                    const SetCell& c = sc[h];
+                    float d2 = 0.f;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        const float d = fmaxf(0.f, fmaxf(bl[k] - c.u[k], c.u[k] - bh[k]));
+                        d2 = fmaf(d, d, d2);
+                    }
+                    in[h] = d2 > c.tu;
+                    tc[h] = !in[h] && !(d2 < c.tl);
+                }
+                // Opening angles of 1/sqrt(3) and more: a cell whose cube
+                // overlaps the box is rejected.  (Below, a cube that overlaps
+                // the box puts its centre of mass within sqrt(3) l of the box,
+                // below l / theta + s, so the distance alone rejects it.)
+                if (kGen && overlap) {
+#pragma unroll
+                    for (int h = 0; h < kWalkHalves; ++h) {
+                        const SetCell& c = sc[h];
+                        bool sep = false, ovl = true;
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            const float lo = __fsub_rn(c.u[k], c.e[k]);
+                            const float hi = __fadd_rn(lo, c.side);
+                            sep = sep || (lo > bh[k] + c.del) || (bl[k] > hi + c.del);
+                            ovl = ovl && (lo < bh[k] - c.del) && (bl[k] < hi - c.del);
+                        }
+                        tc[h] = a.exact ? tc[h] : !ovl && (!sep || tc[h]);
+                        in[h] = in[h] && sep;
+                    }
+                }
+#pragma unroll
+                for (int h = 0; h < kWalkHalves; ++h) {
+                    const bool m = (cm[h] >> j) & 1u;
+                    if (m && tc[h])  // too close to call
+                        in[h] = sw ? sw_exact(a.cell64, node[h], q.blo, q.bhi)
+                                        : mac_exact(a.cell64, node[h], q.blo, q.bhi, q.theta);
+                    in[h] = in[h] && m;
+                    acc[h] |= in[h] ? 1u << j : 0u;
+                }
+                if (drop) continue;
+                int n = __shfl_sync(kFull, my_nc, j);
+                int32_t* o = nullptr;
+                if (kWrite) o = list + q.off_c;
+#pragma unroll
+                for (int h = 0; h < kWalkHalves; ++h) {
+                    const unsigned am = __ballot_sync(kFull, in[h]);
+                    if (kWrite) {
                         const int32_t r = n + __popc(am & lt);
-                        if (r < wc) list[kMode == 2 ? oc - r : oc + r] = (int32_t)(a.n_part + st.node[h]);
+                        if (in[h] && r < q.want_c) o[kMode == 2 ? -r : r] = (int32_t)(a.n_part + node[h]);
                     }
                     n += __popc(am);
                 }
                 if (lane == j) my_nc = n;
             }
-            // particles of rejected leaves, per group, in position order
-#pragma unroll 1
-            for (unsigned gm = leaf_any; gm; gm &= gm - 1u) {
-                const int j = __ffs(gm) - 1;
-                const int64_t op = sg[j].off_p;
-                const int32_t wp = sg[j].want_p;
-                int n = __shfl_sync(kFull, my_np, j);
+            // rejected leaves, in position order; one run per inner cell some
+            // group rejected, with the mask of the groups that rejected it, the
+            // lowest position's run on top (the last positions are pushed first)
 #pragma unroll
-                for (int h = 0; h < kWalkHalves; ++h) {
-                    const bool mine = st.nch[h] == 0 && ((st.rej[h] >> j) & 1u);
-                    if (!__any_sync(kFull, mine)) continue;
-                    const int np = mine ? st.pe[h] - st.pb[h] : 0;
-                    const int pin = warp_incl_scan(np, lane);
-                    if (kWrite && np > 0) {
-                        const int32_t base = n + pin - np;
-                        for (int k = 0; k < np; ++k)
-                            if (base + k < wp) list[op + base + k] = st.pb[h] + k;
-                    }
-                    n += __shfl_sync(kFull, pin, 31);
+            for (int h = 0; h < kWalkHalves; ++h) {
+                cm[h] &= ~acc[h];
+                const bool leaf = num[h] >= 0 && cm[h] != 0u;
+                const unsigned lm = __ballot_sync(kFull, leaf);
+                if (leaf) {
+                    const int i = (head + held + __popc(lm & lt)) & (kLeafRing - 1);
+                    ring.range[i] = make_int2(at[h], num[h]);
+                    ring.mask[i] = (uint8_t)cm[h];
                 }
-                if (lane == j) my_np = n;
+                held += __popc(lm);
             }
-            set_push(stk, msk, sp, st, lt);
+#pragma unroll
+            for (int h = kWalkHalves - 1; h >= 0; --h) {
+                const bool op = num[h] < 0 && cm[h] != 0u;
+                const unsigned om = __ballot_sync(kFull, op);
+                const int no = __popc(om);
+                if (op) {
+                    const int i = sp + no - 1 - __popc(om & lt);
+                    stk[i] = run(at[h], -num[h]);
+                    msk[i] = (uint8_t)cm[h];
+                }
+                sp += no;
+            }
+            for (; held >= 32; held -= 32, head += 32) set_flush<kWrite>(ring, head, 32, lane, sg, list, my_np);
+            __syncwarp();
         }
+        set_flush<kWrite>(ring, head, held, lane, sg, list, my_np);
         if (failed && lane == 0) atomicOr(status, kWalkOverflow);
         // the groups' records (lane j writes group j's)
-        const int nc = my_nc, npt = my_np;
-        const bool mine = lane < ng && ((valid >> lane) & 1u);
         if (mine) {
             const SetGroup& q = sg[lane];
+            const int nc = my_nc, npt = my_np;
             if (kCount) {
                 otoo_group r;
-                r.first = q.first;
-                r.count = q.count;
+                r.first = a.gfirst[g0 + lane];
+                r.count = a.gcount[g0 + lane];
                 r.n_cell = nc;
                 r.n_part = npt;
+                // pass 0: the offsets come from the scan that follows
                 r.list_off = kMode == 2 ? (nc <= q.want_c && npt <= q.want_p ? q.off_p - nc : -1) : 0;
                 r.eps2 = a.eps2;
-                r.cx = q.c[0];
-                r.cy = q.c[1];
-                r.cz = q.c[2];
+                r.cx = __dmul_rn(__dadd_rn(q.blo[0], q.bhi[0]), 0.5);
+                r.cy = __dmul_rn(__dadd_rn(q.blo[1], q.bhi[1]), 0.5);
+                r.cz = __dmul_rn(__dadd_rn(q.blo[2], q.bhi[2]), 0.5);
                 r.theta = (float)q.theta;
                 r.sys = 0;
                 groups[g0 + lane] = r;
                 const int64_t len = (int64_t)nc + npt;
                 atomicAdd(reinterpret_cast<unsigned long long*>(a.totals), (unsigned long long)len);
-                atomicAdd(reinterpret_cast<unsigned long long*>(a.totals + 1), (unsigned long long)(len * q.count));
+                atomicAdd(reinterpret_cast<unsigned long long*>(a.totals + 1), (unsigned long long)(len * r.count));
                 atomicAdd(reinterpret_cast<unsigned long long*>(a.totals + 2),
-                          (unsigned long long)((int64_t)nc * q.count));
+                          (unsigned long long)((int64_t)nc * r.count));
                 atomicMax(reinterpret_cast<unsigned long long*>(a.totals + 3), (unsigned long long)nc);
                 atomicMax(reinterpret_cast<unsigned long long*>(a.totals + 4), (unsigned long long)npt);
                 if (kMode == 2 && (nc > q.want_c || npt > q.want_p))
@@ -1029,7 +997,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32, OTOO_WALK_MIN_BLOCKS)
 }
 
 // ---- the walk fused with the force (the paper's GPU design) ------------------
-// One warp per group walks the tree as k_walk does, but the entries do not go
+// One warp per group walks the tree as k_walk_set does one group, but the entries do not go
 // to a list in device memory: accepted cells and the particles of rejected
 // leaves collect in two shared-memory index buffers, and whenever one holds a
 // tile of entries the warp stages the tile as pair records (the layout of
@@ -1704,39 +1672,54 @@ WalkArgs walk_args(const otoo_dev_walk* w)
     return a;
 }
 
-template <int kMode>
-int launch_walk(const otoo_dev_walk* w, otoo_group* groups, int32_t* list, int64_t capacity, cudaStream_t s,
-                int64_t pcap = 0)
+// One threshold rule for every group and no cube test: the absolute MAC, the SPH
+// radius, or one opening angle below the limit of group flag 2.
+bool plain_rule(const otoo_dev_walk* w)
+{
+    return w->mac == OTOO_MAC_SW || w->mac == OTOO_MAC_SPH || (!w->theta_per_group && w->theta < kCubeAngle);
+}
+
+template <int kMode, bool kGen>
+int launch_walk_form(const otoo_dev_walk* w, otoo_group* groups, int32_t* list, int64_t capacity, cudaStream_t s,
+                     int64_t pcap)
 {
     int dev = 0, sms = 0, occ = 0;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // groups per warp: as asked, or (0) up to kSet while every resident warp
-    // still gets about three sets to balance the load
+    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_walk_set<kMode, kGen>, kWalkWarps * 32, 0));
+    if (occ < 1) occ = 1;
+    // groups per warp: as asked, or (0) about as many as give every resident
+    // warp one set (a quarter more goes to a second round rather than to larger
+    // sets), kSet at most: a larger set shares more of its cells, fewer sets
+    // than warps leave warps idle.  Microseconds with 1 / 2 / 3 / 4 / 6 / 8 groups on
+    // 3648 warps: 5353 groups (King 100003, theta 0.75) 126 / 115 / 126 / 142 /
+    // 169 / 205; 11162 groups (Plummer 200000) 407 / 321 / 260 / 298 / 339 / 399;
+    // 21230 groups (Hernquist 400000) 765 / 534 / 476 / 482 / 432 / 517; 27005 groups
+    // (Plummer 2^20) 1113 / 793 / 724 / 664 / 726 / 686.
     int gs = w->set;
     if (gs == 0) {
-        CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_walk_set<kMode>, kWalkWarps * 32, 0));
-        const int64_t warps = (int64_t)sms * (occ < 1 ? 1 : occ) * kWalkWarps;
-        const int64_t fit = (int64_t)w->n_groups / (3 * warps);
+        const int64_t warps = (int64_t)sms * occ * kWalkWarps;
+        const int64_t fit = ((int64_t)w->n_groups - warps / 4 + warps - 1) / warps;
         gs = fit < 1 ? 1 : fit > kSet ? kSet : (int)fit;
     }
-    const bool sets = gs > 1;
-    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &occ, sets ? (const void*)k_walk_set<kMode> : (const void*)k_walk<kMode>, kWalkWarps * 32, 0));
-    if (occ < 1) occ = 1;
-    int64_t blocks = (int64_t)sms * occ;
+    // one set per warp, spread over all SMs, while there are fewer sets than warps
     const int64_t units = ((int64_t)w->n_groups + gs - 1) / gs;
-    const int64_t need = (units + kWalkWarps - 1) / kWalkWarps;
-    if (blocks > need) blocks = need;
-    if (blocks < 1) blocks = 1;
+    const int64_t blocks = units < (int64_t)sms * occ ? units : (int64_t)sms * occ;
+    const int64_t need = (units + blocks - 1) / blocks;
+    const int nw = need < kWalkWarps ? (int)need : kWalkWarps;
     CUDA_TRY(cudaMemsetAsync(w->counter, 0, sizeof(uint32_t), s));
-    if (sets)
-        k_walk_set<kMode><<<(unsigned)blocks, kWalkWarps * 32, 0, s>>>(walk_args(w), (int32_t)units, gs, groups,
-                                                                      list, capacity, pcap);
-    else
-        k_walk<kMode><<<(unsigned)blocks, kWalkWarps * 32, 0, s>>>(walk_args(w), groups, list, capacity, pcap);
+    k_walk_set<kMode, kGen><<<(unsigned)blocks, nw * 32, 0, s>>>(walk_args(w), (int32_t)units, gs, groups, list, capacity,
+                                                                 pcap);
     CUDA_TRY(cudaGetLastError());
     return OTOO_OK;
+}
+
+template <int kMode>
+int launch_walk(const otoo_dev_walk* w, otoo_group* groups, int32_t* list, int64_t capacity, cudaStream_t s,
+                int64_t pcap = 0)
+{
+    return plain_rule(w) ? launch_walk_form<kMode, false>(w, groups, list, capacity, s, pcap)
+                         : launch_walk_form<kMode, true>(w, groups, list, capacity, s, pcap);
 }
 
 }  // namespace
