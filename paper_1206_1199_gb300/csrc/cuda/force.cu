@@ -346,23 +346,22 @@ using Kernel = void (*)(const otoo_dev_system, double*, double*);
 // at every size measured (merger, N = 10^6, n_crit 64: 2.94 ms against 2.72 ms,
 // tiles of 128 entries), so both values run the packed arithmetic.
 struct ForceKernel {
-    Kernel one, team;  // a work item per warp; a work item per CTA of kTeamWarps warps
+    Kernel one, team;  // a work item per warp; that or a work item per CTA of kTeamWarps warps
     int team_smem;
+    bool opt_in;  // the team's shared memory passes 48 KB
 };
 constexpr int kTeamWarps = 4;
-// Items per SM up to which a CTA of four warps takes one item: below, the
-// longest items (64 targets against the whole list) set the launch's time;
-// above, the team's barriers cost more than its shorter tail gives.  One item
-// per warp / per CTA (128, 2, 128 tuning, theta 0.6, quadrupole cells): N = 4096
-// (307 items) 92 / 48 us, 30000 (2039) 265 / 115, 100003 (6615) 408 / 283,
-// 200000 (8759) 831 / 731, 400000 (18094) 1426 / 1523, 2^20 (46109) 3951 / 4303.
+// Items per SM up to which the kernel with both forms is launched, which decides
+// on the device (team_pays): above, a work item per warp is always the better
+// one (18094 items 1426 us against 1523 with a CTA per item, 46109 3951 / 4303).
 constexpr int64_t kTeamItems = 80;
 
 template <int NW, int IB, int SPL>
 constexpr ForceKernel force_kernel()
 {
-    return {k_force_warp2<NW, IB, SPL>, k_force_warp2<kTeamWarps, IB, SPL, true>,
-            (int)sizeof(TeamPart<IB>) * kTeamWarps};
+    constexpr int smem = (int)sizeof(TeamPart<IB>) * kTeamWarps;
+    return {k_force_warp2<NW, IB, SPL>, k_force_warp2<kTeamWarps, IB, SPL, true>, smem,
+            smem + kTeamWarps * kCellRecF4 * 16 * SPL * (int)sizeof(float4) + 64 > 48 * 1024};
 }
 
 ForceKernel pick_f32(int B, int IB, int tile, int packed)
@@ -376,7 +375,7 @@ ForceKernel pick_f32(int B, int IB, int tile, int packed)
         PICK(4, 2, 2) PICK(4, 4, 4) PICK(4, 4, 8) PICK(2, 4, 4) PICK(8, 2, 4) PICK(8, 1, 4)
     }
 #undef PICK
-    return {nullptr, nullptr, 0};
+    return {nullptr, nullptr, 0, false};
 }
 
 // FP64 form: B threads per CTA for a plan made with iblock targets per lane
@@ -435,7 +434,7 @@ int enqueue_force(const otoo_dev_system* sys, double* accel, double* pot, int pr
                   cudaStream_t s)
 {
     const bool fp64 = precision == OTOO_FP64;
-    const ForceKernel fk = fp64 ? ForceKernel{pick_f64(t->iblock), nullptr, 0}
+    const ForceKernel fk = fp64 ? ForceKernel{pick_f64(t->iblock), nullptr, 0, false}
                                 : pick_f32(t->block, t->iblock, t->tile, t->packed);
     int dev = 0, nsm = 0, occ = 0;
     CUDA_TRY(cudaGetDevice(&dev));
@@ -444,7 +443,7 @@ int enqueue_force(const otoo_dev_system* sys, double* accel, double* pot, int pr
     Kernel fn = team ? fk.team : fk.one;
     const int block = fp64 ? 128 : team ? 32 * kTeamWarps : t->block;
     const int smem = team ? fk.team_smem : 0;
-    if (team) CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    if (team && fk.opt_in) CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, smem));
     if (occ < 1) return set_error(OTOO_EINVAL, "force kernel does not fit on an SM");
     const int per_sm = t->ctas_per_sm > 0 ? std::min(t->ctas_per_sm, occ) : occ;

@@ -39,3 +39,24 @@ def test_small_and_large_launches_give_the_same_bits(block, iblock, tile, packed
     for k in (0, copies // 2, copies - 1):
         np.testing.assert_array_equal(am[off[k]:off[k + 1]], a)
         np.testing.assert_array_equal(pm[off[k]:off[k + 1]], p)
+
+
+@pytest.mark.parametrize("block,iblock,tile,packed", [(128, 2, 128, 0), (128, 2, 256, 1), (128, 4, 128, 0), (64, 1, 128, 1)])
+def test_short_items_below_the_line(block, iblock, tile, packed):
+    # few enough items for the kernel with both forms, too short for a CTA each
+    L.load()
+    import torch
+    line = 80 * torch.cuda.get_device_properties(0).multi_processor_count
+    pos, mass = ic.plummer(70000, 82)
+    lists = S.Tree(pos, mass, 8).lists(1.0, 32, 1e-2, True)
+    plan = lists.plan(L.Tune(block=block, iblock=iblock, tile=tile, split=8192, ctas_per_sm=0, packed=packed))
+    a, p = (t.cpu().numpy() for t in S.force(S.DeviceSystem.upload(lists, plan, "cuda")))
+    copies = line // plan.n_items + 2
+    many = S.Lists.pack([lists] * copies)
+    mplan = many.plan(plan.tune)
+    assert plan.n_items <= line < mplan.n_items
+    am, pm = (t.cpu().numpy() for t in S.force(S.DeviceSystem.upload(many, mplan, "cuda")))
+    off = many.sys_part_off
+    for k in (0, copies - 1):
+        np.testing.assert_array_equal(am[off[k]:off[k + 1]], a)
+        np.testing.assert_array_equal(pm[off[k]:off[k + 1]], p)
