@@ -70,16 +70,66 @@ __global__ void __launch_bounds__(256) k_direct_range(const otoo_src* __restrict
 // half's sums join the first's at the end.  The float sums are moved into FP64
 // every kTfFold tiles.  Bound by the FP32 pipe: about 195 packed operations per
 // source and two targets.
-// N = 2^19, 5003 targets: 24.2 ms (1.09e11 pairs/s) against 110 ms for the FP64
-// form.  Relative error (2-norm over 40 targets, against extended precision) of
-// the accelerations and potentials, two-float / FP64 form: N = 20000 1.2e-15 /
-// 7.0e-16 and 1.6e-16 / 3.0e-16, 60000 1.0e-15 / 1.0e-15 and 2.3e-16 / 4.7e-16,
-// 200000 3.2e-16 / 1.9e-15 and 1.2e-16 / 1.2e-15, 10^6 3.9e-16 / 4.5e-15 and
-// 1.3e-16 / 1.4e-15 (the FP64 form's sums of a chunk's pairs lose more the
-// longer they are).  The line is where the two-float form is no less exact.
+// N = 2^19, 5003 targets: 25.1 ms (1.05e11 pairs/s) against 110 ms for the FP64
+// form.  Relative error (2-norm over 40 targets, against extended precision) over
+// N = 66000, 90000, 130000 and 400000, four models and softenings 1e-4 and 1e-2,
+// two-float / FP64 form: accelerations 3.3e-16 to 1.2e-15 / 8.0e-16 to 5.8e-15,
+// potentials 0.9e-16 to 2.5e-16 / 3.9e-16 to 1.7e-15, for each input the
+// two-float form's no larger (one of 32 equal, 8.3e-16 / 8.0e-16): the FP64 form's
+// sums of a chunk's pairs lose more the longer they are.  N = 20000 1.2e-15 / 7.0e-16:
+// the line is where the two-float form is no less exact.
 constexpr int64_t kTfMinSources = 65536;
 constexpr int kTfTile = 256;
 constexpr int kTfFold = 8;  // the longest run (1024 sources) the float sums take before FP64
+
+constexpr unsigned kTfPos = kTfFold * kTfTile - 1;  // position in a run
+static_assert(((kTfPos + 1) & kTfPos) == 0, "a run's length is a power of two");
+
+// What the heaviest pair of each target of a run (run0 + the low bits of top)
+// lacks: its FP64 value less the two-float one.  A close pair at a small
+// softening can be most of a target's acceleration, and its 2^-47, or the grid's
+// spacing against its distance, would then be the sum's error (Hernquist, eps
+// 1e-4, N = 130000: 6.4e-15 without this, 3.8e-16 with it, all FP64 1.6e-15).
+__device__ __forceinline__ void tf_refine(const otoo_src* __restrict__ src, int64_t run0, int64_t j1,
+                                          const unsigned top[2], const int64_t ti[2], const long long x[2],
+                                          const long long y[2], const long long z[2], const TfScale& sc, float ms,
+                                          double eps2, const F2x2& e2, double fix[4][2])
+{
+    long long d[3][2];
+    float m[2];
+    const double es = eps2 * tf_pow2(-2 * sc.ex), sx = tf_pow2(-sc.ex);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        int64_t j = run0 + (top[k] & kTfPos);
+        j = j < j1 ? j : j1 - 1;
+        const otoo_src q = src[j];
+        d[0][k] = tf_fixed(q.x, sc.ex) - x[k];
+        d[1][k] = tf_fixed(q.y, sc.ex) - y[k];
+        d[2][k] = tf_fixed(q.z, sc.ex) - z[k];
+        m[k] = j == ti[k] || top[k] == 0u ? 0.f : q.m * ms;  // (0: no pair)
+        // (from the coordinates themselves: near the origin they are finer than the grid)
+        const otoo_src t = src[ti[k] < 0 ? j : ti[k]];
+        const double rx = (q.x - t.x) * sx, ry = (q.y - t.y) * sx, rz = (q.z - t.z) * sx;
+        const double inv = rsqrt(fma(rx, rx, fma(ry, ry, fma(rz, rz, es))));
+        const double mi = (double)m[k] * inv, mi3 = mi * inv * inv;
+        fix[0][k] = mi3 * rx;
+        fix[1][k] = mi3 * ry;
+        fix[2][k] = mi3 * rz;
+        fix[3][k] = mi;
+    }
+    F2x3 A[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) A[c].zero();
+    tf_pair_mono(tf_diff(d[0][0], d[0][1]), tf_diff(d[1][0], d[1][1]), tf_diff(d[2][0], d[2][1]), f2pack(m[0], m[1]), e2,
+                 A);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        double v0, v1;
+        A[c].value(v0, v1);
+        fix[c][0] -= v0;
+        fix[c][1] -= v1;
+    }
+}
 
 __global__ void __launch_bounds__(256, 2) k_direct_tf(const otoo_src* __restrict__ src, int64_t n_src,
                                                       const int64_t* __restrict__ tgt, int64_t n_tgt, double eps2,
@@ -129,6 +179,8 @@ __global__ void __launch_bounds__(256, 2) k_direct_tf(const otoo_src* __restrict
         sum[c][0] = sum[c][1] = 0.0;
     }
     int fold = 0;
+    int64_t run0 = j0;            // first source of the run being summed
+    unsigned top[2] = {0u, 0u};   // the run's heaviest pair: m q^2's bits above its position in the run
     for (int64_t b = j0; b < j1; b += kTfTile) {
         const int64_t j = b + threadIdx.x;
         if (j < j1) {
@@ -148,18 +200,27 @@ __global__ void __launch_bounds__(256, 2) k_direct_tf(const otoo_src* __restrict
             const F2x2 dx = tf_diff(xy.x - x[0], xy.x - x[1]);
             const F2x2 dy = tf_diff(xy.y - y[0], xy.y - y[1]);
             const F2x2 dz = tf_diff(zm.x - z[0], zm.x - z[1]);
-            tf_pair_mono(dx, dy, dz, f2pack(k == self0 ? 0.f : m, k == self1 ? 0.f : m), e2, A);
+            float w0, w1;
+            f2unpack(tf_pair_mono(dx, dy, dz, f2pack(k == self0 ? 0.f : m, k == self1 ? 0.f : m), e2, A), w0, w1);
+            const unsigned at = (unsigned)(fold * kTfTile + k);
+            top[0] = max(top[0], (__float_as_uint(w0) & ~kTfPos) | at);
+            top[1] = max(top[1], (__float_as_uint(w1) & ~kTfPos) | at);
         }
         if (++fold == kTfFold || b + kTfTile >= j1) {
             fold = 0;
+            // the heaviest pair of the run again in FP64, less what was added for it
+            double fix[4][2];
+            tf_refine(src, run0, j1, top, ti, x, y, z, sc, ms, eps2, e2, fix);
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 double v0, v1;
                 A[c].value(v0, v1);
-                sum[c][0] += v0;
-                sum[c][1] += v1;
+                sum[c][0] += v0 + fix[c][0];
+                sum[c][1] += v1 + fix[c][1];
                 A[c].zero();
             }
+            top[0] = top[1] = 0u;
+            run0 = b + kTfTile;
         }
         __syncthreads();
     }

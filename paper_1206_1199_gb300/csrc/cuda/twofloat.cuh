@@ -184,9 +184,10 @@ struct F2x3 {
 };
 
 // One source of mass m (per target) at difference (x, y, z) from two targets:
-// A[0..2] += m q^3 r, A[3] += m q.
-__device__ __forceinline__ void tf_pair_mono(const F2x2& x, const F2x2& y, const F2x2& z, f2 m, const F2x2& e2,
-                                             F2x3 A[4])
+// A[0..2] += m q^3 r, A[3] += m q.  Returns m q^2 (single floats), the pair's
+// weight in the acceleration.
+__device__ __forceinline__ f2 tf_pair_mono(const F2x2& x, const F2x2& y, const F2x2& z, f2 m, const F2x2& e2,
+                                           F2x3 A[4])
 {
     const F2x2 q = tf_rsqrt(tf_r2(x, y, z, e2));
     F2x2 t = two_prod(q.h, q.h);
@@ -202,6 +203,7 @@ __device__ __forceinline__ void tf_pair_mono(const F2x2& x, const F2x2& y, const
     A[0].add(tf_mul(g, x));
     A[1].add(tf_mul(g, y));
     A[2].add(tf_mul(g, z));
+    return f2mul(mq.h, q.h);
 }
 
 // ---- one value per operand (the quadrupole part of the FP64 form) ------------
