@@ -31,6 +31,7 @@
 #include <mutex>
 
 #include "../common.h"
+#include "../narrow.h"
 
 using namespace otoo;
 
@@ -120,6 +121,8 @@ __device__ __forceinline__ void write_component(const otoo_dev_system& sys, cons
 // within a factor of two of c (Sterbenz), so near entries keep the accuracy of
 // an FP64 subtraction rounded once to FP32, and far entries stay within about
 // one FP32 ulp of it.
+// (narrow2: with conversions it was bound by the FP64 pipe, 12 operations a
+// source; 12.4 million sources 222 -> 92 us.)
 // counter (or NULL): the work ticket and status word of the force kernel that
 // follows, cleared here instead of by a launch of its own.
 __global__ void k_split(const otoo_src* __restrict__ src, float4* __restrict__ out, int64_t n,
@@ -131,10 +134,14 @@ __global__ void k_split(const otoo_src* __restrict__ src, float4* __restrict__ o
     double x, y, z;
     float m;
     load_src(src, s, x, y, z, m);
-    const float hx = __double2float_rn(x), hy = __double2float_rn(y), hz = __double2float_rn(z);
-    out[2 * s] = make_float4(hx, hy, hz, m);
-    out[2 * s + 1] = make_float4(__double2float_rn(x - (double)hx), __double2float_rn(y - (double)hy),
-                                 __double2float_rn(z - (double)hz), 0.f);
+    float4 h, l;
+    narrow2(x, h.x, l.x);
+    narrow2(y, h.y, l.y);
+    narrow2(z, h.z, l.z);
+    h.w = m;
+    l.w = 0.f;
+    out[2 * s] = h;
+    out[2 * s + 1] = l;
 }
 
 // Centre-relative coordinates of n sources as the FP32 force kernels stage

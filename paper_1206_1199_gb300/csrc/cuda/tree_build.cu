@@ -164,6 +164,9 @@ __global__ void __launch_bounds__(256) k_bbox(const double* __restrict__ pos, co
 
 // ---- keys ---------------------------------------------------------------------
 
+// Bound by the FP64 pipe while floor, clamp and conversion ran there (seven FP64
+// operations per axis); two are left: N = 2^23 294 -> 224 us, 2^20 41 -> 33 us, now
+// by the key's integer operations.
 // One key per particle, and the counts of all eight digits of all keys
 // (ghist[pass][digit], zero before the launch) that the sort's passes start
 // from: shared-memory counts per block (increments of one address by a whole
@@ -428,10 +431,10 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_tile(const uint64_t* __re
 
 // ---- tree order ------------------------------------------------------------------
 
+// (The grid coordinates of a cell's first particle, which the records need, are
+// worked out there; one triple per particle here cost 282 us for 250 at N = 2^23.)
 __global__ void k_permute(const double* __restrict__ pos, const float* __restrict__ mass,
-                          const uint32_t* __restrict__ order, int64_t n, const Geom* __restrict__ g,
-                          otoo_src* __restrict__ src, int64_t* __restrict__ perm, int32_t* __restrict__ gq,
-                          uint32_t* __restrict__ status)
+                          const uint32_t* __restrict__ order, int64_t n, otoo_src* __restrict__ src, int64_t* __restrict__ perm, uint32_t* __restrict__ status)
 {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
@@ -448,9 +451,6 @@ __global__ void k_permute(const double* __restrict__ pos, const float* __restric
     s.pad = 0;
     src[k] = s;
     perm[k] = i;
-    gq[3 * k] = (int32_t)quantize(s.x, g->lo[0], g->scale);
-    gq[3 * k + 1] = (int32_t)quantize(s.y, g->lo[1], g->scale);
-    gq[3 * k + 2] = (int32_t)quantize(s.z, g->lo[2], g->scale);
 }
 
 // ---- cells, one level at a time ---------------------------------------------------
@@ -1131,7 +1131,7 @@ struct RecArgs {
 // every n_crit particles inside a leaf that holds more (one bit per particle
 // in bits).
 __device__ __forceinline__ void cell_records(const RecArgs& ra, int32_t cell, const Geom* __restrict__ g,
-                                             const Cells& c, const Moments& mo, const int32_t* __restrict__ gq,
+                                             const Cells& c, const Moments& mo,
                                              otoo_src* __restrict__ src, otoo_quad* __restrict__ quad,
                                              otoo_wcell* __restrict__ wc, otoo_wcell64* __restrict__ wc64,
                                              int32_t* __restrict__ level_out, uint32_t* __restrict__ bits)
@@ -1146,10 +1146,12 @@ __device__ __forceinline__ void cell_records(const RecArgs& ra, int32_t cell, co
     }
     const int sh = kLevels - L;
     const double side = cube_side(g->h, L);
+    const otoo_src p0 = src[b];
+    const double first[3] = {p0.x, p0.y, p0.z};
     double lo[3], gc[3], com[3];
     for (int a = 0; a < 3; ++a) {
-        const int64_t gcoord = gq[3 * (int64_t)b + a];
-        const int64_t org = sh >= kLevels ? 0 : (gcoord >> sh) << sh;
+        // (sh = 21: the root)
+        const uint32_t org = quantize(first[a], g->lo[a], g->scale) >> sh << sh;
         lo[a] = cube_lo(g->lo[a], org, g->h);
         gc[a] = cube_centre(lo[a], side);
         com[a] = mo.com[3 * (int64_t)cell + a];
@@ -1159,7 +1161,7 @@ __device__ __forceinline__ void cell_records(const RecArgs& ra, int32_t cell, co
     s.x = com[0];
     s.y = com[1];
     s.z = com[2];
-    s.m = (float)m;
+    s.m = narrow(m);
     s.pad = 0;
     src[ra.n_part + cell] = s;
     otoo_quad qd;
@@ -1167,13 +1169,13 @@ __device__ __forceinline__ void cell_records(const RecArgs& ra, int32_t cell, co
     // Q = 3 C - tr(C) I from the central second moment C
     const double* cm = mo.q + 6 * (int64_t)cell;
     const double tr = mo.b2[cell];
-    qd.xx = u ? (float)(3.0 * cm[0] - tr) : 0.f;
-    qd.yy = u ? (float)(3.0 * cm[1] - tr) : 0.f;
-    qd.zz = u ? (float)(3.0 * cm[2] - tr) : 0.f;
-    qd.xy = u ? (float)(3.0 * cm[3]) : 0.f;
-    qd.xz = u ? (float)(3.0 * cm[4]) : 0.f;
-    qd.yz = u ? (float)(3.0 * cm[5]) : 0.f;
-    qd.b2 = u ? (float)tr : 0.f;
+    qd.xx = u ? narrow(3.0 * cm[0] - tr) : 0.f;
+    qd.yy = u ? narrow(3.0 * cm[1] - tr) : 0.f;
+    qd.zz = u ? narrow(3.0 * cm[2] - tr) : 0.f;
+    qd.xy = u ? narrow(3.0 * cm[3]) : 0.f;
+    qd.xz = u ? narrow(3.0 * cm[4]) : 0.f;
+    qd.yz = u ? narrow(3.0 * cm[5]) : 0.f;
+    qd.b2 = u ? narrow(tr) : 0.f;
     qd.pad = 0.f;
     quad[cell] = qd;
     const double dm = __longlong_as_double((long long)mo.dmax2[cell]);
@@ -1186,7 +1188,7 @@ __device__ __forceinline__ void cell_records(const RecArgs& ra, int32_t cell, co
     w.child0 = w.nchild > 0 ? c.child0[cell] : 0;
     w.begin = b;
     w.end = e;
-    w.rb = (float)rb;
+    w.rb = narrow(rb);
     wc[cell] = w;
     otoo_wcell64 w64;
     for (int a = 0; a < 3; ++a) w64.lo[a] = lo[a], w64.com[a] = com[a], w64.gc[a] = gc[a];
@@ -1198,14 +1200,13 @@ __device__ __forceinline__ void cell_records(const RecArgs& ra, int32_t cell, co
 }
 
 __global__ void __launch_bounds__(128) k_records(RecArgs ra, const Head* __restrict__ head, Cells c, Moments mo,
-                                                 const int32_t* __restrict__ gq, otoo_src* __restrict__ src,
-                                                 otoo_quad* __restrict__ quad, otoo_wcell* __restrict__ wc,
+                                                 otoo_src* __restrict__ src, otoo_quad* __restrict__ quad, otoo_wcell* __restrict__ wc,
                                                  otoo_wcell64* __restrict__ wc64, int32_t* __restrict__ level_out,
                                                  uint32_t* __restrict__ bits)
 {
     const int32_t n_cell = head->lev[kLv];
     for (int32_t cell = blockIdx.x * blockDim.x + threadIdx.x; cell < n_cell; cell += gridDim.x * blockDim.x)
-        cell_records(ra, cell, &head->g, c, mo, gq, src, quad, wc, wc64, level_out, bits);
+        cell_records(ra, cell, &head->g, c, mo, src, quad, wc, wc64, level_out, bits);
 }
 
 // Groups in tree order from their first particles' bits: words of 32 particles,
@@ -1402,7 +1403,7 @@ int scan32(int32_t* a, int64_t n, int64_t* bsum, int64_t* total, cudaStream_t s)
 
 // Scratch layout (byte offsets, each part 256-byte aligned).
 struct Layout {
-    size_t keys0, keys1, vals0, vals1, head, bits, hist, bsum, part, gq, cells[6], mom_m, mom_com, mom_q, mom_b2,
+    size_t keys0, keys1, vals0, vals1, head, bits, hist, bsum, part, cells[6], mom_m, mom_com, mom_q, mom_b2,
         mom_dmax, dig, total;
 };
 
@@ -1433,7 +1434,6 @@ Layout layout(int64_t n, int64_t cap)
     // block sums of the cells' scan, later the groups' per block
     l.bsum = take(8 * ((256 * nblk + n) / kScanThreads + 8));
     l.part = take(8 * 6 * 1024);
-    l.gq = take(12 * n);
     for (int k = 0; k < 6; ++k) l.cells[k] = take(4 * cap);
     l.mom_m = take(8 * cap);
     l.mom_com = take(24 * cap);
@@ -1489,7 +1489,6 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     Geom* geom = &head->g;
     uint32_t* bits = reinterpret_cast<uint32_t*>(base + ly.bits);
     const int64_t nw = (n + 31) / 32;
-    int32_t* gq = reinterpret_cast<int32_t*>(base + ly.gq);
     Cells c;
     c.begin = reinterpret_cast<int32_t*>(base + ly.cells[0]);
     c.end = reinterpret_cast<int32_t*>(base + ly.cells[1]);
@@ -1534,7 +1533,7 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
                 look[(p & 1) ^ 1], keys[cur ^ 1], vals[cur ^ 1], status);
     }
     CUDA_TRY(cudaGetLastError());
-    k_permute<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(pos, mass, vals[cur], n, geom, t->src, t->perm, gq,
+    k_permute<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(pos, mass, vals[cur], n, t->src, t->perm,
                                                           status);
     CUDA_TRY(cudaGetLastError());
     const uint64_t* skeys = keys[cur];
@@ -1601,7 +1600,7 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     ra.n_crit = t->n_crit;
     ra.delta = t->delta;
     ra.m_limit = t->m_limit;
-    k_records<<<cg, 128, 0, s>>>(ra, head, c, mo, gq, t->src, t->quad, t->cell, t->cell64, t->cell_level, bits);
+    k_records<<<cg, 128, 0, s>>>(ra, head, c, mo, t->src, t->quad, t->cell, t->cell64, t->cell_level, bits);
     // groups
     int32_t* gsum = reinterpret_cast<int32_t*>(bsum);
     const unsigned gg = (unsigned)((nw + kGroupWords - 1) / kGroupWords);

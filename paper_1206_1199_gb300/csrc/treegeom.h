@@ -8,6 +8,7 @@
 
 #include <cmath>
 
+#include "narrow.h"
 #include "otoo.h"
 
 #ifdef __CUDACC__
@@ -82,10 +83,31 @@ OTOO_HD void root_cube(const double mn[3], const double mx[3], double lo[3], dou
 // Grid coordinate of x on an axis (Section III-B, step 2), clamped.
 OTOO_HD uint32_t quantize(double x, double lo, double scale)
 {
+#ifdef __CUDA_ARCH__
+    // floor, clamp and conversion on the bits (two FP64 operations instead of seven)
+    const double v = dmul(dsub(x, lo), scale);
+    const int hi = __double2hiint(v), e = hi >> 20;  // (the sign gives a negative e)
+    const uint32_t top = (uint32_t)((hi & 0xfffff) | 0x100000);
+    if (e >= 1023 + kLevels) return v == v ? (uint32_t)kGrid - 1u : 0u;
+    return e >= 1023 ? top >> (1043 - e) : 0u;
+#else
     double q = floor(dmul(dsub(x, lo), scale));
     if (q < 0.0) q = 0.0;
     if (q > kGrid - 1.0) q = kGrid - 1.0;
     return (uint32_t)q;
+#endif
+}
+
+// Bit b of a 21-bit value to bit 3 b, by halving the runs of bits.
+OTOO_HD uint64_t spread3(uint32_t v)
+{
+    uint64_t x = v & 0x1fffffu;
+    x = (x | x << 32) & 0x001f00000000ffffull;
+    x = (x | x << 16) & 0x001f0000ff0000ffull;
+    x = (x | x << 8) & 0x100f00f00f00f00full;
+    x = (x | x << 4) & 0x10c30c30c30c30c3ull;
+    x = (x | x << 2) & 0x1249249249249249ull;
+    return x;
 }
 
 // Hilbert index of a point on the 2^21 grid: Skilling's transpose method
@@ -116,16 +138,13 @@ OTOO_HD uint64_t hilbert_key(uint32_t x0, uint32_t x1, uint32_t x2)
     for (uint32_t Q = M; Q > 1; Q >>= 1)
         if (X[2] & Q) t ^= Q - 1;
     for (int i = 0; i < 3; ++i) X[i] ^= t;
-    uint64_t key = 0;
-    for (int b = kLevels - 1; b >= 0; --b)
-        for (int i = 0; i < 3; ++i) key = (key << 1) | ((X[i] >> b) & 1u);
-    return key;
+    return (spread3(X[0]) << 2) | (spread3(X[1]) << 1) | spread3(X[2]);
 }
 
 // Cube of a cell at `level` whose integer origin on the grid is org:
 // side = h 2^(21 - level), lower corner = lo + org h, centre = corner + side/2.
-OTOO_HD double cube_side(double h, int level) { return dmul(h, (double)((int64_t)1 << (kLevels - level))); }
-OTOO_HD double cube_lo(double root_lo, int64_t org, double h) { return dadd(root_lo, dmul((double)org, h)); }
+OTOO_HD double cube_side(double h, int level) { return dmul(h, pow2(kLevels - level)); }
+OTOO_HD double cube_lo(double root_lo, uint32_t org, double h) { return dadd(root_lo, dmul(small_int(org), h)); }
 OTOO_HD double cube_centre(double lo, double side) { return dadd(lo, dmul(0.5, side)); }
 
 // Bounding radius of the absolute MAC (Eq. SW_MAC): where the monopole error
@@ -147,14 +166,13 @@ OTOO_HD void wcell_geometry(const double com[3], const double lo[3], const doubl
 {
     double s2 = 0;
     for (int a = 0; a < 3; ++a) {
-        w->com_hi[a] = (float)com[a];
-        w->com_lo[a] = (float)dsub(com[a], (double)w->com_hi[a]);
-        w->e[a] = (float)dsub(com[a], lo[a]);
+        narrow2(com[a], w->com_hi[a], w->com_lo[a]);
+        w->e[a] = narrow(dsub(com[a], lo[a]));
         const double e = dsub(com[a], gc[a]);
         s2 = dadd(s2, dmul(e, e));
     }
-    w->side = (float)side;
-    w->s = (float)dsqrt(s2);
+    w->side = narrow(side);
+    w->s = narrow(dsqrt(s2));
 }
 
 }  // namespace otoo
