@@ -1707,7 +1707,7 @@ int launch_walk_form(const otoo_dev_walk* w, otoo_group* groups, int32_t* list, 
     const int64_t blocks = units < (int64_t)sms * occ ? units : (int64_t)sms * occ;
     const int64_t need = (units + blocks - 1) / blocks;
     const int nw = need < kWalkWarps ? (int)need : kWalkWarps;
-    CUDA_TRY(cudaMemsetAsync(w->counter, 0, sizeof(uint32_t), s));
+    if (kMode == 1) CUDA_TRY(cudaMemsetAsync(w->counter, 0, sizeof(uint32_t), s));  // (the others start with clear_walk)
     k_walk_set<kMode, kGen><<<(unsigned)blocks, nw * 32, 0, s>>>(walk_args(w), (int32_t)units, gs, groups, list, capacity,
                                                                  pcap);
     CUDA_TRY(cudaGetLastError());
@@ -1728,6 +1728,20 @@ extern "C" {
 
 int64_t otoo_walk_totals_len(int64_t n_groups) { return kTotals + scan_blocks(n_groups < 0 ? 0 : n_groups) + 1; }
 
+// Clears the ticket, the status and the totals before a walk: one operation
+// when the caller keeps the totals right behind the four counter words.
+static int clear_walk(const otoo_dev_walk* w, cudaStream_t s)
+{
+    const size_t nc = 4 * sizeof(uint32_t), nt = kTotals * sizeof(int64_t);
+    if (reinterpret_cast<char*>(w->counter) + nc == reinterpret_cast<char*>(w->totals)) {
+        CUDA_TRY(cudaMemsetAsync(w->counter, 0, nc + nt, s));
+    } else {
+        CUDA_TRY(cudaMemsetAsync(w->counter, 0, nc, s));
+        CUDA_TRY(cudaMemsetAsync(w->totals, 0, nt, s));
+    }
+    return OTOO_OK;
+}
+
 int otoo_walk_count(const otoo_dev_walk* w, otoo_group* groups, void* stream)
 {
     otoo::Range range_("otoo_walk_count");
@@ -1735,8 +1749,8 @@ int otoo_walk_count(const otoo_dev_walk* w, otoo_group* groups, void* stream)
     if (rc) return rc;
     OTOO_REQUIRE(groups, OTOO_EINVAL, "otoo_walk_count: groups is NULL");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    CUDA_TRY(cudaMemsetAsync(w->counter, 0, 4 * sizeof(uint32_t), s));
-    CUDA_TRY(cudaMemsetAsync(w->totals, 0, kTotals * sizeof(int64_t), s));
+    const int r1 = clear_walk(w, s);
+    if (r1) return r1;
     const int r2 = launch_walk<0>(w, groups, nullptr, 0, s);
     if (r2) return r2;
     CUDA_TRY(excl_scan(GroupLen{groups}, GroupOff{groups}, w->n_groups, w->totals + kTotals, nullptr, s));
@@ -1754,8 +1768,8 @@ int otoo_walk_single(const otoo_dev_walk* w, otoo_group* groups, int32_t* slots,
                  "otoo_walk_single: slot sizes out of range");
     OTOO_REQUIRE(w->n_groups <= INT64_MAX / (cell_cap + part_cap), OTOO_EINVAL, "otoo_walk_single: slots too large");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    CUDA_TRY(cudaMemsetAsync(w->counter, 0, 4 * sizeof(uint32_t), s));
-    CUDA_TRY(cudaMemsetAsync(w->totals, 0, kTotals * sizeof(int64_t), s));
+    const int r1 = clear_walk(w, s);
+    if (r1) return r1;
     return launch_walk<2>(w, groups, slots, cell_cap, s, part_cap);
 }
 

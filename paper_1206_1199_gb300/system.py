@@ -438,7 +438,7 @@ class DeviceTree:
                      cell64=torch.empty(cap * 96, dtype=u8, device=device),
                      first=torch.empty(n, dtype=i32, device=device), count=torch.empty(n, dtype=i32, device=device),
                      perm=torch.empty(n, dtype=i64, device=device), level=torch.empty(cap, dtype=i32, device=device),
-                     status=torch.zeros(2, dtype=i32, device=device))
+                     status=torch.empty(2, dtype=i32, device=device))
             t = L.DevTree()
             t.n_part, t.cap_cell, t.leaf_size, t.n_crit = n, cap, int(leaf_size), int(n_crit)
             t.use_quad, t.mac = int(bool(use_quad)), MAC_KINDS[mac]
@@ -562,8 +562,11 @@ class DeviceLists:
         self.n_part, self.n_src, self.n_groups = dtree.n_part, dtree.n_src, G
         self.use_quad = dtree.use_quad
         alloc = _alloc(pool, dev)
-        b = dict(groups=alloc("groups", G * 64, torch.uint8), counter=alloc("wcounter", 4, torch.int32),
-                 totals=alloc("totals", L.load().otoo_walk_totals_len(G), torch.int64))
+        # the plan's totals [4], the walk's counter words [2] and its totals: what
+        # the host reads, side by side so that one copy brings it
+        head = alloc("whead", 6 + L.load().otoo_walk_totals_len(G), torch.int64)
+        b = dict(groups=alloc("groups", G * 64, torch.uint8), head=head, counter=head[4:6].view(torch.int32),
+                 totals=head[6:])
         if theta_per_group is not None:
             tpg = np.ascontiguousarray(theta_per_group, dtype=np.float32)
             assert tpg.shape == (G,)
@@ -590,11 +593,11 @@ class DeviceLists:
             ccap, pcap = slots
             spool = alloc("slots", G * (ccap + pcap), torch.int32)
             L.call("otoo_walk_single", ctypes.byref(w), gp, spool.data_ptr(), ccap, pcap, st)
-        tot = [int(x) for x in b["totals"][:6].tolist()] if slots else None
+        tot, status = self.read_head(4, 12, stream) if slots else (None, 0)
         self.one_pass = bool(slots) and tot[5] == 0
         if not self.one_pass:
             L.call("otoo_walk_count", ctypes.byref(w), gp, st)
-            tot = [int(x) for x in b["totals"][:6].tolist()]
+            tot, _ = self.read_head(4, 12, stream)
         self.n_list, self.interactions, self.cell_interactions = tot[:3]
         if max_entries is not None and self.n_list > max_entries:
             raise ValueError("walk: %d list entries exceed max_entries %d" % (self.n_list, max_entries))
@@ -602,15 +605,26 @@ class DeviceLists:
             self.slots = (ccap, pcap)
             b["list"] = spool
             self.list_len = G * (ccap + pcap)
+            if status:
+                L.call("otoo_walk_check_status", ctypes.byref(w), st)
         else:
             b["list"] = alloc("list", self.n_list, torch.int32)
             self.list_len = self.n_list
             L.call("otoo_walk_fill", ctypes.byref(w), gp, b["list"].data_ptr(), self.n_list, st)
-        L.call("otoo_walk_check_status", ctypes.byref(w), st)
+            L.call("otoo_walk_check_status", ctypes.byref(w), st)
         if pool is not None and single:
             ccap, pcap = int(1.25 * tot[3]) + 64, int(1.25 * tot[4]) + 64
             if 4 * G * (ccap + pcap) <= self.SLOT_BYTES_MAX:
                 pool.meta[key] = (ccap, pcap)
+
+    def read_head(self, lo, hi, stream=None):
+        """Words [lo, hi) of the head, but for the counter words, and the
+        walk's status bits, in one copy on the stream that wrote them."""
+        import torch
+        with torch.cuda.stream(stream):  # (None: the current stream)
+            v = self.bufs["head"][lo:hi].tolist()
+        status = (v[4 - lo] >> 32) & 0xffffffff
+        return v[:4 - lo] + v[6 - lo:], status
 
     @property
     def groups(self):
@@ -668,18 +682,39 @@ class DevicePlan:
         st = _stream(stream, dev)
         alloc = _alloc(dl.pool, dev)
         scratch = alloc("pscratch", L.load().otoo_plan_scratch_ints(G), torch.int32)
-        ptot = alloc("ptotals", 4, torch.int64)
+        head = dl.bufs["head"]
+        ptot = head.data_ptr()
         gp = dl.bufs["groups"].data_ptr()
-        L.call("otoo_plan_count", gp, G, ctypes.byref(tune), scratch.data_ptr(), ptot.data_ptr(), st)
-        n_items, n_splits, slots, ncm = (int(x) for x in ptot.tolist())
+        counter = dl.bufs["counter"]
+
+        def count():
+            L.call("otoo_plan_count", gp, G, ctypes.byref(tune), scratch.data_ptr(), ptot, st)
+
+        def fill(items, n_items, splits, n_splits):
+            L.call("otoo_plan_fill", gp, G, ctypes.byref(tune), scratch.data_ptr(), ptot, items.data_ptr(), n_items,
+                   splits.data_ptr(), n_splits, counter.data_ptr(), st)
+
+        count()
+        # with buffers kept from an earlier step the fill needs no host read before
+        # it (it writes nothing past their ends); one that outgrew them is made again
+        kept = [dl.pool.bufs.get(k) for k in ("items", "splits")] if dl.pool is not None else [None]
+        filled = all(t is not None and t.dtype == torch.uint8 for t in kept)
+        if filled:
+            fill(kept[0], kept[0].numel() // 32, kept[1], kept[1].numel() // 16)
+        (n_items, n_splits, slots, ncm), status = dl.read_head(0, 6, stream)
+        if filled and (n_items > kept[0].numel() // 32 or n_splits > kept[1].numel() // 16):
+            with torch.cuda.stream(stream):
+                counter.zero_()
+            count()
+            filled = False
         self.n_items, self.n_splits, self.n_crit_max = n_items, n_splits, max(ncm, 1)
         self.partial_doubles = slots * 4 * self.n_crit_max
         self.items_buf = alloc("items", n_items * 32, torch.uint8)
         self.splits_buf = alloc("splits", n_splits * 16, torch.uint8)
-        L.call("otoo_plan_fill", gp, G, ctypes.byref(tune), scratch.data_ptr(), ptot.data_ptr(),
-               self.items_buf.data_ptr(), n_items, self.splits_buf.data_ptr(), n_splits,
-               dl.bufs["counter"].data_ptr(), st)
-        L.call("otoo_walk_check_status", ctypes.byref(dl.struct), st)
+        if not filled:
+            fill(self.items_buf, n_items, self.splits_buf, n_splits)
+        if not filled or status:
+            L.call("otoo_walk_check_status", ctypes.byref(dl.struct), st)
 
     @property
     def items(self):
