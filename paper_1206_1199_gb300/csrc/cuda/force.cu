@@ -359,9 +359,11 @@ struct ForceKernel {
 };
 constexpr int kTeamWarps = 4;
 // Items per SM up to which the kernel with both forms is launched, which decides
-// on the device (team_pays): above, a work item per warp is always the better
-// one (18094 items 1426 us against 1523 with a CTA per item, 46109 3951 / 4303).
-constexpr int64_t kTeamItems = 80;
+// on the device (team_pays): above (four items per resident warp) that takes a
+// CTA per item only for items of more than 600 record steps, and the kernel of the
+// one form leaves more of an SM's memory to L1 (11321 items of 106 steps 167 us
+// against 171).
+constexpr int64_t kTeamItems = 64;
 
 template <int NW, int IB, int SPL>
 constexpr ForceKernel force_kernel()

@@ -58,25 +58,27 @@ struct TeamPart {
 
 // Whether a CTA per item pays for a launch on `warps` resident warps, from 32
 // items spread over the plan (which is ordered by cost).  An item takes L record
-// steps of a warp (the mean of the 32); the team's barriers and the idle warps of its last
-// round cost what about 200 steps cost, so it pays while the items per warp stay
-// below 6 L / (L + 200).  Fitted to 324 plans (N = 4096 to 400000, n_crit 32 to
-// 128, theta 0.45 to 1, three models, both tile sizes), both forms measured: the
-// rule's choice is 0.2% slower than the better form on average, 11% at worst; a
-// limit on the number of items alone (80 per SM) 3.4% and 65%.  Microseconds with
-// one warp / a CTA per item: N = 4096 (n_crit 64, King, theta 0.75, L 152) 69 / 46;
-// 50000 (n_crit 128, L 740) 426 / 234; 100003 (n_crit 32, theta 1, L 87) 149 /
-// 200; 200000 (n_crit 64, theta 0.75, L 137) 341 / 396.  (Changing to single warps
-// within a launch, once the items left pass the rule, measured worse than either.)
+// steps of a warp (the mean of the 32; a step without quadrupoles is half a
+// one); the team's barriers and the idle warps of its last round cost what about
+// 75 steps cost, so it pays while the items per warp stay below 4.5 L / (L + 75).
+// Fitted to 324 plans (N = 4096 to 400000, n_crit 32 to 128, theta 0.45 to 1, three
+// models, both tile sizes), both forms measured: the rule's choice is 0.1% slower
+// than the better form on average, 9% at worst; a limit on the number of items
+// alone (80 per SM) 3.4% and 65%.  Microseconds with one warp / a CTA per item:
+// N = 4096 (n_crit 64, King, theta 0.75, L 76) 69 / 46; 50000 (n_crit 128, L 740)
+// 426 / 234; 100003 (n_crit 64, theta 0.75, L 132) 210 / 195, (n_crit 32, theta 1, L
+// 54) 149 / 200; 200000 (n_crit 64, theta 0.75, L 137) 341 / 396.  (Changing to
+// single warps within a launch, once the items left pass the rule, measured worse
+// than either.)
 template <int IB>
 __device__ __forceinline__ bool team_pays(const otoo_dev_system& sys, int warps, int lane)
 {
     const otoo_item item = sys.items[(int)(((int64_t)sys.n_items * (2 * lane + 1)) >> 6)];
     const int ni = min(max(item.ni, 1), 32 * IB), len = max(item.j1 - item.j0, 0);
-    float L = (float)len / (float)(64 * (32 / ((ni + IB - 1) / IB)));
+    float L = (sys.quad ? 1.f : 0.5f) * (float)len / (float)(64 * (32 / ((ni + IB - 1) / IB)));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(kFull, L, o);
-    return (float)sys.n_items * (L + 200.f) < 6.f * L * (float)warps;
+    return (float)sys.n_items * (L + 75.f) < 4.5f * L * (float)warps;
 }
 
 // One item on the calling warp, or (kTeam) on the CTA's NW warps.
