@@ -637,8 +637,7 @@ int64_t otoo_devtree_scratch_bytes(int64_t n_part, int64_t cap_cell);
 
 /* Builds the tree of pos (device [n_part][3] FP64, caller order) and mass
    (device [n_part] FP32 > 0) on stream and fills tree's device arrays and
-   out fields; synchronises stream once per tree level (the host reads each
-   level's cell count).  Errors: OTOO_EINVAL (sizes, NULL pointers, scratch
+   out fields; synchronises stream once, at the end (the host reads the counts).  Errors: OTOO_EINVAL (sizes, NULL pointers, scratch
    too small or not 16-byte aligned, a non-finite position or a mass <= 0),
    OTOO_ENOMEM (more cells than cap_cell: n_cell = -1; call again with a
    larger capacity), OTOO_ECUDA. */

@@ -1,7 +1,8 @@
 """Autotuner for the force step.
 
 Knobs: the group size n_crit (it changes the host walk, so every candidate
-re-walks the tree), packed two-wide FP32 arithmetic or not (packed), target
+re-walks the tree), packed (part of a variant's name: every variant computes
+with packed two-wide FP32), target
 particles per lane (iblock), list entries per staged tile (tile),
 list-split threshold (split) and threads per CTA (block).  Objective: device time of one FP32 force step at fixed theta, the
 minimum over repeated CUDA-event timings.  The search is coordinate descent

@@ -2,8 +2,8 @@
 // force kernels (force.cu) and the walk fused with the force (walk.cu):
 // Plummer-softened particle / monopole pairs and quadrupole cell pairs
 // (Section II: a cell acts as a virtual particle at its centre of mass; the
-// quadrupole term is this library's extension), scalar and packed two-wide
-// FP32 forms, compensated running sums and the merge of a warp's lane
+// quadrupole term is this library's extension), FP64 monopole and packed
+// two-wide FP32 forms, compensated running sums and the merge of a warp's lane
 // subsets.  Included inside each translation unit's anonymous namespace.
 #pragma once
 

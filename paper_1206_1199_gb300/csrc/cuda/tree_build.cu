@@ -19,8 +19,7 @@
 //                           per pass: one launch per pass with a decoupled
 //                           look-back between tiles, or all passes in one
 //                           block for at most one tile.
-//   k_permute               particles in tree order (sources, permutation,
-//                           grid coordinates).
+//   k_permute               particles in tree order (sources, permutation).
 //   k_levels / k_cells      every cell of every level at once, from the
 //                           number of key digits that neighbouring particles
 //                           share.
