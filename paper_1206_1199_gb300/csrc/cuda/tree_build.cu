@@ -680,8 +680,9 @@ __device__ __forceinline__ double widen(float f)
 // records take the quadrupole Q = 3 C - tr(C) I.  GB300's FP64 pipe (1/76 of
 // the FP32 rate) bounds both kernels at large N, latency at small N.
 
-// The end of a cell and, for a leaf (nch = 0), its moments.
-__device__ __forceinline__ void close_cell(int32_t cell, int32_t b, int lvl, int32_t nch,
+// The end of a cell, and the moments of a leaf (nch = 0) of one particle; returns
+// the number of particles of a leaf of several, else 0.
+__device__ __forceinline__ int32_t close_cell(int32_t cell, int32_t b, int lvl, int32_t nch,
                                            const uint64_t* __restrict__ keys, int64_t n, int64_t leaf_size,
                                            const otoo_src* __restrict__ src, const Cells& c, const Moments& mo)
 {
@@ -703,18 +704,28 @@ __device__ __forceinline__ void close_cell(int32_t cell, int32_t b, int lvl, int
     const int32_t e = (int32_t)hi;
     c.end[cell] = e;
     mo.dmax2[cell] = 0ull;
-    if (nch > 0) return;
+    if (nch > 0) return 0;
+    if (e - b == 1) {
+        const otoo_src p0 = src[b];
+        double* q = mo.q + 6 * (int64_t)cell;
+        double* com = mo.com + 3 * (int64_t)cell;
+        mo.m[cell] = widen(p0.m);
+        com[0] = p0.x, com[1] = p0.y, com[2] = p0.z;
+        q[0] = q[1] = q[2] = q[3] = q[4] = q[5] = 0.0;
+        mo.b2[cell] = 0.0;
+        return 0;
+    }
+    return e - b;
+}
+
+// The moments of a leaf of several particles [b, e).
+__device__ __forceinline__ void leaf_moments(int32_t cell, int32_t b, int32_t e, const otoo_src* __restrict__ src,
+                                             const Moments& mo)
+{
     const otoo_src p0 = src[b];
     double m = widen(p0.m);
     double* q = mo.q + 6 * (int64_t)cell;
     double* com = mo.com + 3 * (int64_t)cell;
-    if (e - b == 1) {
-        mo.m[cell] = m;
-        com[0] = p0.x, com[1] = p0.y, com[2] = p0.z;
-        q[0] = q[1] = q[2] = q[3] = q[4] = q[5] = 0.0;
-        mo.b2[cell] = 0.0;
-        return;
-    }
     double s1[3] = {0, 0, 0}, s2[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll 1
     for (int32_t i = b + 1; i < e; ++i) {
@@ -744,19 +755,30 @@ __device__ __forceinline__ void close_cell(int32_t cell, int32_t b, int lvl, int
 // a galloping search over the keys' leading digits; a cell that splits holds
 // at least leaf_size + 1 particles), and for a leaf its moments.  The
 // reference particle's own terms are zero and are left out (a leaf of leaf size
-// 8 holds 2.7 particles on average): 17 us at N = 4096, 93-97 us at 2^20, 0.57
-// to 0.64 ms at 2^23 with leaves of 16, links included.
-__global__ void __launch_bounds__(128) k_leaves(const int32_t* __restrict__ lev, const uint64_t* __restrict__ keys,
-                                                int64_t n, int64_t leaf_size, const otoo_src* __restrict__ src,
-                                                Cells c, Moments mo, int32_t* __restrict__ plist,
-                                                int32_t* __restrict__ pcount)
+// 8 holds 2.7 particles on average).  An FP64 instruction costs its warp the
+// same for one lane as for 32, so the block sorts its leaves of several
+// particles by their number (counting sort in shared memory) and a warp takes
+// leaves of about one size.  Bound by the FP64 pipe: N = 2^20 96 -> 64 us, 2^23
+// with leaves of 16 635 -> 440 us against a thread per cell in cell order (16.6 of
+// 32 lanes in an instruction, N = 2^22); 4096 17 -> 18 us, links included.
+constexpr int kLeafThreads = 256;  // cells per block at most
+
+__global__ void __launch_bounds__(kLeafThreads) k_leaves(const int32_t* __restrict__ lev,
+                                                         const uint64_t* __restrict__ keys, int64_t n,
+                                                         int64_t leaf_size, const otoo_src* __restrict__ src, Cells c,
+                                                         Moments mo, int32_t* __restrict__ plist,
+                                                         int32_t* __restrict__ pcount)
 {
+    constexpr int kBins = 64;  // leaves of 64 particles and more first, of 2 last
+    __shared__ int32_t bins[kBins], total;
+    __shared__ int32_t leaf[kLeafThreads][3];  // cell, first particle, one past the last
     const int32_t n_cell = lev[kLv];
     const int lane = threadIdx.x & 31;
-    for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); w0 < n_cell;
-         w0 += (int64_t)gridDim.x * blockDim.x) {
-        const bool in = w0 + lane < n_cell;
-        const int32_t cell = (int32_t)(in ? w0 + lane : w0);
+    for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x; w0 < n_cell; w0 += (int64_t)gridDim.x * blockDim.x) {
+        for (int j = threadIdx.x; j < kBins; j += blockDim.x) bins[j] = 0;
+        __syncthreads();
+        const bool in = w0 + threadIdx.x < n_cell;
+        const int32_t cell = (int32_t)(in ? w0 + threadIdx.x : w0);
         int32_t k = 0;
         const int32_t c0 = in ? c.child0[cell] : 0;
         if (c0 > 0)
@@ -771,11 +793,38 @@ __global__ void __launch_bounds__(128) k_leaves(const int32_t* __restrict__ lev,
         if (k > 0 && lane == lead) at = atomicAdd(pcount + lvl, __popc(peers));
         at = __shfl_sync(kFull, at, lead);
         if (k > 0) plist[lev[lvl] + at + __popc(peers & ((1u << lane) - 1u))] = cell;
+        int32_t np = 0, rank = 0, b = 0;
         if (in) {
             c.nchild[cell] = k;
-            close_cell(cell, c.begin[cell], lvl, k, keys, n, leaf_size, src, c, mo);
+            b = c.begin[cell];
+            np = close_cell(cell, b, lvl, k, keys, n, leaf_size, src, c, mo);
         }
-        __syncwarp();
+        const int bin = np < kBins ? kBins - np : 0;
+        if (np > 0) rank = atomicAdd(bins + bin, 1);
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            const int32_t n0 = bins[2 * lane], n1 = bins[2 * lane + 1];
+            int32_t incl = n0 + n1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t t = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += t;
+            }
+            bins[2 * lane] = incl - n0 - n1;
+            bins[2 * lane + 1] = incl - n1;
+            if (lane == 31) total = incl;
+        }
+        __syncthreads();
+        if (np > 0) {
+            int32_t* q = leaf[bins[bin] + rank];
+            q[0] = cell, q[1] = b, q[2] = b + np;
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < total) {
+            const int32_t* q = leaf[threadIdx.x];
+            leaf_moments(q[0], q[1], q[2], src, mo);
+        }
+        __syncthreads();
     }
 }
 
@@ -1567,7 +1616,10 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
     // cells: their number is on the device)
     const unsigned cg = (unsigned)std::min<int64_t>((cap + 127) / 128, (int64_t)sms * 16);
     int32_t* pcount = head->pcount;
-    k_leaves<<<cg, 128, 0, s>>>(lev, skeys, n, leaf, t->src, c, mo, dig, pcount);
+    // (small trees: smaller blocks use more SMs)
+    const int lt = n < 32768 ? 64 : n < 262144 ? 128 : kLeafThreads;
+    k_leaves<<<(unsigned)std::min<int64_t>((cap + lt - 1) / lt, (int64_t)sms * 8 * kLeafThreads / lt), lt, 0, s>>>(
+        lev, skeys, n, leaf, t->src, c, mo, dig, pcount);
     if (n > leaf) {
         uint32_t* bar = &head->bar;
         void* args[] = {&lev, &c, &mo, &dig, &pcount, &bar, &status};

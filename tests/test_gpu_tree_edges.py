@@ -63,3 +63,12 @@ def test_repeated_builds_are_bit_equal(mac):
         if ref is None:
             ref = got
         assert all(torch.equal(a, b) for a, b in zip(ref, got))
+
+
+@pytest.mark.parametrize("n", [32767, 32769, 262143, 262145])
+@pytest.mark.parametrize("leaf,mac", [(8, "theta"), (70, "theta"), (16, "sw")])
+def test_leaves_across_block_sizes(n, leaf, mac):
+    # the block sizes of the leaf kernel; leaves of 1, of a few and of more than 64 particles
+    pos, mass = ic.plummer(n, 64)
+    kw = dict(mac="sw", delta=1e-3) if mac == "sw" else {}
+    check_tree(pos, mass, leaf, 64 if leaf < 64 else 128, **kw)
