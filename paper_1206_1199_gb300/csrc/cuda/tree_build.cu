@@ -1036,66 +1036,149 @@ __device__ __forceinline__ float bmax_dist(const float4 cc, const float4 p, floa
 // particles.
 //
 // kW lanes (8 or 32) share the particles [i0, i1) of one cell; the lanes of a
-// warp run the same number of rounds (trips, uniform).  Returns the bits of
-// the kW lanes' maximum in every lane.
+// warp run the same number of rounds (trips, uniform).  SPH: returns, in each of
+// the kW lanes, the largest of their particles' radius bounds.
 template <int kW>
-__device__ __forceinline__ unsigned long long bmax_of(int64_t i0, int64_t i1, int trips, int j, float4 cc,
-                                                      const double* __restrict__ com,
-                                                      const otoo_src* __restrict__ src,
-                                                      const float4* __restrict__ pk, int sph)
+__device__ __forceinline__ float bmax_sph(int i0, int i1, int trips, int j, float4 cc, const float4* __restrict__ pk)
 {
-    float lo = 0.f;
+    float hi = 0.f;
+#pragma unroll 4
     for (int t = 0; t < trips; ++t) {
-        const int64_t i = i0 + (int64_t)t * kW + j;
+        const int i = i0 + t * kW + j;
         if (i < i1) {
             const float4 p = pk[i];
             float ej;
             const float d = bmax_dist(cc, p, ej);
-            lo = fmaxf(lo, sph ? d + (p.w + ej) : d * (1.0f - 0x1p-20f) - 2.0f * (ej + cc.w));
+            hi = fmaxf(hi, d + (p.w + ej));
         }
     }
     __syncwarp();
 #pragma unroll
-    for (int o = kW / 2; o > 0; o >>= 1) lo = fmaxf(lo, __shfl_xor_sync(kFull, lo, o));
-    if (sph) return (unsigned long long)__float_as_uint((lo + cc.w) * (1.0f + 0x1p-20f));
-    const double cx = com[0], cy = com[1], cz = com[2];
-    unsigned long long d2max = 0;
+    for (int o = kW / 2; o > 0; o >>= 1) hi = fmaxf(hi, __shfl_xor_sync(kFull, hi, o));
+    return (hi + cc.w) * (1.0f + 0x1p-20f);
+}
+
+// A distance within 2^-22 (the margins allow 2^-20).
+__device__ __forceinline__ float bmax_dist_approx(const float4 cc, const float4 p, float& ej)
+{
+    const float dx = cc.x - p.x, dy = cc.y - p.y, dz = cc.z - p.z;
+    ej = 0x1p-23f * (fabsf(p.x) + fabsf(p.y) + fabsf(p.z));
+    float d;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(d) : "f"(fmaf(dx, dx, fmaf(dy, dy, dz * dz))));
+    return d;
+}
+
+// Absolute MAC, first pass: the kW lanes' largest lower bound lo, and of the
+// lane's own particles the largest upper bound u1 with its particle, and the
+// second largest u2 (infinite when a bound is not finite).
+struct BmaxLane {
+    float lo, u1, u2;
+    int i1;
+};
+template <int kW>
+__device__ __forceinline__ BmaxLane bmax_scan(int i0, int i1, int trips, int j, float4 cc, const float4* __restrict__ pk)
+{
+    BmaxLane r = {0.f, -1.f, -1.f, i0};
+#pragma unroll 4
     for (int t = 0; t < trips; ++t) {
-        const int64_t i = i0 + (int64_t)t * kW + j;
+        const int i = i0 + t * kW + j;
+        if (i < i1) {
+            float ej;
+            const float d = bmax_dist_approx(cc, pk[i], ej);
+            const float e2 = 2.0f * (ej + cc.w), u = (d + e2) * (1.0f + 0x1p-20f);
+            r.lo = fmaxf(r.lo, d * (1.0f - 0x1p-20f) - e2);
+            r.u2 = u <= 3.0e38f ? fmaxf(r.u2, fminf(r.u1, u)) : __int_as_float(0x7f800000);
+            r.i1 = u > r.u1 ? i : r.i1;
+            r.u1 = fmaxf(r.u1, u);
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = kW / 2; o > 0; o >>= 1) r.lo = fmaxf(r.lo, __shfl_xor_sync(kFull, r.lo, o));
+    return r;
+}
+
+// The (cell, particle) pairs whose FP64 distance is to be taken, a queue per
+// warp: an FP64 instruction costs the warp the same for one pair as for 32, so
+// the pairs of several cells are taken together.
+struct BmaxQueue {
+    int2 q[64];
+};
+
+__device__ __forceinline__ void bmax_flush(const BmaxQueue& s, int n, int lane, const double* __restrict__ com,
+                                           const otoo_src* __restrict__ src, unsigned long long* __restrict__ dmax2)
+{
+    __syncwarp();
+    if (lane < n) {
+        const int2 c = s.q[lane];
+        const otoo_src p = src[c.y];
+        const double* x = com + 3 * (int64_t)c.x;
+        const double dx = x[0] - p.x, dy = x[1] - p.y, dz = x[2] - p.z;
+        atomicMax(dmax2 + c.x, (unsigned long long)__double_as_longlong(dx * dx + dy * dy + dz * dz));
+    }
+    __syncwarp();
+}
+
+__device__ __forceinline__ void bmax_push(BmaxQueue& s, int& held, bool near, int32_t cell, int i, int lane,
+                                          const double* __restrict__ com, const otoo_src* __restrict__ src,
+                                          unsigned long long* __restrict__ dmax2)
+{
+    const unsigned m = __ballot_sync(kFull, near);
+    if (near) s.q[held + __popc(m & ((1u << lane) - 1u))] = make_int2(cell, i);
+    held += __popc(m);
+    if (held >= 32) {
+        bmax_flush(s, 32, lane, com, src, dmax2);
+        int2 rest = make_int2(0, 0);
+        if (lane < held - 32) rest = s.q[32 + lane];
+        __syncwarp();
+        if (lane < held - 32) s.q[lane] = rest;
+        held -= 32;
+    }
+}
+
+// Absolute MAC, the candidates of a cell: nearly always a lane has at most one, the
+// one that the first pass kept; if some lane may have a second, all particles
+// are gone through again.
+template <int kW>
+__device__ __forceinline__ void bmax_candidates(BmaxQueue& s, int& held, int32_t cell, const BmaxLane& r, int i0, int i1,
+                                                int trips, int j, int lane, float4 cc, const double* __restrict__ com,
+                                                const otoo_src* __restrict__ src, const float4* __restrict__ pk,
+                                                unsigned long long* __restrict__ dmax2)
+{
+    if (!__any_sync(kFull, r.u2 >= r.lo && trips > 0)) {
+        bmax_push(s, held, r.u1 >= r.lo, cell, r.i1, lane, com, src, dmax2);
+        return;
+    }
+    for (int t = 0; t < trips; ++t) {
+        const int i = i0 + t * kW + j;
         bool near = false;
         if (i < i1) {
             float ej;
-            const float d = bmax_dist(cc, pk[i], ej);
-            near = !((d + 2.0f * (ej + cc.w)) * (1.0f + 0x1p-20f) < lo);  // NaN bounds count as candidates
+            const float d = bmax_dist_approx(cc, pk[i], ej);
+            near = !((d + 2.0f * (ej + cc.w)) * (1.0f + 0x1p-20f) < r.lo);  // NaN bounds count as candidates
         }
-        if (near) {
-            const otoo_src p = src[i];
-            const double dx = cx - p.x, dy = cy - p.y, dz = cz - p.z;
-            const unsigned long long v = (unsigned long long)__double_as_longlong(dx * dx + dy * dy + dz * dz);
-            d2max = v > d2max ? v : d2max;
-        }
+        bmax_push(s, held, near, cell, i, lane, com, src, dmax2);
     }
-    __syncwarp();
-#pragma unroll
-    for (int o = kW / 2; o > 0; o >>= 1) {
-        const unsigned long long v = __shfl_xor_sync(kFull, d2max, o);
-        d2max = v > d2max ? v : d2max;
-    }
-    return d2max;
 }
 
-// Cells of up to kBmaxSmall particles, four per warp (eight lanes each: an
-// FP64 instruction on the narrow pipe serves four cells, where one warp per
-// cell left most of its lanes idle); larger cells as the work items
-// items[0, head->extra) = (cell, chunk of kBmaxChunk particles), one warp each,
-// folded into the cell by an atomic max on the bits (non-negative
-// floating-point values order like their bit patterns).
+// Cells of up to kBmaxSmall particles, four per warp (eight lanes each); larger
+// cells as the work items items[0, head->extra) = (cell, chunk of kBmaxChunk
+// particles), one warp each.  The results fold into dmax2 (zero before) by an
+// atomic max on the bits (non-negative floating-point values order like their
+// bit patterns).  Bound by the loads of the particles' FP32 records and the
+// instructions around them: one pass over them instead of two, approximate square
+// roots inside the bounds' margins and 32-bit indices took the absolute MAC's
+// radii at N = 2^23 (leaves of 16) from 841 to 465 us and the SPH radii at 2^20 from
+// 64 to 53 us; the FP64 distances, in rounds of 32, no longer count.
 constexpr int kBmaxSmall = 64;
 
 __global__ void __launch_bounds__(256) k_bmax(const Head* __restrict__ head, const int2* __restrict__ items,
                                               const otoo_src* __restrict__ src, const float4* __restrict__ pk,
                                               const float4* __restrict__ cf, Cells c, Moments mo, int sph)
 {
+    __shared__ BmaxQueue queue[8];
+    BmaxQueue& s = queue[threadIdx.x >> 5];
+    int held = 0;  // (uniform)
     const int lane = threadIdx.x & 31;
     const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int32_t n_cell = head->lev[kLv];
@@ -1103,11 +1186,16 @@ __global__ void __launch_bounds__(256) k_bmax(const Head* __restrict__ head, con
     for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < n_units; w += nwarp) {
         if (w < nbig) {
             const int2 it = items[w];
-            const int64_t i0 = c.begin[it.x] + (int64_t)it.y * kBmaxChunk, e = c.end[it.x];
-            const int64_t i1 = i0 + kBmaxChunk < e ? i0 + kBmaxChunk : e;
-            const unsigned long long v = bmax_of<32>(i0, i1, (int)((i1 - i0 + 31) / 32), lane, cf[it.x],
-                                                     mo.com + 3 * (int64_t)it.x, src, pk, sph);
-            if (lane == 0) atomicMax(mo.dmax2 + it.x, v);
+            const int i0 = c.begin[it.x] + it.y * kBmaxChunk, e = c.end[it.x];
+            const int i1 = min(i0 + kBmaxChunk, e), trips = (i1 - i0 + 31) / 32;
+            const float4 cc = cf[it.x];
+            if (sph) {
+                const float h = bmax_sph<32>(i0, i1, trips, lane, cc, pk);
+                if (lane == 0) atomicMax(mo.dmax2 + it.x, (unsigned long long)__float_as_uint(h));
+            } else {
+                const BmaxLane r = bmax_scan<32>(i0, i1, trips, lane, cc, pk);
+                bmax_candidates<32>(s, held, it.x, r, i0, i1, trips, lane, lane, cc, mo.com, src, pk, mo.dmax2);
+            }
         } else {
             const int64_t k = 4 * (w - nbig) + (lane >> 3);
             const int32_t cell = (int32_t)(k < n_cell ? k : n_cell - 1);
@@ -1115,11 +1203,18 @@ __global__ void __launch_bounds__(256) k_bmax(const Head* __restrict__ head, con
             // a single particle is its own centre of mass: distance 0
             const bool on = k < n_cell && e - b <= kBmaxSmall && (sph || e - b > 1);
             const int trips = __reduce_max_sync(kFull, on ? (e - b + 7) / 8 : 0);
-            const unsigned long long v = bmax_of<8>(b, on ? e : b, trips, lane & 7, cf[cell],
-                                                    mo.com + 3 * (int64_t)cell, src, pk, sph);
-            if (on && (lane & 7) == 0) mo.dmax2[cell] = v;
+            const int i1 = on ? e : b;
+            const float4 cc = cf[cell];
+            if (sph) {
+                const float h = bmax_sph<8>(b, i1, trips, lane & 7, cc, pk);
+                if (on && (lane & 7) == 0) mo.dmax2[cell] = (unsigned long long)__float_as_uint(h);
+            } else {
+                const BmaxLane r = bmax_scan<8>(b, i1, trips, lane & 7, cc, pk);
+                bmax_candidates<8>(s, held, cell, r, b, i1, trips, lane & 7, lane, cc, mo.com, src, pk, mo.dmax2);
+            }
         }
     }
+    bmax_flush(s, held, lane, mo.com, src, mo.dmax2);
 }
 
 // The work items of the cells of more than kBmaxSmall particles (any order;

@@ -72,3 +72,30 @@ def test_leaves_across_block_sizes(n, leaf, mac):
     pos, mass = ic.plummer(n, 64)
     kw = dict(mac="sw", delta=1e-3) if mac == "sw" else {}
     check_tree(pos, mass, leaf, 64 if leaf < 64 else 128, **kw)
+
+
+@pytest.mark.parametrize("kind", ["lattice", "shell", "pairs"])
+@pytest.mark.parametrize("shift", [0.0, 3e4, -1e7])
+@pytest.mark.parametrize("leaf", [8, 40, 300])
+def test_radii_with_many_candidates(kind, shift, leaf):
+    # many particles at a cell's largest distance, or within the FP32 bounds of
+    # it (large coordinates): the FP64 radius about the record's own centre of
+    # mass (the host's differs from it by the rounding of large coordinates).
+    # With a huge delta the record's r_b is that radius: b / 2 + sqrt(b^2 / 4).
+    if kind == "lattice":
+        g = np.arange(16) / 16.0
+        pos = np.stack(np.meshgrid(g, g, g, indexing="ij"), -1).reshape(-1, 3)
+    elif kind == "shell":
+        v = np.random.default_rng(7).standard_normal((5000, 3))
+        pos = v / np.linalg.norm(v, axis=1)[:, None]
+    else:
+        pos = np.repeat(ic.plummer(1500, 65)[0], 3, axis=0)
+    pos = pos + shift
+    from paper_1206_1199_gb300 import system as S
+    d = S.DeviceTree.build(pos, np.full(len(pos), 1.0 / len(pos), np.float32), leaf, 64, True, "cuda", "sw", 1e290).bufs
+    w = d["cell"].cpu().numpy().view(np.dtype(L.WCell))
+    w64 = d["cell64"].cpu().numpy().view(np.dtype(L.WCell64))
+    p = pos[d["perm"].cpu().numpy()]
+    b = np.array([np.sqrt(((w64["com"][k] - p[w["begin"][k]:w["end"][k]]) ** 2).sum(1).max()) for k in range(len(w))])
+    # (the squared distance's, the square root's and r_b's roundings)
+    assert np.all(np.abs(w64["rb"] - b) <= 8 * 2.0 ** -53 * b + 1e-140)
