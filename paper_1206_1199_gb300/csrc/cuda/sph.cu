@@ -9,8 +9,9 @@
 //   k_sph_prep        once per step, per source in tree order: its position
 //                     as a float pair (hi = x rounded to FP32, lo = the
 //                     remainder), m_j 8/(pi h_j^3) and 1/h_j (h through the
-//                     permutation): the step's only FP64 work, as in the
-//                     force step's float-pair split.
+//                     permutation), as in the force step's float-pair split
+//                     (N = 2^20: 27 us with conversions on the FP64 pipe, 16
+//                     with narrow2).
 //   k_density<IB>     one work item (group, target chunk, list chunk) per warp
 //                     from an atomic ticket, IB targets per lane in lane
 //                     subsets that share out the kept entries of a tile (as
@@ -37,6 +38,7 @@
 #include <cstdint>
 
 #include "../common.h"
+#include "../narrow.h"
 
 using namespace otoo;
 
@@ -66,10 +68,14 @@ __global__ void k_sph_prep(const otoo_src* __restrict__ src, const float* __rest
     }
     const otoo_src s = src[k];
     const float ih = 1.0f / hk;
-    const float hx = __double2float_rn(s.x), hy = __double2float_rn(s.y), hz = __double2float_rn(s.z);
-    out[2 * k] = make_float4(hx, hy, hz, s.m * kNorm * ih * ih * ih);
-    out[2 * k + 1] = make_float4(__double2float_rn(s.x - (double)hx), __double2float_rn(s.y - (double)hy),
-                                 __double2float_rn(s.z - (double)hz), ih);
+    float4 p, l;
+    narrow2(s.x, p.x, l.x);
+    narrow2(s.y, p.y, l.y);
+    narrow2(s.z, p.z, l.z);
+    p.w = s.m * kNorm * ih * ih * ih;
+    l.w = ih;
+    out[2 * k] = p;
+    out[2 * k + 1] = l;
 }
 
 // Square roots of both halves of a float pair (the hardware approximation,
