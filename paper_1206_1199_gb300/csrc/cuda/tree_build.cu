@@ -38,6 +38,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <cstring>
 
 #include "../common.h"
 #include "../treegeom.h"
