@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(256, 2) k_direct_tf(const otoo_src* __restrict
         e2.h = f2dup(eh);
         e2.l = f2dup(__double2float_rn(e - (double)eh));
     }
-    const float ms = __int_as_float((127 - (sc.em > 126 ? 126 : sc.em < -126 ? -126 : sc.em)) << 23);
+    const float ms = __int_as_float((127 - sc.em) << 23);  // 2^-em (em from -125 to 126)
     F2x3 A[4];
     double sum[4][2];
 #pragma unroll

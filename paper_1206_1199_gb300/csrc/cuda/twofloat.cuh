@@ -25,8 +25,9 @@ struct TfScale {
 
 // xmax, mmax: bit patterns of the largest |coordinate| (FP64) and mass (FP32
 // widened).  The form needs finite values, exponents that leave room for
-// r^2 and r^-3, and a softening of at least 2^-30 of the largest coordinate
-// (r^-3 stays far inside the FP32 range).
+// r^2 and r^-3, masses whose power of two has a reciprocal in FP32's normal range
+// (below 2^126), and a softening of at least 2^-30 of the largest coordinate (r^-3
+// stays far inside the FP32 range).
 __device__ __forceinline__ TfScale tf_scale(unsigned long long xmax, uint32_t mmax, double eps2)
 {
     TfScale s;
@@ -34,7 +35,7 @@ __device__ __forceinline__ TfScale tf_scale(unsigned long long xmax, uint32_t mm
     s.ex = xe - 1022;
     s.em = me - 126;
     const int ee = (int)(((unsigned long long)__double_as_longlong(eps2) >> 52) & 2047) - 1023;  // eps2 >= 2^ee
-    s.ok = xe > 0 && me > 0 && me < 255 && s.ex > -300 && s.ex < 300 && ee - 2 * s.ex >= -60 && ee - 2 * s.ex < 60;
+    s.ok = xe > 0 && me > 0 && s.em <= 126 && s.ex > -300 && s.ex < 300 && ee - 2 * s.ex >= -60 && ee - 2 * s.ex < 60;
     return s;
 }
 
