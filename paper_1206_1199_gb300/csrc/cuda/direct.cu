@@ -42,15 +42,14 @@ __global__ void __launch_bounds__(256) k_direct_range(const otoo_src* __restrict
     unsigned long long x = 0;
     uint32_t m = 0;
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
-        const double2* ps = reinterpret_cast<const double2*>(src + i);
-        const double2 a = __ldg(ps), b = __ldg(ps + 1);
-        const double v[3] = {a.x, a.y, b.x};
+        const otoo_src q = src[i];  // (8-byte loads: the sources may start on any 8-byte boundary)
+        const double v[3] = {q.x, q.y, q.z};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const unsigned long long u = (unsigned long long)__double_as_longlong(v[k]) & 0x7fffffffffffffffull;
             x = u > x ? u : x;
         }
-        const uint32_t w = (uint32_t)__double_as_longlong(b.y) & 0x7fffffffu;
+        const uint32_t w = __float_as_uint(q.m) & 0x7fffffffu;
         m = w > m ? w : m;
     }
 #pragma unroll
