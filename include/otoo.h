@@ -389,15 +389,17 @@ int64_t otoo_force_static_capacity(void);
      accel[t] = sum_{j != i} m_j r / (r^2 + eps2)^(3/2),
      pot[t]   = -sum_{j != i} m_j / (r^2 + eps2)^(1/2),   r = x_j - x_i,
    over the n_src sources src[0, n_src) (pass the particles only).  From 65536
-   sources on, pairs are evaluated in two-float arithmetic (relative error of a
-   pair about 2^-47, unbiased; sums in three floats and FP64), whose sums are
-   closer to the exact ones than FP64 pairs summed one after another; systems
-   whose softening is below 2^-30 of the largest coordinate, or whose scale
-   leaves the FP32 exponents, take FP64 pairs at every size.
+   sources on, pairs are evaluated in two-float arithmetic (exact differences of
+   the coordinates whatever the system's extent, relative error of a pair about
+   2^-48, unbiased; the heaviest pairs in FP64, sums in three floats and FP64),
+   whose sums are closer to the exact ones than FP64 pairs summed one after
+   another; systems whose softening is below 2^-30 of the largest coordinate, or
+   whose coordinates or masses leave the FP32 exponents, take FP64 pairs at every
+   size.
    Device arrays: src [n_src], targets [n_tgt] int64, accel [n_tgt][3],
    pot [n_tgt], scratch >= 4 * otoo_direct_chunks(n_src, n_tgt) * n_tgt
    doubles, status one uint32 (bit 2 set when a target index is out of
-   range).  Asynchronous on stream; deterministic (chunk sums in order). */
+   range).  Asynchronous on stream; deterministic (chunk sums in a fixed order). */
 int64_t otoo_direct_chunks(int64_t n_src, int64_t n_tgt);
 int otoo_direct(const otoo_src* src, int64_t n_src, const int64_t* targets, int64_t n_tgt, double eps2,
                 double* accel, double* pot, double* scratch, uint32_t* status, void* stream);

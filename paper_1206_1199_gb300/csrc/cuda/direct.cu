@@ -1,5 +1,5 @@
 // Direct summation on the device: chosen targets against every particle of
-// a system, in FP64 -- the exact reference the learned opening angle is
+// a system, to FP64's accuracy -- the exact reference the learned opening angle is
 // trained against (the measured group errors are this sum's, the paper's
 // O(N^2) brute force of Section II), and a check of the tree force.
 //
@@ -8,10 +8,12 @@
 //                  scale, then the pairs in two-float arithmetic
 //                  (twofloat.cuh), 256 targets per block.
 //   k_direct_part  fewer sources, or a scale the two-float form does not take
-//                  (k_direct_tf then returns at once, else this one does): block (target tile of 128, source chunk): the chunk's
-//                  sources staged through shared memory, FP64 pairs, one
-//                  partial sum per (chunk, target).
-//   k_direct_sum   the chunk partials of each target summed in chunk order.
+//                  (k_direct_tf then returns at once, else this one does): block
+//                  (target tile of 128, source chunk): the chunk's sources staged
+//                  through shared memory, FP64 pairs, one partial sum per (chunk,
+//                  target).
+//   k_direct_sum / k_direct_tree  the chunk partials of each target, in chunk
+//                  order or by the lanes of a warp.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -28,19 +30,25 @@ namespace {
 constexpr int kTgt = 128;     // targets per block
 constexpr int kTile = 128;    // sources staged per tile
 
-// Largest |coordinate| and mass of the sources (order-preserving bit
-// patterns; range is zero before the launch): the scales of the two-float
-// form.  An infinite or NaN coordinate gives the largest pattern.
+// Largest |coordinate|, largest and smallest mass of the sources
+// (order-preserving bit patterns; range is zero before the launch): the scales of
+// the two-float form.  An infinite or NaN coordinate gives the largest pattern.
 struct DirectRange {
     unsigned long long xmax;
-    uint32_t mmax, pad;
+    uint32_t mmax;
+    uint32_t mlow;  // 0x7f800000 less the smallest positive mass's pattern
 };
+
+__device__ __forceinline__ TfScale direct_scale(const DirectRange* __restrict__ r, double eps2)
+{
+    return tf_scale(r->xmax, r->mmax, 0x7f800000u - r->mlow, eps2);
+}
 
 __global__ void __launch_bounds__(256) k_direct_range(const otoo_src* __restrict__ src, int64_t n,
                                                       DirectRange* __restrict__ range)
 {
     unsigned long long x = 0;
-    uint32_t m = 0;
+    uint32_t m = 0, ml = 0;
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
         const otoo_src q = src[i];  // (8-byte loads: the sources may start on any 8-byte boundary)
         const double v[3] = {q.x, q.y, q.z};
@@ -51,6 +59,7 @@ __global__ void __launch_bounds__(256) k_direct_range(const otoo_src* __restrict
         }
         const uint32_t w = __float_as_uint(q.m) & 0x7fffffffu;
         m = w > m ? w : m;
+        if (w - 1u < 0x7f7fffffu) ml = max(ml, 0x7f800000u - w);  // (neither zero, infinite nor NaN)
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -58,75 +67,119 @@ __global__ void __launch_bounds__(256) k_direct_range(const otoo_src* __restrict
         x = u > x ? u : x;
     }
     m = __reduce_max_sync(kFull, m);
+    ml = __reduce_max_sync(kFull, ml);
     if ((threadIdx.x & 31) == 0) {
         atomicMax(&range->xmax, x);
         atomicMax(&range->mmax, m);
+        atomicMax(&range->mlow, ml);
     }
 }
 
 // The two-float form: 256 targets per block, two per thread; the block's
 // halves of 128 threads take the halves of every staged tile, and the second
 // half's sums join the first's at the end.  The float sums are moved into FP64
-// every kTfFold tiles.  Bound by the FP32 pipe: about 195 packed operations per
+// every kTfFold tiles.  Bound by the FP32 pipe: about 260 packed operations per
 // source and two targets.
-// N = 2^19, 5003 targets: 25.1 ms (1.05e11 pairs/s) against 110 ms for the FP64
+// N = 2^19, 5003 targets: 32.6 ms (8.0e10 pairs/s) against 110 ms for the FP64
 // form.  Relative error (2-norm over 40 targets, against extended precision) over
-// N = 66000, 90000, 130000 and 400000, four models and softenings 1e-4 and 1e-2,
-// two-float / FP64 form: accelerations 3.3e-16 to 1.2e-15 / 8.0e-16 to 5.8e-15,
-// potentials 0.9e-16 to 2.5e-16 / 3.9e-16 to 1.7e-15, for each input the
-// two-float form's no larger (one of 32 equal, 8.3e-16 / 8.0e-16): the FP64 form's
-// sums of a chunk's pairs lose more the longer they are.  N = 20000 1.2e-15 / 7.0e-16:
-// the line is where the two-float form is no less exact.
+// N = 66000 and 130000, four models, softenings 1e-4 and 1e-2, and 40, 600 and 5000
+// targets, two-float / FP64 form: accelerations 0.6e-16 to 1.2e-16 / 2.5e-16 to
+// 9.2e-16, potentials 0.5e-16 to 1.2e-16 / 1.9e-16 to 7.4e-16; with one particle 1e3
+// to 1e7 core radii out 0.8e-16 to 2.1e-16 / 2.5e-16 to 6.7e-16; with a fifth of the
+// system in close groups of 2 to 1000, 1.5e-16 to 8.0e-16 / 7.8e-16 to 3.0e-15.
+// (Before, with coordinates on one grid of 2^-62 of the extent, r^2 summed in plain
+// floats and one pair of a run again in FP64: 25.1 ms; 2.9e-16 to 1.3e-15, 4e-16 to
+// 7e-13 and 3e-16 to 2e-13, larger than the FP64 form's in most of them.)
+// Below 65536 sources the FP64 form stays: the line is not a matter of accuracy.
 constexpr int64_t kTfMinSources = 65536;
 constexpr int kTfTile = 256;
-constexpr int kTfFold = 8;  // the longest run (1024 sources) the float sums take before FP64
+constexpr int kTfFold = 8;  // the longest run (1024 sources of each half) the float sums take before FP64
 
 constexpr unsigned kTfPos = kTfFold * kTfTile - 1;  // position in a run
 static_assert(((kTfPos + 1) & kTfPos) == 0, "a run's length is a power of two");
 
-// What the heaviest pair of each target of a run (run0 + the low bits of top)
-// lacks: its FP64 value less the two-float one.  A close pair at a small
-// softening can be most of a target's acceleration, and its 2^-47, or the grid's
-// spacing against its distance, would then be the sum's error (Hernquist, eps
-// 1e-4, N = 130000: 6.4e-15 without this, 3.8e-16 with it, all FP64 1.6e-15).
-__device__ __forceinline__ void tf_refine(const otoo_src* __restrict__ src, int64_t run0, int64_t j1,
-                                          const unsigned top[2], const int64_t ti[2], const long long x[2],
-                                          const long long y[2], const long long z[2], const TfScale& sc, float ms,
-                                          double eps2, const F2x2& e2, double fix[4][2])
+// The pairs of a run that are evaluated again in FP64: the four heaviest of its even
+// and the four of its odd positions (two lists of four cost half the comparisons of
+// one of eight).
+constexpr int kTfTop = 4;
+constexpr int kTfLists = 2;
+
+// A target's coordinates, negated, and another's, one field per operand.
+struct TfTargets {
+    f2 n[3][4];
+};
+__device__ __forceinline__ f2 tf_pack_neg(float a, float b) { return f2pack(-a, -b); }
+__device__ __forceinline__ void tf_targets(const TfCoord c0[3], const TfCoord c1[3], TfTargets& t)
 {
-    long long d[3][2];
-    float m[2];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        t.n[a][0] = tf_pack_neg(c0[a].a, c1[a].a);
+        t.n[a][1] = tf_pack_neg(c0[a].b, c1[a].b);
+        t.n[a][2] = tf_pack_neg(c0[a].c, c1[a].c);
+        t.n[a][3] = tf_pack_neg(c0[a].d, c1[a].d);
+    }
+}
+
+// What one heavy pair of each target of a run (run0 + the low bits of top) lacks:
+// its FP64 value less the two-float one, added to sum.  A few close pairs at a
+// small softening can be most of a target's acceleration, and their 2^-48 would
+// then be the sum's error.
+__device__ __forceinline__ void tf_refine(const otoo_src* __restrict__ src, int64_t run0, int64_t j1, unsigned top0,
+                                          unsigned top1, const int64_t ti[2], const TfTargets& tg, const TfScale& sc,
+                                          float ms, double eps2, const F2v3& e2, double sum[4][2])
+{
     const double es = eps2 * tf_pow2(-2 * sc.ex), sx = tf_pow2(-sc.ex);
+    TfCoord c[2][3];
+    float m[2];
+    double fix[4][2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        int64_t j = run0 + (top[k] & kTfPos);
+        const unsigned top = k ? top1 : top0;
+        int64_t j = run0 + (top & kTfPos);
         j = j < j1 ? j : j1 - 1;
         const otoo_src q = src[j];
-        d[0][k] = tf_fixed(q.x, sc.ex) - x[k];
-        d[1][k] = tf_fixed(q.y, sc.ex) - y[k];
-        d[2][k] = tf_fixed(q.z, sc.ex) - z[k];
-        m[k] = j == ti[k] || top[k] == 0u ? 0.f : q.m * ms;  // (0: no pair)
-        // (from the coordinates themselves: near the origin they are finer than the grid)
+        c[k][0] = tf_split(q.x, sc.ex);
+        c[k][1] = tf_split(q.y, sc.ex);
+        c[k][2] = tf_split(q.z, sc.ex);
+        m[k] = j == ti[k] || top == 0u ? 0.f : q.m * ms;  // (0: no pair)
         const otoo_src t = src[ti[k] < 0 ? j : ti[k]];
         const double rx = (q.x - t.x) * sx, ry = (q.y - t.y) * sx, rz = (q.z - t.z) * sx;
-        const double inv = rsqrt(fma(rx, rx, fma(ry, ry, fma(rz, rz, es))));
-        const double mi = (double)m[k] * inv, mi3 = mi * inv * inv;
+        const double r2 = fma(rx, rx, fma(ry, ry, fma(rz, rz, es)));
+        // (the library's rsqrt is within an ulp, three of them in its cube: corrected
+        // by its residual e = 1 - r^2 y^2)
+        const double y = rsqrt(r2), yy = y * y, e = fma(-r2, fma(y, y, -yy), fma(-r2, yy, 1.0));
+        const double my = (double)m[k] * y, myyy = my * yy, mi3 = fma(1.5 * myyy, e, myyy);
         fix[0][k] = mi3 * rx;
         fix[1][k] = mi3 * ry;
         fix[2][k] = mi3 * rz;
-        fix[3][k] = mi;
+        fix[3][k] = fma(0.5 * my, e, my);
     }
+    F2x2 d[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        d[a] = tf_diff(f2add(f2pack(c[0][a].a, c[1][a].a), tg.n[a][0]), f2add(f2pack(c[0][a].b, c[1][a].b), tg.n[a][1]),
+                       f2add(f2pack(c[0][a].c, c[1][a].c), tg.n[a][2]), f2add(f2pack(c[0][a].d, c[1][a].d), tg.n[a][3]));
     F2x3 A[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) A[c].zero();
-    tf_pair_mono(tf_diff(d[0][0], d[0][1]), tf_diff(d[1][0], d[1][1]), tf_diff(d[2][0], d[2][1]), f2pack(m[0], m[1]), e2,
-                 A);
+    for (int k = 0; k < 4; ++k) A[k].zero();
+    tf_pair_mono(d[0], d[1], d[2], f2pack(m[0], m[1]), e2, A);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int k = 0; k < 4; ++k) {
         double v0, v1;
-        A[c].value(v0, v1);
-        fix[c][0] -= v0;
-        fix[c][1] -= v1;
+        A[k].value(v0, v1);
+        sum[k][0] += fix[k][0] - v0;
+        sum[k][1] += fix[k][1] - v1;
+    }
+}
+
+// Keeps the kTfTop largest of the values w has taken, in order.
+__device__ __forceinline__ void tf_keep(unsigned top[kTfTop], unsigned w)
+{
+#pragma unroll
+    for (int r = 0; r < kTfTop; ++r) {
+        const unsigned hi = max(top[r], w);
+        w = min(top[r], w);
+        top[r] = hi;
     }
 }
 
@@ -136,38 +189,46 @@ __global__ void __launch_bounds__(256, 2) k_direct_tf(const otoo_src* __restrict
                                                       const DirectRange* __restrict__ range,
                                                       uint32_t* __restrict__ status)
 {
-    __shared__ longlong2 s_xy[kTfTile];
-    __shared__ longlong2 s_zm[kTfTile];
+    __shared__ ulonglong2 s_c[6][kTfTile];  // the fields (a, b) and (c, d) of x, y, z, each twice
+    __shared__ float s_m[kTfTile];
     __shared__ double s_sum[128][9];
-    const TfScale sc = tf_scale(range->xmax, range->mmax, eps2);
+    const TfScale sc = direct_scale(range, eps2);
     if (!sc.ok) return;  // k_direct_part runs
     const int lt = threadIdx.x & 127, half = threadIdx.x >> 7;
     const int64_t j0 = (int64_t)blockIdx.y * chunk;
     const int64_t j1 = j0 + chunk < n_src ? j0 + chunk : n_src;
     int64_t ti[2];
-    long long x[2] = {0, 0}, y[2] = {0, 0}, z[2] = {0, 0};
+    TfTargets tg;
+    {
+        TfCoord c[2][3];
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const int64_t t = (int64_t)blockIdx.x * 256 + 128 * k + lt;
-        ti[k] = -1;
-        if (t < n_tgt) {
-            ti[k] = tgt[t];
-            if (ti[k] < 0 || ti[k] >= n_src) {
-                atomicOr(status, 2u);
-                ti[k] = -1;
-            } else {
-                x[k] = tf_fixed(src[ti[k]].x, sc.ex);
-                y[k] = tf_fixed(src[ti[k]].y, sc.ex);
-                z[k] = tf_fixed(src[ti[k]].z, sc.ex);
+        for (int k = 0; k < 2; ++k) {
+            const int64_t t = (int64_t)blockIdx.x * 256 + 128 * k + lt;
+            ti[k] = -1;
+            c[k][0] = c[k][1] = c[k][2] = TfCoord{0.f, 0.f, 0.f, 0.f};
+            if (t < n_tgt) {
+                ti[k] = tgt[t];
+                if (ti[k] < 0 || ti[k] >= n_src) {
+                    atomicOr(status, 2u);
+                    ti[k] = -1;
+                } else {
+                    const otoo_src q = src[ti[k]];
+                    c[k][0] = tf_split(q.x, sc.ex);
+                    c[k][1] = tf_split(q.y, sc.ex);
+                    c[k][2] = tf_split(q.z, sc.ex);
+                }
             }
         }
+        tf_targets(c[0], c[1], tg);
     }
-    F2x2 e2;
+    F2v3 e2;
     {
         const double e = eps2 * tf_pow2(-2 * sc.ex);  // exact
-        const float eh = __double2float_rn(e);
+        const float eh = __double2float_rn(e), el = __double2float_rn(e - (double)eh);
         e2.h = f2dup(eh);
-        e2.l = f2dup(__double2float_rn(e - (double)eh));
+        e2.l = f2dup(el);
+        // (in two floats it would be off by the same 2^-50 in every pair)
+        e2.t = f2dup(__double2float_rn((e - (double)eh) - (double)el));
     }
     const float ms = __int_as_float((127 - sc.em) << 23);  // 2^-em (em from -125 to 126)
     F2x3 A[4];
@@ -179,13 +240,24 @@ __global__ void __launch_bounds__(256, 2) k_direct_tf(const otoo_src* __restrict
     }
     int fold = 0;
     int64_t run0 = j0;            // first source of the run being summed
-    unsigned top[2] = {0u, 0u};   // the run's heaviest pair: m q^2's bits above its position in the run
+    // the run's heaviest pairs per list and target: m r^-2's bits above the position in the run
+    unsigned top[kTfLists][2][kTfTop];
+#pragma unroll
+    for (int r = 0; r < kTfTop; ++r)
+#pragma unroll
+        for (int u = 0; u < kTfLists; ++u) top[u][0][r] = top[u][1][r] = 0u;
     for (int64_t b = j0; b < j1; b += kTfTile) {
         const int64_t j = b + threadIdx.x;
         if (j < j1) {
             const otoo_src q = src[j];
-            s_xy[threadIdx.x] = make_longlong2(tf_fixed(q.x, sc.ex), tf_fixed(q.y, sc.ex));
-            s_zm[threadIdx.x] = make_longlong2(tf_fixed(q.z, sc.ex), (long long)__float_as_uint(q.m * ms));
+            const double x[3] = {q.x, q.y, q.z};
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const TfCoord c = tf_split(x[a], sc.ex);
+                s_c[2 * a][threadIdx.x] = make_ulonglong2(f2dup(c.a), f2dup(c.b));
+                s_c[2 * a + 1][threadIdx.x] = make_ulonglong2(f2dup(c.c), f2dup(c.d));
+            }
+            s_m[threadIdx.x] = q.m * ms;
         }
         __syncthreads();
         const int cnt = j1 - b < kTfTile ? (int)(j1 - b) : kTfTile;
@@ -193,32 +265,50 @@ __global__ void __launch_bounds__(256, 2) k_direct_tf(const otoo_src* __restrict
         const int self0 = ti[0] >= b && ti[0] < b + cnt ? (int)(ti[0] - b) : -1;  // j != i
         const int self1 = ti[1] >= b && ti[1] < b + cnt ? (int)(ti[1] - b) : -1;
 #pragma unroll 1
-        for (int k = k0; k < k1; ++k) {
-            const longlong2 xy = s_xy[k], zm = s_zm[k];
-            const float m = __uint_as_float((unsigned)zm.y);
-            const F2x2 dx = tf_diff(xy.x - x[0], xy.x - x[1]);
-            const F2x2 dy = tf_diff(xy.y - y[0], xy.y - y[1]);
-            const F2x2 dz = tf_diff(zm.x - z[0], zm.x - z[1]);
-            float w0, w1;
-            f2unpack(tf_pair_mono(dx, dy, dz, f2pack(k == self0 ? 0.f : m, k == self1 ? 0.f : m), e2, A), w0, w1);
-            const unsigned at = (unsigned)(fold * kTfTile + k);
-            top[0] = max(top[0], (__float_as_uint(w0) & ~kTfPos) | at);
-            top[1] = max(top[1], (__float_as_uint(w1) & ~kTfPos) | at);
+        for (int k2 = k0; k2 < k1; k2 += kTfLists) {
+#pragma unroll
+            for (int u = 0; u < kTfLists; ++u) {
+                const int k = k2 + u;
+                if (k >= k1) break;
+                const float m = s_m[k];
+                F2x2 d[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const ulonglong2 p = s_c[2 * a][k], q = s_c[2 * a + 1][k];
+                    d[a] = tf_diff(f2add(p.x, tg.n[a][0]), f2add(p.y, tg.n[a][1]), f2add(q.x, tg.n[a][2]),
+                                   f2add(q.y, tg.n[a][3]));
+                }
+                float w0, w1;
+                f2unpack(tf_pair_mono(d[0], d[1], d[2], f2pack(k == self0 ? 0.f : m, k == self1 ? 0.f : m), e2, A), w0,
+                         w1);
+                const unsigned at = (unsigned)(fold * kTfTile + k);
+                tf_keep(top[u][0], (__float_as_uint(w0) & ~kTfPos) | at);
+                tf_keep(top[u][1], (__float_as_uint(w1) & ~kTfPos) | at);
+            }
         }
         if (++fold == kTfFold || b + kTfTile >= j1) {
             fold = 0;
-            // the heaviest pair of the run again in FP64, less what was added for it
-            double fix[4][2];
-            tf_refine(src, run0, j1, top, ti, x, y, z, sc, ms, eps2, e2, fix);
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 double v0, v1;
                 A[c].value(v0, v1);
-                sum[c][0] += v0 + fix[c][0];
-                sum[c][1] += v1 + fix[c][1];
+                sum[c][0] += v0;
+                sum[c][1] += v1;
                 A[c].zero();
             }
-            top[0] = top[1] = 0u;
+            // the heaviest pairs of the run again in FP64, less what was added for them
+#pragma unroll 1
+            for (int r = 0; r < kTfTop; ++r)
+#pragma unroll
+                for (int u = 0; u < kTfLists; ++u) {
+                    tf_refine(src, run0, j1, top[u][0][0], top[u][1][0], ti, tg, sc, ms, eps2, e2, sum);
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+#pragma unroll
+                        for (int q = 0; q + 1 < kTfTop; ++q) top[u][k][q] = top[u][k][q + 1];
+                        top[u][k][kTfTop - 1] = 0u;
+                    }
+                }
             run0 = b + kTfTile;
         }
         __syncthreads();
@@ -250,7 +340,7 @@ __global__ void __launch_bounds__(kTgt) k_direct_part(const otoo_src* __restrict
                                                       uint32_t* __restrict__ status)
 {
     __shared__ double4 s[kTile];
-    if (kAfterTf && tf_scale(range->xmax, range->mmax, eps2).ok) return;
+    if (kAfterTf && direct_scale(range, eps2).ok) return;
     const int64_t t = (int64_t)blockIdx.x * kTgt + threadIdx.x;
     const int64_t j0 = (int64_t)blockIdx.y * chunk;
     const int64_t j1 = j0 + chunk < n_src ? j0 + chunk : n_src;
@@ -315,6 +405,28 @@ __global__ void k_direct_sum(const double* __restrict__ part, int64_t n_tgt, int
     pot[t] = a[3];
 }
 
+// The same by a warp per target (at least kTfMinSources sources): lane l the chunks
+// l, l + 32, ..., then the lanes pairwise.  One after another, the up to 608 partials of
+// a few targets lose more digits than the pairs (N = 66000, 40 targets: 8.2e-16 of the
+// acceleration).
+__global__ void __launch_bounds__(128) k_direct_tree(const double* __restrict__ part, int64_t n_tgt, int n_chunk,
+                                                     double* __restrict__ accel, double* __restrict__ pot)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (t >= n_tgt) return;
+    double a[4] = {0, 0, 0, 0};
+    for (int c = lane; c < n_chunk; c += 32)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a[k] += part[((int64_t)c * n_tgt + t) * 4 + k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a[k] += __shfl_xor_sync(kFull, a[k], o);
+    if (lane < 3) accel[3 * t + lane] = lane == 0 ? a[0] : lane == 1 ? a[1] : a[2];
+    if (lane == 3) pot[t] = a[3];
+}
+
 #define CUDA_TRY(expr)                                                                                 \
     do {                                                                                               \
         cudaError_t e_ = (expr);                                                                       \
@@ -364,7 +476,10 @@ int otoo_direct(const otoo_src* src, int64_t n_src, const int64_t* targets, int6
         k_direct_part<false><<<grid, kTgt, 0, s>>>(src, n_src, targets, n_tgt, eps2, chunk, scratch, nullptr, status);
     }
     CUDA_TRY(cudaGetLastError());
-    k_direct_sum<<<(unsigned)((n_tgt + 127) / 128), 128, 0, s>>>(scratch, n_tgt, (int)nch, accel, pot);
+    if (n_src >= kTfMinSources)
+        k_direct_tree<<<(unsigned)((n_tgt + 3) / 4), 128, 0, s>>>(scratch, n_tgt, (int)nch, accel, pot);
+    else
+        k_direct_sum<<<(unsigned)((n_tgt + 127) / 128), 128, 0, s>>>(scratch, n_tgt, (int)nch, accel, pot);
     CUDA_TRY(cudaGetLastError());
     return OTOO_OK;
 }

@@ -4,16 +4,12 @@
 // clock and SM; conversions to and from FP64 at the same 1.6, measured), so an
 // FP64 pair of 19 operations costs as much pipe time as 1500 FP32 operations.
 // Here a value is an unevaluated sum of two floats (48 bits; Dekker 1971, Knuth
-// TAOCP 2 4.2.2: error-free sums and products), a pair takes about 195 FP32
-// operations, and two targets share every packed two-wide instruction.  A
-// pair's relative error is about 2^-47 and unbiased, and sums are kept in three
-// floats, so the error of a sum over many pairs is below that of FP64 pairs
-// summed one after another; each use states its measurement.
-//
-// Coordinates enter as 64-bit integers on a grid of 2^-62 of the system's
-// largest coordinate (a power of two above it), so a difference is exact; the
-// difference becomes a float pair through three exact pieces.  Included after
-// pair.cuh inside each translation unit's anonymous namespace.
+// TAOCP 2 4.2.2: error-free sums and products) and two targets share every packed
+// two-wide instruction.  Differences of coordinates and r^2 + eps^2 are exact to
+// 2^-60, r^-3 comes from one correction of m y^3 (y the approximate reciprocal
+// root), and sums are kept in three floats: a pair's relative error is 2^-48
+// (rms), without bias.  Included after pair.cuh inside each translation unit's
+// anonymous namespace.
 #pragma once
 
 // Power-of-two scales of one system, from the largest coordinate and mass.
@@ -23,36 +19,58 @@ struct TfScale {
     bool ok;      // the two-float form holds (else the FP64 form runs)
 };
 
-// xmax, mmax: bit patterns of the largest |coordinate| (FP64) and mass (FP32
-// widened).  The form needs finite values, exponents that leave room for
-// r^2 and r^-3, masses whose power of two has a reciprocal in FP32's normal range
-// (below 2^126), and a softening of at least 2^-30 of the largest coordinate (r^-3
-// stays far inside the FP32 range).
-__device__ __forceinline__ TfScale tf_scale(unsigned long long xmax, uint32_t mmax, double eps2)
+// xmax, mmax, mmin: bit patterns of the largest |coordinate| (FP64), the largest
+// and the smallest positive mass (FP32).  The form needs finite values, exponents
+// that leave room for r^2 and r^-3, masses whose power of two has a reciprocal in
+// FP32's normal range (below 2^126), a softening of at least 2^-30 of the largest
+// coordinate (r^-3 stays far inside the FP32 range), and of the lightest source a
+// smallest m r^-3 of 2^-90 in these units (its low parts stay above 2^-149).
+__device__ __forceinline__ TfScale tf_scale(unsigned long long xmax, uint32_t mmax, uint32_t mmin, double eps2)
 {
     TfScale s;
-    const int xe = (int)(xmax >> 52), me = (int)(mmax >> 23);
+    const int xe = (int)(xmax >> 52), me = (int)(mmax >> 23), ml = (int)(mmin >> 23);
     s.ex = xe - 1022;
     s.em = me - 126;
     const int ee = (int)(((unsigned long long)__double_as_longlong(eps2) >> 52) & 2047) - 1023;  // eps2 >= 2^ee
-    s.ok = xe > 0 && me > 0 && s.em <= 126 && s.ex > -300 && s.ex < 300 && ee - 2 * s.ex >= -60 && ee - 2 * s.ex < 60;
+    const int eo = ee - 2 * s.ex;
+    s.ok = xe > 0 && me > 0 && ml > 0 && s.em <= 126 && s.ex > -300 && s.ex < 300 && eo >= -60 && eo < 60 &&
+           2 * (me - ml) + 3 * max(4, eo + 2) <= 180;
     return s;
 }
 
-// x on the grid: x 2^(62 - ex) rounded to an integer (|x| < 2^ex).
-__device__ __forceinline__ long long tf_fixed(double x, int ex)
+// A coordinate in units of 2^ex as a sum of four floats on fixed grids: |x| 2^-ex
+// cut off at 2^-92, its fields of 22, 23, 23 and 24 bits.  Equal fields of two
+// coordinates differ by at most 24 bits, so their difference is exact whatever the
+// coordinates are: one particle far out, which makes the units large, takes
+// nothing from pairs near the origin (2^-92 of the extent is 2^-62 of the smallest
+// softening the form takes).
+struct TfCoord {
+    float a, b, c, d;
+};
+__device__ __forceinline__ TfCoord tf_split(double x, int ex)
 {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int e = (int)((b >> 52) & 2047);
-    unsigned long long m = b & 0xfffffffffffffull;
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    const int e = (int)((u >> 52) & 2047);
+    unsigned long long m = u & 0xfffffffffffffull;
     if (e > 0) m |= 1ull << 52;
-    const int sh = (e > 0 ? e : 1) - 1075 + 62 - ex;  // x = m 2^(sh - 62 + ex)
-    unsigned long long v;
-    if (sh >= 0)
-        v = sh < 11 ? m << sh : 0ull;
-    else
-        v = sh > -55 ? ((m >> (-sh - 1)) + 1ull) >> 1 : 0ull;
-    return (long long)b < 0 ? -(long long)v : (long long)v;
+    const int sh = (e > 0 ? e : 1) - 1075 + 92 - ex;  // |x| 2^(92 - ex) = m 2^sh; below 2^92: sh <= 39
+    unsigned long long lo = 0, hi = 0;
+    if (sh >= 0) {
+        lo = m << (sh & 63);
+        hi = (m >> 1) >> ((63 - sh) & 63);
+    } else if (sh > -64) {
+        lo = m >> -sh;
+    }
+    const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
+    auto field = [&](unsigned v, float unit) {  // +- v unit, exact (v below 2^24)
+        return __uint_as_float(__float_as_uint(__fmul_rn((float)(int)v, unit)) ^ sign);
+    };
+    TfCoord r;
+    r.a = field((unsigned)(hi >> 6) & 0x3fffffu, 0x1p-22f);
+    r.b = field(((unsigned)hi & 63u) << 17 | (unsigned)(lo >> 47), 0x1p-45f);
+    r.c = field((unsigned)(lo >> 24) & 0x7fffffu, 0x1p-68f);
+    r.d = field((unsigned)lo & 0xffffffu, 0x1p-92f);
+    return r;
 }
 
 // 2^k as a double, -1022 <= k <= 1023.
@@ -84,69 +102,60 @@ __device__ __forceinline__ F2x2 two_prod(f2 a, f2 b)
     return r;
 }
 
-// The differences d0, d1 of two targets (in units of 2^-62) as float pairs:
-// 24, 24 and 16 bits of the integer, each exact.
-__device__ __forceinline__ F2x2 tf_diff(long long d0, long long d1)
+// s + e = a + b exactly, for |a| >= |b| or a = 0
+__device__ __forceinline__ F2x2 fast_two_sum(f2 a, f2 b)
 {
-    const f2 ca = f2dup(0x1p-30f), cb = f2dup(0x1p-46f), cc = f2dup(0x1p-62f);
-    const int h0 = (int)(d0 >> 32), h1 = (int)(d1 >> 32);
-    const unsigned l0 = (unsigned)d0, l1 = (unsigned)d1;
-    const f2 a = f2mul(f2pack((float)(h0 & ~0xff), (float)(h1 & ~0xff)), ca);
-    const f2 b = f2mul(f2pack((float)(int)(((h0 & 0xff) << 16) | (l0 >> 16)), (float)(int)(((h1 & 0xff) << 16) | (l1 >> 16))),
-                       cb);
-    const f2 c = f2pack((float)(int)(l0 & 0xffffu), (float)(int)(l1 & 0xffffu));
     F2x2 r;
     r.h = f2add(a, b);
-    r.l = f2fma(c, cc, f2sub(b, f2sub(r.h, a)));
+    r.l = f2sub(b, f2sub(r.h, a));
     return r;
 }
 
-// r^2 + eps^2 of two targets from the difference's float pairs.
-__device__ __forceinline__ F2x2 tf_r2(const F2x2& x, const F2x2& y, const F2x2& z, const F2x2& e2)
+// The difference of two coordinates from its fields' differences (exact), the low
+// part cut at 2^-48 of the high one.
+__device__ __forceinline__ F2x2 tf_diff(f2 a, f2 b, f2 c, f2 d)
 {
-    F2x2 px = two_prod(x.h, x.h), py = two_prod(y.h, y.h), pz = two_prod(z.h, z.h);
-    // (the squares of the low parts too: they are small but never negative)
-    px.l = f2fma(f2add(x.h, x.h), x.l, f2fma(x.l, x.l, px.l));
-    py.l = f2fma(f2add(y.h, y.h), y.l, f2fma(y.l, y.l, py.l));
-    pz.l = f2fma(f2add(z.h, z.h), z.l, f2fma(z.l, z.l, pz.l));
+    const F2x2 u = fast_two_sum(a, b);
+    F2x2 r = fast_two_sum(u.h, f2add(u.l, c));
+    r.l = f2add(r.l, d);
+    return r;
+}
+
+// A value as a sum of three floats, each at most about 2^-23 of the one before.
+struct F2v3 {
+    f2 h, l, t;
+};
+
+// r^2 + eps^2 of two targets from the difference's float pairs, exact to 2^-60:
+// the squares' high parts by exact sums, then the ten terms of 2^-24 (their errors,
+// the squares' and the cross products' low parts) added to a constant of 2^-18 that
+// takes their bits down to 2^-41 without rounding, and what is left below in plain
+// floats.  (Added in plain floats those ten terms left an error of 2^-48.5, and a
+// bias up to 2^-50: squares end in few bit patterns, so that their sums meet ties
+// which all round the same way.)
+__device__ __forceinline__ F2v3 tf_r2(const F2x2& x, const F2x2& y, const F2x2& z, const F2v3& e2)
+{
+    const F2x2 px = two_prod(x.h, x.h), py = two_prod(y.h, y.h), pz = two_prod(z.h, z.h);
+    const F2x2 bx = two_prod(f2add(x.h, x.h), x.l), by = two_prod(f2add(y.h, y.h), y.l),
+               bz = two_prod(f2add(z.h, z.h), z.l);
+    f2 t = f2fma(x.l, x.l, f2fma(y.l, y.l, f2fma(z.l, z.l, e2.t)));
+    t = f2add(t, f2add(f2add(bx.l, by.l), bz.l));
     const F2x2 s1 = two_sum(px.h, py.h), s2 = two_sum(s1.h, pz.h), s3 = two_sum(s2.h, e2.h);
-    const f2 low = f2add(f2add(f2add(px.l, py.l), f2add(pz.l, e2.l)), f2add(f2add(s1.l, s2.l), s3.l));
-    F2x2 r;
-    r.h = f2add(s3.h, low);
-    r.l = f2sub(low, f2sub(r.h, s3.h));
-    return r;
-}
-
-// q = r2^(-1/2): the hardware approximation y (relative error 2^-22) and one
-// step of third order, y + y (e / 2 + 3 e^2 / 8) with e = 1 - r2 y^2 kept as an
-// exact part eh and a remainder, renormalised: relative error about 2^-48.
-__device__ __forceinline__ F2x2 tf_rsqrt(const F2x2& r2)
-{
-    const f2 one = f2dup(1.f);
-    const f2 y = f2rsqrt(r2.h);
-    const F2x2 t = two_prod(y, y);
-    F2x2 p = two_prod(r2.h, t.h);
-    p.l = f2fma(r2.h, t.l, p.l);
-    p.l = f2fma(r2.l, t.h, p.l);
-    const f2 eh = f2sub(one, p.h);  // exact
-    const f2 hy = f2mul(y, f2dup(0.5f));
-    const F2x2 c = two_prod(hy, eh);
-    const f2 e = f2sub(eh, p.l);
-    f2 low = f2fma(hy, f2neg(p.l), c.l);
-    low = f2fma(f2mul(e, e), f2mul(hy, f2dup(0.75f)), low);
-    F2x2 q;
-    q.h = f2add(y, c.h);
-    const f2 x = f2sub(c.h, f2sub(q.h, y));
-    q.l = f2add(x, low);
-    return q;
-}
-
-// the same value with a low part of at most half an ulp of the high one
-__device__ __forceinline__ F2x2 tf_norm(const F2x2& a)
-{
-    F2x2 r;
-    r.h = f2add(a.h, a.l);
-    r.l = f2sub(a.l, f2sub(r.h, a.h));
+    // 1.5 x 2^-18 of each half's power of two (r^2 >= 2^-60: no borrow between the halves)
+    const f2 big = ((s3.h & 0x7f8000007f800000ull) - 0x0900000009000000ull) | 0x0040000000400000ull;
+    f2 T = big;
+    const f2 v[10] = {px.l, py.l, pz.l, bx.h, by.h, bz.h, s1.l, s2.l, s3.l, e2.l};
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+        const f2 u = f2add(T, v[k]);
+        t = f2add(t, f2sub(v[k], f2sub(u, T)));
+        T = u;
+    }
+    const F2x2 u = fast_two_sum(s3.h, f2sub(T, big));
+    F2v3 r;
+    r.h = u.h;
+    r.l = f2add(u.l, t);
+    r.t = f2sub(t, f2sub(r.l, u.l));
     return r;
 }
 
@@ -184,27 +193,44 @@ struct F2x3 {
     }
 };
 
+// w (1 + c), c = (ch, cl) small, of the float pair w
+__device__ __forceinline__ F2x2 tf_corrected(const F2x2& w, f2 ch, f2 cl)
+{
+    const F2x2 k = two_prod(w.h, ch);
+    F2x2 r = fast_two_sum(w.h, k.h);
+    r.l = f2add(r.l, f2add(w.l, f2fma(w.l, ch, f2fma(w.h, cl, k.l))));
+    return r;
+}
+
 // One source of mass m (per target) at difference (x, y, z) from two targets:
-// A[0..2] += m q^3 r, A[3] += m q.  Returns m q^2 (single floats), the pair's
-// weight in the acceleration.
-__device__ __forceinline__ f2 tf_pair_mono(const F2x2& x, const F2x2& y, const F2x2& z, f2 m, const F2x2& e2,
+// A[0..2] += m r^-3 (x, y, z), A[3] += m r^-1.  With y the hardware's approximate
+// r^-1 (relative error 2^-22) and e = 1 - r^2 y^2 as a float pair, m r^-1 =
+// m y (1 + e / 2 + 3 e^2 / 8) and m r^-3 = m y^3 (1 + 3 e / 2 + 15 e^2 / 8), which rounds
+// once where a cube of r^-1 has its error three times.  Returns m r^-2 (single
+// floats), the pair's weight in the acceleration.
+__device__ __forceinline__ f2 tf_pair_mono(const F2x2& x, const F2x2& y, const F2x2& z, f2 m, const F2v3& e2,
                                            F2x3 A[4])
 {
-    const F2x2 q = tf_rsqrt(tf_r2(x, y, z, e2));
-    F2x2 t = two_prod(q.h, q.h);
-    t.l = f2fma(q.l, q.l, t.l);
-    t.l = f2fma(f2add(q.h, q.h), q.l, t.l);
-    t = tf_norm(t);
-    F2x2 mq = two_prod(m, q.h);
-    mq.l = f2fma(m, q.l, mq.l);
+    const F2v3 R = tf_r2(x, y, z, e2);
+    const f2 iy = f2rsqrt(R.h);
+    const F2x2 t = two_prod(iy, iy), p = two_prod(R.h, t.h);
+    const f2 low = f2fma(R.l, t.h, f2fma(R.h, t.l, p.l));
+    F2x2 e = fast_two_sum(f2sub(f2dup(1.f), p.h), f2neg(low));
+    e.l = f2fma(f2neg(R.t), t.h, e.l);
+    const f2 ee = f2mul(e.h, e.h);
+    const F2x2 u = two_prod(m, iy);
+    const F2x2 mq = tf_corrected(u, f2mul(e.h, f2dup(0.5f)), f2fma(ee, f2dup(0.375f), f2mul(e.l, f2dup(0.5f))));
     A[3].add(mq);
-    F2x2 g = tf_mul(mq, t);
-    g.l = f2fma(mq.l, t.l, g.l);
-    g = tf_norm(g);
+    F2x2 v = two_prod(u.h, t.h);
+    v.l = f2fma(u.l, t.h, f2fma(u.h, t.l, v.l));
+    const f2 c15 = f2dup(1.5f), ch = f2mul(e.h, c15);
+    const f2 cl = f2fma(ee, f2dup(1.875f), f2fma(e.l, c15, f2fma(e.h, c15, f2neg(ch))));
+    F2x2 g = tf_corrected(v, ch, cl);
+    g = fast_two_sum(g.h, g.l);
     A[0].add(tf_mul(g, x));
     A[1].add(tf_mul(g, y));
     A[2].add(tf_mul(g, z));
-    return f2mul(mq.h, q.h);
+    return f2mul(mq.h, iy);
 }
 
 // ---- one value per operand (the quadrupole part of the FP64 form) ------------
