@@ -581,16 +581,21 @@ __global__ void __launch_bounds__(kLvThreads) k_levels(const uint64_t* __restric
 
 // Writes the cells that start in the tile.  offs: the exclusive scan of
 // k_levels' counts, *total their sum; block 0 writes the levels' first cells
-// lev[0 .. 22].  More than cap cells: nothing is written and stop is set.
+// lev[0 .. 22].  More than cap cells, or an error found before (status: a position
+// that is not finite would put every particle into one leaf, which one thread sums
+// for a second at N = 2^23): nothing is written, so that every later kernel finds no
+// cells, and stop is set.
 __global__ void __launch_bounds__(kLvThreads) k_cells(int64_t n, const uint16_t* __restrict__ lv,
                                                        const int32_t* __restrict__ offs,
                                                        const int64_t* __restrict__ total, int64_t cap, Cells c,
-                                                       int32_t* __restrict__ lev, uint32_t* __restrict__ stop)
+                                                       int32_t* __restrict__ lev,
+                                                       const uint32_t* __restrict__ status,
+                                                       uint32_t* __restrict__ stop)
 {
     __shared__ int32_t wcnt[kLvWarps][kLv];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    if (*total > cap) {
+    if (*total > cap || *status != 0u) {
         if (blockIdx.x == 0 && threadIdx.x == 0) *stop = 1u;
         return;
     }
@@ -1724,7 +1729,7 @@ int otoo_devtree_build(const double* pos, const float* mass, otoo_devtree* t, vo
         const int r = scan32(hist, (int64_t)kLv * nblk, bsum, &head->cells, s);
         if (r) return r;
     }
-    k_cells<<<nblk, kLvThreads, 0, s>>>(n, lv, hist, &head->cells, cap, c, lev, &head->stop);
+    k_cells<<<nblk, kLvThreads, 0, s>>>(n, lv, hist, &head->cells, cap, c, lev, status, &head->stop);
     CUDA_TRY(cudaGetLastError());
 
     // links, leaves, then the parents level by level (grid-stride over the
