@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kBackThreads) k_mlp_backward(const uint16_t* _
         float z = sh.w[OB1 + i];
 #pragma unroll
         for (int k = 0; k < NI; ++k) z = fmaf(sh.w[OW1 + i * NI + k], xr[k], z);
-        h1[u] = tanhf(z);
+        h1[u] = on ? tanhf(z) : 0.f;  // (an infinite weight against the zeros of a row past the last is NaN)
     }
 #pragma unroll
     for (int u = 0; u < kU; u += 4)
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kBackThreads) k_mlp_backward(const uint16_t* _
             z[4] = fmaf(wb.x, h, z[4]), z[5] = fmaf(wb.y, h, z[5]), z[6] = fmaf(wb.z, h, z[6]), z[7] = fmaf(wb.w, h, z[7]);
         }
 #pragma unroll
-        for (int u = 0; u < kU; ++u) h2[u] = tanhf(z[u]);
+        for (int u = 0; u < kU; ++u) h2[u] = on ? tanhf(z[u]) : 0.f;
 #pragma unroll
         for (int u = 0; u < kU; u += 4)
             *reinterpret_cast<float4*>(&sh.h2[row][u0 + u]) = make_float4(h2[u], h2[u + 1], h2[u + 2], h2[u + 3]);
@@ -197,11 +197,11 @@ __global__ void __launch_bounds__(kBackThreads) k_mlp_backward(const uint16_t* _
             yv = fmaf(sh.w[OW3 + j], h.x, yv), yv = fmaf(sh.w[OW3 + j + 1], h.y, yv);
             yv = fmaf(sh.w[OW3 + j + 2], h.z, yv), yv = fmaf(sh.w[OW3 + j + 3], h.w, yv);
         }
-        // rows past the last: no residual, so every delta is zero
+        // rows past the last: no residual; their hidden values and deltas are zero
         const float dy = on ? 2.0f * (yv - target) * inv_n : 0.f;
         float d[kU];
 #pragma unroll
-        for (int u = 0; u < kU; ++u) d[u] = dy * sh.w[OW3 + u0 + u] * (1.0f - h2[u] * h2[u]);
+        for (int u = 0; u < kU; ++u) d[u] = on ? dy * sh.w[OW3 + u0 + u] * (1.0f - h2[u] * h2[u]) : 0.f;
 #pragma unroll
         for (int u = 0; u < kU; u += 4)
             *reinterpret_cast<float4*>(&sh.d2[row][u0 + u]) = make_float4(d[u], d[u + 1], d[u + 2], d[u + 3]);
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kBackThreads) k_mlp_backward(const uint16_t* _
             sd[4] = fmaf(wb.x, d, sd[4]), sd[5] = fmaf(wb.y, d, sd[5]), sd[6] = fmaf(wb.z, d, sd[6]), sd[7] = fmaf(wb.w, d, sd[7]);
         }
 #pragma unroll
-        for (int u = 0; u < kU; ++u) sd[u] *= 1.0f - h1[u] * h1[u];
+        for (int u = 0; u < kU; ++u) sd[u] = on ? sd[u] * (1.0f - h1[u] * h1[u]) : 0.f;
 #pragma unroll
         for (int u = 0; u < kU; u += 4)
             *reinterpret_cast<float4*>(&sh.d1[row][u0 + u]) = make_float4(sd[u], sd[u + 1], sd[u + 2], sd[u + 3]);
