@@ -50,8 +50,8 @@ extern "C" {
 
 /* precision of otoo_force */
 #define OTOO_FP32K 0      /* FP32 centre-relative pairs, per-thread Kahan sums, FP64 final sums */
-#define OTOO_FP64  1      /* every pair in FP64 (comparison form; the quadrupole part of a cell as
-                             sums of two floats, relative error about 2^-47 of that part) */
+#define OTOO_FP64  1      /* every pair in FP64 (comparison form; the quadrupole part of a cell in
+                             62-bit fixed point, whose error is below that of FP64 operations) */
 
 /* ---- parameters ----------------------------------------------------------- */
 /* acceptance rule of the walk (otoo_params.mac) */

@@ -20,7 +20,7 @@
 //                 sums between Kahan-compensated flushes, FP64 merge of the
 //                 lane-level j-split and FP64 outputs.
 //   k_force_f64   FP64 form (comparison form): one work item per CTA, FP64
-//                 pairs (the quadrupole part in two-float arithmetic).
+//                 pairs (the quadrupole part in fixed point).
 //   k_merge       FP64 sum of the chunk partials of split lists, in chunk
 //                 order (deterministic).
 #include <cuda_runtime.h>
@@ -32,6 +32,7 @@
 
 #include "../common.h"
 #include "../narrow.h"
+#include "../quadfix.h"
 
 using namespace otoo;
 
@@ -42,7 +43,6 @@ constexpr uint32_t kBadItem = 1u;
 constexpr uint32_t kBadIndex = 2u;
 
 #include "pair.cuh"
-#include "twofloat.cuh"
 
 __device__ __forceinline__ void load_src(const otoo_src* src, int64_t idx, double& x, double& y, double& z, float& m)
 {
@@ -159,24 +159,60 @@ __global__ void k_centre_relative(const float4* __restrict__ pairs, int64_t n, f
 
 #include "force_warp2.cuh"
 
-// FP64 form: one work item per CTA of B threads, IB targets per thread,
-// B entries staged per tile; particles and monopoles in FP64, of a quadrupole
-// cell the monopole part (pair_quad_mixed).  Bound by the FP64 pipe, 18
-// operations per pair.  N = 2^17 (4.7e8 pairs, 70% with cells): 17.1 ms against
-// 28.3 ms with the quadrupole part in FP64 too (38 operations); error against
-// extended precision on the same lists (2-norm, accelerations) 4.5e-16 both, the
-// potentials' 1.7e-16 and 1.6e-16; over four models, theta 0.5 to 0.9,
-// softenings 1e-4 to 0.3 and lengths of 1 and 1e12 accelerations 1.3e-16 to
-// 5.5e-16 (within 6% of each other), potentials 1.3e-16 to 1.8e-16 (0.92 to 1.07).
-template <int B, int IB>
+// A quadrupole cell of the FP64 form (pair_quad2's law): the monopole part in FP64,
+// the quadrupole part in fixed point (quadfix.h).
+__device__ __forceinline__ void pair_quad_f64(const V4<double>& s, const QuadFix& c, double xi, double yi, double zi,
+                                              double eps2, double p[4], QuadSum& Q)
+{
+    const double rx = s.x - xi, ry = s.y - yi, rz = s.z - zi;
+    const double r2 = fma(rx, rx, fma(ry, ry, fma(rz, rz, eps2)));
+    const double q = rsqrt(r2);
+    const double q2 = q * q;
+    const double mq = s.w * q;
+    const double mq3 = mq * q2;
+    p[3] -= mq;
+    p[0] = fma(mq3, rx, p[0]);
+    p[1] = fma(mq3, ry, p[1]);
+    p[2] = fma(mq3, rz, p[2]);
+    if (((__double2hiint(q) >> 20) & 2047) == 0) return;  // r^2 past the FP64 range
+    if (c.kind == 1) {
+        quad_fix_pair(c, rx, ry, rz, q, eps2 * q2, Q, p);
+    } else if (c.kind == 2) {  // a field that is not finite
+        double v[7];
+#pragma unroll
+        for (int k = 0; k < 7; ++k) v[k] = (double)__int_as_float(c.h[k]);
+        const double n0 = fma(v[0], rx, fma(v[3], ry, v[4] * rz)), n1 = fma(v[3], rx, fma(v[1], ry, v[5] * rz));
+        const double n2 = fma(v[4], rx, fma(v[5], ry, v[2] * rz));
+        const double q5 = q * (q2 * q2), t = fma(rx, n0, fma(ry, n1, fma(rz, n2, -v[6] * eps2))) * q5;
+        p[3] = fma(-0.5, t, p[3]);
+        p[0] = fma(2.5 * t * q2, rx, fma(-q5, n0, p[0]));
+        p[1] = fma(2.5 * t * q2, ry, fma(-q5, n1, p[1]));
+        p[2] = fma(2.5 * t * q2, rz, fma(-q5, n2, p[2]));
+    }
+}
+
+// FP64 form: one work item per CTA of B threads, a target per thread (items of
+// more than B targets, kMax at most, in passes of B), the threads' subsets share
+// out the entries of a tile of B; particles and monopoles in FP64, of a quadrupole
+// cell the monopole part (pair_quad_f64).  Bound by the
+// FP64 pipe, 19 operations per pair (39 with the quadrupole part in FP64).  N = 2^17,
+// theta 0.5 (4.7e8 pairs, 70% with cells): 16.8 ms against 28.3 ms all in FP64, 17.1
+// with the quadrupole part in two-float arithmetic, whose 2^-47 showed at theta 0.9
+// (King, N = 5000: 1.9e-16).  Error against extended precision on the same lists (2-norm
+// over 200 targets, twelve models, sizes, theta 0.4 to 1, softenings 1e-9 to 0.3,
+// lengths of 1 and 1e12, masses 1e-20 next to 1), here / all in FP64: accelerations
+// 0.7e-16 to 1.2e-16 / 1.5e-16 to 2.0e-16, potentials 0.5e-16 to 0.9e-16 / 1.4e-16 to
+// 1.7e-16 (eps 1e-9: 2.2e-16 / 2.3e-16).
+// (With two or four targets a thread the kernel needs 192 or 250 registers: 19.3
+// and 24.8 ms.)
+template <int B, int kMax>
 __global__ void __launch_bounds__(B) k_force_f64(const otoo_dev_system sys, double* __restrict__ accel,
                                                  double* __restrict__ pot)
 {
     __shared__ V4<double> s_src[B];
-    __shared__ float4 s_qa[B];
-    __shared__ float4 s_qb[B];
+    __shared__ QuadFix s_quad[B];
     __shared__ int s_idx[B];  // particle entries: their source index
-    __shared__ double s_red[B * IB * 4];
+    __shared__ double s_red[B * 4];
     __shared__ int s_ticket;
 
     const int tid = threadIdx.x;
@@ -192,120 +228,109 @@ __global__ void __launch_bounds__(B) k_force_f64(const otoo_dev_system sys, doub
 
         const otoo_item item = sys.items[it];
         otoo_group grp;
-        if (!item_ok(sys, item, grp, B * IB)) {
+        if (!item_ok(sys, item, grp, kMax)) {
             if (tid == 0) atomicOr(status, kBadItem);
             continue;
         }
-        const int ni = item.ni;
-        const int P = (ni + IB - 1) / IB;
-        const int nsplit = B / P;
-        const int islot = tid % P, js = tid / P;
-        const bool active = js < nsplit;
         const double eps2 = grp.eps2;
         const double cx = grp.cx, cy = grp.cy, cz = grp.cz;
-
-        double xi[IB], yi[IB], zi[IB];
-        Acc<double> acc[IB];
-        QuadSum qsum[IB];
-        int self[IB];  // the target's own source index
-#pragma unroll
-        for (int k = 0; k < IB; ++k) {
-            const int i = islot + k * P;
-            qsum[k].zero();
-            self[k] = active && i < ni ? grp.first + item.i0 + i : -1;
-            xi[k] = yi[k] = zi[k] = 0.0;
-            if (active && i < ni) {
-                double x, y, z;
-                float m;
-                load_src(sys.src, (int64_t)grp.first + item.i0 + i, x, y, z, m);
-                xi[k] = x - cx;
-                yi[k] = y - cy;
-                zi[k] = z - cz;
-            }
-            acc[k].zero();
-        }
-
         const int32_t* lst = sys.list + grp.list_off;
-        for (int seg = 0; seg < 2; ++seg) {
-            const bool is_cell = seg == 0;
-            const int s0 = is_cell ? item.j0 : max(item.j0, grp.n_cell);
-            const int s1 = is_cell ? min(item.j1, grp.n_cell) : item.j1;
-            const bool quad = is_cell && has_quad;
-            for (int base = s0; base < s1; base += B) {
-                const int cnt = min(B, s1 - base);
-                if (tid < cnt) {
-                    const int idx = __ldg(lst + base + tid);
-                    const bool good = is_cell ? (idx >= sys.n_part && idx < sys.n_src) : (idx >= 0 && idx < sys.n_part);
-                    V4<double> v = {0, 0, 0, 0};
-                    if (good) {
-                        double x, y, z;
-                        float m;
-                        load_src(sys.src, idx, x, y, z, m);
-                        v = V4<double>{x - cx, y - cy, z - cz, (double)m};
-                    } else {
-                        atomicOr(status, kBadIndex);
-                    }
-                    s_src[tid] = v;
-                    s_idx[tid] = good ? idx : -2;
-                    if (quad) {
-                        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-                        if (good) {
-                            const float4* qp = reinterpret_cast<const float4*>(sys.quad + (idx - sys.n_part));
-                            a = __ldg(qp);
-                            b = __ldg(qp + 1);
-                        }
-                        s_qa[tid] = a;
-                        s_qb[tid] = b;
-                    }
-                }
-                __syncthreads();
-                if (active) {
-                    double p[IB][4];
-#pragma unroll
-                    for (int k = 0; k < IB; ++k) p[k][0] = p[k][1] = p[k][2] = p[k][3] = 0.0;
-                    if (quad) {
-                        for (int j = js; j < cnt; j += nsplit) {
-                            const V4<double> s = s_src[j];
-                            const float4 qa = s_qa[j], qb = s_qb[j];
-#pragma unroll
-                            for (int k = 0; k < IB; ++k)
-                                pair_quad_mixed(s, qa, qb, xi[k], yi[k], zi[k], eps2, p[k], qsum[k]);
-                        }
-                    } else {
-                        for (int j = js; j < cnt; j += nsplit) {
-                            const V4<double> s = s_src[j];
-                            const int idx = s_idx[j];
-#pragma unroll
-                            for (int k = 0; k < IB; ++k)
-                                pair_mono(V4<double>{s.x, s.y, s.z, idx == self[k] ? 0.0 : s.w}, xi[k], yi[k], zi[k],
-                                          eps2, p[k]);  // j != i
-                        }
-                    }
-#pragma unroll
-                    for (int k = 0; k < IB; ++k) acc[k].add(p[k]);
-                }
-                __syncthreads();
+#pragma unroll 1
+        for (int i0 = 0; i0 < item.ni; i0 += B) {
+            const int P = min(B, item.ni - i0);
+            const int nsplit = B / P;
+            const int islot = tid % P, js = tid / P;
+            const bool active = js < nsplit;
+            const int64_t t = (int64_t)grp.first + item.i0 + i0 + islot;  // the target's own source index
+            double xi, yi, zi;
+            {
+                float m;
+                load_src(sys.src, t, xi, yi, zi, m);
+                xi -= cx, yi -= cy, zi -= cz;
             }
-        }
+            Acc<double> acc;
+            acc.zero();
+            QuadSum qsum;
+            qsum.zero();
+            int terms = 0;  // quadrupole terms since the last fold, at most
 
-        if (active) {
+            for (int seg = 0; seg < 2; ++seg) {
+                const bool is_cell = seg == 0;
+                const int s0 = is_cell ? item.j0 : max(item.j0, grp.n_cell);
+                const int s1 = is_cell ? min(item.j1, grp.n_cell) : item.j1;
+                const bool quad = is_cell && has_quad;
+                for (int base = s0; base < s1; base += B) {
+                    const int cnt = min(B, s1 - base);
+                    if (tid < cnt) {
+                        const int idx = __ldg(lst + base + tid);
+                        const bool good =
+                            is_cell ? (idx >= sys.n_part && idx < sys.n_src) : (idx >= 0 && idx < sys.n_part);
+                        V4<double> v = {0, 0, 0, 0};
+                        if (good) {
+                            double x, y, z;
+                            float m;
+                            load_src(sys.src, idx, x, y, z, m);
+                            v = V4<double>{x - cx, y - cy, z - cz, (double)m};
+                        } else {
+                            atomicOr(status, kBadIndex);
+                        }
+                        s_src[tid] = v;
+                        s_idx[tid] = good ? idx : -2;
+                        if (quad) {
+                            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+                            if (good) {
+                                const float4* qp = reinterpret_cast<const float4*>(sys.quad + (idx - sys.n_part));
+                                a = __ldg(qp);
+                                b = __ldg(qp + 1);
+                            }
+                            const float v7[7] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z};
+                            s_quad[tid] = quad_fix(v7);
+                        }
+                    }
+                    __syncthreads();
+                    if (active) {
+                        double p[4] = {0.0, 0.0, 0.0, 0.0};
+                        if (quad) {
+                            for (int j = js; j < cnt; j += nsplit)
+                                pair_quad_f64(s_src[j], s_quad[j], xi, yi, zi, eps2, p, qsum);
+                            terms += (B + nsplit - 1) / nsplit;
+                            if (terms > kQuadTerms - B) {
+                                terms = 0;
+                                qsum.fold(p);
+                            }
+                        } else {
+                            for (int j = js; j < cnt; j += nsplit) {
+                                const V4<double> s = s_src[j];
+                                pair_mono(V4<double>{s.x, s.y, s.z, s_idx[j] == t ? 0.0 : s.w}, xi, yi, zi, eps2,
+                                          p);  // j != i
+                            }
+                        }
+                        acc.add(p);
+                    }
+                    __syncthreads();
+                }
+            }
+
+            if (active) {
+                qsum.fold(acc.s);
 #pragma unroll
-            for (int k = 0; k < IB; ++k) qsum[k].fold(acc[k].s);
-#pragma unroll
-            for (int k = 0; k < IB; ++k)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) s_red[((js * P + islot) * IB + k) * 4 + c] = acc[k].value(c);
+                for (int c = 0; c < 4; ++c) s_red[(js * P + islot) * 4 + c] = acc.value(c);
+            }
+            __syncthreads();
+            // the subsets' sums, each addition's error carried along: a component of a
+            // target per thread (by the targets' threads alone its dependent FP64
+            // operations held the other warps up by 15% on short lists)
+            for (int r = tid; r < 4 * P; r += B) {
+                double a = 0.0, e = 0.0;
+                for (int j = 0; j < nsplit; ++j) {
+                    const double v = s_red[4 * j * P + r], u = __dadd_rn(a, v), w = __dsub_rn(u, a);
+                    e += __dadd_rn(__dsub_rn(a, __dsub_rn(u, w)), __dsub_rn(v, w));
+                    a = u;
+                }
+                write_component(sys, grp, item, i0 + (r >> 2), r & 3, a + e, accel, pot);
+            }
+            __syncthreads();
         }
-        __syncthreads();
-        for (int i = tid; i < ni; i += B) {
-            const int sl = i % P, k = i / P;
-            double a[4] = {0, 0, 0, 0};
-            for (int j = 0; j < nsplit; ++j)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) a[c] += s_red[((j * P + sl) * IB + k) * 4 + c];
-            write_target(sys, grp, item, i, a, accel, pot);
-        }
-        __syncthreads();
     }
 }
 
@@ -387,13 +412,19 @@ ForceKernel pick_f32(int B, int IB, int tile, int packed)
     return {nullptr, nullptr, 0, false};
 }
 
-// FP64 form: B threads per CTA for a plan made with iblock targets per lane
-// (items of at most 32 * iblock targets).
+// FP64 form: B threads per CTA, items of up to the 128 iblock targets that were
+// taken with iblock targets a thread.  256 threads up to 14 items per SM, where the
+// longest items set the time and twice the threads share an item's entries.
+// Microseconds with 128 / 256 threads: 0.7 items per SM 314 / 278, 2.5 1135 / 685, 5.6 2451 /
+// 1206, 9 2512 / 1278, 14 2628 / 1772, 15 (short lists) 833 / 857, 27 2548 / 2690 (before
+// the subsets' sums were added component by component).
+constexpr int64_t kWideItems = 14;
+template <int B>
 Kernel pick_f64(int IB)
 {
-    if (IB == 1) return k_force_f64<128, 1>;
-    if (IB == 2) return k_force_f64<128, 2>;
-    return k_force_f64<128, 4>;
+    if (IB == 1) return k_force_f64<B, 128>;
+    if (IB == 2) return k_force_f64<B, 256>;
+    return k_force_f64<B, 512>;
 }
 
 int check_tune(const otoo_tune* t)
@@ -443,14 +474,15 @@ int enqueue_force(const otoo_dev_system* sys, double* accel, double* pot, int pr
                   cudaStream_t s)
 {
     const bool fp64 = precision == OTOO_FP64;
-    const ForceKernel fk = fp64 ? ForceKernel{pick_f64(t->iblock), nullptr, 0, false}
-                                : pick_f32(t->block, t->iblock, t->tile, t->packed);
     int dev = 0, nsm = 0, occ = 0;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const bool wide = fp64 && sys->n_items <= kWideItems * nsm;
+    const ForceKernel fk = fp64 ? ForceKernel{wide ? pick_f64<256>(t->iblock) : pick_f64<128>(t->iblock), nullptr, 0, false}
+                                : pick_f32(t->block, t->iblock, t->tile, t->packed);
     const bool team = !fp64 && sys->n_items <= kTeamItems * nsm;
     Kernel fn = team ? fk.team : fk.one;
-    const int block = fp64 ? 128 : team ? 32 * kTeamWarps : t->block;
+    const int block = fp64 ? (wide ? 256 : 128) : team ? 32 * kTeamWarps : t->block;
     const int smem = team ? fk.team_smem : 0;
     if (team && fk.opt_in) CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, smem));

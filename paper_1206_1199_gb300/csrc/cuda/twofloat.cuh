@@ -232,165 +232,3 @@ __device__ __forceinline__ f2 tf_pair_mono(const F2x2& x, const F2x2& y, const F
     A[2].add(tf_mul(g, z));
     return f2mul(mq.h, iy);
 }
-
-// ---- one value per operand (the quadrupole part of the FP64 form) ------------
-
-struct F2s {
-    float h, l;
-};
-
-__device__ __forceinline__ F2s sum2(float a, float b)
-{
-    F2s r;
-    r.h = __fadd_rn(a, b);
-    const float bb = __fsub_rn(r.h, a);
-    r.l = __fadd_rn(__fsub_rn(a, __fsub_rn(r.h, bb)), __fsub_rn(b, bb));
-    return r;
-}
-__device__ __forceinline__ F2s prod2(float a, float b)
-{
-    F2s r;
-    r.h = __fmul_rn(a, b);
-    r.l = __fmaf_rn(a, b, -r.h);
-    return r;
-}
-__device__ __forceinline__ F2s mul2(const F2s& a, const F2s& b)
-{
-    F2s r = prod2(a.h, b.h);
-    r.l = __fmaf_rn(a.h, b.l, r.l);
-    r.l = __fmaf_rn(a.l, b.h, r.l);
-    return r;
-}
-__device__ __forceinline__ F2s mul2(float a, const F2s& b)
-{
-    F2s r = prod2(a, b.h);
-    r.l = __fmaf_rn(a, b.l, r.l);
-    return r;
-}
-// the same value with a low part of at most half an ulp of the high one
-__device__ __forceinline__ F2s norm2(const F2s& a)
-{
-    F2s r;
-    r.h = __fadd_rn(a.h, a.l);
-    r.l = __fsub_rn(a.l, __fsub_rn(r.h, a.h));
-    return r;
-}
-__device__ __forceinline__ F2s add2(const F2s& a, const F2s& b)
-{
-    F2s r = sum2(a.h, b.h);
-    r.l = __fadd_rn(r.l, __fadd_rn(a.l, b.l));
-    return r;
-}
-
-// x 2^k as a float pair by integer operations on x's bits (the FP64 pipe, which
-// a conversion would occupy, bounds the kernels that use this): the top 24
-// bits of the mantissa, truncated, and the rest, then renormalised (a low part
-// of one sign would bias the products that leave out the low parts' product).
-// |x 2^k| below 2^-73 gives 0; it must stay below 2^127.
-__device__ __forceinline__ F2s split2(double x, int k)
-{
-    const int hi = __double2hiint(x), lo = __double2loint(x);
-    const int a = (hi & 0x7fffffff) + ((k - 896) << 20);  // float exponent field above 20 mantissa bits
-    const unsigned sign = (unsigned)hi & 0x80000000u;
-    const bool tiny = a < (54 << 20);
-    const float h = tiny ? 0.f : __uint_as_float(__funnelshift_l((unsigned)lo, (unsigned)a, 3) | sign);
-    const float ulp = tiny ? 0.f : __uint_as_float(((((unsigned)a >> 20) - 52u) << 23) | sign);
-    const float l = __fmul_rn((float)(lo & 0x1fffffff), ulp);
-    F2s r;
-    r.h = __fadd_rn(h, l);
-    r.l = __fsub_rn(l, __fsub_rn(r.h, h));
-    return r;
-}
-
-// A running sum of three floats (F2x3 for one value).
-struct F3s {
-    float h, m, l;
-    __device__ __forceinline__ void zero() { h = m = l = 0.f; }
-    __device__ __forceinline__ void add(const F2s& p)
-    {
-        const F2s t = sum2(h, p.h), u = sum2(m, t.l), v = sum2(u.h, p.l);
-        h = t.h;
-        m = v.h;
-        l = __fadd_rn(l, __fadd_rn(u.l, v.l));
-    }
-    __device__ __forceinline__ double value() const { return (double)h + ((double)m + (double)l); }
-};
-
-// The quadrupole terms of one target: sums of three floats in units of powers
-// of two taken from a cell of the list (mass 2^km, q = 2^kq), in which the
-// terms that matter stay far inside the FP32 range: a cell whose acceleration is
-// beyond 2^24 times the unit folds the sums and gives the next units, and a
-// term far below the unit is as far below the cell that gave it.
-struct QuadSum {
-    F3s s[4];
-    int km, kq;  // km + 2 kq: the unit of the acceleration
-    __device__ __forceinline__ void zero()
-    {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) s[c].zero();
-        km = kq = kOff;
-    }
-    static constexpr int kOff = -4096;
-    // adds the sums to p in the caller's units, and clears them
-    __device__ __forceinline__ void fold(double p[4])
-    {
-        if (km == kOff) return;
-        const double sa = scalbn(1.0, km + 2 * kq), sp = scalbn(1.0, km + kq);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            p[c] = fma(s[c].value(), c < 3 ? sa : -sp, p[c]);
-            s[c].zero();
-        }
-    }
-};
-
-// A quadrupole cell (pair_quad2's law) with the monopole part in FP64 and the
-// quadrupole part, a few percent of it, in two-float arithmetic (relative error
-// 2^-47, so 2^-50 or less of the pair): with u = r q, n = Q u and w = u.n - B_2 eps^2 q^2,
-//   phi -= m q + (1/2) w q^3,  a += m q^3 r + q^4 ((5/2) w u - n).
-// 18 FP64 operations and about 340 FP32 and integer ones, which the FP64 pipe's
-// time (80 FP32 operations each) hides; all in FP64 it is 38.
-__device__ __forceinline__ void pair_quad_mixed(const V4<double>& s, const float4 qa, const float4 qb, double xi,
-                                                double yi, double zi, double eps2, double p[4], QuadSum& Q)
-{
-    const double rx = s.x - xi, ry = s.y - yi, rz = s.z - zi;
-    const double r2 = fma(rx, rx, fma(ry, ry, fma(rz, rz, eps2)));
-    const double q = rsqrt(r2);
-    const double q2 = q * q;
-    const double mq = s.w * q;
-    const double mq3 = mq * q2;
-    p[3] -= mq;
-    p[0] = fma(mq3, rx, p[0]);
-    p[1] = fma(mq3, ry, p[1]);
-    p[2] = fma(mq3, rz, p[2]);
-    const int em = (__double2hiint(s.w) >> 20) & 2047, eq = (__double2hiint(q) >> 20) & 2047;
-    if (em == 0 || eq == 0) return;  // no mass, or r^2 past the FP64 range
-    if (em + 2 * eq - 3 * 1023 > Q.km + 2 * Q.kq + 24) {
-        Q.fold(p);
-        Q.km = em - 1023;
-        Q.kq = eq - 1023;
-    }
-    const F2s qs = split2(q, -Q.kq);
-    const F2s ux = norm2(mul2(split2(rx, Q.kq), qs)), uy = norm2(mul2(split2(ry, Q.kq), qs));
-    const F2s uz = norm2(mul2(split2(rz, Q.kq), qs));
-    const F2s et = split2(eps2 * q2, 0);  // (eps q)^2 <= 1
-    // Q and B_2 in units of 2^(km - 2 kq), the power applied in two exact halves
-    const int kk = 2 * Q.kq - Q.km, k1 = max(-126, min(126, kk / 2)), k2 = max(-126, min(126, kk - k1));
-    const float f1 = __int_as_float((127 + k1) << 23), f2_ = __int_as_float((127 + k2) << 23);
-    const float xx = qa.x * f1 * f2_, yy = qa.y * f1 * f2_, zz = qa.z * f1 * f2_, xy = qa.w * f1 * f2_;
-    const float xz = qb.x * f1 * f2_, yz = qb.y * f1 * f2_, bb = qb.z * f1 * f2_;
-    const F2s n0 = norm2(add2(add2(mul2(xx, ux), mul2(xy, uy)), mul2(xz, uz)));
-    const F2s n1 = norm2(add2(add2(mul2(xy, ux), mul2(yy, uy)), mul2(yz, uz)));
-    const F2s n2 = norm2(add2(add2(mul2(xz, ux), mul2(yz, uy)), mul2(zz, uz)));
-    const F2s w = norm2(add2(add2(mul2(ux, n0), mul2(uy, n1)), add2(mul2(uz, n2), mul2(-bb, et))));
-    F2s qq = mul2(qs, qs);
-    qq.l = __fmaf_rn(qs.l, qs.l, qq.l);
-    qq = norm2(qq);
-    const F2s q3 = norm2(mul2(qq, qs)), q4 = norm2(mul2(qq, qq));
-    const F2s hw = {0.5f * w.h, 0.5f * w.l}, cw = mul2(2.5f, w);
-    Q.s[3].add(mul2(hw, q3));
-    const F2s m0 = {-n0.h, -n0.l}, m1 = {-n1.h, -n1.l}, m2 = {-n2.h, -n2.l};
-    Q.s[0].add(mul2(norm2(add2(mul2(cw, ux), m0)), q4));
-    Q.s[1].add(mul2(norm2(add2(mul2(cw, uy), m1)), q4));
-    Q.s[2].add(mul2(norm2(add2(mul2(cw, uz), m2)), q4));
-}
