@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(B) k_force_f64(const otoo_dev_system sys, doub
     __shared__ V4<double> s_src[B];
     __shared__ QuadFix s_quad[B];
     __shared__ int s_idx[B];  // particle entries: their source index
-    __shared__ double s_red[B * 4];
+    __shared__ double s_red[B * 4], s_err[B * 4];
     __shared__ int s_ticket;
 
     const int tid = threadIdx.x;
@@ -314,21 +314,29 @@ __global__ void __launch_bounds__(B) k_force_f64(const otoo_dev_system sys, doub
             if (active) {
                 qsum.fold(acc.s);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) s_red[(js * P + islot) * 4 + c] = acc.value(c);
+                for (int c = 0; c < 4; ++c) {
+                    s_red[(js * P + islot) * 4 + c] = acc.value(c);
+                    s_err[(js * P + islot) * 4 + c] = 0.0;
+                }
+            }
+            // the subsets' sums pairwise, each addition's error carried along, a component
+            // of a target per thread (one after another by the targets' threads alone, these
+            // dependent FP64 operations held the other warps up by 15% on short lists, and
+            // took 40 us for one target's 256 subsets)
+            for (int left = nsplit; left > 1;) {
+                const int keep = (left + 1) / 2;
+                __syncthreads();
+                for (int r = tid; r < 4 * P * (left - keep); r += B) {
+                    const double x = s_red[r], v = s_red[4 * P * keep + r];
+                    const double u = __dadd_rn(x, v), w = __dsub_rn(u, x);
+                    s_red[r] = u;
+                    s_err[r] += s_err[4 * P * keep + r] + __dadd_rn(__dsub_rn(x, __dsub_rn(u, w)), __dsub_rn(v, w));
+                }
+                left = keep;
             }
             __syncthreads();
-            // the subsets' sums, each addition's error carried along: a component of a
-            // target per thread (by the targets' threads alone its dependent FP64
-            // operations held the other warps up by 15% on short lists)
-            for (int r = tid; r < 4 * P; r += B) {
-                double a = 0.0, e = 0.0;
-                for (int j = 0; j < nsplit; ++j) {
-                    const double v = s_red[4 * j * P + r], u = __dadd_rn(a, v), w = __dsub_rn(u, a);
-                    e += __dadd_rn(__dsub_rn(a, __dsub_rn(u, w)), __dsub_rn(v, w));
-                    a = u;
-                }
-                write_component(sys, grp, item, i0 + (r >> 2), r & 3, a + e, accel, pot);
-            }
+            for (int r = tid; r < 4 * P; r += B)
+                write_component(sys, grp, item, i0 + (r >> 2), r & 3, s_red[r] + s_err[r], accel, pot);
             __syncthreads();
         }
     }
@@ -416,8 +424,7 @@ ForceKernel pick_f32(int B, int IB, int tile, int packed)
 // taken with iblock targets a thread.  256 threads up to 14 items per SM, where the
 // longest items set the time and twice the threads share an item's entries.
 // Microseconds with 128 / 256 threads: 0.7 items per SM 314 / 278, 2.5 1135 / 685, 5.6 2451 /
-// 1206, 9 2512 / 1278, 14 2628 / 1772, 15 (short lists) 833 / 857, 27 2548 / 2690 (before
-// the subsets' sums were added component by component).
+// 1206, 9 2512 / 1278, 14 2628 / 1772, 15 (short lists) 833 / 857, 27 2548 / 2690.
 constexpr int64_t kWideItems = 14;
 template <int B>
 Kernel pick_f64(int IB)
