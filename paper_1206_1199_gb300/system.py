@@ -523,7 +523,7 @@ class FusedStep:
         w.src, w.cell, w.cell64 = tb["src"].data_ptr(), tb["cell"].data_ptr(), tb["cell64"].data_ptr()
         w.group_first, w.group_count = tb["first"].data_ptr(), tb["count"].data_ptr()
         w.theta_per_group = b["tpg"].data_ptr() if "tpg" in b else None
-        w.counter, w.totals = b["counter"].data_ptr(), b["totals"].data_ptr()
+        w.counter, w.totals = head.data_ptr() + 32, head.data_ptr() + 48
         self.struct = w
         self.bufs = b
 
@@ -542,6 +542,22 @@ class FusedStep:
         """(list entries, interactions, cell interactions) of the last step."""
         t = [int(x) for x in self.bufs["totals"][:3].tolist()]
         return tuple(t)
+
+
+class _WalkBufs(dict):
+    """A walk's buffers; the views of its head (the walk's counter words and
+    totals) are made when asked for (each costs as much as an allocation)."""
+
+    def __missing__(self, key):
+        import torch
+        if key == "counter":
+            v = self["head"][4:6].view(torch.int32)
+        elif key == "totals":
+            v = self["head"][6:]
+        else:
+            raise KeyError(key)
+        self[key] = v
+        return v
 
 
 class DeviceLists:
@@ -565,8 +581,7 @@ class DeviceLists:
         # the plan's totals [4], the walk's counter words [2] and its totals: what
         # the host reads, side by side so that one copy brings it
         head = alloc("whead", 6 + L.load().otoo_walk_totals_len(G), torch.int64)
-        b = dict(groups=alloc("groups", G * 64, torch.uint8), head=head, counter=head[4:6].view(torch.int32),
-                 totals=head[6:])
+        b = _WalkBufs(groups=alloc("groups", G * 64, torch.uint8), head=head)
         if theta_per_group is not None:
             tpg = np.ascontiguousarray(theta_per_group, dtype=np.float32)
             assert tpg.shape == (G,)
@@ -581,7 +596,7 @@ class DeviceLists:
         w.src, w.cell, w.cell64 = tb["src"].data_ptr(), tb["cell"].data_ptr(), tb["cell64"].data_ptr()
         w.group_first, w.group_count = tb["first"].data_ptr(), tb["count"].data_ptr()
         w.theta_per_group = b["tpg"].data_ptr() if "tpg" in b else None
-        w.counter, w.totals = b["counter"].data_ptr(), b["totals"].data_ptr()
+        w.counter, w.totals = head.data_ptr() + 32, head.data_ptr() + 48
         self.struct = w
         self.bufs = b
         st = _stream(stream, dev)
@@ -620,9 +635,13 @@ class DeviceLists:
     def read_head(self, lo, hi, stream=None):
         """Words [lo, hi) of the head, but for the counter words, and the
         walk's status bits, in one copy on the stream that wrote them."""
-        import torch
-        with torch.cuda.stream(stream):  # (None: the current stream)
-            v = self.bufs["head"][lo:hi].tolist()
+        h = self.bufs["head"][lo:hi]
+        if stream is None:
+            v = h.tolist()
+        else:
+            import torch
+            with torch.cuda.stream(stream):
+                v = h.tolist()
         status = (v[4 - lo] >> 32) & 0xffffffff
         return v[:4 - lo] + v[6 - lo:], status
 
@@ -685,14 +704,14 @@ class DevicePlan:
         head = dl.bufs["head"]
         ptot = head.data_ptr()
         gp = dl.bufs["groups"].data_ptr()
-        counter = dl.bufs["counter"]
+        counter = dl.struct.counter
 
         def count():
             L.call("otoo_plan_count", gp, G, ctypes.byref(tune), scratch.data_ptr(), ptot, st)
 
         def fill(items, n_items, splits, n_splits):
             L.call("otoo_plan_fill", gp, G, ctypes.byref(tune), scratch.data_ptr(), ptot, items.data_ptr(), n_items,
-                   splits.data_ptr(), n_splits, counter.data_ptr(), st)
+                   splits.data_ptr(), n_splits, counter, st)
 
         count()
         # with buffers kept from an earlier step the fill needs no host read before
@@ -704,7 +723,7 @@ class DevicePlan:
         (n_items, n_splits, slots, ncm), status = dl.read_head(0, 6, stream)
         if filled and (n_items > kept[0].numel() // 32 or n_splits > kept[1].numel() // 16):
             with torch.cuda.stream(stream):
-                counter.zero_()
+                dl.bufs["counter"].zero_()
             count()
             filled = False
         self.n_items, self.n_splits, self.n_crit_max = n_items, n_splits, max(ncm, 1)
