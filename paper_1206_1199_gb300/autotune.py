@@ -1,14 +1,15 @@
 """Autotuner for the force step.
 
 Knobs: the group size n_crit (it changes the host walk, so every candidate
-re-walks the tree), packed (part of a variant's name: every variant computes
-with packed two-wide FP32), target
-particles per lane (iblock), list entries per staged tile (tile),
-list-split threshold (split) and threads per CTA (block).  Objective: device time of one FP32 force step at fixed theta, the
-minimum over repeated CUDA-event timings.  The search is coordinate descent
-per n_crit (packed, then iblock, tile, split, block) over the compiled
-kernel variants; the winner over all n_crit is cached per GPU name and
-workload in tune_cache.json next to this file.
+re-walks the tree), target particles per lane (iblock), list entries per
+staged tile (tile), list-split threshold (split) and threads per CTA (block).
+Objective: device time of one FP32 force step at fixed theta, the minimum over
+repeated CUDA-event timings.  The search is coordinate descent per n_crit
+(iblock, then tile, split, block) over the compiled kernel variants; the winner
+over all n_crit is cached per GPU name and workload in tune_cache.json next to
+this file.  packed is part of a variant's name and nothing else (every variant
+computes with packed two-wide FP32), so a kernel named by both of its values is
+timed once, under packed = 1.
 
 Command line (writes the cache; --out also writes a copy elsewhere):
     python -m paper_1206_1199_gb300.autotune --workload hernquist8m [--out path]
@@ -95,10 +96,14 @@ def search(pos, mass, w, n_crits=(32, 64, 128, 256), device="cuda", log=print):
         lists = tree.lists(w["theta"], nc, w["eps"], w["use_quad"])
         cache = {}
 
-        def run(block, ib, tile, split, packed):
-            key = (block, ib, tile, split, packed)
+        def packed_of(block, ib, tile):
+            return 1 if (block, ib, tile, 1) in VARIANTS else 0
+
+        def run(block, ib, tile, split):
+            key = (block, ib, tile, split)
             if key in cache:
                 return cache[key]
+            packed = packed_of(block, ib, tile)
             if (block, ib, tile, packed) not in VARIANTS:
                 cache[key] = float("inf")
                 return cache[key]
@@ -114,8 +119,8 @@ def search(pos, mass, w, n_crits=(32, 64, 128, 256), device="cuda", log=print):
             log(json.dumps(row))
             return ms
 
-        cur = [128, 2, 128, 4096, 1]
-        for pos_k, cands in ((4, (0, 1)), (1, (1, 2, 4)), (2, (64, 128, 256)), (3, (2048, 4096, 8192, 16384)),
+        cur = [128, 2, 128, 4096]
+        for pos_k, cands in ((1, (1, 2, 4)), (2, (64, 128, 256)), (3, (2048, 4096, 8192, 16384)),
                              (0, (64, 128, 256))):
             res = []
             for v in cands:
@@ -126,7 +131,7 @@ def search(pos, mass, w, n_crits=(32, 64, 128, 256), device="cuda", log=print):
         ms = run(*cur)
         if best is None or ms < best["ms"]:
             best = dict(n_crit=nc, tune=dict(block=cur[0], iblock=cur[1], tile=cur[2], split=cur[3], ctas_per_sm=0,
-                                             packed=cur[4]),
+                                             packed=packed_of(*cur[:3])),
                         ms=ms, interactions=lists.interactions)
     return best, table
 
