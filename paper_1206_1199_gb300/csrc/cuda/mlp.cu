@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(kChooseBlock) k_theta_choose(const ThetaArgs a
         }
         // the group's threads stop together, after the round with its first passing angle
         const unsigned m = __ballot_sync(0xffffffffu, pass) >> (threadIdx.x & 31 & ~(S - 1));
-        done = done || (safe && (m & (S < 32 ? (1u << S) - 1u : 0xffffffffu)) != 0u);
+        done = done || (safe && (m & ((1u << S) - 1u)) != 0u);
     }
 #pragma unroll
     for (int o = S / 2; o > 0; o >>= 1) {
@@ -826,7 +826,10 @@ int otoo_learned_theta(const otoo_theta_net* net, const otoo_theta_rule* rule, c
     CUDA_TRY(cudaGetLastError());
     // threads per group: as many as keep the launch within the threads that are
     // resident at once (about 500 per SM), where more would only wait
-    const int64_t resident = 152 * 500;
+    int dev = 0, sms = 0;
+    CUDA_TRY(cudaGetDevice(&dev));
+    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int64_t resident = (int64_t)sms * 500;
     if (8 * n_groups <= resident)
         k_theta_choose<8><<<(unsigned)((n_groups + kChooseBlock / 8 - 1) / (kChooseBlock / 8)), kChooseBlock, 0, s>>>(
             a, wg, lambda, grid, n_theta, rule->fallback, log10_target, theta_out);
