@@ -13,8 +13,8 @@
 // as fast for unchanged arguments, but a time loop's counts change from step to
 // step, and recording it anew took 50 us at N = 4096):
 //   k_split       FP32 form only: each source position as a float pair
-//                 (hi, lo), once per step -- the FP64 work of the step; clears
-//                 the work ticket and the status word.
+//                 (hi, lo), once per step; clears the work ticket and the status
+//                 word.
 //   k_force_warp2 FP32 form: one work item per warp (small launches: per CTA);
 //                 packed two-wide FP32 pairs on group-centre-relative coordinates, plain FP32
 //                 sums between Kahan-compensated flushes, FP64 merge of the

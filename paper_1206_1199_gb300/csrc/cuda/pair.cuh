@@ -8,7 +8,6 @@
 #pragma once
 
 template <typename R> struct V4;
-template <> struct __align__(16) V4<float> { float x, y, z, w; };
 template <> struct __align__(32) V4<double> { double x, y, z, w; };
 
 // FP32 reciprocal square root: the hardware approximation (PTX
