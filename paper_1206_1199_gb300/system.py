@@ -523,7 +523,7 @@ class FusedStep:
         w.src, w.cell, w.cell64 = tb["src"].data_ptr(), tb["cell"].data_ptr(), tb["cell64"].data_ptr()
         w.group_first, w.group_count = tb["first"].data_ptr(), tb["count"].data_ptr()
         w.theta_per_group = b["tpg"].data_ptr() if "tpg" in b else None
-        w.counter, w.totals = head.data_ptr() + 32, head.data_ptr() + 48
+        w.counter, w.totals = b["counter"].data_ptr(), b["totals"].data_ptr()
         self.struct = w
         self.bufs = b
 
