@@ -110,7 +110,7 @@ constexpr int kSt = NH + 4;  // floats per row of a unit array (16-byte aligned 
 
 struct BackShared {
     float h1[kRowsPerCta][kSt], h2[kRowsPerCta][kSt], d1[kRowsPerCta][kSt], d2[kRowsPerCta][kSt];
-    float x[kRowsPerCta][8];  // the row's inputs, 1, 0 (zeros past the last row)
+    float x[kRowsPerCta][8];  // the row's inputs, 1 (past the last row 0), 0
     float dy[kRowsPerCta];
     float w2t[NH][NH];        // second layer's weights, transposed
     float w[NP + 3];
@@ -142,9 +142,10 @@ __global__ void __launch_bounds__(kBackThreads) k_mlp_backward(const uint16_t* _
     const int64_t r = r0 + row;
     const bool on = r < n;
     const float inv_n = 1.0f / (float)n;
+    const float* __restrict__ xp = on ? x + r * NI : x;
     float xr[NI], target = 0.f;
 #pragma unroll
-    for (int k = 0; k < NI; ++k) xr[k] = on ? x[r * NI + k] : 0.f;
+    for (int k = 0; k < NI; ++k) xr[k] = xp[k];
     if (on) target = tgt[r];
     for (int k = tid; k < NP; k += kBackThreads) {
         const float w = bf16_to_f(wbf16[k]);
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(kBackThreads) k_mlp_backward(const uint16_t* _
         float z = sh.w[OB1 + i];
 #pragma unroll
         for (int k = 0; k < NI; ++k) z = fmaf(sh.w[OW1 + i * NI + k], xr[k], z);
-        h1[u] = on ? tanhf(z) : 0.f;  // (an infinite weight against the zeros of a row past the last is NaN)
+        h1[u] = tanhf(z);
     }
 #pragma unroll
     for (int u = 0; u < kU; u += 4)
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(kBackThreads) k_mlp_backward(const uint16_t* _
             z[4] = fmaf(wb.x, h, z[4]), z[5] = fmaf(wb.y, h, z[5]), z[6] = fmaf(wb.z, h, z[6]), z[7] = fmaf(wb.w, h, z[7]);
         }
 #pragma unroll
-        for (int u = 0; u < kU; ++u) h2[u] = on ? tanhf(z[u]) : 0.f;
+        for (int u = 0; u < kU; ++u) h2[u] = tanhf(z[u]);
 #pragma unroll
         for (int u = 0; u < kU; u += 4)
             *reinterpret_cast<float4*>(&sh.h2[row][u0 + u]) = make_float4(h2[u], h2[u + 1], h2[u + 2], h2[u + 3]);
@@ -197,11 +198,12 @@ __global__ void __launch_bounds__(kBackThreads) k_mlp_backward(const uint16_t* _
             yv = fmaf(sh.w[OW3 + j], h.x, yv), yv = fmaf(sh.w[OW3 + j + 1], h.y, yv);
             yv = fmaf(sh.w[OW3 + j + 2], h.z, yv), yv = fmaf(sh.w[OW3 + j + 3], h.w, yv);
         }
-        // rows past the last: no residual; their hidden values and deltas are zero
+        // places past the last row repeat the first without a residual: every delta is zero
+        // (with zero inputs an infinite weight would make their hidden values NaN)
         const float dy = on ? 2.0f * (yv - target) * inv_n : 0.f;
         float d[kU];
 #pragma unroll
-        for (int u = 0; u < kU; ++u) d[u] = on ? dy * sh.w[OW3 + u0 + u] * (1.0f - h2[u] * h2[u]) : 0.f;
+        for (int u = 0; u < kU; ++u) d[u] = dy * sh.w[OW3 + u0 + u] * (1.0f - h2[u] * h2[u]);
 #pragma unroll
         for (int u = 0; u < kU; u += 4)
             *reinterpret_cast<float4*>(&sh.d2[row][u0 + u]) = make_float4(d[u], d[u + 1], d[u + 2], d[u + 3]);
@@ -220,7 +222,7 @@ __global__ void __launch_bounds__(kBackThreads) k_mlp_backward(const uint16_t* _
             sd[4] = fmaf(wb.x, d, sd[4]), sd[5] = fmaf(wb.y, d, sd[5]), sd[6] = fmaf(wb.z, d, sd[6]), sd[7] = fmaf(wb.w, d, sd[7]);
         }
 #pragma unroll
-        for (int u = 0; u < kU; ++u) sd[u] = on ? sd[u] * (1.0f - h1[u] * h1[u]) : 0.f;
+        for (int u = 0; u < kU; ++u) sd[u] *= 1.0f - h1[u] * h1[u];
 #pragma unroll
         for (int u = 0; u < kU; u += 4)
             *reinterpret_cast<float4*>(&sh.d1[row][u0 + u]) = make_float4(sd[u], sd[u + 1], sd[u + 2], sd[u + 3]);
