@@ -383,7 +383,7 @@ int otoo_force_static_status(void* stream);
 /* Size in bytes of the array otoo_force_static uses. */
 int64_t otoo_force_static_capacity(void);
 
-/* FP64 direct sum (Section II: the O(N^2) sum a tree code approximates),
+/* Direct sum to FP64's accuracy (Section II: the O(N^2) sum a tree code approximates),
    used as the exact reference of the learned opening angle's training
    errors:  for each target t, i = targets[t] (an index into src),
      accel[t] = sum_{j != i} m_j r / (r^2 + eps2)^(3/2),

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(256) k_direct_range(const otoo_src* __restrict
 // half's sums join the first's at the end.  The float sums are moved into FP64
 // every kTfFold tiles.  Bound by the FP32 pipe: about 260 packed operations per
 // source and two targets.
-// N = 2^19, 5003 targets: 32.6 ms (8.0e10 pairs/s) against 110 ms for the FP64
+// N = 2^19, 5003 targets: 32.9 ms (8.0e10 pairs/s) against 110 ms for the FP64
 // form.  Relative error (2-norm over 40 targets, against extended precision) over
 // N = 66000 and 130000, four models, softenings 1e-4 and 1e-2, and 40, 600 and 5000
 // targets, two-float / FP64 form: accelerations 0.6e-16 to 1.2e-16 / 2.5e-16 to
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kTgt) k_direct_part(const otoo_src* __restrict
         for (int k = 0; k < cnt; ++k) {
             const double4 q = s[k];
             const double rx = q.x - xi, ry = q.y - yi, rz = q.z - zi;
-            // (18 FP64 operations per pair, rsqrt 5 of them: 1.6 per clock and SM bound this kernel)
+            // (18 FP64 operations per pair, rsqrt 5 of them: 1.7 per clock and SM bound this kernel)
             const double r2 = fma(rx, rx, fma(ry, ry, fma(rz, rz, eps2)));
             const double inv = rsqrt(r2);
             const double mi = (k == kself ? 0.0 : q.w) * inv;

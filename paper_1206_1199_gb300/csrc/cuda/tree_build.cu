@@ -683,7 +683,7 @@ __device__ __forceinline__ double widen(float f)
 // loses about log2((M - m_0) / m_0) bits: under 3 for a parent (the heaviest
 // of up to 8 children), about log2 of the leaf size for equal masses in a
 // leaf.  Stored: m, com, C (Cxx Cyy Czz Cxy Cxz Cyz) and B_2 = tr C; the
-// records take the quadrupole Q = 3 C - tr(C) I.  GB300's FP64 pipe (1/80 of
+// records take the quadrupole Q = 3 C - tr(C) I.  GB300's FP64 pipe (1/76 of
 // the FP32 rate) bounds both kernels at large N, latency at small N.
 
 // The end of a cell, and the moments of a leaf (nch = 0) of one particle; returns

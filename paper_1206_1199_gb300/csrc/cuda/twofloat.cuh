@@ -1,8 +1,8 @@
 // Pairs in two-float arithmetic: the FP64 forms' pair law on the FP32 pipe.
 //
-// GB300 runs FP64 at 1/80 of its FP32 rate (1.6 against 128 operations per
-// clock and SM; conversions to and from FP64 at the same 1.6, measured), so an
-// FP64 pair of 19 operations costs as much pipe time as 1500 FP32 operations.
+// GB300 runs FP64 at 1/76 of its FP32 rate (1.7 against 128 operations per
+// clock and SM; conversions to and from FP64 at the same rate, measured), so an
+// FP64 pair of 19 operations costs as much pipe time as 1450 FP32 operations.
 // Here a value is an unevaluated sum of two floats (48 bits; Dekker 1971, Knuth
 // TAOCP 2 4.2.2: error-free sums and products) and two targets share every packed
 // two-wide instruction.  Differences of coordinates and r^2 + eps^2 are exact to

@@ -1,5 +1,5 @@
 // FP64 to FP32 and back by integer operations on the device.  GB300 converts at
-// its FP64 rate, 1.6 per clock and SM: one conversion takes the time of about
+// its FP64 rate, 1.7 per clock and SM: one conversion takes the time of about
 // fifty integer operations (128 per clock and SM for two instructions of three),
 // and the kernels that turn coordinates into float pairs are bound by it.  The
 // results are those of the conversions, bit for bit; values outside FP32's

@@ -1,8 +1,8 @@
 // The quadrupole part of a cell pair in 62-bit fixed point, for the FP64 form of
 // the force.
 //
-// GB300 runs FP64 at 1/80 of its FP32 rate, so the 20 FP64 operations of the
-// quadrupole part would take as long as 1600 of other kinds.  All its factors are
+// GB300 runs FP64 at 1/76 of its FP32 rate, so the 20 FP64 operations of the
+// quadrupole part would take as long as 1500 of other kinds.  All its factors are
 // bounded: with q = (r^2 + eps^2)^(-1/2), u = r q has length below 1, and a cell's
 // Q and B_2 divided by a power of two are below 1/2.  So the part is evaluated in
 // integers of 2^-60 (two limbs of 31 bits, products of limbs in 64 bits), about

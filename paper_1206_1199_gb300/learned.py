@@ -93,7 +93,7 @@ class Evaluator:
         return acc.cpu().numpy(), pot.cpu().numpy(), ms
 
     def direct(self, targets, on_device=False):
-        """FP64 direct sum on the device for tree-order targets (device
+        """Direct sum to FP64's accuracy on the device for tree-order targets (device
         tensors when on_device, else host arrays)."""
         torch = _torch()
         if self._src_dev is None:

@@ -280,7 +280,7 @@ def _particle_sources(pos, mass, device):
 
 
 def direct_sum(pos, mass, eps, targets, device="cuda"):
-    """FP64 direct sum on the device (otoo_direct) for the given particle
+    """Direct sum to FP64's accuracy on the device (otoo_direct) for the given particle
     indices (caller order): returns (acc [k][3], pot [k]) as numpy."""
     import torch
     src = _particle_sources(pos, mass, device)
