@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(256) k_direct_range(const otoo_src* __restrict
 // half's sums join the first's at the end.  The float sums are moved into FP64
 // every kTfFold tiles.  Bound by the FP32 pipe: about 260 packed operations per
 // source and two targets.
-// N = 2^19, 5003 targets: 32.9 ms (8.0e10 pairs/s) against 110 ms for the FP64
+// N = 2^19, 5003 targets: 24.0 ms (1.09e11 pairs/s) against 110 ms for the FP64
 // form.  Relative error (2-norm over 40 targets, against extended precision) over
 // N = 66000 and 130000, four models, softenings 1e-4 and 1e-2, and 40, 600 and 5000
 // targets, two-float / FP64 form: accelerations 0.6e-16 to 1.2e-16 / 2.5e-16 to
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(256) k_direct_range(const otoo_src* __restrict
 // to 1e7 core radii out 0.8e-16 to 2.1e-16 / 2.5e-16 to 6.7e-16; with a fifth of the
 // system in close groups of 2 to 1000, 1.5e-16 to 8.0e-16 / 7.8e-16 to 3.0e-15.
 // (Before, with coordinates on one grid of 2^-62 of the extent, r^2 summed in plain
-// floats and one pair of a run again in FP64: 25.1 ms; 2.9e-16 to 1.3e-15, 4e-16 to
+// floats and one pair of a run again in FP64, 25.1 ms in a wave and a twentieth: 2.9e-16 to 1.3e-15, 4e-16 to
 // 7e-13 and 3e-16 to 2e-13, larger than the FP64 form's in most of them.)
 // Below 65536 sources the FP64 form stays: the line is not a matter of accuracy.
 constexpr int64_t kTfMinSources = 65536;
@@ -427,6 +427,30 @@ __global__ void __launch_bounds__(128) k_direct_tree(const double* __restrict__ 
     if (lane == 3) pot[t] = a[3];
 }
 
+// Sources per chunk of the two-float form: as many chunks (nc at most) as fill one to
+// four waves of its blocks (256 targets each, two resident per SM), or the FP64
+// form's number, whichever takes the least time.  A wave takes its chunk's sources
+// and about 128 more for a block's start and the pairs evaluated again, one of a few
+// blocks half of that (140 blocks took as long as 304: they are not spread over the
+// SMs one by one).  N = 2^19, 5003 targets: 24.0 ms in one wave of 300 blocks, 32.9 ms
+// with the 320 that the FP64 form's rule gives.
+int64_t direct_tf_chunk(int64_t n_src, int64_t n_tgt, int64_t nc, int nsm)
+{
+    const int64_t tb = (n_tgt + 255) / 256, resident = 2 * (int64_t)nsm;
+    int64_t best = 0;
+    double cost = 1e300;
+    for (int w = 0; w <= 4; ++w) {
+        const int64_t c = w == 0 ? nc : w * resident / tb;
+        if (c < 1 || c > nc) continue;
+        const int64_t chunk = ((n_src + c - 1) / c + kTile - 1) / kTile * kTile;
+        const int64_t blocks = tb * ((n_src + chunk - 1) / chunk), rest = blocks % resident;
+        const double waves = (double)(blocks / resident) + (rest == 0 ? 0.0 : rest > resident / 8 ? 1.0 : 0.5);
+        const double t = waves * (double)(chunk + 128);
+        if (t < cost) cost = t, best = chunk;
+    }
+    return best;
+}
+
 #define CUDA_TRY(expr)                                                                                 \
     do {                                                                                               \
         cudaError_t e_ = (expr);                                                                       \
@@ -456,7 +480,13 @@ int otoo_direct(const otoo_src* src, int64_t n_src, const int64_t* targets, int6
     OTOO_REQUIRE(n_src >= 1 && n_tgt >= 1 && n_tgt <= ((int64_t)1 << 31), OTOO_EINVAL, "otoo_direct: bad sizes");
     OTOO_REQUIRE(eps2 > 0.0, OTOO_EINVAL, "otoo_direct: eps2 must be > 0");
     const int64_t nc = otoo_direct_chunks(n_src, n_tgt);
-    const int64_t chunk = ((n_src + nc - 1) / nc + kTile - 1) / kTile * kTile;
+    int64_t chunk = ((n_src + nc - 1) / nc + kTile - 1) / kTile * kTile;
+    if (n_src >= kTfMinSources) {
+        int dev = 0, nsm = 0;
+        CUDA_TRY(cudaGetDevice(&dev));
+        CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+        chunk = direct_tf_chunk(n_src, n_tgt, nc, nsm);
+    }
     const int64_t nch = (n_src + chunk - 1) / chunk;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(uint32_t), s));
